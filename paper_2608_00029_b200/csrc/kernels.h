@@ -103,8 +103,18 @@ cudaError_t launch_lmhead(const CUtensorMap& tmX, const CUtensorMap& tmW, const 
                           void* workspace, int num_sms, int* dev_status, cudaStream_t stream);
 cudaError_t configure_lmhead();
 size_t lmhead_workspace_bytes(int M, int N);
+float* lmhead_target_logits(void* workspace, int M, int N);  // the part of the workspace behind the partial pairs
 // Rows of the X and W boxes; returns the box width in k elements.
 int lmhead_boxes(int* box_rows_x, int* box_rows_w);
+
+// The same for at most kLmHeadFewRows rows (lmhead_rows.cu).  lmhead_rows_plan chooses the number of CTAs, the height
+// of a W tile (rows of the box of `tmW`) and the rows of the box of `tmX`; both boxes are 64 k elements wide.
+constexpr int kLmHeadFewRows = 64;
+cudaError_t configure_lmhead_rows();
+void lmhead_rows_plan(int M, int N, int num_sms, int* ctas, int* tile_h, int* m_pad);
+cudaError_t launch_lmhead_rows(const CUtensorMap& tmX, const CUtensorMap& tmW, const int* targets, void* logits,
+                               float* lse, float* loss, int M, int N, int K, int ctas, int tile_h, int m_pad,
+                               void* workspace, float* tgt_logit, int* dev_status, cudaStream_t stream);
 
 // Clears `bytes` (a multiple of 16) at the 16-byte aligned `ptr`.
 cudaError_t launch_zero(void* ptr, size_t bytes, int num_sms, cudaStream_t stream);

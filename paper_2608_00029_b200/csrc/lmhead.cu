@@ -57,18 +57,6 @@ struct Tiles {
     }
 };
 
-__device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(smem_u32(smem_dst)), "l"(m), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
-                 : "memory");
-}
-
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, const void* smem_src, int c0, int c1) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(m),
-                 "r"(smem_u32(smem_src)), "r"(c0), "r"(c1)
-                 : "memory");
-}
-
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
               const __grid_constant__ CUtensorMap tmL, const int* __restrict__ targets, int store_logits,
@@ -681,6 +669,11 @@ size_t lmhead_workspace_bytes(int M, int N) {
     return (bytes + 255) & ~size_t(255);
 }
 
+float* lmhead_target_logits(void* workspace, int M, int N) {
+    const size_t n_part = (static_cast<size_t>(N) + kPart - 1) / kPart;
+    return reinterpret_cast<float*>(static_cast<float2*>(workspace) + n_part * M);
+}
+
 cudaError_t configure_lmhead() {
     cudaError_t e = cudaFuncSetAttribute(lmhead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
@@ -692,7 +685,7 @@ cudaError_t launch_lmhead(const CUtensorMap& tmX, const CUtensorMap& tmW, const 
                           void* workspace, int num_sms, int* dev_status, cudaStream_t stream) {
     const int n_part = (N + kPart - 1) / kPart;
     float2* partials = static_cast<float2*>(workspace);
-    float* tgt_logit = reinterpret_cast<float*>(partials + static_cast<size_t>(n_part) * M);
+    float* tgt_logit = lmhead_target_logits(workspace, M, N);
     const int m_tiles = (M + kBM - 1) / kBM;
     const long long n_tiles = static_cast<long long>(m_tiles) * ((N + kBN - 1) / kBN);
     cudaError_t e;

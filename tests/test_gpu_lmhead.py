@@ -68,6 +68,21 @@ def test_edge_shapes(M, N, K):
     _check(cfg, *W.make_lmhead_inputs(cfg))
 
 
+# At most 64 rows: the kernel that streams W past swapped operands.  Group edges of the rows (16, 32), equal tile
+# heights below 128 (18952 = 148 * 128 + 8 entries: two rounds), a lone entry beyond a tile, a ragged k block, and
+# the first row count that goes to the other kernel.
+FEW_ROWS = [(1, 136, 8), (16, 18952, 64), (17, 2056, 72), (32, 50304, 128), (33, 1000, 200), (64, 18944, 64), (65, 264, 64)]
+
+
+@pytest.mark.parametrize("M,N,K", FEW_ROWS)
+def test_few_rows(M, N, K):
+    cfg = W.LmHeadConfig("few", M=M, N=N, K=K, seed=7 + M + N + K, w_factor=0.3, ignored_every=5)
+    X, Wm, t = W.make_lmhead_inputs(cfg)
+    t[-1] = N - 1  # the last entry of the vocabulary as a target
+    _check(cfg, X, Wm, t)
+    _check(cfg, X, Wm, t, want_logits=False)
+
+
 def test_without_logits_and_run_to_run_determinism():
     cfg = W.LmHeadConfig("nolog", M=384, N=3000 // 8 * 8, K=256, seed=5, w_factor=0.1)
     X, Wm, t = W.make_lmhead_inputs(cfg)
