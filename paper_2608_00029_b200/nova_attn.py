@@ -1,4 +1,6 @@
-"""ctypes binding of libnova_attn.so: same names as the C ABI, argument marshalling only.
+"""Binding of libnova_attn.so: same names as the C ABI, argument checks and marshalling only.  The calls of a
+training or inference loop go through the native module `_binding` (csrc/binding.cpp), which checks the tensors
+and calls the C ABI; what is called once in a while goes through ctypes.
 
 Every step of the attention path runs inside the CUDA library; PyTorch is used here for device
 memory and streams.  There is no CPU fallback: if the shared library is missing or a call fails, an
@@ -14,6 +16,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libnova_attn.so")
 _lib = None
+_native = None
 
 OK = 0
 ERR_NULL, ERR_SHAPE, ERR_UNSUPPORTED, ERR_ALIGNMENT, ERR_SCALE, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(-1, -9, -1)
@@ -83,36 +86,20 @@ def load():
     return lib
 
 
+def _binding():
+    """The native module of the calls that loops make (once)."""
+    global _native
+    if _native is None:
+        load()  # raises if the library has not been built
+        from . import _binding as native
+        _native = native
+    return _native
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
-
-
-def _ptr(t) -> int:
-    return 0 if t is None else int(t.data_ptr())
-
-
-def _check_bf16(name, t, shape=None):
-    if t.dtype != torch.bfloat16 or not t.is_cuda or not t.is_contiguous():
-        raise TypeError(f"{name} must be a contiguous CUDA bf16 tensor")
-    if shape is not None and tuple(t.shape) != tuple(shape):
-        raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
-
-
-def _view_strides(name, t, shape=None) -> Strides:
-    """Strides of a [B,H,T,D]-shaped bf16 CUDA view whose last dimension is contiguous (the view may be a
-    slice / permutation of a larger buffer, e.g. of a fused projection output)."""
-    if t.dtype != torch.bfloat16 or not t.is_cuda or t.dim() != 4 or t.stride(3) != 1:
-        raise TypeError(f"{name} must be a 4-D CUDA bf16 view [B,H,T,D] with a contiguous last dimension")
-    if shape is not None and tuple(t.shape) != tuple(shape):
-        raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
-    return Strides(t.stride(0), t.stride(1), t.stride(2))
-
-
-def _check_f32(name, t, shape):
-    if t.dtype != torch.float32 or not t.is_cuda or not t.is_contiguous() or tuple(t.shape) != tuple(shape):
-        raise TypeError(f"{name} must be a contiguous CUDA fp32 tensor of shape {tuple(shape)}")
 
 
 def nova_attn_status_string(status: int) -> str:
@@ -125,38 +112,21 @@ def nova_attn_bwd_workspace_bytes(B: int, H: int, T: int, D: int) -> int:
 
 def nova_attn_fwd(Q, K, V, O, LSE, scale: float, causal: bool = True, stream=None) -> None:
     """O, LSE <- attention(Q, K, V); tensors are [B,H,T,D] bf16, LSE [B,H,T] fp32, all preallocated."""
-    _check_bf16("Q", Q)
-    B, H, T, D = Q.shape
-    for n, t in (("K", K), ("V", V), ("O", O)):
-        _check_bf16(n, t, Q.shape)
-    _check_f32("LSE", LSE, (B, H, T))
-    rc = load().nova_attn_fwd(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(LSE), B, H, T, D, float(scale),
-                              int(bool(causal)), _stream_ptr(stream))
+    rc = _binding().attn_fwd(Q, K, V, O, LSE, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_fwd")
 
 
 def nova_attn_bwd_preprocess(O, dO, Delta, stream=None) -> None:
     """Delta <- rowsum(dO * O)."""
-    _check_bf16("O", O)
-    _check_bf16("dO", dO, O.shape)
-    B, H, T, D = O.shape
-    _check_f32("Delta", Delta, (B, H, T))
-    rc = load().nova_attn_bwd_preprocess(_ptr(O), _ptr(dO), _ptr(Delta), B, H, T, D, _stream_ptr(stream))
+    rc = _binding().preprocess(O, dO, Delta, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_preprocess")
 
 
 def nova_attn_bwd_preprocess_exact(Q, K, V, dO, LSE, Delta, scale: float, causal: bool = True, stream=None) -> None:
     """Delta <- sum_j P_ij (dO_i . V_j) with P rebuilt from LSE: independent of the rounding of O."""
-    _check_bf16("Q", Q)
-    B, H, T, D = Q.shape
-    for n, t in (("K", K), ("V", V), ("dO", dO)):
-        _check_bf16(n, t, Q.shape)
-    _check_f32("LSE", LSE, (B, H, T))
-    _check_f32("Delta", Delta, (B, H, T))
-    rc = load().nova_attn_bwd_preprocess_exact(_ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(LSE), _ptr(Delta), B, H, T,
-                                               D, float(scale), int(bool(causal)), _stream_ptr(stream))
+    rc = _binding().preprocess_exact(Q, K, V, dO, LSE, Delta, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_preprocess_exact")
 
@@ -170,21 +140,7 @@ def nova_attn_bwd(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: 
     """dQ, dK, dV <- gradients of sum(O*dO); `workspace` is a CUDA byte/float tensor of at least
     nova_attn_bwd_workspace_bytes(B,H,T,D) bytes (allocated here if omitted).  `steps` other than
     BWD_STEP_ALL goes through nova_attn_bwd_steps (a timing aid)."""
-    _check_bf16("Q", Q)
-    B, H, T, D = Q.shape
-    for n, t in (("K", K), ("V", V), ("O", O), ("dO", dO), ("dQ", dQ), ("dK", dK), ("dV", dV)):
-        _check_bf16(n, t, Q.shape)
-    _check_f32("LSE", LSE, (B, H, T))
-    _check_f32("Delta", Delta, (B, H, T))
-    if workspace is None:
-        workspace = torch.empty(nova_attn_bwd_workspace_bytes(B, H, T, D), dtype=torch.uint8, device=Q.device)
-    ws_bytes = workspace.numel() * workspace.element_size()
-    args = (_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(LSE), _ptr(Delta), _ptr(dQ), _ptr(dK), _ptr(dV),
-            B, H, T, D, float(scale), int(bool(causal)), _ptr(workspace), ws_bytes, _stream_ptr(stream))
-    if steps == BWD_STEP_ALL:
-        rc = load().nova_attn_bwd(*args)
-    else:
-        rc = load().nova_attn_bwd_steps(*args, int(steps))
+    rc = _binding().bwd(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale, causal, workspace, stream, steps)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd")
 
@@ -200,15 +156,7 @@ def nova_attn_bwd_static_scratch(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale: 
     or in the library.  The dQ accumulator is a fixed 32 MiB array inside the library, shared by all
     calls on the device, so B*H*T*D must not exceed 8 Mi elements and calls must not overlap on the
     GPU.  Make the first call on a device before any stream capture."""
-    _check_bf16("Q", Q)
-    B, H, T, D = Q.shape
-    for n, t in (("K", K), ("V", V), ("O", O), ("dO", dO), ("dQ", dQ), ("dK", dK), ("dV", dV)):
-        _check_bf16(n, t, Q.shape)
-    _check_f32("LSE", LSE, (B, H, T))
-    _check_f32("Delta", Delta, (B, H, T))
-    rc = load().nova_attn_bwd_static_scratch(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(LSE), _ptr(Delta),
-                                             _ptr(dQ), _ptr(dK), _ptr(dV), B, H, T, D, float(scale),
-                                             int(bool(causal)), _stream_ptr(stream))
+    rc = _binding().bwd_static_scratch(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_static_scratch")
 
@@ -247,24 +195,14 @@ def nova_attn_poll_device_status(stream=None) -> int:
 def nova_attn_fwd_strided(Q, K, V, O, LSE, scale: float, causal: bool = True, stream=None) -> None:
     """nova_attn_fwd on [B,H,T,D]-shaped VIEWS: strides are taken from the tensors, so Q, K, V may be slices
     of a fused projection output and O a permuted view of a [B,T,H,D] buffer.  LSE is contiguous [B,H,T]."""
-    sq = _view_strides("Q", Q)
-    B, H, T, D = Q.shape
-    sk, sv, so = (_view_strides(n, t, Q.shape) for n, t in (("K", K), ("V", V), ("O", O)))
-    _check_f32("LSE", LSE, (B, H, T))
-    rc = load().nova_attn_fwd_strided(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(LSE), B, H, T, D, sq, sk, sv, so,
-                                      float(scale), int(bool(causal)), _stream_ptr(stream))
+    rc = _binding().attn_fwd_strided(Q, K, V, O, LSE, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_fwd_strided")
 
 
 def nova_attn_bwd_preprocess_strided(O, dO, Delta, stream=None) -> None:
     """nova_attn_bwd_preprocess on [B,H,T,D]-shaped views."""
-    so = _view_strides("O", O)
-    sdo = _view_strides("dO", dO, O.shape)
-    B, H, T, D = O.shape
-    _check_f32("Delta", Delta, (B, H, T))
-    rc = load().nova_attn_bwd_preprocess_strided(_ptr(O), _ptr(dO), _ptr(Delta), B, H, T, D, so, sdo,
-                                                 _stream_ptr(stream))
+    rc = _binding().preprocess_strided(O, dO, Delta, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_preprocess_strided")
 
@@ -272,18 +210,7 @@ def nova_attn_bwd_preprocess_strided(O, dO, Delta, stream=None) -> None:
 def nova_attn_bwd_strided(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: bool = True, workspace=None,
                           stream=None) -> None:
     """nova_attn_bwd on [B,H,T,D]-shaped views (dQ, dK, dV may be slices of one fused gradient buffer)."""
-    sq = _view_strides("Q", Q)
-    B, H, T, D = Q.shape
-    rest = [_view_strides(n, t, Q.shape) for n, t in (("K", K), ("V", V), ("dO", dO), ("dQ", dQ), ("dK", dK), ("dV", dV))]
-    _check_f32("LSE", LSE, (B, H, T))
-    _check_f32("Delta", Delta, (B, H, T))
-    need = nova_attn_bwd_workspace_bytes(B, H, T, D)
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=Q.device)
-    rc = load().nova_attn_bwd_strided(_ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(LSE), _ptr(Delta), _ptr(dQ), _ptr(dK),
-                                      _ptr(dV), B, H, T, D, sq, *rest, float(scale), int(bool(causal)),
-                                      _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                      _stream_ptr(stream))
+    rc = _binding().bwd_strided(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale, causal, workspace, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_strided")
 
@@ -291,14 +218,6 @@ def nova_attn_bwd_strided(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, cau
 def nova_attn_bwd_deterministic(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: bool = True,
                                 stream=None) -> None:
     """dQ, dK, dV by the two-kernel backward: bitwise reproducible, no workspace, slower than nova_attn_bwd."""
-    _check_bf16("Q", Q)
-    B, H, T, D = Q.shape
-    for n, t in (("K", K), ("V", V), ("dO", dO), ("dQ", dQ), ("dK", dK), ("dV", dV)):
-        _check_bf16(n, t, Q.shape)
-    _check_f32("LSE", LSE, (B, H, T))
-    _check_f32("Delta", Delta, (B, H, T))
-    rc = load().nova_attn_bwd_deterministic(_ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(LSE), _ptr(Delta), _ptr(dQ),
-                                            _ptr(dK), _ptr(dV), B, H, T, D, float(scale), int(bool(causal)),
-                                            _stream_ptr(stream))
+    rc = _binding().bwd_deterministic(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_deterministic")

@@ -167,3 +167,19 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(na, "LIB_PATH", str(tmp_path / "libnova_attn.so"))
     with pytest.raises(ImportError):
         na.load()
+
+
+@pytest.mark.parametrize("bad", ["device", "dtype", "not a tensor"])
+def test_binding_rejects_wrong_tensors(bad):
+    """The native binding raises before anything is called (no GPU involved)."""
+    import torch
+    from paper_2608_00029_b200 import nova_attn as na, nova_lmhead as nl
+    x = {"device": torch.zeros(1, 1, 4, 64, dtype=torch.bfloat16), "dtype": torch.zeros(1, 1, 4, 64),
+         "not a tensor": None}[bad]
+    for call in (lambda: na.nova_attn_fwd(x, x, x, x, x, 0.125), lambda: na.nova_attn_fwd_strided(x, x, x, x, x, 0.125),
+                 lambda: na.nova_attn_bwd_preprocess(x, x, x),
+                 lambda: na.nova_attn_bwd(x, x, x, x, x, x, x, x, x, x, 0.125),
+                 lambda: na.nova_attn_bwd_deterministic(x, x, x, x, x, x, x, x, x, 0.125),
+                 lambda: nl.nova_lmhead_fwd(x, x, x, x, x, x)):
+        with pytest.raises(TypeError):
+            call()
