@@ -645,6 +645,18 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
     if (!Cfg::kBulkdQ && cwarp == 0 && lane == 0) bulk_wait_group<0>();
 }
 
+// 32 accumulator columns of a thread's row, scaled and rounded to bf16, into 16-byte chunks ch0..ch0+3 of its 128-byte
+// swizzled staging row.
+__device__ __forceinline__ void bwd_pack_row32(const uint32_t* a, float f, uint8_t* row_ptr, int ch0, int sw) {
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch)
+        *reinterpret_cast<uint4*>(row_ptr + (((ch0 + ch) ^ sw) << 4)) =
+            make_uint4(pack_bf16x2(__uint_as_float(a[8 * ch + 0]) * f, __uint_as_float(a[8 * ch + 1]) * f),
+                       pack_bf16x2(__uint_as_float(a[8 * ch + 2]) * f, __uint_as_float(a[8 * ch + 3]) * f),
+                       pack_bf16x2(__uint_as_float(a[8 * ch + 4]) * f, __uint_as_float(a[8 * ch + 5]) * f),
+                       pack_bf16x2(__uint_as_float(a[8 * ch + 6]) * f, __uint_as_float(a[8 * ch + 7]) * f));
+}
+
 // dQ warps at D=64.  One thread per row.  Per query tile they move the partial dQ tile from TMEM into
 // a swizzled shared-memory staging buffer, and a leader thread sends it to the fp32 accumulator with
 // two TMA reduce-add operations.  At the end of a work item the same warps pull dV and dK out of
@@ -652,7 +664,9 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
 // warps move on to the next item at once.  Nothing waits for a reduction or a store to complete
 // except the end of the kernel; before the staging buffer is refilled, the leader checks that the copy
 // engine has read it.
-template <bool kStrided>
+// kDirect: the head has a single key tile, so the tile of dQ is complete: it goes out scaled, as bf16, through the
+// map of dQ itself (`tmAcc`).
+template <bool kStrided, bool kDirect>
 __device__ __forceinline__ void bwd_dq_tma(uint8_t* smem, BwdBars* bars, uint32_t tmem_base, const CUtensorMap* tmAcc,
                                            const CUtensorMap* tmdK, const CUtensorMap* tmdV, float scale,
                                            const WorkList& wl, int qwarp, int lane) {
@@ -673,7 +687,7 @@ __device__ __forceinline__ void bwd_dq_tma(uint8_t* smem, BwdBars* bars, uint32_
     int w = 0, g = 0, u = 0;  // items, query tiles, uses of the staging buffer so far
 
     // Hands the filled staging buffer to the leader, who issues the copies of `kind`
-    // (0: dQ reduce-add, 1: dV/dK store) at row `row` of head `bh`.
+    // (0: dQ reduce-add or store, 1: dV/dK store) at row `row` of head `bh`.
     auto flush = [&](int kind, int row, int bh) -> bool {
         fence_proxy_async_smem();
         __syncwarp();
@@ -682,7 +696,10 @@ __device__ __forceinline__ void bwd_dq_tma(uint8_t* smem, BwdBars* bars, uint32_
         if (leader) {
             leader_ok = mbar_wait(&bars->stage_full, u & 1, abort_flag);
             if (leader_ok) {
-                if (kind == 0) {
+                if (kind == 0 && kDirect) {
+                    tma_store_tile<kStrided>(tmAcc, stage, (wl.orders() >> 24) & 15, 0, row, kStrided ? bh % wl.H() : 0,
+                                             kStrided ? bh / wl.H() : 0, bh);
+                } else if (kind == 0) {
                     tma_reduce_add_3d(tmAcc, stage, 0, row, bh);
                     tma_reduce_add_3d(tmAcc, stage + kHalfTileBytes, 32, row, bh);
                 } else {
@@ -728,6 +745,10 @@ __device__ __forceinline__ void bwd_dq_tma(uint8_t* smem, BwdBars* bars, uint32_
                 uint32_t a[32];
                 tmem_ld_x32(t_dq + 32 * hb, a);
                 tmem_wait_ld();
+                if constexpr (kDirect) {
+                    bwd_pack_row32(a, scale, row0, 4 * hb, sw);
+                    continue;
+                }
                 uint8_t* rowp = hb ? row1 : row0;
                 // fp32 [128 rows x 32 columns] per box: eight 16-byte chunks per row, 128-byte swizzle
 #pragma unroll
@@ -790,8 +811,11 @@ __device__ __forceinline__ void bwd_dq_tma(uint8_t* smem, BwdBars* bars, uint32_
 // against 2600 clocks of tensor work, so the copy engine must never idle: every box is a bulk group of its
 // own, boxes 0 and 1 are issued together, box 2 goes into the first half as soon as box 0 has been read
 // (box 1 still being read), box 3 into the second half once box 1 has been.
+// kDirect as above: both halves of the staging buffer hold 64 bf16 columns and go out as two stores.
+template <bool kStrided, bool kDirect>
 __device__ __forceinline__ void bwd_dq_tma_wide(uint8_t* smem, BwdBars* bars, uint32_t tmem_base,
-                                                const CUtensorMap* tmAcc, const WorkList& wl, int qwarp, int lane) {
+                                                const CUtensorMap* tmAcc, float scale, const WorkList& wl, int qwarp,
+                                                int lane) {
     constexpr int D = 128;
     using Cfg = BwdCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
@@ -823,7 +847,11 @@ __device__ __forceinline__ void bwd_dq_tma_wide(uint8_t* smem, BwdBars* bars, ui
             leader_ok = mbar_wait(&bars->stage_full, nf & 1, abort_flag);
             if (leader_ok) {
                 for (int k = 0; k < n; ++k) {
-                    tma_reduce_add_3d(tmAcc, stage + (first + k) * kHalfTileBytes, col + 32 * k, row, bh);
+                    if (kDirect)
+                        tma_store_tile<kStrided>(tmAcc, stage + k * kHalfTileBytes, (wl.orders() >> 24) & 15, kBoxCols * k, row,
+                                                 kStrided ? bh % wl.H() : 0, kStrided ? bh / wl.H() : 0, bh);
+                    else
+                        tma_reduce_add_3d(tmAcc, stage + (first + k) * kHalfTileBytes, col + 32 * k, row, bh);
                     bulk_commit_group();
                 }
             }
@@ -858,6 +886,23 @@ __device__ __forceinline__ void bwd_dq_tma_wide(uint8_t* smem, BwdBars* bars, ui
             if (g > 0) ok = reusable(std::integral_constant<int, 0>{});  // boxes 2, 3 of the previous tile
             tmem_wait_ld();
             if (!ok) break;
+            if constexpr (kDirect) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    bwd_pack_row32(a, scale, row_ptr + h * kHalfTileBytes, 0, sw);
+                    bwd_pack_row32(a + 32, scale, row_ptr + h * kHalfTileBytes, 4, sw);
+                    if (h == 0) {
+                        tmem_ld_x32(t_dq + 64, a);
+                        tmem_ld_x32(t_dq + 96, a + 32);
+                        tmem_wait_ld();
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars->dq_free);
+                ok = send(0, 2, 0, row, bh);
+                continue;
+            }
             fill(a, 0);
             fill(a + 32, 1);
             tmem_ld_x32(t_dq + 64, a);
@@ -882,7 +927,7 @@ __device__ __forceinline__ void bwd_dq_tma_wide(uint8_t* smem, BwdBars* bars, ui
     if (leader) bulk_wait_group<0>();
 }
 
-template <int D, bool kCausal, bool kStrided>
+template <int D, bool kCausal, bool kStrided, bool kDirect>
 __global__ void __launch_bounds__(BwdCfg<D>::kThreads, 1)
 attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
@@ -976,9 +1021,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         bwd_compute<D, kCausal, kStrided>(smem, bars, tmem_base, &tmdK, &tmdV, T, scale, wl, warp - 4, lane);
     } else {
         if constexpr (Cfg::kBulkdQ)
-            bwd_dq_tma<kStrided>(smem, bars, tmem_base, &tmAcc, &tmdK, &tmdV, scale, wl, warp - 4 - Cfg::kComputeWarps, lane);
+            bwd_dq_tma<kStrided, kDirect>(smem, bars, tmem_base, &tmAcc, &tmdK, &tmdV, scale, wl, warp - 4 - Cfg::kComputeWarps, lane);
         else
-            bwd_dq_tma_wide(smem, bars, tmem_base, &tmAcc, wl, warp - 4 - Cfg::kComputeWarps, lane);
+            bwd_dq_tma_wide<kStrided, kDirect>(smem, bars, tmem_base, &tmAcc, scale, wl, warp - 4 - Cfg::kComputeWarps, lane);
     }
 
     tc_fence_before();
@@ -990,7 +1035,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 template <int D, bool kCausal>
 cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                        const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
-                       const CUtensorMap& tmdV, bool strided, uint32_t orders, bool no_dq, const float* LSE,
+                       const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,
                        const float* Delta, __nv_bfloat16* dK, __nv_bfloat16* dV, const TensorStrides& sdk,
                        const TensorStrides& sdv, const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream) {
     static_assert(kBlockK == 128 && kBlockQ == 128, "the work plan counts 128-row tiles");
@@ -998,19 +1043,22 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     int n_tiles = 0, n_ctas = 0;
     const WorkPlan plan = bwd_work_plan(BH, s.T, D, kCausal, num_sms, &n_tiles, &n_ctas);
     const dim3 grid(static_cast<unsigned>(n_ctas));  // one persistent CTA per SM
-    const WorkArgs wa{BH, n_tiles, s.H, orders, no_dq ? 1 : 0, plan};
-    if (strided)
-        return launch_overlapped(attn_bwd_kernel<D, kCausal, true>, grid, dim3(BwdCfg<D>::kThreads), BwdCfg<D>::kSmemBytes,
-                                 stream, tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, LSE, Delta, dK, dV, sdk, sdv, s.T, wa,
-                                 s.scale, dev_status);
-    return launch_overlapped(attn_bwd_kernel<D, kCausal, false>, grid, dim3(BwdCfg<D>::kThreads), BwdCfg<D>::kSmemBytes, stream,
-                             tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, LSE, Delta, dK, dV, sdk, sdv, s.T, wa, s.scale,
-                             dev_status);
+    const WorkArgs wa{BH, n_tiles, s.H, orders, dq == DqMode::kNone ? 1 : 0, plan};
+    auto go = [&](auto kernel) {
+        return launch_overlapped(kernel, grid, dim3(BwdCfg<D>::kThreads), BwdCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO,
+                                 tmAcc, tmdK, tmdV, LSE, Delta, dK, dV, sdk, sdv, s.T, wa, s.scale, dev_status);
+    };
+    if (dq == DqMode::kDirect)
+        return strided ? go(attn_bwd_kernel<D, kCausal, true, true>) : go(attn_bwd_kernel<D, kCausal, false, true>);
+    return strided ? go(attn_bwd_kernel<D, kCausal, true, false>) : go(attn_bwd_kernel<D, kCausal, false, false>);
 }
 
 template <int D, bool kCausal, bool kStrided>
 cudaError_t configure_one() {
-    return cudaFuncSetAttribute(attn_bwd_kernel<D, kCausal, kStrided>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(attn_bwd_kernel<D, kCausal, kStrided, false>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<D>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(attn_bwd_kernel<D, kCausal, kStrided, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 BwdCfg<D>::kSmemBytes);
 }
 
@@ -1028,16 +1076,16 @@ cudaError_t configure_attn_bwd() {
 
 cudaError_t launch_attn_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                             const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
-                            const CUtensorMap& tmdV, bool strided, uint32_t orders, bool no_dq, const float* LSE,
+                            const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,
                             const float* Delta, __nv_bfloat16* dK, __nv_bfloat16* dV, const TensorStrides& sdk,
                             const TensorStrides& sdv, const AttnShape& s, int num_sms, int* dev_status,
                             cudaStream_t stream) {
     if (s.D == 64) {
-        return s.causal ? launch_one<64, true>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, no_dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream)
-                        : launch_one<64, false>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, no_dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream);
+        return s.causal ? launch_one<64, true>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream)
+                        : launch_one<64, false>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream);
     }
-    return s.causal ? launch_one<128, true>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, no_dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream)
-                    : launch_one<128, false>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, no_dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream);
+    return s.causal ? launch_one<128, true>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream)
+                    : launch_one<128, false>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream);
 }
 
 }  // namespace nova

@@ -82,15 +82,22 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
                            const AttnShape& s, int* dev_status, cudaStream_t stream);
 cudaError_t configure_attn_dq();
 
+// What the backward main kernel does with its partial tiles of dQ.
+enum class DqMode {
+    kAccumulate,  // adds them, unscaled, into the fp32 accumulator
+    kNone,        // nothing: dK and dV only (the dK/dV half of the two-kernel backward)
+    kDirect,      // T <= kBlockK, a head has one key tile: its dQ tile is complete and is written scaled, as bf16
+};
+
 // Backward main kernel: adds unscaled dQ partial tiles into the fp32 accumulator [B,H,T,D] (zero on
 // entry) described by `tmAcc` (fp32 [D, T, B*H], box [32, 128, 1], 128-byte swizzle) and writes dK and dV
 // (`tmdK`, `tmdV`: the bf16 maps of the outputs, used for TMA stores at D=64; at D=128 the rows go out
 // with plain stores through `dK`, `dV` and their strides).  `strided`, `orders`: as in the forward, for
-// Q, K, V, dO, dK, dV.  `no_dq`: write dK and dV only (the dK/dV half of the two-kernel backward); `tmAcc` is
-// then never used.  Persistent: launches at most `num_sms` CTAs.
+// Q, K, V, dO, dK, dV (and dQ).  `dq`: see above; `tmAcc` is the bf16 map of dQ with kDirect and never used with
+// kNone.  Persistent: launches at most `num_sms` CTAs.
 cudaError_t launch_attn_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                             const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
-                            const CUtensorMap& tmdV, bool strided, uint32_t orders, bool no_dq, const float* LSE, const float* Delta,
+                            const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE, const float* Delta,
                             __nv_bfloat16* dK, __nv_bfloat16* dV, const TensorStrides& sdk, const TensorStrides& sdv,
                             const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream);
 cudaError_t configure_attn_bwd();

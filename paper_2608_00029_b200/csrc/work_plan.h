@@ -29,7 +29,7 @@ struct WorkCursor {
 // this kernel is at its register limit).
 struct WorkArgs {
     int BH, n_tiles, H;
-    uint32_t orders;  // coordinate orders of the Q, K, V, dO, dK, dV tensor maps, four bits each
+    uint32_t orders;  // coordinate orders of the Q, K, V, dO, dK, dV, dQ tensor maps, four bits each
     int no_dq;        // dK/dV half of the two-kernel backward: no dQ product, no accumulator traffic
     WorkPlan plan;
 };

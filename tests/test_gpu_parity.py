@@ -321,6 +321,39 @@ def test_fused_projection_layout(B, H, T, D, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"fused T={T} D={D}: ", dO=ref["dO_in"])
 
 
+@pytest.mark.parametrize("T", [1, 17, 64, 127, 128])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_single_key_tile_writes_dq_directly(T, D, causal):
+    """T <= 128: the backward writes dQ without the fp32 accumulator.  One contribution per tile added to zero, scaled
+    and rounded once is the same number either way, so the three steps issued one by one (which go through the
+    accumulator) give the same bits, as do the deterministic entry point and, on a fused layout, the strided one;
+    more heads than SMs, so that a CTA reuses its staging buffer."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("direct", B=4, H=50, T=T, D=D, seed=700 + T + D, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    got = h.run_gpu(Q, K, V, dO, cfg.scale, causal)
+    q, k, v, do = (x.to(dev) for x in (Q, K, V, dO))
+    o, lse, delta = got["O"].to(dev), got["LSE"].to(dev), got["Delta"].to(dev)
+    ws = torch.full((nova_attn.nova_attn_bwd_workspace_bytes(cfg.B, cfg.H, T, D),), 255, dtype=torch.uint8, device=dev)
+    a, b = ([torch.full_like(q, 7.0) for _ in range(3)] for _ in range(2))
+    for step in (nova_attn.BWD_STEP_ZERO, nova_attn.BWD_STEP_MAIN, nova_attn.BWD_STEP_CONVERT):
+        nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *a, cfg.scale, causal, ws, steps=step)
+    nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *b, cfg.scale, causal)
+    dqkv = torch.full((cfg.B, T, 3, cfg.H, D), 7.0, dtype=torch.bfloat16, device=dev)
+    c = [dqkv[:, :, i].permute(0, 2, 1, 3) for i in range(3)]
+    nova_attn.nova_attn_bwd_strided(q, k, v, do, lse, delta, *c, cfg.scale, causal, ws)
+    nova_attn.nova_attn_poll_device_status()
+    for name, x, y, z in zip(("dQ", "dK", "dV"), a, b, c):
+        for other in (x, y, z):
+            assert torch.equal(other.cpu(), got[name]), name
+    heads = [(0, 0), (3, 49)]
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal, heads=heads)
+    h.compare(h.select_heads(got, heads), ref, label=f"direct T={T} D={D}: ", dO=ref["dO_in"])
+
+
 DETERMINISTIC = [  # (B, H, T, D, causal)
     (1, 2, 64, 64, True),
     (2, 3, 300, 64, True),
