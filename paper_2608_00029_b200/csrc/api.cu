@@ -76,7 +76,6 @@ int device_state(DeviceState** out) {
         }
         e = configure_attn_fwd();
         if (e == cudaSuccess) e = configure_attn_bwd();
-        if (e == cudaSuccess) e = configure_attn_delta();
         if (e == cudaSuccess) e = configure_attn_dq();
         if (e == cudaSuccess) e = configure_lmhead();
         if (e == cudaSuccess) e = configure_lmhead_rows();
@@ -92,7 +91,7 @@ int device_state(DeviceState** out) {
 // call to a lookup when the same buffers are used step after step.
 struct MapKey {
     const void* ptr;
-    int D, T, BH, dev, elem_bytes;
+    int D, T, BH, dev, elem_bytes, box_rows;
     long long st, sh;
 };
 struct MapEntry {
@@ -105,26 +104,26 @@ MapEntry g_maps[kMapCache];
 
 // 3-D map [D, T, B*H] of a tensor whose heads and batches merge into one dimension of stride `sh`
 // elements (0: contiguous, sh = T*D) with token stride `st` (0: D).
-// elem_bytes 2: bf16 tensor, box [64, 128, 1]; elem_bytes 4: fp32 tensor, box [32, 128, 1].
+// elem_bytes 2: bf16 tensor, box [64, box_rows, 1]; elem_bytes 4: fp32 tensor, box [32, box_rows, 1].
 int get_tensor_map(const void* ptr, int D, long long T, long long BH, CUtensorMap* out, int elem_bytes = 2,
-                   long long st = 0, long long sh = 0) {
+                   long long st = 0, long long sh = 0, int box_rows = kBlockQ) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (st == 0) st = D;
     if (sh == 0) sh = T * D;
-    const MapKey key{ptr, D, static_cast<int>(T), static_cast<int>(BH), dev, elem_bytes, st, sh};
-    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull + uint64_t(T) * 31 + uint64_t(BH) * 131 + D;
+    const MapKey key{ptr, D, static_cast<int>(T), static_cast<int>(BH), dev, elem_bytes, box_rows, st, sh};
+    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull + (uint64_t(T) * 31 + uint64_t(BH) * 131 + D + box_rows) * 0xD6E8FEB86659FD93ull;
     std::lock_guard<std::mutex> lock(g_mutex);
     MapEntry& e = g_maps[(h >> 32) % kMapCache];
     if (e.valid && e.key.ptr == key.ptr && e.key.D == key.D && e.key.T == key.T && e.key.BH == key.BH &&
-        e.key.dev == key.dev && e.key.elem_bytes == key.elem_bytes && e.key.st == key.st && e.key.sh == key.sh) {
+        e.key.dev == key.dev && e.key.elem_bytes == key.elem_bytes && e.key.box_rows == box_rows && e.key.st == key.st && e.key.sh == key.sh) {
         *out = e.map;
         return NOVA_ATTN_OK;
     }
     // [D, T, B*H], D contiguous; 128-byte box rows; rows past T read as zero and are clipped on writes.
     const cuuint64_t dims[3] = {cuuint64_t(D), cuuint64_t(T), cuuint64_t(BH)};
     const cuuint64_t strides[2] = {cuuint64_t(st) * elem_bytes, cuuint64_t(sh) * elem_bytes};
-    const cuuint32_t box[3] = {cuuint32_t(128 / elem_bytes), cuuint32_t(kBlockQ), 1};
+    const cuuint32_t box[3] = {cuuint32_t(128 / elem_bytes), cuuint32_t(box_rows), 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     CUtensorMap m;
     const CUresult r = g_encode(&m, elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
@@ -144,7 +143,7 @@ int get_tensor_map(const void* ptr, int D, long long T, long long BH, CUtensorMa
 // tokens.  `*order` receives which of the three sits where (the code tma_order_coords understands).
 struct Map4Key {
     const void* ptr;
-    int D, T, H, B, dev;
+    int D, T, H, B, dev, box_rows;
     long long sb, sh, st;
 };
 struct Map4Entry {
@@ -155,16 +154,18 @@ struct Map4Entry {
 };
 Map4Entry g_maps4[kMapCache];
 
-int get_tensor_map4(const void* ptr, const AttnShape& s, const TensorStrides& st, CUtensorMap* out, uint32_t* order) {
+int get_tensor_map4(const void* ptr, const AttnShape& s, const TensorStrides& st, CUtensorMap* out, uint32_t* order,
+                    int box_rows) {
     int dev = 0;
     cudaGetDevice(&dev);
-    const Map4Key key{ptr, s.D, s.T, s.H, s.B, dev, st.b, st.h, st.t};
-    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull + uint64_t(s.T) * 31 +
-                       uint64_t(s.B) * 131 + uint64_t(s.H) * 17 + uint64_t(st.t) * 7 + s.D;
+    const Map4Key key{ptr, s.D, s.T, s.H, s.B, dev, box_rows, st.b, st.h, st.t};
+    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull + 
+                       (uint64_t(s.T) * 31 + uint64_t(s.B) * 131 + uint64_t(s.H) * 17 + uint64_t(st.t) * 7 + s.D + box_rows) *
+                           0xD6E8FEB86659FD93ull;
     std::lock_guard<std::mutex> lock(g_mutex);
     Map4Entry& e = g_maps4[(h >> 32) % kMapCache];
     if (e.valid && e.key.ptr == key.ptr && e.key.D == key.D && e.key.T == key.T && e.key.H == key.H &&
-        e.key.B == key.B && e.key.dev == key.dev && e.key.sb == key.sb && e.key.sh == key.sh && e.key.st == key.st) {
+        e.key.B == key.B && e.key.dev == key.dev && e.key.box_rows == box_rows && e.key.sb == key.sb && e.key.sh == key.sh && e.key.st == key.st) {
         *out = e.map;
         *order = static_cast<uint32_t>(e.order);
         return NOVA_ATTN_OK;
@@ -187,7 +188,7 @@ int get_tensor_map4(const void* ptr, const AttnShape& s, const TensorStrides& st
     for (int i = 0; i < 3; ++i) {
         dims[1 + i] = cuuint64_t(extent_of[which[i]]);
         strides[i] = cuuint64_t(stride_of[which[i]]) * sizeof(__nv_bfloat16);
-        if (which[i] == 0) box[1 + i] = cuuint32_t(kBlockQ);
+        if (which[i] == 0) box[1 + i] = cuuint32_t(box_rows);
     }
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUtensorMap m;
@@ -230,10 +231,10 @@ bool merges(const AttnShape& s, const TensorStrides& st) {
 
 // The map of a bf16 tensor for the plain (3-D) or the strided (4-D) build of the kernels.
 int get_bf16_map(const void* ptr, const AttnShape& s, const TensorStrides& st, bool strided, CUtensorMap* out,
-                 uint32_t* order) {
-    if (strided) return get_tensor_map4(ptr, s, st, out, order);
+                 uint32_t* order, int box_rows = kBlockQ) {
+    if (strided) return get_tensor_map4(ptr, s, st, out, order, box_rows);
     *order = 0;
-    return get_tensor_map(ptr, s.D, s.T, static_cast<long long>(s.B) * s.H, out, 2, st.t, st.h);
+    return get_tensor_map(ptr, s.D, s.T, static_cast<long long>(s.B) * s.H, out, 2, st.t, st.h, box_rows);
 }
 
 TensorStrides contiguous_strides(int H, int T, int D) {
@@ -368,8 +369,8 @@ int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, 
     const long long BH = static_cast<long long>(B) * H;
     CUtensorMap tmQ, tmK, tmV, tmdO;
     if (int rc = get_tensor_map(Q, D, T, BH, &tmQ)) return rc;
-    if (int rc = get_tensor_map(K, D, T, BH, &tmK)) return rc;
-    if (int rc = get_tensor_map(V, D, T, BH, &tmV)) return rc;
+    if (int rc = get_tensor_map(K, D, T, BH, &tmK, 2, 0, 0, kKeyStep)) return rc;
+    if (int rc = get_tensor_map(V, D, T, BH, &tmV, 2, 0, 0, kKeyStep)) return rc;
     if (int rc = get_tensor_map(dO, D, T, BH, &tmdO)) return rc;
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const cudaError_t e =
@@ -465,22 +466,23 @@ int nova_attn_bwd_deterministic(const void* Q, const void* K, const void* V, con
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const TensorStrides c = contiguous_strides(H, T, D);
-    CUtensorMap tmQ, tmK, tmV, tmdO, tmdK, tmdV;
+    CUtensorMap tmQ, tmK, tmV, tmKs, tmVs, tmdO, tmdQ, tmdK, tmdV;
     if (int rc = get_tensor_map(Q, D, T, BH, &tmQ)) return rc;
     if (int rc = get_tensor_map(K, D, T, BH, &tmK)) return rc;
     if (int rc = get_tensor_map(V, D, T, BH, &tmV)) return rc;
     if (int rc = get_tensor_map(dO, D, T, BH, &tmdO)) return rc;
     if (int rc = get_tensor_map(dK, D, T, BH, &tmdK)) return rc;
     if (int rc = get_tensor_map(dV, D, T, BH, &tmdV)) return rc;
+    if (int rc = get_tensor_map(dQ, D, T, BH, &tmdQ)) return rc;
     if (T <= kBlockK) {  // one key tile per head: nothing is summed across blocks, the fused kernel is deterministic too
-        CUtensorMap tmdQ;
-        if (int rc = get_tensor_map(dQ, D, T, BH, &tmdQ)) return rc;
         const cudaError_t e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmdQ, tmdK, tmdV, false, 0u, DqMode::kDirect, LSE, Delta,
                                               static_cast<__nv_bfloat16*>(dK), static_cast<__nv_bfloat16*>(dV), c, c, s,
                                               st->num_sms, st->dev_status, cs);
         return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
     }
-    cudaError_t e = launch_attn_dq(tmQ, tmK, tmV, tmdO, LSE, Delta, static_cast<__nv_bfloat16*>(dQ), s, st->dev_status, cs);
+    if (int rc = get_tensor_map(K, D, T, BH, &tmKs, 2, 0, 0, kKeyStep)) return rc;
+    if (int rc = get_tensor_map(V, D, T, BH, &tmVs, 2, 0, 0, kKeyStep)) return rc;
+    cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, false, 0u, LSE, Delta, s, st->dev_status, cs);
     if (e != cudaSuccess) return fail_cuda(e);
     // the dK/dV half: the fused kernel without its dQ product (the accumulator map is never used: any map will do)
     e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmQ, tmdK, tmdV, false, 0u, DqMode::kNone, LSE, Delta, static_cast<__nv_bfloat16*>(dK),

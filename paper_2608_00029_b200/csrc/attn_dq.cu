@@ -1,257 +1,545 @@
-// Deterministic dQ for the two-kernel backward of the paper (Section 4.2, "The Backward Pass": one kernel
-// reduces dQ over keys, the other reduces dK and dV over queries; the probability matrix is rebuilt from
-// the saved log-sum-exp in both).  One CTA owns a 128-row query tile of one head and walks the key tiles
-// in order, so every dQ row is summed by one thread block in a fixed order: no atomics, no workspace,
-// bitwise reproducible.  Per key tile:
-//   S  = Q K_j^T,  dP = dO V_j^T            (smem x smem -> two TMEM accumulators)
-//   dS = exp2(S*c - LSE*log2e) * (dP - Delta)   (one thread per query row; bf16 back into TMEM over S)
-//   dQ += dS K_j                             (TMEM x smem, K read MN-major; accumulator in TMEM)
-// and at the end dQ * scale is rounded once to bf16 and stored.  Costs two contractions more than the
-// fused backward (S and dP are computed here and again in the dK/dV kernel): the price of determinism.
-//   warp 0      TMA producer (Q and dO once, K and V tiles through a ring)
-//   warp 1      UMMA issuer
-//   warps 2..5  one thread per query row
-// TMEM columns: S / dS [0,128)  dP [128,256)  dQ [256, 256+D).
+// Query-major passes of the backward (paper Section 4.2, "The Backward Pass": one kernel reduces dQ over keys, the
+// other reduces dK and dV over queries; the probability matrix is rebuilt from the saved log-sum-exp, never stored):
+//   attn_dq_kernel     dQ_i = scale * sum_j dS_ij K_j,  dS = exp2(S*c - LSE*log2e) * (dP - Delta).  Every dQ row is
+//                      summed by one thread block in key order: no atomics, no workspace, bitwise reproducible.
+//   attn_delta_kernel  Delta_i = sum_j P_ij (dO_i . V_j): the exact softmax-Jacobian row term.  The cheap route to the
+//                      same quantity, rowsum(dO * O), inherits the bf16 rounding of the stored O, which with sharply
+//                      peaked rows (|O| ~ |V|) is the largest term in dQ and dK.
+// Both form S = Q K_j^T and dP = dO V_j^T tile by tile and differ in what becomes of the tile, so they are two builds of
+// one kernel.
+//
+// A work item is a block of 256 query rows of one head: two 128-row tiles, A and B, that share every K and V tile
+// they both need.  The keys go by in steps of 64.  Items are handed out dynamically, heaviest first, as in the
+// forward (WorkRing).  384 threads:
+//   warp 0      TMA producer: Q and dO per tile of an item, K and V through a ring of 64-key stages
+//   warps 1, 3  UMMA issuers, one per query tile, so that neither tile waits for the other's products and A may be in
+//               the next item while B finishes this one
+//   warps 4-7   rows of tile A, warps 8-11 rows of tile B: one thread per query row takes 64 keys of S and dP out of
+//               tensor memory and writes dS back as bf16 (or adds P*dP into its Delta)
+//
+// What bounds it: one tile in flight is a serial chain (products -> tensor memory -> arithmetic -> tensor memory ->
+// product), during which the tensor cores idle; two tiles fill each other's gaps.  64 keys per step is what tensor memory
+// allows two tiles at D=128: dQ takes 128 of a tile's 256 columns, S and dP 64 each.  A product of N=64 with both
+// operands in shared memory costs 49 clocks per 16 k elements against 65 for twice the keys, so a 128 x 128 block takes
+// 2100 clocks of tensor time at D=128 (1560 with N=128).
+#include <type_traits>
+
 #include "kernels.h"
 #include "ptx.cuh"
 
 namespace nova {
 namespace {
 
-constexpr int kDqThreads = 192;
-constexpr int kDqTmemCols = 512;
+constexpr int kThreads = 384;
+constexpr int kTmemCols = 512;
+constexpr int kStep = kKeyStep;                  // keys per step
+constexpr int kBlockRows = 2 * kBlockQ;          // query rows per work item
+constexpr int kHalfStepBytes = kStep * 128;      // one [64 keys x 64 bf16] box
+constexpr int kWorkConsumers = 2 + 8;            // issuers + row warps
 
 template <int D>
 struct DqCfg {
     static constexpr int kHalves = D / kBoxCols;
     static constexpr int kTileBytes = kHalves * kHalfTileBytes;
-    static constexpr int kStages = (D == 64) ? 2 : 1;
-    static constexpr int kOffQ = 0;
-    static constexpr int kOffdO = kTileBytes;
-    static constexpr int kOffK = 2 * kTileBytes;
-    static constexpr int kOffV = kOffK + kStages * kTileBytes;
-    static constexpr int kOffBar = kOffV + kStages * kTileBytes;
-    // One CTA per SM (it takes all 512 TMEM columns): ask for more than half of the shared memory so
-    // that a second CTA is never made resident only to wait for TMEM.
-    static constexpr int kSmemBytes = (kOffBar + 256 + 1024) > 120 * 1024 ? (kOffBar + 256 + 1024) : 120 * 1024;
-    static constexpr int kColS = 0, kColdP = 128, kColdQ = 256;
+    static constexpr int kStepBytes = kHalves * kHalfStepBytes;
+    static constexpr int kQStages = (D == 64) ? 2 : 1;  // Q and dO of an item
+    static constexpr int kKVStages = (D == 64) ? 5 : 3;
+    static constexpr int kOffQ = 0;                                     // [kQStages][2 tiles] of Q, then of dO
+    static constexpr int kOffdO = kQStages * 2 * kTileBytes;
+    static constexpr int kOffK = 2 * kOffdO;                            // [kKVStages] of K, then of V
+    static constexpr int kOffV = kOffK + kKVStages * kStepBytes;
+    static constexpr int kOffBar = kOffV + kKVStages * kStepBytes;
+    static constexpr int kSmemBytes = kOffBar + 512 + 1024;
+    static_assert(kSmemBytes <= 232448, "exceeds the shared memory of one CTA");
+    // Columns of a tile (256 per tile).  dQ first.  D=64: S, dP, and two buffers of dS (32 columns each), so that S and
+    // dP of the next step are queued as soon as the row warps have read them.  D=128: S and dP, and dS lies over S.
+    static constexpr bool kSepdS = (D == 64);
+    static constexpr int kColS = D, kColdP = D + 64;
+    static constexpr int kColdS = kSepdS ? 192 : kColS;
 };
 
 struct DqBars {
-    uint64_t q_full;
-    uint64_t kv_full[2], kv_empty[2];
-    uint64_t acc_full;   // UMMA -> rows: S and dP of the tile are complete
-    uint64_t ds_ready;   // rows (one arrival per warp) -> UMMA: dS is in TMEM
-    uint64_t dq_done;    // UMMA -> rows: the last dQ product is complete
-    uint64_t drain;
+    uint64_t q_full[2][2], q_empty[2][2];  // [stage][tile]
+    uint64_t kv_full[5], kv_empty[5];
+    uint64_t sp_full[2][2], sp_free[2][2];  // [buffer][tile]; the second buffer is used by the Delta build only
+    // Two ds_ready per tile, used in turn: where dS has columns of its own the row warps may finish step j + 1 before the
+    // issuer has seen step j, and a single barrier two phases on looks as if it had not moved.
+    uint64_t ds_ready[2][2];                     // [step & 1][tile]
+    uint64_t dq_done[2], dq_free[2], staged[2];  // per tile
+    uint64_t drain[2];
+    WorkRing ring;
     uint32_t tmem_base;
     int abort_flag;
 };
+static_assert(sizeof(DqBars) <= 512, "barrier block");
 
-template <int D>
+// Work items: 256-row query blocks, heaviest first (the last block of a causal problem sees every key).
+struct DqWork {
+    int BH, n_blocks, T, H;
+    uint32_t orders;  // coordinate orders of the Q, K, V, dO, dQ tensor maps, four bits each
+    bool causal;
+    // Block index, head, and the number of key steps each tile visits (0: the tile lies past the end of the sequence).
+    __device__ __forceinline__ void get(int idx, int* blk, int* bh, int* n_a, int* n_b) const {
+        *blk = n_blocks - 1 - idx / BH;
+        *bh = idx % BH;
+        const int n_all = (T + kStep - 1) / kStep;
+        const int qt_a = 2 * (*blk), qt_b = qt_a + 1;
+        *n_a = causal ? min((qt_a + 1) * (kBlockQ / kStep), n_all) : n_all;
+        *n_b = (qt_b * kBlockQ < T) ? (causal ? min((qt_b + 1) * (kBlockQ / kStep), n_all) : n_all) : 0;
+    }
+};
+
+template <int D, bool kStrided>
 __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, int qt, int bh,
-                                            int n_kv) {
+                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork& wk) {
     using Cfg = DqCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
-    int armed[2] = {-1, -1};
-    mbar_expect_tx(&bars->q_full, 2 * Cfg::kTileBytes);
+    constexpr long long limit = kWaitLimitCycles;
+    int armed_q[2][2] = {{-1, -1}, {-1, -1}}, armed_kv[Cfg::kKVStages];
+    for (int s = 0; s < Cfg::kKVStages; ++s) armed_kv[s] = -1;
+    bool ok = true, clc_pending = false;
+    int w = 0, st = 0;  // items so far, K/V stage
+    uint32_t ph = 0;    // and its phase
+    int item = blockIdx.x;
+    for (;;) {
+        ok = bars->ring.publish(w, item, abort_flag, limit);
+        if (!ok || item < 0) break;
+        int blk, bh, n_a, n_b;
+        wk.get(item, &blk, &bh, &n_a, &n_b);
+        const int head = kStrided ? bh % wk.H : 0, batch = kStrided ? bh / wk.H : 0;
+        const int qs = w % Cfg::kQStages;
+        const uint32_t qph = (w / Cfg::kQStages) & 1;
+        const int n = max(n_a, n_b);
+        // Tile A's Q and dO, the first keys, tile B's Q and dO (whose buffers tile B hands back later than A), the rest.
+        auto load_q = [&](int t) -> bool {
+            if (!mbar_wait(&bars->q_empty[qs][t], qph ^ 1, abort_flag)) return false;
+            mbar_expect_tx(&bars->q_full[qs][t], 2 * Cfg::kTileBytes);  // rows past T arrive as zeros
+            armed_q[qs][t] = qph;
 #pragma unroll
-    for (int h = 0; h < Cfg::kHalves; ++h) {
-        tma_load_3d(smem + Cfg::kOffQ + h * kHalfTileBytes, tmQ, &bars->q_full, h * kBoxCols, qt * kBlockQ, bh);
-        tma_load_3d(smem + Cfg::kOffdO + h * kHalfTileBytes, tmdO, &bars->q_full, h * kBoxCols, qt * kBlockQ, bh);
-    }
-    bool ok = true;
-    for (int j = 0; j < n_kv; ++j) {
-        const int st = j % Cfg::kStages;
-        const uint32_t ph = (j / Cfg::kStages) & 1;
-        ok = mbar_wait(&bars->kv_empty[st], ph ^ 1, abort_flag);
+            for (int h = 0; h < Cfg::kHalves; ++h) {
+                const int off = (qs * 2 + t) * Cfg::kTileBytes + h * kHalfTileBytes;
+                tma_load_tile<kStrided>(smem + Cfg::kOffQ + off, tmQ, &bars->q_full[qs][t], wk.orders & 15, h * kBoxCols,
+                                        blk * kBlockRows + t * kBlockQ, head, batch, bh);
+                tma_load_tile<kStrided>(smem + Cfg::kOffdO + off, tmdO, &bars->q_full[qs][t], (wk.orders >> 12) & 15,
+                                        h * kBoxCols, blk * kBlockRows + t * kBlockQ, head, batch, bh);
+            }
+            return true;
+        };
+        ok = load_q(0);
         if (!ok) break;
-        mbar_expect_tx(&bars->kv_full[st], 2 * Cfg::kTileBytes);
-        armed[st] = ph;
+        for (int j = 0; j < n; ++j) {
+            ok = mbar_wait(&bars->kv_empty[st], ph ^ 1, abort_flag);
+            if (!ok) break;
+            mbar_expect_tx(&bars->kv_full[st], 2 * Cfg::kStepBytes);
+            armed_kv[st] = ph;
 #pragma unroll
-        for (int h = 0; h < Cfg::kHalves; ++h) {
-            tma_load_3d(smem + Cfg::kOffK + st * Cfg::kTileBytes + h * kHalfTileBytes, tmK, &bars->kv_full[st],
-                        h * kBoxCols, j * kBlockK, bh);
-            tma_load_3d(smem + Cfg::kOffV + st * Cfg::kTileBytes + h * kHalfTileBytes, tmV, &bars->kv_full[st],
-                        h * kBoxCols, j * kBlockK, bh);
+            for (int h = 0; h < Cfg::kHalves; ++h) {
+                tma_load_tile<kStrided>(smem + Cfg::kOffK + st * Cfg::kStepBytes + h * kHalfStepBytes, tmK,
+                                        &bars->kv_full[st], (wk.orders >> 4) & 15, h * kBoxCols, j * kStep, head, batch, bh);
+                tma_load_tile<kStrided>(smem + Cfg::kOffV + st * Cfg::kStepBytes + h * kHalfStepBytes, tmV,
+                                        &bars->kv_full[st], (wk.orders >> 8) & 15, h * kBoxCols, j * kStep, head, batch, bh);
+            }
+            if (++st == Cfg::kKVStages) {
+                st = 0;
+                ph ^= 1;
+            }
+            if (j == 0) {
+                ok = load_q(1);
+                if (!ok) break;
+            }
         }
+        if (!ok) break;
+        // all loads of this item are on their way: claim the next one now, and no earlier
+        bars->ring.request();
+        clc_pending = true;
+        ok = bars->ring.answer(w, &item, abort_flag, limit);
+        if (!ok) break;
+        clc_pending = false;
+        ++w;
     }
-    if (!ok) {  // giving up: let the copies in flight land before the CTA's shared memory goes away
+    if (!ok) {  // giving up: let what is in flight land before the CTA's shared memory goes away
         int none = 0;
-        (void)mbar_wait(&bars->q_full, 0, &none);
-        for (int st = 0; st < Cfg::kStages; ++st)
-            if (armed[st] >= 0) (void)mbar_wait(&bars->kv_full[st], armed[st], &none);
+        if (clc_pending) (void)mbar_wait(&bars->ring.answer_bar, w & 1, &none);
+        for (int s = 0; s < 2; ++s)
+            for (int t = 0; t < 2; ++t)
+                if (armed_q[s][t] >= 0) (void)mbar_wait(&bars->q_full[s][t], armed_q[s][t], &none);
+        for (int s = 0; s < Cfg::kKVStages; ++s)
+            if (armed_kv[s] >= 0) (void)mbar_wait(&bars->kv_full[s], armed_kv[s], &none);
     }
 }
 
-template <int D>
-__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, int n_kv) {
+// The issuer of query tile t: the whole warp in uniform control flow, one elected lane issues.
+template <int D, bool kDelta>
+__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork& wk, int t) {
     using Cfg = DqCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
-    constexpr uint32_t kIdescT = umma_idesc_bf16(128, 128, 0, 0);  // S, dP
-    constexpr uint32_t kIdescdQ = umma_idesc_bf16(128, D, 0, 1);   // dQ: A from TMEM, B (K) MN-major
+    constexpr uint32_t kIdescT = umma_idesc_bf16(128, kStep, 0, 0);  // S, dP
+    constexpr uint32_t kIdescdQ = umma_idesc_bf16(128, D, 0, 1);     // dQ: A from TMEM, B (K) MN-major
     const uint32_t hi = umma_desc_hi_sw128(1024);
-    const uint32_t q_k = umma_desc_lo(smem_u32(smem + Cfg::kOffQ), 16);
-    const uint32_t do_k = umma_desc_lo(smem_u32(smem + Cfg::kOffdO), 16);
-    const uint32_t t_s = tmem_base + Cfg::kColS, t_dp = tmem_base + Cfg::kColdP, t_dq = tmem_base + Cfg::kColdQ;
-    // The whole warp runs this role in uniform control flow; one elected lane issues.
+    const uint32_t k_k0 = umma_desc_lo(smem_u32(smem + Cfg::kOffK), 16);
+    const uint32_t v_k0 = umma_desc_lo(smem_u32(smem + Cfg::kOffV), 16);
+    const uint32_t k_m0 = umma_desc_lo(smem_u32(smem + Cfg::kOffK), kHalfStepBytes);
+    const uint32_t t_dq = tmem_base + 256 * t;
     const bool el = elect_one();
-    bool ok = mbar_wait(&bars->q_full, 0, abort_flag);
-    for (int j = 0; j < n_kv && ok; ++j) {
-        const int st = j % Cfg::kStages;
-        ok = mbar_wait(&bars->kv_full[st], (j / Cfg::kStages) & 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t k_k = umma_desc_lo(smem_u32(smem + Cfg::kOffK + st * Cfg::kTileBytes), 16);
-        const uint32_t v_k = umma_desc_lo(smem_u32(smem + Cfg::kOffV + st * Cfg::kTileBytes), 16);
-        const uint32_t k_m = umma_desc_lo(smem_u32(smem + Cfg::kOffK + st * Cfg::kTileBytes), kHalfTileBytes);
-        // S and dP columns are free: the dQ product of the previous tile, which read dS out of them, was
-        // queued before this point (the pipe executes in order), after the rows had finished with dP.
-        if (el) {
+    const int lane = threadIdx.x & 31;
+    bool ok = true;
+    int w = 0, wt = 0;  // items; items in which the tile took part
+    int c = 0, cq = 0;  // steps of this tile finished; steps whose S and dP have been issued
+    int st = 0;         // K/V stage of the current step
+    uint32_t ph = 0;    // and its phase
+    uint32_t q_k = 0, do_k = 0;
+
+    // acc[64 columns] = A_t B^T with both operands K-major, 16 head-dim elements (32 bytes) per instruction
+    auto product = [&](uint32_t t_acc, uint32_t a, uint32_t b) {
 #pragma unroll
-            for (int k = 0; k < D / 16; ++k) {
-                const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
-                umma_ss(t_s, umma_desc_join(q_k + off, hi), umma_desc_join(k_k + off, hi), kIdescT, k > 0 ? 1u : 0u);
-            }
-#pragma unroll
-            for (int k = 0; k < D / 16; ++k) {
-                const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
-                umma_ss(t_dp, umma_desc_join(do_k + off, hi), umma_desc_join(v_k + off, hi), kIdescT, k > 0 ? 1u : 0u);
-            }
-            tc_commit(&bars->acc_full);
+        for (int k = 0; k < D / 16; ++k)
+            umma_ss(t_acc, umma_desc_join(a + (((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4), hi),
+                    umma_desc_join(b + (((k / 4) * kHalfStepBytes + (k % 4) * 32) >> 4), hi), kIdescT, k > 0 ? 1u : 0u);
+    };
+    auto next_stage = [&](int* s, uint32_t* p) {
+        if (++*s == Cfg::kKVStages) {
+            *s = 0;
+            *p ^= 1;
         }
-        __syncwarp();
-        ok = mbar_wait(&bars->ds_ready, j & 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        // dQ += dS K_j: dS from TMEM (16 keys = 8 packed columns per instruction), K MN-major (rows = keys,
-        // 64 head-dim elements per 128-byte row, the second 64-wide half 16 KB further).
-        if (el) {
-#pragma unroll
-            for (int k = 0; k < kBlockK / 16; ++k)
-                umma_ts(t_dq, t_s + k * 8, umma_desc_join(k_m + k * 128, hi), kIdescdQ, (j > 0 || k > 0) ? 1u : 0u);
-            tc_commit(&bars->kv_empty[st]);  // K_j and V_j are no longer read
-            if (j + 1 == n_kv) tc_commit(&bars->dq_done);
+    };
+
+    for (;;) {
+        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
+        if (item < 0) {
+            ok = (item == -1);
+            break;
         }
-        __syncwarp();
+        int blk, bh, n_a, n_b;
+        wk.get(item, &blk, &bh, &n_a, &n_b);
+        const int n_t = t == 0 ? n_a : n_b, n = max(n_a, n_b);
+        const int qs = w % Cfg::kQStages;
+        q_k = umma_desc_lo(smem_u32(smem + Cfg::kOffQ + (qs * 2 + t) * Cfg::kTileBytes), 16);
+        do_k = umma_desc_lo(smem_u32(smem + Cfg::kOffdO + (qs * 2 + t) * Cfg::kTileBytes), 16);
+        if (n_t > 0) {
+            ok = mbar_wait(&bars->q_full[qs][t], (w / Cfg::kQStages) & 1, abort_flag);
+            if (!ok) break;
+        }
+        if constexpr (kDelta) {
+            for (int j = 0; j < n_t; ++j, ++cq) {
+                ok = mbar_wait(&bars->kv_full[st], ph, abort_flag);
+                // the row warps have read what this buffer held two steps ago
+                if (ok) ok = mbar_wait(&bars->sp_free[cq & 1][t], ((cq >> 1) & 1) ^ 1, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                if (el) {
+                    const uint32_t t_s = tmem_base + 256 * t + 128 * (cq & 1);
+                    product(t_s, q_k, k_k0 + st * (Cfg::kStepBytes >> 4));
+                    product(t_s + 64, do_k, v_k0 + st * (Cfg::kStepBytes >> 4));
+                    tc_commit(&bars->sp_full[cq & 1][t]);
+                    tc_commit(&bars->kv_empty[st]);
+                    if (j + 1 == n_t) tc_commit(&bars->q_empty[qs][t]);
+                }
+                __syncwarp();
+                next_stage(&st, &ph);
+            }
+        } else {
+            const uint32_t t_s = t_dq + Cfg::kColS, t_dp = t_dq + Cfg::kColdP;
+            int st_n = st;  // stage of the step whose S and dP come next
+            uint32_t ph_n = ph;
+            // S and dP of the item's first step.  Their columns are free: the row warps have read the previous step's
+            // (sp_free was awaited below, or is here), and a dS that lies over S was consumed by a dQ product queued
+            // earlier.
+            if (n_t > 0) {
+                ok = mbar_wait(&bars->kv_full[st_n], ph_n, abort_flag);
+                if (ok && cq > 0) ok = mbar_wait(&bars->sp_free[0][t], (cq - 1) & 1, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                if (el) {
+                    product(t_s, q_k, k_k0 + st_n * (Cfg::kStepBytes >> 4));
+                    product(t_dp, do_k, v_k0 + st_n * (Cfg::kStepBytes >> 4));
+                    tc_commit(&bars->sp_full[0][t]);
+                }
+                __syncwarp();
+                ++cq;
+                next_stage(&st_n, &ph_n);
+            }
+            for (int j = 0; j < n_t; ++j, ++c) {
+                const bool more = j + 1 < n_t;
+                if (more) {  // dP (and S, where dS has columns of its own) of the next step, once this step's have been read
+                    ok = mbar_wait(&bars->kv_full[st_n], ph_n, abort_flag);
+                    if (ok) ok = mbar_wait(&bars->sp_free[0][t], (cq - 1) & 1, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (el) {
+                        if (Cfg::kSepdS) product(t_s, q_k, k_k0 + st_n * (Cfg::kStepBytes >> 4));
+                        product(t_dp, do_k, v_k0 + st_n * (Cfg::kStepBytes >> 4));
+                        if (Cfg::kSepdS) tc_commit(&bars->sp_full[0][t]);
+                    }
+                    __syncwarp();
+                }
+                ok = mbar_wait(&bars->ds_ready[c & 1][t], (c >> 1) & 1, abort_flag);
+                // the previous item's dQ must have been read out of TMEM before it is overwritten
+                if (ok && j == 0 && wt > 0) ok = mbar_wait(&bars->dq_free[t], (wt - 1) & 1, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                // dQ += dS K_j: dS from TMEM (16 keys = 8 packed columns per instruction), K MN-major (rows = keys,
+                // 64 head-dim elements per 128-byte row, the second 64-wide half kHalfStepBytes further).
+                if (el) {
+                    const uint32_t t_ds = t_dq + Cfg::kColdS + (Cfg::kSepdS ? 32 * (c & 1) : 0);
+                    const uint32_t k_m = k_m0 + st * (Cfg::kStepBytes >> 4);
+#pragma unroll
+                    for (int k = 0; k < kStep / 16; ++k)
+                        umma_ts(t_dq, t_ds + k * 8, umma_desc_join(k_m + k * 128, hi), kIdescdQ, (j > 0 || k > 0) ? 1u : 0u);
+                    tc_commit(&bars->kv_empty[st]);
+                    if (!more) tc_commit(&bars->dq_done[t]);
+                    if (!Cfg::kSepdS && more) {  // S of the next step, over the dS that the product above reads
+                        product(t_s, q_k, k_k0 + st_n * (Cfg::kStepBytes >> 4));
+                        tc_commit(&bars->sp_full[0][t]);
+                    }
+                }
+                __syncwarp();
+                if (more) {
+                    ++cq;
+                    next_stage(&st_n, &ph_n);
+                }
+                next_stage(&st, &ph);
+            }
+        }
+        if (!ok) break;
+        // Steps that only the other tile visits: this tile's share of their release, each once it has landed (an earlier
+        // arrival could fall into the stage's previous use).
+        for (int j = n_t; j < n; ++j) {
+            ok = mbar_wait(&bars->kv_full[st], ph, abort_flag);
+            if (!ok) break;
+            if (lane == 0) mbar_arrive(&bars->kv_empty[st]);
+            __syncwarp();
+            next_stage(&st, &ph);
+        }
+        if (!ok) break;
+        if (n_t > 0) ++wt;
+        ++w;
     }
     if (!ok) {
         int none = 0;
-        if (el) tc_commit(&bars->drain);
+        if (el) tc_commit(&bars->drain[t]);
         __syncwarp();
-        (void)mbar_wait(&bars->drain, 0, &none);
+        (void)mbar_wait(&bars->drain[t], 0, &none);
     }
 }
 
-template <int D, bool kCausal>
-__device__ __forceinline__ void dq_rows(DqBars* bars, uint32_t tmem_base, const float* __restrict__ LSE,
-                                        const float* __restrict__ Delta, __nv_bfloat16* __restrict__ dQ, int T, int qt,
-                                        int bh, int n_kv, float scale, int warp, int lane) {
+// The row warps of query tile t.
+template <int D, bool kCausal, bool kStrided, bool kDelta>
+__device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const CUtensorMap* tmdQ,
+                                        const float* __restrict__ LSE, const float* __restrict__ Delta,
+                                        float* __restrict__ Delta_out, float scale, const DqWork& wk, int t, int rwarp,
+                                        int lane) {
     using Cfg = DqCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
-    const uint32_t lane_base = 32u * (warp & 3);
+    const uint32_t lane_base = 32u * rwarp;
     const int row_local = lane_base + lane;
-    const int row = qt * kBlockQ + row_local;
-    const uint32_t t_s = tmem_addr(tmem_base, lane_base, Cfg::kColS);
-    const uint32_t t_dp = tmem_addr(tmem_base, lane_base, Cfg::kColdP);
-    const uint32_t t_dq = tmem_addr(tmem_base, lane_base, Cfg::kColdQ);
+    const bool leader = (rwarp == 0 && lane == 0);
+    const uint32_t t_dq = tmem_addr(tmem_base, lane_base, 256 * t);
     const float c = scale * kLog2e;
-    const size_t idx = static_cast<size_t>(bh) * T + row;
-    // Rows past the end of the sequence: LSE = +inf gives P = 0 everywhere.
-    const float lse2 = (row < T) ? LSE[idx] * kLog2e : INFINITY;
-    const float delta = (row < T) ? Delta[idx] : 0.f;
+    const uint64_t c2 = f32x2_pack(c, c);
+    const int T = wk.T;
     bool ok = true;
-    for (int j = 0; j < n_kv; ++j) {
-        ok = mbar_wait(&bars->acc_full, j & 1, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        const bool diag = kCausal && (j == qt);
-        const int keys_left = T - j * kBlockK;
-        const int lim = diag ? min(row_local, keys_left - 1) : min(keys_left, kBlockK) - 1;
-        // 32 keys at a time: their bf16 dS pairs (16 columns) land on S columns that have already been read.
-#pragma unroll 1
-        for (int cb = 0; cb < 128; cb += 32) {
-            uint32_t sv[32], dv[32], ds[16];
-            tmem_ld_x32(t_s + cb, sv);
-            tmem_ld_x32(t_dp + cb, dv);
+    int w = 0, wt = 0, cnt = 0;  // items, items this tile took part in, steps processed by this tile
+    int pending_qs = -1;         // Q stage whose dQ store was issued at the end of the previous item
+
+    for (;;) {
+        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
+        if (item < 0) {
+            ok = (item == -1);
+            break;
+        }
+        int blk, bh, n_a, n_b;
+        wk.get(item, &blk, &bh, &n_a, &n_b);
+        const int n_t = (t == 0) ? n_a : n_b;
+        const int qt = 2 * blk + t;
+        const int row = qt * kBlockQ + row_local;
+        const size_t idx = static_cast<size_t>(bh) * T + row;
+        const int qs = w % Cfg::kQStages;
+        if (n_t == 0) {  // tile past the end of the sequence: only release its buffers, once they have been filled
+            bool leader_ok = true;
+            if (leader) {
+                if (pending_qs >= 0) {
+                    bulk_wait_group_read<0>();
+                    mbar_arrive(&bars->q_empty[pending_qs][t]);
+                }
+                leader_ok = mbar_wait(&bars->q_full[qs][t], (w / Cfg::kQStages) & 1, abort_flag);
+                if (leader_ok) mbar_arrive(&bars->q_empty[qs][t]);
+            }
+            pending_qs = -1;
+            ok = __all_sync(0xffffffffu, leader_ok);
+            if (!ok) break;
+            ++w;
+            continue;
+        }
+        // Rows past the end of the sequence: LSE = +inf gives P = 0 everywhere.
+        const float nlse2 = (row < T) ? -LSE[idx] * kLog2e : -INFINITY;
+        const float ndelta = (!kDelta && row < T) ? -Delta[idx] : 0.f;
+        const uint64_t nlse = f32x2_pack(nlse2, nlse2), nd = f32x2_pack(ndelta, ndelta);
+        uint64_t acc0 = 0, acc1 = 0;
+
+        for (int j = 0; j < n_t; ++j, ++cnt) {
+            const int buf = kDelta ? (cnt & 1) : 0;
+            ok = mbar_wait(&bars->sp_full[buf][t], (kDelta ? (cnt >> 1) : cnt) & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t t_s = t_dq + (kDelta ? 128 * buf : Cfg::kColS);
+            const uint32_t t_dp = kDelta ? t_s + 64 : t_dq + Cfg::kColdP;
+            uint32_t sv[kStep], dv[kStep];
+            tmem_ld_x32(t_s, sv);
+            tmem_ld_x32(t_s + 32, sv + 32);
+            tmem_ld_x32(t_dp, dv);
+            tmem_ld_x32(t_dp + 32, dv + 32);
             tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->sp_free[buf][t]);
+            // Mask from indices only: causal keeps key <= query, the end of the sequence key < T.
+            const int lim = (kCausal ? min(row, T - 1) : T - 1) - j * kStep;  // last kept key of the step
+            if ((kCausal && (j + 1) * kStep > qt * kBlockQ) || (j + 1) * kStep > T) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-                float p0 = ex2_approx(fmaf(__uint_as_float(sv[i + 0]), c, -lse2));
-                float p1 = ex2_approx(fmaf(__uint_as_float(sv[i + 1]), c, -lse2));
-                if (cb + i + 0 > lim) p0 = 0.f;
-                if (cb + i + 1 > lim) p1 = 0.f;
-                ds[i / 2] = pack_bf16x2(p0 * (__uint_as_float(dv[i + 0]) - delta), p1 * (__uint_as_float(dv[i + 1]) - delta));
+                for (int i = 0; i < kStep; ++i)
+                    if (i > lim) sv[i] = 0xff800000u;  // -inf: P = 0
             }
-            tmem_st_x16(t_s + cb / 2, ds);
-        }
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->ds_ready);
-    }
-    if (!ok) return;
-    // dQ row = scale * accumulator, rounded once
-    ok = mbar_wait(&bars->dq_done, 0, abort_flag);
-    if (!ok) return;
-    tc_fence_after();
-    uint4* out = reinterpret_cast<uint4*>(dQ + idx * D);
+            uint32_t ds[kStep / 2];
 #pragma unroll
-    for (int cb = 0; cb < D; cb += 32) {
-        uint32_t a[32];
-        tmem_ld_x32(t_dq + cb, a);
-        tmem_wait_ld();
-        if (row < T) {
-#pragma unroll
-            for (int x = 0; x < 32; x += 8) {
-                uint4 v;
-                v.x = pack_bf16x2(__uint_as_float(a[x + 0]) * scale, __uint_as_float(a[x + 1]) * scale);
-                v.y = pack_bf16x2(__uint_as_float(a[x + 2]) * scale, __uint_as_float(a[x + 3]) * scale);
-                v.z = pack_bf16x2(__uint_as_float(a[x + 4]) * scale, __uint_as_float(a[x + 5]) * scale);
-                v.w = pack_bf16x2(__uint_as_float(a[x + 6]) * scale, __uint_as_float(a[x + 7]) * scale);
-                out[(cb + x) / 8] = v;
+            for (int i = 0; i < kStep; i += 4) {
+                float x0, x1, x2, x3;
+                f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sv[i + 0]), __uint_as_float(sv[i + 1])), c2, nlse), x0, x1);
+                f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3])), c2, nlse), x2, x3);
+                const uint64_t p01 = f32x2_pack(ex2_approx(x0), ex2_approx(x1)), p23 = f32x2_pack(ex2_approx(x2), ex2_approx(x3));
+                const uint64_t d01 = f32x2_pack(__uint_as_float(dv[i + 0]), __uint_as_float(dv[i + 1]));
+                const uint64_t d23 = f32x2_pack(__uint_as_float(dv[i + 2]), __uint_as_float(dv[i + 3]));
+                if constexpr (kDelta) {
+                    acc0 = f32x2_fma(p01, d01, acc0);
+                    acc1 = f32x2_fma(p23, d23, acc1);
+                } else {
+                    f32x2_unpack(f32x2_mul(p01, f32x2_add(d01, nd)), x0, x1);
+                    f32x2_unpack(f32x2_mul(p23, f32x2_add(d23, nd)), x2, x3);
+                    ds[i / 2] = pack_bf16x2(x0, x1);
+                    ds[i / 2 + 1] = pack_bf16x2(x2, x3);
+                }
+            }
+            if constexpr (!kDelta) {
+                // D=64: the dQ product of two steps ago, which read this buffer, was queued before S of this step, and
+                // the tensor pipe completes in order.
+                tmem_st_x32(t_dq + Cfg::kColdS + (Cfg::kSepdS ? 32 * (cnt & 1) : 0), ds);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars->ds_ready[cnt & 1][t]);
+                if (pending_qs >= 0) {
+                    if (leader) {
+                        bulk_wait_group_read<0>();
+                        mbar_arrive(&bars->q_empty[pending_qs][t]);
+                    }
+                    pending_qs = -1;
+                    __syncwarp();
+                }
             }
         }
+        if (!ok) break;
+        if constexpr (kDelta) {
+            float a0, a1, a2, a3;
+            f32x2_unpack(acc0, a0, a1);
+            f32x2_unpack(acc1, a2, a3);
+            if (row < T) Delta_out[idx] = (a0 + a1) + (a2 + a3);
+            __syncwarp();
+        } else {
+            // ---- end of the item: scale * dQ_t as bf16 into this tile's Q buffer (no longer read: the last dQ product
+            // completed after every S of the tile), then TMA stores
+            ok = mbar_wait(&bars->dq_done[t], wt & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            uint8_t* stage = smem + Cfg::kOffQ + (qs * 2 + t) * Cfg::kTileBytes;
+#pragma unroll
+            for (int cb = 0; cb < D; cb += 32) {
+                uint32_t a[32];
+                tmem_ld_x32(t_dq + cb, a);
+                tmem_wait_ld();
+                uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + row_local * 128;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
+                    uint4 v;
+                    v.x = pack_bf16x2(__uint_as_float(a[8 * x + 0]) * scale, __uint_as_float(a[8 * x + 1]) * scale);
+                    v.y = pack_bf16x2(__uint_as_float(a[8 * x + 2]) * scale, __uint_as_float(a[8 * x + 3]) * scale);
+                    v.z = pack_bf16x2(__uint_as_float(a[8 * x + 4]) * scale, __uint_as_float(a[8 * x + 5]) * scale);
+                    v.w = pack_bf16x2(__uint_as_float(a[8 * x + 6]) * scale, __uint_as_float(a[8 * x + 7]) * scale);
+                    *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (row_local & 7)) << 4)) = v;
+                }
+            }
+            tc_fence_before();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&bars->dq_free[t]);
+                mbar_arrive(&bars->staged[t]);
+            }
+            bool leader_ok = true;
+            if (leader) {
+                leader_ok = mbar_wait(&bars->staged[t], wt & 1, abort_flag);
+                if (leader_ok) {
+#pragma unroll
+                    for (int h = 0; h < Cfg::kHalves; ++h)
+                        tma_store_tile<kStrided>(tmdQ, stage + h * kHalfTileBytes, (wk.orders >> 16) & 15, h * kBoxCols,
+                                                 qt * kBlockQ, kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
+                    bulk_commit_group();
+                    if (Cfg::kQStages == 1) {  // the next item's Q tile needs this very buffer
+                        bulk_wait_group_read<0>();
+                        mbar_arrive(&bars->q_empty[qs][t]);
+                    }
+                }
+            }
+            if (Cfg::kQStages > 1) pending_qs = qs;  // handed back after the next item's first step, as in the forward
+            ok = __all_sync(0xffffffffu, leader_ok);
+            if (!ok) break;
+        }
+        ++w;
+        ++wt;
     }
+    if (!kDelta && leader) bulk_wait_group<0>();  // dQ must be complete before the kernel ends
 }
 
-template <int D, bool kCausal>
-__global__ void __launch_bounds__(kDqThreads, 1)
-attn_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-               const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
-               const float* __restrict__ LSE, const float* __restrict__ Delta, __nv_bfloat16* __restrict__ dQ, int T,
-               int BH, int n_q_tiles, float scale, int* __restrict__ dev_status) {
+// Set-up and roles, shared by the two builds below.
+template <int D, bool kCausal, bool kStrided, bool kDelta>
+__device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
+                                        const CUtensorMap* tmdO, const CUtensorMap* tmdQ, const float* __restrict__ LSE,
+                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork& wk,
+                                        float scale, int* __restrict__ dev_status) {
     using Cfg = DqCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     DqBars* bars = reinterpret_cast<DqBars*>(smem + Cfg::kOffBar);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // heaviest query tiles (most key tiles under the causal clamp) first
-    const int qt = n_q_tiles - 1 - static_cast<int>(blockIdx.x) / BH;
-    const int bh = static_cast<int>(blockIdx.x) % BH;
-    const int n_kv_all = (T + kBlockK - 1) / kBlockK;
-    const int n_kv = kCausal ? min(qt + 1, n_kv_all) : n_kv_all;
 
     if (threadIdx.x == 0) {
-        mbar_init(&bars->q_full, 1);
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&bars->kv_full[s], 1);
-            mbar_init(&bars->kv_empty[s], 1);
+        for (int t = 0; t < 2; ++t) {
+            for (int s = 0; s < 2; ++s) {
+                mbar_init(&bars->q_full[s][t], 1);
+                mbar_init(&bars->q_empty[s][t], 1);
+                mbar_init(&bars->sp_full[s][t], 1);
+                mbar_init(&bars->sp_free[s][t], 4);
+                mbar_init(&bars->ds_ready[s][t], 4);
+            }
+            mbar_init(&bars->dq_done[t], 1);
+            mbar_init(&bars->dq_free[t], 4);
+            mbar_init(&bars->staged[t], 4);
+            mbar_init(&bars->drain[t], 1);
         }
-        mbar_init(&bars->acc_full, 1);
-        mbar_init(&bars->ds_ready, 4);
-        mbar_init(&bars->dq_done, 1);
-        mbar_init(&bars->drain, 1);
+        for (int s = 0; s < Cfg::kKVStages; ++s) {
+            mbar_init(&bars->kv_full[s], 1);
+            mbar_init(&bars->kv_empty[s], 2);  // the two issuers
+        }
+        bars->ring.init(kWorkConsumers);
         bars->abort_flag = 0;
         fence_mbar_init();
-        tma_prefetch_desc(&tmQ);
-        tma_prefetch_desc(&tmK);
-        tma_prefetch_desc(&tmV);
-        tma_prefetch_desc(&tmdO);
+        tma_prefetch_desc(tmQ);
+        tma_prefetch_desc(tmK);
+        tma_prefetch_desc(tmV);
+        tma_prefetch_desc(tmdO);
+        if (!kDelta) tma_prefetch_desc(tmdQ);
     }
     if (warp == 1) {
-        tmem_alloc(&bars->tmem_base, kDqTmemCols);
+        tmem_alloc(&bars->tmem_base, kTmemCols);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -262,55 +550,98 @@ attn_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     griddep_wait();  // everything above overlaps the previous kernel of the stream
 
     if (warp == 0) {
-        if (lane == 0) dq_producer<D>(&tmQ, &tmK, &tmV, &tmdO, smem, bars, qt, bh, n_kv);
-    } else if (warp == 1) {
-        dq_mma<D>(smem, bars, tmem_base, n_kv);
-    } else {
-        dq_rows<D, kCausal>(bars, tmem_base, LSE, Delta, dQ, T, qt, bh, n_kv, scale, warp, lane);
+        if (lane == 0) dq_producer<D, kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
+    } else if (warp == 1 || warp == 3) {
+        dq_mma<D, kDelta>(smem, bars, tmem_base, wk, warp >> 1);
+    } else if (warp >= 4) {
+        dq_rows<D, kCausal, kStrided, kDelta>(smem, bars, tmem_base, tmdQ, LSE, Delta, Delta_out, scale, wk,
+                                              (warp - 4) >> 2, warp & 3, lane);
     }
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, kDqTmemCols);
+    if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
     if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
 }
 
-template <int D, bool kCausal>
-cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
-                       const CUtensorMap& tmdO, const float* LSE, const float* Delta, __nv_bfloat16* dQ,
-                       const AttnShape& s, int* dev_status, cudaStream_t stream) {
-    const int n_q_tiles = (s.T + kBlockQ - 1) / kBlockQ;
-    const int BH = s.B * s.H;
-    return launch_overlapped(attn_dq_kernel<D, kCausal>, dim3(static_cast<unsigned>(n_q_tiles) * BH), dim3(kDqThreads),
-                             DqCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO, LSE, Delta, dQ, s.T, BH, n_q_tiles,
-                             s.scale, dev_status);
+template <int D, bool kCausal, bool kStrided>
+__global__ void __launch_bounds__(kThreads, 1)
+attn_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+               const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
+               const __grid_constant__ CUtensorMap tmdQ, const float* __restrict__ LSE, const float* __restrict__ Delta,
+               int T, int BH, int H, uint32_t orders, int n_blocks, float scale, int* __restrict__ dev_status) {
+    dq_body<D, kCausal, kStrided, false>(&tmQ, &tmK, &tmV, &tmdO, &tmdQ, LSE, Delta, nullptr,
+                                         DqWork{BH, n_blocks, T, H, orders, kCausal}, scale, dev_status);
 }
 
 template <int D, bool kCausal>
+__global__ void __launch_bounds__(kThreads, 1)
+attn_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
+                  const float* __restrict__ LSE, float* __restrict__ Delta, int T, int BH, int n_blocks, float scale,
+                  int* __restrict__ dev_status) {
+    dq_body<D, kCausal, false, true>(&tmQ, &tmK, &tmV, &tmdO, nullptr, LSE, nullptr, Delta,
+                                     DqWork{BH, n_blocks, T, 1, 0u, kCausal}, scale, dev_status);
+}
+
+int n_blocks_of(const AttnShape& s) { return (s.T + kBlockRows - 1) / kBlockRows; }
+// One CTA per item; those that do not start at once are taken over by those that did.
+dim3 grid_of(const AttnShape& s) { return dim3(static_cast<unsigned>(n_blocks_of(s)) * s.B * s.H); }
+
+template <int D, bool kCausal>
 cudaError_t configure_one() {
-    return cudaFuncSetAttribute(attn_dq_kernel<D, kCausal>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                DqCfg<D>::kSmemBytes);
+    auto set = [](auto kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<D>::kSmemBytes);
+    };
+    cudaError_t e = set(attn_dq_kernel<D, kCausal, false>);
+    if (e == cudaSuccess) e = set(attn_dq_kernel<D, kCausal, true>);
+    if (e == cudaSuccess) e = set(attn_delta_kernel<D, kCausal>);
+    return e;
+}
+
+// Calls f with the head dimension and the mask as compile-time constants.
+template <typename F>
+cudaError_t dispatch(const AttnShape& s, F&& f) {
+    using D64 = std::integral_constant<int, 64>;
+    using D128 = std::integral_constant<int, 128>;
+    if (s.D == 64) return s.causal ? f(D64{}, std::true_type{}) : f(D64{}, std::false_type{});
+    return s.causal ? f(D128{}, std::true_type{}) : f(D128{}, std::false_type{});
 }
 
 }  // namespace
 
 cudaError_t configure_attn_dq() {
-    const cudaError_t r[4] = {configure_one<64, true>(), configure_one<64, false>(), configure_one<128, true>(),
-                              configure_one<128, false>()};
-    for (cudaError_t e : r)
-        if (e != cudaSuccess) return e;
-    return cudaSuccess;
+    cudaError_t e = configure_one<64, true>();
+    if (e == cudaSuccess) e = configure_one<64, false>();
+    if (e == cudaSuccess) e = configure_one<128, true>();
+    if (e == cudaSuccess) e = configure_one<128, false>();
+    return e;
 }
 
 cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
-                           const CUtensorMap& tmdO, const float* LSE, const float* Delta, __nv_bfloat16* dQ,
-                           const AttnShape& s, int* dev_status, cudaStream_t stream) {
-    if (s.D == 64) {
-        return s.causal ? launch_one<64, true>(tmQ, tmK, tmV, tmdO, LSE, Delta, dQ, s, dev_status, stream)
-                        : launch_one<64, false>(tmQ, tmK, tmV, tmdO, LSE, Delta, dQ, s, dev_status, stream);
-    }
-    return s.causal ? launch_one<128, true>(tmQ, tmK, tmV, tmdO, LSE, Delta, dQ, s, dev_status, stream)
-                    : launch_one<128, false>(tmQ, tmK, tmV, tmdO, LSE, Delta, dQ, s, dev_status, stream);
+                           const CUtensorMap& tmdO, const CUtensorMap& tmdQ, bool strided, uint32_t orders,
+                           const float* LSE, const float* Delta, const AttnShape& s, int* dev_status,
+                           cudaStream_t stream) {
+    return dispatch(s, [&](auto d, auto causal) {
+        constexpr int D = decltype(d)::value;
+        constexpr bool kCausal = decltype(causal)::value;
+        auto go = [&](auto kernel) {
+            return launch_overlapped(kernel, grid_of(s), dim3(kThreads), DqCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO,
+                                     tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, n_blocks_of(s), s.scale, dev_status);
+        };
+        return strided ? go(attn_dq_kernel<D, kCausal, true>) : go(attn_dq_kernel<D, kCausal, false>);
+    });
+}
+
+cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                              const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s,
+                              int* dev_status, cudaStream_t stream) {
+    return dispatch(s, [&](auto d, auto causal) {
+        constexpr int D = decltype(d)::value;
+        constexpr bool kCausal = decltype(causal)::value;
+        return launch_overlapped(attn_delta_kernel<D, kCausal>, grid_of(s), dim3(kThreads), DqCfg<D>::kSmemBytes, stream, tmQ,
+                                 tmK, tmV, tmdO, LSE, Delta, s.T, s.B * s.H, n_blocks_of(s), s.scale, dev_status);
+    });
 }
 
 }  // namespace nova

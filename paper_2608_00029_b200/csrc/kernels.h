@@ -69,17 +69,19 @@ cudaError_t launch_attn_bwd_preprocess(const __nv_bfloat16* O, const __nv_bfloat
                                        const AttnShape& s, const TensorStrides& so, const TensorStrides& sdo,
                                        int num_sms, cudaStream_t stream);
 
+// The query-major passes of the backward (attn_dq.cu): K and V maps with boxes of kKeyStep rows.
+constexpr int kKeyStep = 64;
 // Exact Delta_i = sum_j P_ij (dO_i . V_j) with P rebuilt from LSE (two contractions + exp2 per tile).
 cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                               const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s,
                               int* dev_status, cudaStream_t stream);
-cudaError_t configure_attn_delta();
-
-// Deterministic dQ (the dQ half of the paper's two-kernel backward): one CTA per 128-row query tile walks
-// the key tiles in order and writes dQ = bf16(scale * sum_j dS_j K_j).  3-D [D, T, B*H] maps; dQ contiguous.
+// Deterministic dQ (the dQ half of the paper's two-kernel backward): one CTA per pair of 128-row query tiles walks
+// the keys in order and writes dQ = bf16(scale * sum_j dS_j K_j) through `tmdQ`.  `strided`, `orders`: as in the
+// forward, for Q, K, V, dO, dQ.
 cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
-                           const CUtensorMap& tmdO, const float* LSE, const float* Delta, __nv_bfloat16* dQ,
-                           const AttnShape& s, int* dev_status, cudaStream_t stream);
+                           const CUtensorMap& tmdO, const CUtensorMap& tmdQ, bool strided, uint32_t orders,
+                           const float* LSE, const float* Delta, const AttnShape& s, int* dev_status,
+                           cudaStream_t stream);
 cudaError_t configure_attn_dq();
 
 // What the backward main kernel does with its partial tiles of dQ.

@@ -354,6 +354,38 @@ def test_single_key_tile_writes_dq_directly(T, D, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"direct T={T} D={D}: ", dO=ref["dO_in"])
 
 
+@pytest.mark.parametrize("T", [129, 191, 193, 256, 257, 385, 449])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_query_major_passes_at_step_edges(T, D, causal):
+    """The deterministic dQ and the exact Delta walk the keys in steps of 64 for pairs of 128-row tiles: sequence lengths
+    around the edges of a step, of a tile and of a pair (a second tile with one row, or none), more items than SMs so
+    that CTAs take over further ones; twelve calls back to back give the same bits every time."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("steps", B=7, H=30, T=T, D=D, seed=900 + T + D, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    got = h.run_gpu(Q, K, V, dO, cfg.scale, causal, exact_delta=True)
+    q, k, v, do = (x.to(dev) for x in (Q, K, V, dO))
+    lse = got["LSE"].to(dev)
+    runs = []
+    for _ in range(12):
+        delta = torch.full_like(lse, 7.0)
+        dq, dk, dv = (torch.full_like(q, 7.0) for _ in range(3))
+        nova_attn.nova_attn_bwd_preprocess_exact(q, k, v, do, lse, delta, cfg.scale, causal)
+        nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, dq, dk, dv, cfg.scale, causal)
+        runs.append((delta, dq, dk, dv))
+    nova_attn.nova_attn_poll_device_status()
+    for r in runs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(r, runs[0]))
+    assert torch.equal(runs[0][0].cpu(), got["Delta"])
+    got.update(dQ=runs[0][1].cpu(), dK=runs[0][2].cpu(), dV=runs[0][3].cpu())
+    heads = [(0, 0), (6, 29)]
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal, heads=heads)
+    h.compare(h.select_heads(got, heads), ref, label=f"steps T={T} D={D}: ", dO=ref["dO_in"])
+
+
 DETERMINISTIC = [  # (B, H, T, D, causal)
     (1, 2, 64, 64, True),
     (2, 3, 300, 64, True),
