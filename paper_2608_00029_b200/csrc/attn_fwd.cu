@@ -1,6 +1,7 @@
 // Fused causal attention forward for sm_100a (paper Section 4.2: score contraction, index mask,
 // base-2 online softmax, value contraction, causal loop clamp, 1/sum epilogue, LSE saved).
 //
+// (Small problems: one tile per item, see launch_one.)
 // A work item is a block of 256 query rows of one (batch, head): two 128-row query tiles, A and B,
 // that share every K/V tile they both need.  The kernel is persistent and its work is handed out
 // dynamically: the grid has one CTA per item, heaviest first (the last query block of a causal problem
@@ -68,8 +69,11 @@ struct FwdBars {
 };
 constexpr int kWorkConsumers = 1 + 8;  // UMMA issuer warp + 8 softmax warps
 
-// Work items: 256-row query blocks, numbered heaviest first.
+// Work items: 256-row query blocks, numbered heaviest first.  kSingle: 128-row blocks, tile A alone.
+template <bool kSingle>
 struct FwdWork {
+    static constexpr int kRows = kSingle ? kBlockQ : kBlockRows;
+    static constexpr int kTiles = kRows / kBlockQ;
     int n_items, BH, n_blocks, n_kv_all, T, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, O tensor maps, four bits each
     bool causal;
@@ -78,17 +82,17 @@ struct FwdWork {
     __device__ __forceinline__ void get(int idx, int* blk, int* bh, int* n_a, int* n_b) const {
         *blk = n_blocks - 1 - idx / BH;
         *bh = idx % BH;
-        const int qt_a = 2 * (*blk), qt_b = qt_a + 1;
+        const int qt_a = kTiles * (*blk), qt_b = qt_a + 1;
         // causal clamp of the key loop: tile qt visits key tiles 0..qt
         *n_a = causal ? min(qt_a + 1, n_kv_all) : n_kv_all;
-        *n_b = (qt_b * kBlockQ < T) ? (causal ? min(qt_b + 1, n_kv_all) : n_kv_all) : 0;
+        *n_b = (!kSingle && qt_b * kBlockQ < T) ? (causal ? min(qt_b + 1, n_kv_all) : n_kv_all) : 0;
     }
 };
 
-template <int D, bool kStrided>
+template <int D, bool kStrided, typename Work>
 __device__ __forceinline__ void fwd_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK,
                                              const CUtensorMap* tmV, uint8_t* smem, FwdBars* bars,
-                                             const FwdWork& wk, long long limit, int inject) {
+                                             const Work& wk, long long limit, int inject) {
     using Cfg = FwdCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
     int armed_q[2] = {-1, -1}, armed_k[2] = {-1, -1}, armed_v[2] = {-1, -1};
@@ -107,14 +111,14 @@ __device__ __forceinline__ void fwd_producer(const CUtensorMap* tmQ, const CUten
         const uint32_t qph = (w / Cfg::kQStages) & 1;
         ok = mbar_wait(&bars->q_empty[qs], qph ^ 1, abort_flag, limit);
         if (!ok) break;
-        mbar_expect_tx(&bars->q_full[qs], 2 * Cfg::kTileBytes);  // rows past T arrive as zeros
+        mbar_expect_tx(&bars->q_full[qs], Work::kTiles * Cfg::kTileBytes);  // rows past T arrive as zeros
         armed_q[qs] = qph;
 #pragma unroll
-        for (int t = 0; t < 2; ++t)
+        for (int t = 0; t < Work::kTiles; ++t)
 #pragma unroll
             for (int h = 0; h < Cfg::kHalves; ++h)
                 tma_load_tile<kStrided>(smem + Cfg::kOffQ + (qs * 2 + t) * Cfg::kTileBytes + h * kHalfTileBytes, tmQ,
-                              &bars->q_full[qs], wk.orders & 15, h * kBoxCols, blk * kBlockRows + t * kBlockQ, head, batch, bh);
+                              &bars->q_full[qs], wk.orders & 15, h * kBoxCols, blk * Work::kRows + t * kBlockQ, head, batch, bh);
         const int n = max(n_a, n_b);
         for (int j = 0; j < n; ++j, ++g) {
             const int st = g & 1;
@@ -164,8 +168,8 @@ __device__ __forceinline__ void fwd_producer(const CUtensorMap* tmQ, const CUten
     }
 }
 
-template <int D>
-__device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const FwdWork& wk,
+template <int D, typename Work>
+__device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const Work& wk,
                                         long long limit) {
     using Cfg = FwdCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
@@ -342,9 +346,9 @@ __device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t t
     }
 }
 
-template <int D, bool kCausal, bool kStrided>
+template <int D, bool kCausal, bool kStrided, typename Work>
 __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const CUtensorMap* tmO,
-                                            float* __restrict__ LSE, float scale, const FwdWork& wk, int t, int swarp,
+                                            float* __restrict__ LSE, float scale, const Work& wk, int t, int swarp,
                                             int lane, long long limit) {
     using Cfg = FwdCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
@@ -369,7 +373,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
         int blk, bh, n_a, n_b;
         wk.get(item, &blk, &bh, &n_a, &n_b);
         const int n_kv = (t == 0) ? n_a : n_b;
-        const int qt = 2 * blk + t;
+        const int qt = Work::kTiles * blk + t;
         const int row = qt * kBlockQ + row_local;
         const int qs = w % Cfg::kQStages;
         uint8_t* stage = smem + Cfg::kOffQ + (qs * 2 + t) * Cfg::kTileBytes;  // this tile's Q buffer
@@ -565,7 +569,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
     if (leader) bulk_wait_group<0>();  // O must be complete before the kernel ends
 }
 
-template <int D, bool kCausal, bool kStrided>
+template <int D, bool kCausal, bool kStrided, bool kSingle>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -576,7 +580,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     FwdBars* bars = reinterpret_cast<FwdBars*>(smem + Cfg::kOffBar);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const FwdWork wk{n_blocks * BH, BH, n_blocks, (T + kBlockK - 1) / kBlockK, T, H, orders, kCausal};
+    using Work = FwdWork<kSingle>;
+    const Work wk{n_blocks * BH, BH, n_blocks, (T + kBlockK - 1) / kBlockK, T, H, orders, kCausal};
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -619,9 +624,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #pragma unroll
             for (int h = 0; h < Cfg::kHalves; ++h) {
                 tma_prefetch_tile<kStrided>(&tmK, (wk.orders >> 4) & 15, h * kBoxCols, 0, head, batch, bh);
-                tma_prefetch_tile<kStrided>(&tmQ, wk.orders & 15, h * kBoxCols, blk * kBlockRows, head, batch, bh);
+                tma_prefetch_tile<kStrided>(&tmQ, wk.orders & 15, h * kBoxCols, blk * Work::kRows, head, batch, bh);
                 tma_prefetch_tile<kStrided>(&tmV, (wk.orders >> 8) & 15, h * kBoxCols, 0, head, batch, bh);
-                tma_prefetch_tile<kStrided>(&tmQ, wk.orders & 15, h * kBoxCols, blk * kBlockRows + kBlockQ, head, batch, bh);
+                if (!kSingle)
+                    tma_prefetch_tile<kStrided>(&tmQ, wk.orders & 15, h * kBoxCols, blk * Work::kRows + kBlockQ, head, batch, bh);
             }
         }
     }
@@ -646,21 +652,30 @@ template <int D, bool kCausal>
 cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                        const CUtensorMap& tmO, bool strided, uint32_t orders, float* LSE, const AttnShape& s,
                        int num_sms, long long wait_limit, int inject, int* dev_status, cudaStream_t stream) {
-    const int n_blocks = (s.T + kBlockRows - 1) / kBlockRows;
     const int BH = s.B * s.H;
-    const long long n_items = static_cast<long long>(n_blocks) * BH;
-    (void)num_sms;
-    const dim3 grid(static_cast<unsigned>(n_items));  // one CTA per item; those that do not start at once are taken over
-    if (strided)
-        return launch_overlapped(attn_fwd_kernel<D, kCausal, true>, grid, dim3(kFwdThreads), FwdCfg<D>::kSmemBytes,
-                                 stream, tmQ, tmK, tmV, tmO, LSE, s.T, BH, s.H, orders, n_blocks, s.scale, wait_limit, inject, dev_status);
-    return launch_overlapped(attn_fwd_kernel<D, kCausal, false>, grid, dim3(kFwdThreads), FwdCfg<D>::kSmemBytes, stream,
-                             tmQ, tmK, tmV, tmO, LSE, s.T, BH, s.H, orders, n_blocks, s.scale, wait_limit, inject, dev_status);
+    const int n_tiles = (s.T + kBlockQ - 1) / kBlockQ;
+    // Pairs of query tiles share their K and V tiles and fill each other's gaps; but if every tile can have an SM of its
+    // own, a tile is done sooner alone (softmax of one tile: 1450 clocks, of two at a time 2300).  D=64, pairs against
+    // single tiles: B=1, H=12, T=777: 13.6 -> 12.1 us, T=1500: 23.4 -> 18.0 us; H=1, T=8192: 99.5 -> 76.8 us; D=128,
+    // B=1, H=16, T=1024 without the mask: 20.9 -> 18.1 us.
+    const bool single = static_cast<long long>(n_tiles) * BH <= num_sms;
+    const int n_blocks = single ? n_tiles : (n_tiles + 1) / 2;
+    const dim3 grid(static_cast<unsigned>(n_blocks) * BH);  // one CTA per item; those that do not start at once are taken over
+    auto go = [&](auto kernel) {
+        return launch_overlapped(kernel, grid, dim3(kFwdThreads), FwdCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmO, LSE, s.T,
+                                 BH, s.H, orders, n_blocks, s.scale, wait_limit, inject, dev_status);
+    };
+    if (single)
+        return strided ? go(attn_fwd_kernel<D, kCausal, true, true>) : go(attn_fwd_kernel<D, kCausal, false, true>);
+    return strided ? go(attn_fwd_kernel<D, kCausal, true, false>) : go(attn_fwd_kernel<D, kCausal, false, false>);
 }
 
 template <int D, bool kCausal, bool kStrided>
 cudaError_t configure_one() {
-    return cudaFuncSetAttribute(attn_fwd_kernel<D, kCausal, kStrided>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<D, kCausal, kStrided, false>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<D>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(attn_fwd_kernel<D, kCausal, kStrided, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 FwdCfg<D>::kSmemBytes);
 }
 

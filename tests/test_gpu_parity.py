@@ -386,6 +386,31 @@ def test_query_major_passes_at_step_edges(T, D, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"steps T={T} D={D}: ", dO=ref["dO_in"])
 
 
+@pytest.mark.parametrize("T", [1, 127, 129, 256, 257, 384, 500])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_forward_alone_and_in_a_crowd(T, D, causal):
+    """With an SM for every 128-row tile the forward works on one tile per CTA, otherwise on pairs of tiles: a row's
+    arithmetic is the same either way, so 160 copies of a head (pairs, several items per CTA) give the bits of the head
+    alone, on the plain and on a strided layout; the head matches the oracle."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("crowd", B=1, H=1, T=T, D=D, seed=300 + T + D, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    alone = h.run_gpu(Q, K, V, dO, cfg.scale, causal)
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal)
+    h.compare(h.select_heads(alone, None), ref, label=f"alone T={T} D={D}: ", dO=ref["dO_in"])
+    q, k, v = (x.to(dev).expand(8, 20, T, D).contiguous() for x in (Q, K, V))
+    for strided in (False, True):
+        if strided:
+            q, k, v = (x.transpose(1, 2).contiguous().transpose(1, 2) for x in (q, k, v))
+        o, lse = torch.full_like(q, 7.0), torch.full((8, 20, T), 7.0, device=dev)
+        (nova_attn.nova_attn_fwd_strided if strided else nova_attn.nova_attn_fwd)(q, k, v, o, lse, cfg.scale, causal)
+        nova_attn.nova_attn_poll_device_status()
+        assert torch.equal(o.cpu(), alone["O"].expand(8, 20, T, D)) and torch.equal(lse.cpu(), alone["LSE"].expand(8, 20, T))
+
+
 DETERMINISTIC = [  # (B, H, T, D, causal)
     (1, 2, 64, 64, True),
     (2, 3, 300, 64, True),
