@@ -26,19 +26,45 @@ __device__ __forceinline__ float dot8_bf16(const uint4& a, const uint4& b) {
     return acc;
 }
 
-// Offset, in 16-byte units, of row r = (b*H + h)*T + t of a tensor with strides `s`.
-__device__ __forceinline__ long long row_offset16(long long r, int H, int T, const TensorStrides& s) {
-    const long long bh = r / T;
-    const long long t = r - bh * T;
-    const long long b = bh / H;
-    const long long h = bh - b * H;
+// n / d for 0 <= n < 2^31 without a division instruction (Granlund and Montgomery, "Division by Invariant Integers using
+// Multiplication", 1994): with 2^(s-1) < d <= 2^s and m = floor(2^32 (2^s - d) / d) + 1 the quotient is
+// (umulhi(n, m) + n) >> s, and the sum stays below 2^32.
+struct FastDiv {
+    uint32_t m, s, d;
+    explicit FastDiv(int divisor) : m(0), s(0), d(static_cast<uint32_t>(divisor)) {
+        while ((1ull << s) < d) ++s;
+        m = static_cast<uint32_t>(((1ull << 32) * ((1ull << s) - d)) / d + 1);
+    }
+    __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(n, m) + n) >> s; }
+};
+
+// How a row index r = (b*H + h)*T + t is split again for strided tensors.
+struct RowSplit {
+    FastDiv T, H;
+    int wide;  // 2^31 rows or more
+};
+
+// Offset, in 16-byte units, of row r of a tensor with strides `s`.
+__device__ __forceinline__ long long row_offset16(long long r, const RowSplit& rs, const TensorStrides& s) {
+    uint32_t t, b, h;
+    if (rs.wide) {
+        const long long bh = r / rs.T.d;
+        t = static_cast<uint32_t>(r - bh * rs.T.d);
+        b = static_cast<uint32_t>(bh / rs.H.d);
+        h = static_cast<uint32_t>(bh - static_cast<long long>(b) * rs.H.d);
+    } else {
+        const uint32_t r32 = static_cast<uint32_t>(r), bh = rs.T.div(r32);
+        t = r32 - bh * rs.T.d;
+        b = rs.H.div(bh);
+        h = bh - b * rs.H.d;
+    }
     return (b * s.b + h * s.h + t * s.t) >> 3;
 }
 
 // LPR = lanes per row = D/8 (8 for D=64, 16 for D=128); each lane owns 8 consecutive bf16.
 template <int LPR, int UNROLL, bool kContiguous>
 __global__ void __launch_bounds__(256) bwd_preprocess_kernel(const uint4* __restrict__ O, const uint4* __restrict__ dO,
-                                                             float* __restrict__ Delta, long long rows, int H, int T,
+                                                             float* __restrict__ Delta, long long rows, const RowSplit rs,
                                                              const TensorStrides so, const TensorStrides sdo) {
     griddep_launch_dependents();
     griddep_wait();
@@ -53,8 +79,8 @@ __global__ void __launch_bounds__(256) bwd_preprocess_kernel(const uint4* __rest
         for (int u = 0; u < UNROLL; ++u) {
             const long long ru = r + u * rows_per_pass;
             if (ru < rows) {
-                a[u] = __ldg(O + (kContiguous ? ru * LPR : row_offset16(ru, H, T, so)) + sub);
-                b[u] = __ldg(dO + (kContiguous ? ru * LPR : row_offset16(ru, H, T, sdo)) + sub);
+                a[u] = __ldg(O + (kContiguous ? ru * LPR : row_offset16(ru, rs, so)) + sub);
+                b[u] = __ldg(dO + (kContiguous ? ru * LPR : row_offset16(ru, rs, sdo)) + sub);
             } else {
                 a[u] = make_uint4(0, 0, 0, 0);
                 b[u] = make_uint4(0, 0, 0, 0);
@@ -71,13 +97,62 @@ __global__ void __launch_bounds__(256) bwd_preprocess_kernel(const uint4* __rest
     }
 }
 
+// Heads inside tokens (O and dO as [B,T,H,D] views): a block takes kTokTile tokens of kTokHeads heads, reads them in the order
+// in which they lie in memory, kTokHeads * 2 * D bytes at a time, and turns the sums round in shared memory, so that
+// Delta [B,H,T] is written in lines as well.  Head by head through such a layout (128 bytes every 2 KB) reading took
+// 10.8 us at B=8, H=16, T=1024, D=64 and 18.5 us at B=4, H=32, T=1000, D=128, against 8.5 and 14.1 us here; in memory
+// order with the sums written as they come 16 and 28 us.  Tiles of 32 tokens: 7.4 to 10 and 17.6 us.
+constexpr int kTokTile = 16, kTokHeads = 8;
+
+template <int LPR>
+__global__ void __launch_bounds__(256, 4) bwd_preprocess_tokens_kernel(const uint4* __restrict__ O, const uint4* __restrict__ dO,
+                                                                    float* __restrict__ Delta, int H, int T, int t_tiles,
+                                                                    int h_tiles, const TensorStrides so,
+                                                                    const TensorStrides sdo) {
+    constexpr int kRowsPerPass = 256 / LPR, kPasses = kTokTile * kTokHeads / kRowsPerPass, kUnroll = 4;
+    __shared__ float sums[kTokHeads][kTokTile + 1];
+    griddep_launch_dependents();
+    const int h0 = static_cast<int>(blockIdx.x) % h_tiles * kTokHeads;
+    const int bt = static_cast<int>(blockIdx.x) / h_tiles, t0 = bt % t_tiles * kTokTile;
+    const long long b = bt / t_tiles;
+    const int sub = threadIdx.x % LPR, row0 = threadIdx.x / LPR;
+    const uint4* po = O + ((b * so.b) >> 3) + sub;
+    const uint4* pd = dO + ((b * sdo.b) >> 3) + sub;
+    griddep_wait();
+#pragma unroll
+    for (int p = 0; p < kPasses; p += kUnroll) {
+        uint4 x[kUnroll], y[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const int r = row0 + (p + u) * kRowsPerPass, t = t0 + r / kTokHeads, h = h0 + r % kTokHeads;
+            x[u] = y[u] = make_uint4(0, 0, 0, 0);
+            if (t < T && h < H) {
+                x[u] = __ldg(po + ((h * so.h + t * so.t) >> 3));
+                y[u] = __ldg(pd + ((h * sdo.h + t * sdo.t) >> 3));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            float acc = dot8_bf16(x[u], y[u]);
+#pragma unroll
+            for (int off = LPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            const int r = row0 + (p + u) * kRowsPerPass;
+            if (sub == 0) sums[r % kTokHeads][r / kTokHeads] = acc;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x >= kTokTile * kTokHeads) return;
+    const int h = h0 + threadIdx.x / kTokTile, t = t0 + threadIdx.x % kTokTile;
+    if (h < H && t < T) Delta[(b * H + h) * T + t] = sums[threadIdx.x / kTokTile][threadIdx.x % kTokTile];
+}
+
 // Each thread takes kConvertItems groups of 8 elements per pass and issues all their loads before the
 // first store.
 constexpr int kConvertItems = 4;
 
 template <bool kContiguous>
 __global__ void __launch_bounds__(256) dq_convert_kernel(const float4* __restrict__ acc, uint4* __restrict__ dQ,
-                                                         long long n8, float scale, int lpr_shift, int H, int T,
+                                                         long long n8, float scale, int lpr_shift, const RowSplit rs,
                                                          const TensorStrides sdq) {
     griddep_launch_dependents();
     griddep_wait();
@@ -106,7 +181,7 @@ __global__ void __launch_bounds__(256) dq_convert_kernel(const float4* __restric
                 dQ[i] = v;
             } else {
                 const long long r = i >> lpr_shift;
-                dQ[row_offset16(r, H, T, sdq) + (i - (r << lpr_shift))] = v;
+                dQ[row_offset16(r, rs, sdq) + (i - (r << lpr_shift))] = v;
             }
         }
     }
@@ -134,6 +209,9 @@ cudaError_t launch_zero(void* ptr, size_t bytes, int num_sms, cudaStream_t strea
 }
 
 namespace {
+RowSplit split_of(const AttnShape& s) {
+    return RowSplit{FastDiv(s.T), FastDiv(s.H), static_cast<long long>(s.B) * s.H * s.T >= (1ll << 31) ? 1 : 0};
+}
 bool is_contiguous(const AttnShape& s, const TensorStrides& st) {
     return st.t == s.D && st.h == static_cast<long long>(s.T) * s.D && st.b == static_cast<long long>(s.H) * s.T * s.D;
 }
@@ -154,8 +232,17 @@ cudaError_t launch_attn_bwd_preprocess(const __nv_bfloat16* O, const __nv_bfloat
     const uint4* d4 = reinterpret_cast<const uint4*>(dO);
     const dim3 grid(static_cast<unsigned>(blocks));
     const bool contiguous = is_contiguous(s, so) && is_contiguous(s, sdo);
+    const int t_tiles = (s.T + kTokTile - 1) / kTokTile, h_tiles = (s.H + kTokHeads - 1) / kTokHeads;
+    const long long token_blocks = static_cast<long long>(s.B) * t_tiles * h_tiles;
+    if (!contiguous && so.h < so.t && sdo.h < sdo.t && token_blocks <= 0x7fffffff) {
+        auto go = [&](auto kernel) {
+            return launch_overlapped(kernel, dim3(static_cast<unsigned>(token_blocks)), dim3(kThreads), 0, stream, o4, d4,
+                                     Delta, s.H, s.T, t_tiles, h_tiles, so, sdo);
+        };
+        return s.D == 64 ? go(bwd_preprocess_tokens_kernel<8>) : go(bwd_preprocess_tokens_kernel<16>);
+    }
     auto go = [&](auto kernel) {
-        return launch_overlapped(kernel, grid, dim3(kThreads), 0, stream, o4, d4, Delta, rows, s.H, s.T, so, sdo);
+        return launch_overlapped(kernel, grid, dim3(kThreads), 0, stream, o4, d4, Delta, rows, split_of(s), so, sdo);
     };
     if (s.D == 64) return contiguous ? go(bwd_preprocess_kernel<8, kUnroll, true>) : go(bwd_preprocess_kernel<8, kUnroll, false>);
     return contiguous ? go(bwd_preprocess_kernel<16, kUnroll, true>) : go(bwd_preprocess_kernel<16, kUnroll, false>);
@@ -173,7 +260,7 @@ cudaError_t launch_dq_convert(const float* dq_acc, __nv_bfloat16* dQ, const Attn
     const dim3 grid(static_cast<unsigned>(blocks));
     auto go = [&](auto kernel) {
         return launch_overlapped(kernel, grid, dim3(kThreads), 0, stream, reinterpret_cast<const float4*>(dq_acc),
-                                 reinterpret_cast<uint4*>(dQ), n8, scale, lpr_shift, s.H, s.T, sdq);
+                                 reinterpret_cast<uint4*>(dQ), n8, scale, lpr_shift, split_of(s), sdq);
     };
     return is_contiguous(s, sdq) ? go(dq_convert_kernel<true>) : go(dq_convert_kernel<false>);
 }

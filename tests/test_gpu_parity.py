@@ -231,6 +231,24 @@ def test_preprocess_matches_rowsum():
         torch.testing.assert_close(Delta.cpu().double(), ref, rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("B,H,T", [(1, 1, 1), (2, 7, 33), (1, 9, 16), (3, 8, 257), (16, 12, 513), (4, 12, 1024)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_preprocess_with_heads_inside_tokens(B, H, T, D):
+    """O and dO as views of [B,T,H,D] buffers take the path that reads in memory order: tiles of tokens and heads with
+    remainders of both, few and many blocks; the same sums in the same order as the plain path, so the same bits."""
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    g = torch.Generator().manual_seed(B + H + T + D)
+    O, dO = (torch.randn((B, T, H, D), generator=g).to(torch.bfloat16).to(dev).permute(0, 2, 1, 3) for _ in range(2))
+    buf = torch.full((B * H * T + 128,), 3.0, device=dev)
+    Delta, plain = buf[64:-64].view(B, H, T), torch.empty((B, H, T), device=dev)
+    nova_attn.nova_attn_bwd_preprocess_strided(O, dO, Delta)
+    nova_attn.nova_attn_bwd_preprocess(O.contiguous(), dO.contiguous(), plain)
+    nova_attn.nova_attn_poll_device_status()
+    assert torch.equal(Delta, plain)
+    assert bool((buf[:64] == 3.0).all()) and bool((buf[-64:] == 3.0).all())
+
+
 def test_back_to_back_steps_on_shared_buffers():
     """Every kernel may start while its predecessor in the stream is still draining, and waits for it
     before touching global memory.  Twelve forward + backward steps are enqueued without a host
