@@ -22,7 +22,8 @@
 //   warp 1       UMMA issuer, software-pipelined: S^T of the next query tile is issued as soon as the
 //                compute warps have read the current one; dK, dQ and the next dP^T run while they
 //                work on the next P
-//   warps 2-3    row loader: -LSE*log2e and -Delta of the query tile into shared memory
+//   warps 2-3    row loader: -LSE*log2e and -Delta of the query tile into shared memory (D=64: -LSE/scale and -Delta as
+//                operands of the products, see kFold)
 //   warps 4-11   compute: thread = (key row, 64-query half); P phase then dS phase per tile
 //                (at D=128 they also send dV and dK at the end of an item, through the dS^T staging buffer)
 //   warps 12-15  dQ: one thread per row moves the partial dQ tile from TMEM into the fp32 accumulator
@@ -49,6 +50,8 @@ namespace nova {
 namespace {
 
 constexpr int kBwdTmemCols = 512;
+// LSE/scale has to be finite.  Below this scale the scores add nothing to P (|s| < 1e6 at most), with it or without.
+constexpr float kLeastScale = 1e-30f;
 
 template <int D>
 struct BwdCfg {
@@ -70,7 +73,16 @@ struct BwdCfg {
     // dQ warps then send out too: kBulkdQ).
     static constexpr bool kBulkdQ = (D == 64);
     static constexpr int kStageBytes = 2 * kHalfTileBytes;
-    static constexpr int kOffStage = kOffRow + 2 * 2 * 128 * 4;
+    // At D=64 the row terms enter S^T and dP^T through the tensor core: one more instruction per product multiplies a
+    // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale and -Delta, each as three bf16 numbers
+    // that add up to it exactly to 24 bits.  The compute warps then read no rows from shared memory (512 broadcasts of
+    // 16 bytes a tile, some 600 clocks of its one port, which the operands of the products need as well) and have an
+    // fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at B=32, 337 -> 321 us at
+    // B=1, T=8192, 214 -> 182 us at B=4, T=2048 without the mask.  D=128 has no shared memory left for the tiles.
+    static constexpr bool kFold = (D == 64);
+    static constexpr int kExtBytes = 128 * 16 * 2;
+    static constexpr int kOffExt = kOffRow;                           // kFold: 2 stages, then the constants for S^T and dP^T
+    static constexpr int kOffStage = kOffRow + (kFold ? 4 * kExtBytes : 2 * 2 * 128 * 4);
     static constexpr int kOffBar = kOffStage + kStageBytes;
     // At D=128 the tiles fill the 227 KB a CTA can have to within 512 bytes, so there is no room for
     // the padding that would let the kernel align its window itself: the kernel checks that the window
@@ -209,13 +221,22 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     // The whole warp runs this role in uniform control flow; one elected lane issues.
     const bool el = elect_one();
 
+    // The row terms of tile gq: unswizzled tiles, 8 x 16-byte core matrices 128 bytes apart along K, 256 along M and N.
+    const uint32_t ext_hi = umma_desc_hi_plain(256);
+    const uint32_t ext_b = umma_desc_lo(smem_u32(smem + Cfg::kOffExt), 128);
+    constexpr uint32_t kExtStep = Cfg::kExtBytes >> 4;
+    (void)ext_hi, (void)ext_b;
+
     auto issue_st = [&](int gq, uint32_t kd) {  // S^T = K Q^T: K tile `kd`, query tile in Q stage gq % kQStages
         const uint32_t b = q_k0 + (gq % Cfg::kQStages) * kQStageStep;
         if (el) {
+            if (Cfg::kFold)
+                umma_ss(t_s, umma_desc_join(ext_b + 2 * kExtStep, ext_hi), umma_desc_join(ext_b + (gq & 1) * kExtStep, ext_hi),
+                        kIdescT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
                 const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
-                umma_ss(t_s, umma_desc_join(kd + off, hi), umma_desc_join(b + off, hi), kIdescT, k > 0 ? 1u : 0u);
+                umma_ss(t_s, umma_desc_join(kd + off, hi), umma_desc_join(b + off, hi), kIdescT, (Cfg::kFold || k > 0) ? 1u : 0u);
             }
             tc_commit(&bars->s_full);
         }
@@ -224,12 +245,16 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     auto issue_dpt = [&](int gq, uint32_t vd) {  // dP^T = V dO^T: V tile `vd`, query tile in dO stage gq % kdOStages
         const uint32_t b = do_k[gq % Cfg::kdOStages];
         if (el) {
+            if (Cfg::kFold)
+                umma_ss(t_dp, umma_desc_join(ext_b + 3 * kExtStep, ext_hi), umma_desc_join(ext_b + (gq & 1) * kExtStep, ext_hi),
+                        kIdescT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
                 const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
-                umma_ss(t_dp, umma_desc_join(vd + off, hi), umma_desc_join(b + off, hi), kIdescT, k > 0 ? 1u : 0u);
+                umma_ss(t_dp, umma_desc_join(vd + off, hi), umma_desc_join(b + off, hi), kIdescT, (Cfg::kFold || k > 0) ? 1u : 0u);
             }
             tc_commit(&bars->dp_full);
+            if (Cfg::kFold) tc_commit(&bars->row_empty[gq & 1]);
         }
         __syncwarp();
     };
@@ -258,6 +283,8 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
         if (ok) ok = mbar_wait(&bars->q_full[g % Cfg::kQStages], (g / Cfg::kQStages) & 1, abort_flag);
         if (ok && Cfg::kdQAliased && g > 0 && !wl.no_dq()) ok = mbar_wait(&bars->dq_free, (g - 1) & 1, abort_flag);
         if (ok) ok = mbar_wait(&bars->do_full[g % Cfg::kdOStages], (g / Cfg::kdOStages) & 1, abort_flag);
+        // (queued already: its row terms may have been read, and their buffer filled again, by now)
+        if (ok && Cfg::kFold && !first_queued) ok = mbar_wait(&bars->row_full[g & 1], (g >> 1) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
         // The S^T and dP^T columns are free: the last dV / dK (and, at D=128, the dQ read-out) of the
@@ -276,6 +303,7 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
             if (Cfg::kSeparateP && (more || cross)) {  // S^T columns are free as soon as the compute warps have read them
                 if (cross) ok = mbar_wait(&bars->kv_full[ks_n], ((w + 1) / Cfg::kKVStages) & 1, abort_flag);
                 if (ok) ok = mbar_wait(&bars->q_full[(g + 1) % Cfg::kQStages], ((g + 1) / Cfg::kQStages) & 1, abort_flag);
+                if (ok && Cfg::kFold) ok = mbar_wait(&bars->row_full[(g + 1) & 1], ((g + 1) >> 1) & 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 issue_st(g + 1, cross ? k_k_n : k_k);
@@ -385,6 +413,54 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     }
 }
 
+// Three bf16 numbers that add up to v (to 24 bits), as the lower 16 bits of three words.
+__device__ __forceinline__ void split_bf16x3(float v, uint32_t* hi, uint32_t* mid, uint32_t* lo) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    const float r = v - __bfloat162float(h);
+    const __nv_bfloat16 m = __float2bfloat16_rn(r);
+    const __nv_bfloat16 l = __float2bfloat16_rn(r - __bfloat162float(m));
+    *hi = __bfloat16_as_ushort(h);
+    *mid = __bfloat16_as_ushort(m);
+    *lo = __bfloat16_as_ushort(l);
+}
+
+// Row loader where the row terms go through the tensor core (kFold): one row of the (queries x 16) tile per query, 16
+// bytes: -LSE/scale in columns 0-2, -Delta in 3-5.  Queries past the end of the sequence get -1e30, so that their P is 0.
+__device__ __forceinline__ void bwd_rows_folded(BwdBars* bars, uint8_t* ext, const float* __restrict__ LSE,
+                                                const float* __restrict__ Delta, int T, float inv_scale,
+                                                const WorkList& wl, int tid64) {
+    volatile int* abort_flag = &bars->abort_flag;
+    int g = 0;
+    for (WorkCursor cur; !wl.done(cur); wl.advance(cur)) {
+        int kt, bh, i0, n_it;
+        if (!wl.get(cur, &kt, &bh, &i0, &n_it)) continue;
+        const size_t row_base = static_cast<size_t>(bh) * T;
+        for (int it = 0; it < n_it; ++it, ++g) {
+            const int b = g & 1;
+            uint4 v[2];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const int q = (i0 + it) * kBlockQ + tid64 + 64 * x;
+                const float l = (q < T) ? -LSE[row_base + q] * inv_scale : -1e30f;
+                const float d = (q < T) ? -Delta[row_base + q] : 0.f;
+                uint32_t w[6];
+                split_bf16x3(l, w + 0, w + 1, w + 2);
+                split_bf16x3(d, w + 3, w + 4, w + 5);
+                v[x] = make_uint4(w[0] | (w[1] << 16), w[2] | (w[3] << 16), w[4] | (w[5] << 16), 0u);
+            }
+            if (!mbar_wait(&bars->row_empty[b], ((g >> 1) & 1) ^ 1, abort_flag)) return;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const int rl = tid64 + 64 * x;
+                *reinterpret_cast<uint4*>(ext + b * BwdCfg<64>::kExtBytes + (rl >> 3) * 256 + (rl & 7) * 16) = v[x];
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if ((tid64 & 31) == 0) mbar_arrive(&bars->row_full[b]);
+        }
+    }
+}
+
 // Row loader: -LSE*log2e and -Delta of each query tile into the double-buffered row arrays (negated,
 // so that the compute warps fold them in with a packed fma / add).
 __device__ __forceinline__ void bwd_rows(BwdBars* bars, float* row_buf, const float* __restrict__ LSE,
@@ -418,18 +494,24 @@ __device__ __forceinline__ void bwd_rows(BwdBars* bars, float* row_buf, const fl
 // (the dS phase multiplies by the unrounded p: only what feeds a contraction is rounded to bf16, paper
 // Section 4.3).  `s_lse4` holds -lse*log2e; the multiply-add runs on packed fp32 pairs.
 // kMasked: the tile is the diagonal one and/or holds keys past the end of the sequence.
-template <bool kMasked, int N>
+// kFold: the scores arrive as s - lse/scale, and `s_lse4` is not used.
+template <bool kMasked, bool kFold, int N>
 __device__ __forceinline__ void bwd_p_phase(uint32_t (&sv)[N], const float4* s_lse4, float c, bool key_valid, bool diag,
                                             int r, int q_base) {
 #pragma unroll
     for (int g = 0; g < N / 4; ++g) {
-        const float4 l4 = s_lse4[g];
         const uint64_t c2 = f32x2_pack(c, c);
+        const uint64_t s01 = f32x2_pack(__uint_as_float(sv[4 * g + 0]), __uint_as_float(sv[4 * g + 1]));
+        const uint64_t s23 = f32x2_pack(__uint_as_float(sv[4 * g + 2]), __uint_as_float(sv[4 * g + 3]));
         float x0, x1, x2, x3;
-        f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sv[4 * g + 0]), __uint_as_float(sv[4 * g + 1])), c2,
-                               f32x2_pack(l4.x, l4.y)), x0, x1);
-        f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sv[4 * g + 2]), __uint_as_float(sv[4 * g + 3])), c2,
-                               f32x2_pack(l4.z, l4.w)), x2, x3);
+        if constexpr (kFold) {
+            f32x2_unpack(f32x2_mul(s01, c2), x0, x1);
+            f32x2_unpack(f32x2_mul(s23, c2), x2, x3);
+        } else {
+            const float4 l4 = s_lse4[g];
+            f32x2_unpack(f32x2_fma(s01, c2, f32x2_pack(l4.x, l4.y)), x0, x1);
+            f32x2_unpack(f32x2_fma(s23, c2, f32x2_pack(l4.z, l4.w)), x2, x3);
+        }
         float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
         if (kMasked) {
             // keep (query q, key r) iff the key exists and, on the diagonal tile, key <= query
@@ -459,7 +541,7 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
     const int part = cwarp >> 2;             // which kQPT queries of the tile this thread covers
     const int half = (part * kQPT) / 64;     // the 64-query half they lie in (a box of the dS^T staging buffer)
     const int r = lane_base + lane;          // local key row
-    const float c = scale * kLog2e;
+    const float c = (Cfg::kFold ? fmaxf(scale, kLeastScale) : scale) * kLog2e;
     const uint32_t t_s = tmem_addr(tmem_base, lane_base, Cfg::kColS + kQPT * part);
     const uint32_t t_dp = tmem_addr(tmem_base, lane_base, Cfg::kColdP + kQPT * part);
     // bf16 P^T: kQPT / 2 packed columns, in columns of their own or over this thread's own S^T columns
@@ -485,7 +567,7 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
             const float4* s_dl4 = reinterpret_cast<const float4*>(row_buf + b * 256 + 128 + kQPT * part);
             // Three non-blocking probes issued together, so that their latencies overlap; each is followed up by
             // a proper wait only if it failed (-2 % against three waits in a row).
-            const bool row_there = mbar_test(&bars->row_full[b], (g >> 1) & 1);
+            const bool row_there = Cfg::kFold || mbar_test(&bars->row_full[b], (g >> 1) & 1);
             const bool s_there = mbar_test(&bars->s_full, g & 1);
             const bool dp_there = mbar_test(&bars->dp_full, g & 1);
             if (!row_there) ok = mbar_wait(&bars->row_full[b], (g >> 1) & 1, abort_flag);
@@ -501,9 +583,9 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
             {
                 const bool diag = kCausal && (i == kt);
                 if (diag || !tile_keys_valid)
-                    bwd_p_phase<true, kQPT>(pf, s_lse4, c, key_valid, diag, r, kQPT * part);
+                    bwd_p_phase<true, Cfg::kFold, kQPT>(pf, s_lse4, c, key_valid, diag, r, kQPT * part);
                 else
-                    bwd_p_phase<false, kQPT>(pf, s_lse4, c, true, false, r, kQPT * part);
+                    bwd_p_phase<false, Cfg::kFold, kQPT>(pf, s_lse4, c, true, false, r, kQPT * part);
             }
             // P^T as bf16 into TMEM for dV.  Where P^T has columns of its own (kEarlydP) the store must wait
             // until dV of the previous tile has read them: dP^T of this tile was queued after that dV and the
@@ -546,14 +628,16 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
                 uint32_t dd[8];
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
-                    const float4 d4 = s_dl4[x / 4 + y];  // holds -delta
+                    uint64_t e01 = f32x2_pack(__uint_as_float(dv[4 * y + 0]), __uint_as_float(dv[4 * y + 1]));
+                    uint64_t e23 = f32x2_pack(__uint_as_float(dv[4 * y + 2]), __uint_as_float(dv[4 * y + 3]));
+                    if constexpr (!Cfg::kFold) {
+                        const float4 d4 = s_dl4[x / 4 + y];  // holds -delta
+                        e01 = f32x2_add(e01, f32x2_pack(d4.x, d4.y));
+                        e23 = f32x2_add(e23, f32x2_pack(d4.z, d4.w));
+                    }
                     float d0, d1, d2, d3;
-                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(pf[x + 4 * y + 0]), __uint_as_float(pf[x + 4 * y + 1])),
-                                           f32x2_add(f32x2_pack(__uint_as_float(dv[4 * y + 0]), __uint_as_float(dv[4 * y + 1])),
-                                                     f32x2_pack(d4.x, d4.y))), d0, d1);
-                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(pf[x + 4 * y + 2]), __uint_as_float(pf[x + 4 * y + 3])),
-                                           f32x2_add(f32x2_pack(__uint_as_float(dv[4 * y + 2]), __uint_as_float(dv[4 * y + 3])),
-                                                     f32x2_pack(d4.z, d4.w))), d2, d3);
+                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(pf[x + 4 * y + 0]), __uint_as_float(pf[x + 4 * y + 1])), e01), d0, d1);
+                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(pf[x + 4 * y + 2]), __uint_as_float(pf[x + 4 * y + 3])), e23), d2, d3);
                     dd[2 * y + 0] = pack_bf16x2(d0, d1);
                     dd[2 * y + 1] = pack_bf16x2(d2, d3);
                 }
@@ -571,7 +655,7 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&bars->ds_ready);
-                mbar_arrive(&bars->row_empty[b]);
+                if (!Cfg::kFold) mbar_arrive(&bars->row_empty[b]);
             }
         }
         if (!ok) break;
@@ -963,7 +1047,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             mbar_init(&bars->do_full[s], 1);
             mbar_init(&bars->do_empty[s], 1);
             mbar_init(&bars->row_full[s], 2);
-            mbar_init(&bars->row_empty[s], Cfg::kComputeWarps);
+            mbar_init(&bars->row_empty[s], Cfg::kFold ? 1 : Cfg::kComputeWarps);
         }
         mbar_init(&bars->s_full, 1);
         mbar_init(&bars->dp_full, 1);
@@ -986,6 +1070,18 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         tma_prefetch_desc(&tmAcc);
         tma_prefetch_desc(&tmdK);
         tma_prefetch_desc(&tmdV);
+    }
+    if constexpr (Cfg::kFold) {
+        // zeros in the stages, ones in columns 0-2 and 3-5 of the two tiles of constants
+        for (int i = threadIdx.x; i < 4 * Cfg::kExtBytes / 16; i += Cfg::kThreads) {
+            const int tile = i / (Cfg::kExtBytes / 16);
+            const bool first_half = ((i >> 3) & 1) == 0;  // core matrix of columns 0-7
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (first_half && tile == 2) v = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
+            if (first_half && tile == 3) v = make_uint4(0u, 0x3f800000u, 0x3f803f80u, 0u);
+            *reinterpret_cast<uint4*>(smem + Cfg::kOffExt + 16 * i) = v;
+        }
+        fence_proxy_async_smem();
     }
     if (warp == 1) {
         tmem_alloc(&bars->tmem_base, kBwdTmemCols);
@@ -1016,7 +1112,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     } else if (warp == 1) {
         bwd_mma<D>(smem, bars, tmem_base, wl);
     } else if (warp < 4) {
-        bwd_rows(bars, reinterpret_cast<float*>(smem + Cfg::kOffRow), LSE, Delta, T, wl, (warp - 2) * 32 + lane);
+        if constexpr (Cfg::kFold)
+            bwd_rows_folded(bars, smem + Cfg::kOffExt, LSE, Delta, T, 1.0f / fmaxf(scale, kLeastScale), wl, (warp - 2) * 32 + lane);
+        else
+            bwd_rows(bars, reinterpret_cast<float*>(smem + Cfg::kOffRow), LSE, Delta, T, wl, (warp - 2) * 32 + lane);
     } else if (warp < 4 + Cfg::kComputeWarps) {
         bwd_compute<D, kCausal, kStrided>(smem, bars, tmem_base, &tmdK, &tmdV, T, scale, wl, warp - 4, lane);
     } else {

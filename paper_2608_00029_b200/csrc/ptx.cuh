@@ -387,6 +387,11 @@ __device__ __forceinline__ uint64_t umma_smem_desc_sw128(uint32_t smem_addr, uin
 __device__ __forceinline__ uint32_t umma_desc_hi_sw128(uint32_t sbo_bytes) {
     return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);
 }
+// Upper word for an unswizzled operand (8-row x 16-byte core matrices, each 128 contiguous bytes).  K-major: `lbo_bytes`
+// = distance between core matrices along K, `sbo_bytes` = distance between 8-row groups.
+__device__ __forceinline__ uint32_t umma_desc_hi_plain(uint32_t sbo_bytes) {
+    return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14);
+}
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t smem_addr, uint32_t lbo_bytes) {
     return ((smem_addr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }

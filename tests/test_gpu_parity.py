@@ -429,6 +429,22 @@ def test_forward_alone_and_in_a_crowd(T, D, causal):
         assert torch.equal(o.cpu(), alone["O"].expand(8, 20, T, D)) and torch.equal(lse.cpu(), alone["LSE"].expand(8, 20, T))
 
 
+@pytest.mark.parametrize("scale,qk", [(1e-36, 1.0), (1e-20, 1.0), (12.5, 0.01)])
+@pytest.mark.parametrize("T", [100, 300])
+def test_scales_far_from_ordinary(scale, qk, T):
+    """At D=64 the backward subtracts LSE/scale from the scores inside the contraction, as three bf16 numbers: a scale at
+    which that quotient would not be finite (P is uniform there), one at which it dwarfs the scores, and a large one.
+    dQ carries the rounding of dS times scale * |K|, and the harness's bounds are stated for scale * |K| = 1/8 (unit K,
+    D=64): K is scaled down with the large scale so that this holds (at scale 30 and |K| = 0.1 the bound would be 24
+    times theirs)."""
+    h = _harness()
+    cfg = W.AttnConfig("scales", B=1, H=2, T=T, D=64, seed=77, qk_factor=qk)
+    Q, K, V, dO = W.make_inputs(cfg)
+    got = h.run_gpu(Q, K, V, dO, scale, True, exact_delta=True)
+    ref = h.run_oracle(Q, K, V, dO, scale, True)
+    h.compare(h.select_heads(got, None), ref, label=f"scale={scale}: ", dO=ref["dO_in"], rms=scale > 1)
+
+
 DETERMINISTIC = [  # (B, H, T, D, causal)
     (1, 2, 64, 64, True),
     (2, 3, 300, 64, True),
