@@ -77,6 +77,7 @@ int device_state(DeviceState** out) {
         e = configure_attn_fwd();
         if (e == cudaSuccess) e = configure_attn_bwd();
         if (e == cudaSuccess) e = configure_attn_dq();
+        if (e == cudaSuccess) e = configure_attn_dkdv();
         if (e == cudaSuccess) e = configure_lmhead();
         if (e == cudaSuccess) e = configure_lmhead_rows();
         if (e == cudaSuccess) e = cudaGetSymbolAddress(reinterpret_cast<void**>(&st.dev_status), g_dev_status);
@@ -484,6 +485,13 @@ int nova_attn_bwd_deterministic(const void* Q, const void* K, const void* V, con
     if (int rc = get_tensor_map(V, D, T, BH, &tmVs, 2, 0, 0, kKeyStep)) return rc;
     cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, false, 0u, LSE, Delta, s, st->dev_status, cs);
     if (e != cudaSuccess) return fail_cuda(e);
+    if (D == 128) {
+        CUtensorMap tmQs, tmdOs;
+        if (int rc = get_tensor_map(Q, D, T, BH, &tmQs, 2, 0, 0, kKeyStep)) return rc;
+        if (int rc = get_tensor_map(dO, D, T, BH, &tmdOs, 2, 0, 0, kKeyStep)) return rc;
+        e = launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, false, 0u, LSE, Delta, s, st->num_sms, st->dev_status, cs);
+        return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
+    }
     // the dK/dV half: the fused kernel without its dQ product (the accumulator map is never used: any map will do)
     e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmQ, tmdK, tmdV, false, 0u, DqMode::kNone, LSE, Delta, static_cast<__nv_bfloat16*>(dK),
                         static_cast<__nv_bfloat16*>(dV), c, c, s, st->num_sms, st->dev_status, cs);

@@ -1,0 +1,577 @@
+// dK and dV of the two-kernel backward at D = 128 (paper Section 4.2, "The Backward Pass": one kernel reduces dQ over
+// keys, the other reduces dK and dV over queries; the probability matrix is rebuilt from the saved log-sum-exp, never
+// stored; the causal loop bound is raised so that queries above the diagonal are never visited).
+//
+// A work item is one 128-key tile of one head; its queries go by in steps of 64.  As in the fused kernel everything is
+// transposed, keys on the lanes of tensor memory, so that P^T and dS^T feed the tensor cores from where they are made:
+//   S^T  = K_j Q_s^T,  dP^T = V_j dO_s^T                       (smem x smem -> one of two buffers in TMEM)
+//   P^T  = exp2(S^T*c - LSE*log2e),  dS^T = P^T * (dP^T - Delta)   (bf16, over the S^T and dP^T they came from)
+//   dV  += P^T dO_s,  dK += dS^T Q_s                           (TMEM x smem, dO and Q read MN-major)
+// Items are handed out dynamically (WorkRing), heaviest first within a chunk of heads whose tensors stay in L2
+// together.  384 threads:
+//   warp 0      TMA producer: K_j and V_j double-buffered, Q_s and dO_s through a ring of 64-query stages
+//   warp 1      UMMA issuer: S^T and dP^T run two steps ahead of dV and dK, across item boundaries
+//   warp 2      row loader: -LSE*log2e and -Delta of a step into shared memory
+//   warps 4-7   compute group 0, warps 8-11 group 1: the steps alternate between the groups; a thread has one key
+//               row and the 64 queries of its step.  At the end of an item group 0 sends dV out, group 1 dK, through the
+//               item's own V and K buffers, which nothing reads any more.
+#include "kernels.h"
+#include "ptx.cuh"
+
+namespace nova {
+namespace {
+
+constexpr int D = 128;
+constexpr int kThreads = 384;
+constexpr int kTmemCols = 512;
+constexpr int kStep = kKeyStep;              // queries per step
+constexpr int kHalfStepBytes = kStep * 128;  // one [64 rows x 64 bf16] box
+constexpr int kHalves = D / kBoxCols;
+constexpr int kTileBytes = kHalves * kHalfTileBytes;
+constexpr int kStepBytes = kHalves * kHalfStepBytes;
+constexpr int kQStages = 3;
+constexpr int kBufs = 2;                     // buffers of S^T and dP^T, one per compute group
+constexpr int kRowStages = 4;
+constexpr int kWorkConsumers = 2 + 8;        // issuer, row loader, compute warps
+static_assert(kQStages >= kBufs, "the issuer runs kBufs steps ahead");
+
+constexpr int kOffK = 0;                                 // [2]
+constexpr int kOffV = 2 * kTileBytes;                    // [2]
+constexpr int kOffQ = 4 * kTileBytes;                    // [kQStages]
+constexpr int kOffdO = kOffQ + kQStages * kStepBytes;    // [kQStages]
+constexpr int kOffRow = kOffdO + kQStages * kStepBytes;  // [kRowStages] x (-LSE*log2e[64], -Delta[64])
+constexpr int kOffBar = kOffRow + kRowStages * 2 * kStep * 4;
+// There is no room to realign the window: the kernel checks that it starts on a 1024-byte boundary.
+constexpr int kSmemBytes = kOffBar + 512;
+static_assert(kSmemBytes <= 232448, "exceeds the shared memory of one CTA");
+constexpr int kColdV = 0, kColdK = D, kColBuf = 2 * D;   // + 128 * buffer: S^T / P^T, then dP^T / dS^T
+
+struct KvBars {
+    uint64_t kv_full[2], kv_empty[2];
+    uint64_t q_full[kQStages], q_empty[kQStages];
+    uint64_t row_full[kRowStages], row_empty[kRowStages];
+    uint64_t sp_full[kBufs], ready[kBufs];  // per buffer: UMMA -> compute group, compute group -> UMMA
+    uint64_t dkv_full, dkv_free;            // dV and dK of an item complete; read out of TMEM
+    uint64_t staged[2];                     // per group: its rows are staged
+    uint64_t drain;
+    WorkRing ring;
+    uint32_t tmem_base;
+    int abort_flag;
+};
+static_assert(sizeof(KvBars) <= 512, "barrier block");
+
+// Work items: 128-key tiles; heads in chunks, heaviest tiles first within a chunk.
+struct KvWork {
+    int BH, n_tiles, chunk, T, H;
+    uint32_t orders;  // coordinate orders of the Q, K, V, dO, dK, dV tensor maps, four bits each
+    bool causal;
+    // Key tile, head, first step and number of steps of item `idx`.
+    __device__ __forceinline__ void get(int idx, int* kt, int* bh, int* s0, int* n) const {
+        const int per_chunk = chunk * n_tiles;
+        const int ck = idx / per_chunk, in = idx - ck * per_chunk;
+        const int heads = min(chunk, BH - ck * chunk);
+        *kt = in / heads;
+        *bh = ck * chunk + in - *kt * heads;
+        *s0 = causal ? *kt * (kBlockK / kStep) : 0;
+        *n = (T + kStep - 1) / kStep - *s0;
+    }
+};
+
+template <bool kStrided>
+__device__ __forceinline__ void kv_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
+                                            const CUtensorMap* tmdO, uint8_t* smem, KvBars* bars, const KvWork& wk) {
+    volatile int* abort_flag = &bars->abort_flag;
+    int armed_kv[2] = {-1, -1}, armed_q[kQStages];
+    for (int s = 0; s < kQStages; ++s) armed_q[s] = -1;
+    bool ok = true, clc_pending = false;
+    int w = 0, st = 0;
+    uint32_t ph = 0;
+    int item = blockIdx.x;
+    for (;;) {
+        ok = bars->ring.publish(w, item, abort_flag, kWaitLimitCycles);
+        if (!ok || item < 0) break;
+        int kt, bh, s0, n;
+        wk.get(item, &kt, &bh, &s0, &n);
+        const int head = kStrided ? bh % wk.H : 0, batch = kStrided ? bh / wk.H : 0;
+        const int ks = w & 1;
+        ok = mbar_wait(&bars->kv_empty[ks], ((w >> 1) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        mbar_expect_tx(&bars->kv_full[ks], 2 * kTileBytes);  // rows past T arrive as zeros
+        armed_kv[ks] = (w >> 1) & 1;
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h) {
+            tma_load_tile<kStrided>(smem + kOffK + ks * kTileBytes + h * kHalfTileBytes, tmK, &bars->kv_full[ks],
+                                    (wk.orders >> 4) & 15, h * kBoxCols, kt * kBlockK, head, batch, bh);
+            tma_load_tile<kStrided>(smem + kOffV + ks * kTileBytes + h * kHalfTileBytes, tmV, &bars->kv_full[ks],
+                                    (wk.orders >> 8) & 15, h * kBoxCols, kt * kBlockK, head, batch, bh);
+        }
+        for (int s = 0; s < n; ++s) {
+            ok = mbar_wait(&bars->q_empty[st], ph ^ 1, abort_flag);
+            if (!ok) break;
+            mbar_expect_tx(&bars->q_full[st], 2 * kStepBytes);
+            armed_q[st] = ph;
+#pragma unroll
+            for (int h = 0; h < kHalves; ++h) {
+                tma_load_tile<kStrided>(smem + kOffQ + st * kStepBytes + h * kHalfStepBytes, tmQ, &bars->q_full[st],
+                                        wk.orders & 15, h * kBoxCols, (s0 + s) * kStep, head, batch, bh);
+                tma_load_tile<kStrided>(smem + kOffdO + st * kStepBytes + h * kHalfStepBytes, tmdO, &bars->q_full[st],
+                                        (wk.orders >> 12) & 15, h * kBoxCols, (s0 + s) * kStep, head, batch, bh);
+            }
+            if (++st == kQStages) {
+                st = 0;
+                ph ^= 1;
+            }
+        }
+        if (!ok) break;
+        // all loads of this item are on their way: claim the next one now, and no earlier
+        bars->ring.request();
+        clc_pending = true;
+        ok = bars->ring.answer(w, &item, abort_flag, kWaitLimitCycles);
+        if (!ok) break;
+        clc_pending = false;
+        ++w;
+    }
+    if (!ok) {  // giving up: let what is in flight land before the CTA's shared memory goes away
+        int none = 0;
+        if (clc_pending) (void)mbar_wait(&bars->ring.answer_bar, w & 1, &none);
+        for (int s = 0; s < 2; ++s)
+            if (armed_kv[s] >= 0) (void)mbar_wait(&bars->kv_full[s], armed_kv[s], &none);
+        for (int s = 0; s < kQStages; ++s)
+            if (armed_q[s] >= 0) (void)mbar_wait(&bars->q_full[s], armed_q[s], &none);
+    }
+}
+
+// UMMA issuer: the whole warp in uniform control flow, one elected lane issues.
+__device__ __forceinline__ void kv_mma(uint8_t* smem, KvBars* bars, uint32_t tmem_base, const KvWork& wk) {
+    volatile int* abort_flag = &bars->abort_flag;
+    constexpr uint32_t kIdescT = umma_idesc_bf16(128, kStep, 0, 0);  // S^T, dP^T
+    constexpr uint32_t kIdescKV = umma_idesc_bf16(128, D, 0, 1);     // dV, dK: A from TMEM, B MN-major
+    const uint32_t hi = umma_desc_hi_sw128(1024);
+    const uint32_t k_k0 = umma_desc_lo(smem_u32(smem + kOffK), 16), v_k0 = umma_desc_lo(smem_u32(smem + kOffV), 16);
+    const uint32_t q_k0 = umma_desc_lo(smem_u32(smem + kOffQ), 16), do_k0 = umma_desc_lo(smem_u32(smem + kOffdO), 16);
+    const uint32_t q_m0 = umma_desc_lo(smem_u32(smem + kOffQ), kHalfStepBytes);
+    const uint32_t do_m0 = umma_desc_lo(smem_u32(smem + kOffdO), kHalfStepBytes);
+    const bool el = elect_one();
+    const int lane = threadIdx.x & 31;
+    bool ok = true;
+
+    // acc[64 columns] = A B^T, both K-major, 16 head-dim elements (32 bytes) per instruction
+    auto product = [&](uint32_t t_acc, uint32_t a, uint32_t b) {
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k)
+            umma_ss(t_acc, umma_desc_join(a + (((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4), hi),
+                    umma_desc_join(b + (((k / 4) * kHalfStepBytes + (k % 4) * 32) >> 4), hi), kIdescT, k > 0 ? 1u : 0u);
+    };
+
+    // Two cursors over the same sequence of steps: `a` is where S^T and dP^T go next, `c` where dV and dK do.  The first
+    // may be in a later item.  Within an item its loads may be waited for: a stage that a step needs was handed back at
+    // least kQStages steps before, i.e. by what `c` has already done.  For the next item's first step nothing is waited
+    // for while there are steps between the cursors (its loads may depend on stages that only `c` frees).
+    int w_a = 0, left_a = 0;          // items taken by `a`; steps left in the latest
+    bool kv_seen = true, more = true; // its K and V have landed; there may be further items
+    int st_a = 0, buf_a = 0;          // Q stage and buffer of `a`
+    uint32_t ph_a = 0;
+    int n_of[2] = {0, 0};             // steps of item w, by w & 1, for `c`
+    int w_c = 0, done_c = 0;          // item of `c` and its steps so far
+    int st_c = 0, buf_c = 0;
+    uint32_t rdy_ph = 0;              // phase of ready[buf_c]
+    int ahead = 0;                    // steps between the cursors
+
+    for (;;) {
+        // ---- S^T and dP^T, as far ahead as buffers and loads allow
+        while (more && ahead < kBufs) {
+            if (left_a == 0 || !kv_seen) {  // first step of an item
+                const bool block = ahead == 0;
+                if (left_a == 0) {
+                    // `c` may be an item behind, not two: its item's number of steps would be overwritten
+                    if (w_a - w_c >= 2) break;
+                    if (!block && !bars->ring.published(w_a)) break;
+                    const int item = bars->ring.take(w_a, lane, abort_flag, kWaitLimitCycles);
+                    if (item < 0) {
+                        ok = (item == -1);
+                        more = false;
+                        break;
+                    }
+                    int kt, bh, s0, n;
+                    wk.get(item, &kt, &bh, &s0, &n);
+                    left_a = n;
+                    if (w_a & 1) n_of[1] = n;
+                    else n_of[0] = n;
+                    ++w_a;
+                    kv_seen = false;
+                }
+                const uint32_t p = ((w_a - 1) >> 1) & 1;
+                if (block) {
+                    ok = mbar_wait(&bars->kv_full[(w_a - 1) & 1], p, abort_flag);
+                    if (ok) ok = mbar_wait(&bars->q_full[st_a], ph_a, abort_flag);
+                    if (!ok) break;
+                } else {
+                    const bool there = mbar_test(&bars->kv_full[(w_a - 1) & 1], p) && mbar_test(&bars->q_full[st_a], ph_a);
+                    if (!__all_sync(0xffffffffu, there)) break;
+                }
+                kv_seen = true;
+            } else {
+                ok = mbar_wait(&bars->q_full[st_a], ph_a, abort_flag);
+                if (!ok) break;
+            }
+            tc_fence_after();
+            // The buffer is free: the dV and dK products that read its P^T and dS^T were queued before this point.
+            if (el) {
+                const int ks = (w_a - 1) & 1;
+                const uint32_t t_b = tmem_base + kColBuf + 128 * buf_a;
+                product(t_b, k_k0 + ks * (kTileBytes >> 4), q_k0 + st_a * (kStepBytes >> 4));
+                product(t_b + 64, v_k0 + ks * (kTileBytes >> 4), do_k0 + st_a * (kStepBytes >> 4));
+                tc_commit(&bars->sp_full[buf_a]);
+            }
+            __syncwarp();
+            --left_a;
+            ++ahead;
+            if (++st_a == kQStages) {
+                st_a = 0;
+                ph_a ^= 1;
+            }
+            buf_a ^= 1;
+        }
+        if (!ok || ahead == 0) break;  // given up, or no items left
+        // ---- dV and dK of the oldest step
+        ok = mbar_wait(&bars->ready[buf_c], rdy_ph, abort_flag);
+        // the previous item's dV and dK must have been read out of TMEM before they are overwritten
+        if (ok && done_c == 0 && w_c > 0) ok = mbar_wait(&bars->dkv_free, (w_c - 1) & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const bool last = done_c + 1 == ((w_c & 1) ? n_of[1] : n_of[0]);
+        if (el) {
+            const uint32_t t_b = tmem_base + kColBuf + 128 * buf_c;
+            const uint32_t b_v = do_m0 + st_c * (kStepBytes >> 4), b_k = q_m0 + st_c * (kStepBytes >> 4);
+#pragma unroll
+            for (int k = 0; k < kStep / 16; ++k)  // 16 queries: 8 packed columns, 16 smem rows = 2048 bytes
+                umma_ts(tmem_base + kColdV, t_b + k * 8, umma_desc_join(b_v + k * 128, hi), kIdescKV,
+                        (done_c > 0 || k > 0) ? 1u : 0u);
+#pragma unroll
+            for (int k = 0; k < kStep / 16; ++k)
+                umma_ts(tmem_base + kColdK, t_b + 64 + k * 8, umma_desc_join(b_k + k * 128, hi), kIdescKV,
+                        (done_c > 0 || k > 0) ? 1u : 0u);
+            tc_commit(&bars->q_empty[st_c]);
+            if (last) tc_commit(&bars->dkv_full);
+        }
+        __syncwarp();
+        --ahead;
+        if (++st_c == kQStages) st_c = 0;
+        rdy_ph ^= buf_c;  // after the second buffer
+        buf_c ^= 1;
+        if (last) {
+            done_c = 0;
+            ++w_c;
+        } else {
+            ++done_c;
+        }
+    }
+    if (!ok) {
+        int none = 0;
+        if (el) tc_commit(&bars->drain);
+        __syncwarp();
+        (void)mbar_wait(&bars->drain, 0, &none);
+    }
+}
+
+// Row loader (one warp): -LSE*log2e and -Delta of each step, negated so that the compute warps fold them in with a packed
+// fma / add.  Queries past the end of the sequence get -inf, so that their P is exactly 0.  The loads of four steps are
+// in flight together.
+__device__ __forceinline__ void kv_row_loader(KvBars* bars, float* row_buf, const float* __restrict__ LSE,
+                                              const float* __restrict__ Delta, const KvWork& wk, int lane) {
+    volatile int* abort_flag = &bars->abort_flag;
+    constexpr int kDeep = 4;
+    int g = 0;
+    for (int w = 0;; ++w) {
+        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
+        if (item < 0) return;
+        int kt, bh, s0, n;
+        wk.get(item, &kt, &bh, &s0, &n);
+        const size_t base = static_cast<size_t>(bh) * wk.T;
+        for (int s = 0; s < n; s += kDeep) {
+            float l[kDeep][2], d[kDeep][2];
+#pragma unroll
+            for (int u = 0; u < kDeep; ++u)
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    const int q = (s0 + s + u) * kStep + lane + 32 * x;
+                    l[u][x] = (q < wk.T) ? LSE[base + q] : INFINITY;
+                    d[u][x] = (q < wk.T) ? Delta[base + q] : 0.f;
+                }
+#pragma unroll
+            for (int u = 0; u < kDeep; ++u) {
+                if (s + u >= n) break;
+                const int b = g % kRowStages;
+                if (!mbar_wait(&bars->row_empty[b], ((g / kRowStages) & 1) ^ 1, abort_flag)) return;
+                float* r = row_buf + b * 2 * kStep;
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    r[lane + 32 * x] = -l[u][x] * kLog2e;
+                    r[kStep + lane + 32 * x] = -d[u][x];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars->row_full[b]);
+                ++g;
+            }
+        }
+    }
+}
+
+// Compute group `grp` (steps g with g % 2 == grp, which are those of buffer `grp`), warp `cwarp` of it.
+template <bool kCausal, bool kStrided>
+__device__ __forceinline__ void kv_compute(uint8_t* smem, KvBars* bars, uint32_t tmem_base, const CUtensorMap* tmdK,
+                                           const CUtensorMap* tmdV, float scale, const KvWork& wk, int grp, int cwarp,
+                                           int lane) {
+    volatile int* abort_flag = &bars->abort_flag;
+    const uint32_t lane_base = 32u * cwarp;
+    const int r = lane_base + lane;  // local key row
+    const bool leader = (cwarp == 0 && lane == 0);
+    const float c = scale * kLog2e;
+    const uint64_t c2 = f32x2_pack(c, c);
+    const float* row_buf = reinterpret_cast<const float*>(smem + kOffRow);
+    const uint32_t t_s = tmem_addr(tmem_base, lane_base, kColBuf + 128 * grp), t_dp = t_s + 64;
+    bool ok = true;
+    int g = 0;             // steps of all items so far
+    int pending_ks = -1;   // K/V stage whose store was issued at the end of the previous item
+
+    for (int w = 0;; ++w) {
+        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
+        if (item < 0) {
+            ok = (item == -1);
+            break;
+        }
+        int kt, bh, s0, n;
+        wk.get(item, &kt, &bh, &s0, &n);
+        const int key = kt * kBlockK + r;
+        for (int s = (g ^ grp) & 1; s < n; s += 2) {
+            const int gs = g + s;
+            const int rb = gs % kRowStages;
+            ok = mbar_wait(&bars->row_full[rb], (gs / kRowStages) & 1, abort_flag);
+            if (ok) ok = mbar_wait(&bars->sp_full[grp], (gs >> 1) & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            const float4* l4 = reinterpret_cast<const float4*>(row_buf + rb * 2 * kStep);
+            const float4* d4 = l4 + kStep / 4;
+            // Keep key <= query.  Keys past the end of the sequence need no mask: their rows are not stored.
+            const bool masked = kCausal && s < kBlockK / kStep;
+            const int first = key - (s0 + s) * kStep;  // first kept query of the step
+            // Half a step at a time, rolled: the two groups are at different places of this loop.
+#pragma unroll 1
+            for (int q = 0; q < kStep; q += 32) {
+                uint32_t sv[32], dv[32], pk[16];
+                tmem_ld_x32(t_s + q, sv);
+                tmem_ld_x32(t_dp + q, dv);
+                tmem_wait_ld();
+                if (masked) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (q + i < first) sv[i] = 0xff800000u;  // -inf: P = 0
+                }
+#pragma unroll
+                for (int i = 0; i < 32; i += 4) {
+                    const float4 l = l4[(q + i) / 4];
+                    float x0, x1, x2, x3;
+                    f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sv[i + 0]), __uint_as_float(sv[i + 1])), c2,
+                                           f32x2_pack(l.x, l.y)), x0, x1);
+                    f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3])), c2,
+                                           f32x2_pack(l.z, l.w)), x2, x3);
+                    x0 = ex2_approx(x0);
+                    x1 = ex2_approx(x1);
+                    x2 = ex2_approx(x2);
+                    x3 = ex2_approx(x3);
+                    pk[i / 2] = pack_bf16x2(x0, x1);
+                    pk[i / 2 + 1] = pack_bf16x2(x2, x3);
+                    // dS^T from the unrounded P^T: only what feeds a contraction is rounded (paper Section 4.3)
+                    const float4 d = d4[(q + i) / 4];
+                    f32x2_unpack(f32x2_mul(f32x2_pack(x0, x1), f32x2_add(f32x2_pack(__uint_as_float(dv[i + 0]),
+                                                                                    __uint_as_float(dv[i + 1])),
+                                                                         f32x2_pack(d.x, d.y))), x0, x1);
+                    f32x2_unpack(f32x2_mul(f32x2_pack(x2, x3), f32x2_add(f32x2_pack(__uint_as_float(dv[i + 2]),
+                                                                                    __uint_as_float(dv[i + 3])),
+                                                                         f32x2_pack(d.z, d.w))), x2, x3);
+                    dv[i / 2] = pack_bf16x2(x0, x1);
+                    dv[i / 2 + 1] = pack_bf16x2(x2, x3);
+                }
+                tmem_st_x16(t_s + q / 2, pk);
+                tmem_st_x16(t_dp + q / 2, dv);
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&bars->ready[grp]);
+                mbar_arrive(&bars->row_empty[rb]);
+            }
+            if (pending_ks >= 0) {  // the copy engine has long read what was staged at the end of the previous item
+                if (leader) {
+                    bulk_wait_group_read<0>();
+                    mbar_arrive(&bars->kv_empty[pending_ks]);
+                }
+                pending_ks = -1;
+                __syncwarp();
+            }
+        }
+        if (!ok) break;
+        // ---- end of the item: dV (group 0) or dK * scale (group 1) as bf16 into the item's V or K buffer
+        const int ks = w & 1;
+        ok = mbar_wait(&bars->dkv_full, w & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t t_o = tmem_addr(tmem_base, lane_base, grp ? kColdK : kColdV);
+        const float f = grp ? scale : 1.0f;
+        uint8_t* stage = smem + (grp ? kOffK : kOffV) + ks * kTileBytes;
+#pragma unroll
+        for (int cb = 0; cb < D; cb += 32) {
+            uint32_t a[32];
+            tmem_ld_x32(t_o + cb, a);
+            tmem_wait_ld();
+            uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + r * 128;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
+                uint4 v;
+                v.x = pack_bf16x2(__uint_as_float(a[8 * x + 0]) * f, __uint_as_float(a[8 * x + 1]) * f);
+                v.y = pack_bf16x2(__uint_as_float(a[8 * x + 2]) * f, __uint_as_float(a[8 * x + 3]) * f);
+                v.z = pack_bf16x2(__uint_as_float(a[8 * x + 4]) * f, __uint_as_float(a[8 * x + 5]) * f);
+                v.w = pack_bf16x2(__uint_as_float(a[8 * x + 6]) * f, __uint_as_float(a[8 * x + 7]) * f);
+                *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (r & 7)) << 4)) = v;
+            }
+        }
+        tc_fence_before();
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+            mbar_arrive(&bars->dkv_free);
+            mbar_arrive(&bars->staged[grp]);
+        }
+        bool leader_ok = true;
+        if (leader) {
+            // a group that had no step of this item has not handed the previous item's buffer back yet
+            if (pending_ks >= 0) {
+                bulk_wait_group_read<0>();
+                mbar_arrive(&bars->kv_empty[pending_ks]);
+            }
+            leader_ok = mbar_wait(&bars->staged[grp], w & 1, abort_flag);
+            if (leader_ok) {
+                const CUtensorMap* tm = grp ? tmdK : tmdV;
+                const int order = grp ? (wk.orders >> 16) & 15 : (wk.orders >> 20) & 15;
+#pragma unroll
+                for (int h = 0; h < kHalves; ++h)
+                    tma_store_tile<kStrided>(tm, stage + h * kHalfTileBytes, order, h * kBoxCols, kt * kBlockK,
+                                             kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
+                bulk_commit_group();
+            }
+        }
+        pending_ks = ks;
+        ok = __all_sync(0xffffffffu, leader_ok);
+        if (!ok) break;
+        g += n;
+    }
+    if (leader) bulk_wait_group<0>();  // dV and dK must be complete before the kernel ends
+}
+
+template <bool kCausal, bool kStrided>
+__global__ void __launch_bounds__(kThreads, 1)
+attn_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
+                 const __grid_constant__ CUtensorMap tmdK, const __grid_constant__ CUtensorMap tmdV,
+                 const float* __restrict__ LSE, const float* __restrict__ Delta, int T, int BH, int H, uint32_t orders,
+                 int n_tiles, int chunk, float scale, int* __restrict__ dev_status) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    if (smem != smem_raw) {
+        // No room to realign: give up before anything is set up, but only once the predecessor in the stream
+        // has completed (the status word is global memory, and this grid must not finish ahead of it).
+        griddep_wait();
+        if (threadIdx.x == 0) atomicExch(dev_status, kDevTimeout);
+        return;
+    }
+    KvBars* bars = reinterpret_cast<KvBars*>(smem + kOffBar);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const KvWork wk{BH, n_tiles, chunk, T, H, orders, kCausal};
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&bars->kv_full[s], 1);
+            mbar_init(&bars->kv_empty[s], 2);  // the leaders of the two groups
+            mbar_init(&bars->staged[s], 4);
+            mbar_init(&bars->sp_full[s], 1);
+            mbar_init(&bars->ready[s], 4);
+        }
+        for (int s = 0; s < kQStages; ++s) {
+            mbar_init(&bars->q_full[s], 1);
+            mbar_init(&bars->q_empty[s], 1);
+        }
+        for (int s = 0; s < kRowStages; ++s) {
+            mbar_init(&bars->row_full[s], 1);
+            mbar_init(&bars->row_empty[s], 4);
+        }
+        mbar_init(&bars->dkv_full, 1);
+        mbar_init(&bars->dkv_free, 8);
+        mbar_init(&bars->drain, 1);
+        bars->ring.init(kWorkConsumers);
+        bars->abort_flag = 0;
+        fence_mbar_init();
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+        tma_prefetch_desc(&tmdO);
+        tma_prefetch_desc(&tmdK);
+        tma_prefetch_desc(&tmdV);
+    }
+    if (warp == 1) {
+        tmem_alloc(&bars->tmem_base, kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = bars->tmem_base;
+    griddep_launch_dependents();
+    griddep_wait();  // everything above overlaps the previous kernel of the stream
+
+    if (warp == 0) {
+        if (lane == 0) kv_producer<kStrided>(&tmQ, &tmK, &tmV, &tmdO, smem, bars, wk);
+    } else if (warp == 1) {
+        kv_mma(smem, bars, tmem_base, wk);
+    } else if (warp == 2) {
+        kv_row_loader(bars, reinterpret_cast<float*>(smem + kOffRow), LSE, Delta, wk, lane);
+    } else if (warp >= 4) {
+        kv_compute<kCausal, kStrided>(smem, bars, tmem_base, &tmdK, &tmdV, scale, wk, (warp - 4) >> 2, warp & 3, lane);
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
+    if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
+}
+
+}  // namespace
+
+cudaError_t configure_attn_dkdv() {
+    auto set = [](auto kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    };
+    cudaError_t e = set(attn_dkdv_kernel<true, false>);
+    if (e == cudaSuccess) e = set(attn_dkdv_kernel<true, true>);
+    if (e == cudaSuccess) e = set(attn_dkdv_kernel<false, false>);
+    if (e == cudaSuccess) e = set(attn_dkdv_kernel<false, true>);
+    return e;
+}
+
+cudaError_t launch_attn_dkdv(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                             const CUtensorMap& tmdO, const CUtensorMap& tmdK, const CUtensorMap& tmdV, bool strided,
+                             uint32_t orders, const float* LSE, const float* Delta, const AttnShape& s, int num_sms,
+                             int* dev_status, cudaStream_t stream) {
+    const int n_tiles = (s.T + kBlockK - 1) / kBlockK, BH = s.B * s.H;
+    const int chunk = heads_per_chunk(BH, n_tiles, s.T, D, num_sms);
+    const dim3 grid(static_cast<unsigned>(n_tiles) * BH);  // one CTA per item; those that do not start are taken over
+    auto go = [&](auto kernel) {
+        return launch_overlapped(kernel, grid, dim3(kThreads), kSmemBytes, stream, tmQ, tmK, tmV, tmdO, tmdK, tmdV, LSE, Delta,
+                                 s.T, BH, s.H, orders, n_tiles, chunk, s.scale, dev_status);
+    };
+    if (s.causal) return strided ? go(attn_dkdv_kernel<true, true>) : go(attn_dkdv_kernel<true, false>);
+    return strided ? go(attn_dkdv_kernel<false, true>) : go(attn_dkdv_kernel<false, false>);
+}
+
+}  // namespace nova

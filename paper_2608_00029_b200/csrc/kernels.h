@@ -84,6 +84,25 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
                            cudaStream_t stream);
 cudaError_t configure_attn_dq();
 
+// The dK/dV half of the two-kernel backward at D = 128 (attn_dkdv.cu): Q and dO maps with boxes of kKeyStep rows, the
+// others of 128.  `orders` for Q, K, V, dO, dK, dV.
+cudaError_t launch_attn_dkdv(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                             const CUtensorMap& tmdO, const CUtensorMap& tmdK, const CUtensorMap& tmdV, bool strided,
+                             uint32_t orders, const float* LSE, const float* Delta, const AttnShape& s, int num_sms,
+                             int* dev_status, cudaStream_t stream);
+cudaError_t configure_attn_dkdv();
+
+// Heads that the items of the two-kernel backward are taken in together: enough items for two rounds of the SMs, and no
+// more than about 48 MB of Q, K, V and dO, so that what the tiles of a head share stays in L2.
+inline int heads_per_chunk(int BH, int items_per_head, long long T, int D, int num_sms) {
+    long long c = (48ll << 20) / (T * D * 8);
+    const long long c_min = (2ll * num_sms + items_per_head - 1) / items_per_head;
+    if (c < c_min) c = c_min;
+    if (c * 3 / 2 >= BH) return BH;
+    const long long n = (BH + c - 1) / c;
+    return static_cast<int>((BH + n - 1) / n);
+}
+
 // What the backward main kernel does with its partial tiles of dQ.
 enum class DqMode {
     kAccumulate,  // adds them, unscaled, into the fp32 accumulator
