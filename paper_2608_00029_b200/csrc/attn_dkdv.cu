@@ -8,13 +8,14 @@
 //   P^T  = exp2(S^T*c - LSE*log2e),  dS^T = P^T * (dP^T - Delta)   (bf16, over the S^T and dP^T they came from)
 //   dV  += P^T dO_s,  dK += dS^T Q_s                           (TMEM x smem, dO and Q read MN-major)
 // Items are handed out dynamically (WorkRing), heaviest first within a chunk of heads whose tensors stay in L2
-// together.  384 threads:
-//   warp 0      TMA producer: K_j and V_j double-buffered, Q_s and dO_s through a ring of 64-query stages
+// together.  512 threads:
+//   warp 0      TMA producer: K_j double-buffered, V_j, and Q_s and dO_s through a ring of 64-query stages
 //   warp 1      UMMA issuer: S^T and dP^T run two steps ahead of dV and dK, across item boundaries
 //   warp 2      row loader: -LSE*log2e and -Delta of a step into shared memory
 //   warps 4-7   compute group 0, warps 8-11 group 1: the steps alternate between the groups; a thread has one key
-//               row and the 64 queries of its step.  At the end of an item group 0 sends dV out, group 1 dK, through the
-//               item's own V and K buffers, which nothing reads any more.
+//               row and the 64 queries of its step
+//   warps 12-15 send dV and dK of a finished item out, through the item's own K buffer, which nothing reads any more,
+//               while the compute warps are in the next item
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -22,22 +23,24 @@ namespace nova {
 namespace {
 
 constexpr int D = 128;
-constexpr int kThreads = 384;
+constexpr int kThreads = 512;
 constexpr int kTmemCols = 512;
 constexpr int kStep = kKeyStep;              // queries per step
 constexpr int kHalfStepBytes = kStep * 128;  // one [64 rows x 64 bf16] box
 constexpr int kHalves = D / kBoxCols;
 constexpr int kTileBytes = kHalves * kHalfTileBytes;
 constexpr int kStepBytes = kHalves * kHalfStepBytes;
-constexpr int kQStages = 3;
+constexpr int kQStages = 4;
 constexpr int kBufs = 2;                     // buffers of S^T and dP^T, one per compute group
 constexpr int kRowStages = 4;
-constexpr int kWorkConsumers = 2 + 8;        // issuer, row loader, compute warps
+constexpr int kWorkConsumers = 2 + 8 + 4;    // issuer, row loader, compute warps, write-out warps
 static_assert(kQStages >= kBufs, "the issuer runs kBufs steps ahead");
 
+// One V buffer and four stages of Q and dO rather than two and three: with three the loads of a step (32 KB, 1300 clocks
+// from L2 with every SM loading) came too late for it, while V of the next item has the last two steps of this one.
 constexpr int kOffK = 0;                                 // [2]
-constexpr int kOffV = 2 * kTileBytes;                    // [2]
-constexpr int kOffQ = 4 * kTileBytes;                    // [kQStages]
+constexpr int kOffV = 2 * kTileBytes;
+constexpr int kOffQ = 3 * kTileBytes;                    // [kQStages]
 constexpr int kOffdO = kOffQ + kQStages * kStepBytes;    // [kQStages]
 constexpr int kOffRow = kOffdO + kQStages * kStepBytes;  // [kRowStages] x (-LSE*log2e[64], -Delta[64])
 constexpr int kOffBar = kOffRow + kRowStages * 2 * kStep * 4;
@@ -47,12 +50,12 @@ static_assert(kSmemBytes <= 232448, "exceeds the shared memory of one CTA");
 constexpr int kColdV = 0, kColdK = D, kColBuf = 2 * D;   // + 128 * buffer: S^T / P^T, then dP^T / dS^T
 
 struct KvBars {
-    uint64_t kv_full[2], kv_empty[2];
+    uint64_t k_full[2], k_empty[2], v_full, v_empty;
     uint64_t q_full[kQStages], q_empty[kQStages];
     uint64_t row_full[kRowStages], row_empty[kRowStages];
     uint64_t sp_full[kBufs], ready[kBufs];  // per buffer: UMMA -> compute group, compute group -> UMMA
     uint64_t dkv_full, dkv_free;            // dV and dK of an item complete; read out of TMEM
-    uint64_t staged[2];                     // per group: its rows are staged
+    uint64_t staged, stage_free;            // the write-out warps among themselves
     uint64_t drain;
     WorkRing ring;
     uint32_t tmem_base;
@@ -81,7 +84,7 @@ template <bool kStrided>
 __device__ __forceinline__ void kv_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
                                             const CUtensorMap* tmdO, uint8_t* smem, KvBars* bars, const KvWork& wk) {
     volatile int* abort_flag = &bars->abort_flag;
-    int armed_kv[2] = {-1, -1}, armed_q[kQStages];
+    int armed_k[2] = {-1, -1}, armed_v = -1, armed_q[kQStages];
     for (int s = 0; s < kQStages; ++s) armed_q[s] = -1;
     bool ok = true, clc_pending = false;
     int w = 0, st = 0;
@@ -94,17 +97,14 @@ __device__ __forceinline__ void kv_producer(const CUtensorMap* tmQ, const CUtens
         wk.get(item, &kt, &bh, &s0, &n);
         const int head = kStrided ? bh % wk.H : 0, batch = kStrided ? bh / wk.H : 0;
         const int ks = w & 1;
-        ok = mbar_wait(&bars->kv_empty[ks], ((w >> 1) & 1) ^ 1, abort_flag);
+        ok = mbar_wait(&bars->k_empty[ks], ((w >> 1) & 1) ^ 1, abort_flag);
         if (!ok) break;
-        mbar_expect_tx(&bars->kv_full[ks], 2 * kTileBytes);  // rows past T arrive as zeros
-        armed_kv[ks] = (w >> 1) & 1;
+        mbar_expect_tx(&bars->k_full[ks], kTileBytes);  // rows past T arrive as zeros
+        armed_k[ks] = (w >> 1) & 1;
 #pragma unroll
-        for (int h = 0; h < kHalves; ++h) {
-            tma_load_tile<kStrided>(smem + kOffK + ks * kTileBytes + h * kHalfTileBytes, tmK, &bars->kv_full[ks],
+        for (int h = 0; h < kHalves; ++h)
+            tma_load_tile<kStrided>(smem + kOffK + ks * kTileBytes + h * kHalfTileBytes, tmK, &bars->k_full[ks],
                                     (wk.orders >> 4) & 15, h * kBoxCols, kt * kBlockK, head, batch, bh);
-            tma_load_tile<kStrided>(smem + kOffV + ks * kTileBytes + h * kHalfTileBytes, tmV, &bars->kv_full[ks],
-                                    (wk.orders >> 8) & 15, h * kBoxCols, kt * kBlockK, head, batch, bh);
-        }
         for (int s = 0; s < n; ++s) {
             ok = mbar_wait(&bars->q_empty[st], ph ^ 1, abort_flag);
             if (!ok) break;
@@ -121,6 +121,16 @@ __device__ __forceinline__ void kv_producer(const CUtensorMap* tmQ, const CUtens
                 st = 0;
                 ph ^= 1;
             }
+            if (s == 0) {  // V after the first queries: its buffer is the last thing the previous item hands back
+                ok = mbar_wait(&bars->v_empty, (w & 1) ^ 1, abort_flag);
+                if (!ok) break;
+                mbar_expect_tx(&bars->v_full, kTileBytes);
+                armed_v = w & 1;
+#pragma unroll
+                for (int h = 0; h < kHalves; ++h)
+                    tma_load_tile<kStrided>(smem + kOffV + h * kHalfTileBytes, tmV, &bars->v_full, (wk.orders >> 8) & 15,
+                                            h * kBoxCols, kt * kBlockK, head, batch, bh);
+            }
         }
         if (!ok) break;
         // all loads of this item are on their way: claim the next one now, and no earlier
@@ -135,7 +145,8 @@ __device__ __forceinline__ void kv_producer(const CUtensorMap* tmQ, const CUtens
         int none = 0;
         if (clc_pending) (void)mbar_wait(&bars->ring.answer_bar, w & 1, &none);
         for (int s = 0; s < 2; ++s)
-            if (armed_kv[s] >= 0) (void)mbar_wait(&bars->kv_full[s], armed_kv[s], &none);
+            if (armed_k[s] >= 0) (void)mbar_wait(&bars->k_full[s], armed_k[s], &none);
+        if (armed_v >= 0) (void)mbar_wait(&bars->v_full, armed_v, &none);
         for (int s = 0; s < kQStages; ++s)
             if (armed_q[s] >= 0) (void)mbar_wait(&bars->q_full[s], armed_q[s], &none);
     }
@@ -177,62 +188,74 @@ __device__ __forceinline__ void kv_mma(uint8_t* smem, KvBars* bars, uint32_t tme
     uint32_t rdy_ph = 0;              // phase of ready[buf_c]
     int ahead = 0;                    // steps between the cursors
 
-    for (;;) {
-        // ---- S^T and dP^T, as far ahead as buffers and loads allow
-        while (more && ahead < kBufs) {
-            if (left_a == 0 || !kv_seen) {  // first step of an item
-                const bool block = ahead == 0;
-                if (left_a == 0) {
-                    // `c` may be an item behind, not two: its item's number of steps would be overwritten
-                    if (w_a - w_c >= 2) break;
-                    if (!block && !bars->ring.published(w_a)) break;
-                    const int item = bars->ring.take(w_a, lane, abort_flag, kWaitLimitCycles);
-                    if (item < 0) {
-                        ok = (item == -1);
-                        more = false;
-                        break;
-                    }
-                    int kt, bh, s0, n;
-                    wk.get(item, &kt, &bh, &s0, &n);
-                    left_a = n;
-                    if (w_a & 1) n_of[1] = n;
-                    else n_of[0] = n;
-                    ++w_a;
-                    kv_seen = false;
-                }
-                const uint32_t p = ((w_a - 1) >> 1) & 1;
-                if (block) {
-                    ok = mbar_wait(&bars->kv_full[(w_a - 1) & 1], p, abort_flag);
-                    if (ok) ok = mbar_wait(&bars->q_full[st_a], ph_a, abort_flag);
-                    if (!ok) break;
-                } else {
-                    const bool there = mbar_test(&bars->kv_full[(w_a - 1) & 1], p) && mbar_test(&bars->q_full[st_a], ph_a);
-                    if (!__all_sync(0xffffffffu, there)) break;
-                }
-                kv_seen = true;
-            } else {
-                ok = mbar_wait(&bars->q_full[st_a], ph_a, abort_flag);
-                if (!ok) break;
-            }
-            tc_fence_after();
-            // The buffer is free: the dV and dK products that read its P^T and dS^T were queued before this point.
-            if (el) {
-                const int ks = (w_a - 1) & 1;
-                const uint32_t t_b = tmem_base + kColBuf + 128 * buf_a;
-                product(t_b, k_k0 + ks * (kTileBytes >> 4), q_k0 + st_a * (kStepBytes >> 4));
-                product(t_b + 64, v_k0 + ks * (kTileBytes >> 4), do_k0 + st_a * (kStepBytes >> 4));
-                tc_commit(&bars->sp_full[buf_a]);
-            }
-            __syncwarp();
-            --left_a;
-            ++ahead;
-            if (++st_a == kQStages) {
-                st_a = 0;
-                ph_a ^= 1;
-            }
-            buf_a ^= 1;
+    // Are K, V, Q and dO of the next step of `a` there?  False without an error: not yet, or no items left.
+    auto probe = [&]() -> bool {
+        if (!more) return false;
+        if (left_a > 0 && kv_seen) {
+            ok = mbar_wait(&bars->q_full[st_a], ph_a, abort_flag);
+            return ok;
         }
+        const bool block = ahead == 0;
+        if (left_a == 0) {
+            if (w_a - w_c >= 2) return false;  // the number of steps of the item of `c` would be overwritten
+            if (!block && !bars->ring.published(w_a)) return false;
+            const int item = bars->ring.take(w_a, lane, abort_flag, kWaitLimitCycles);
+            if (item < 0) {
+                ok = (item == -1);
+                more = false;
+                return false;
+            }
+            int kt, bh, s0, n;
+            wk.get(item, &kt, &bh, &s0, &n);
+            left_a = n;
+            if (w_a & 1) n_of[1] = n;
+            else n_of[0] = n;
+            ++w_a;
+            kv_seen = false;
+        }
+        const uint32_t p = ((w_a - 1) >> 1) & 1;
+        if (block) {
+            ok = mbar_wait(&bars->k_full[(w_a - 1) & 1], p, abort_flag);
+            if (ok) ok = mbar_wait(&bars->v_full, (w_a - 1) & 1, abort_flag);
+            if (ok) ok = mbar_wait(&bars->q_full[st_a], ph_a, abort_flag);
+            kv_seen = ok;
+        } else {
+            const bool there = mbar_test(&bars->k_full[(w_a - 1) & 1], p) && mbar_test(&bars->v_full, (w_a - 1) & 1) &&
+                               mbar_test(&bars->q_full[st_a], ph_a);
+            kv_seen = __all_sync(0xffffffffu, there);
+        }
+        return kv_seen;
+    };
+    // S^T and dP^T of the next step of `a`.  The buffer is free: the dV and dK products that read its P^T and dS^T were
+    // queued before this point.
+    auto issue_sp = [&]() {
+        tc_fence_after();
+        if (el) {
+            const int ks = (w_a - 1) & 1;
+            const uint32_t t_b = tmem_base + kColBuf + 128 * buf_a;
+            product(t_b, k_k0 + ks * (kTileBytes >> 4), q_k0 + st_a * (kStepBytes >> 4));
+            product(t_b + 64, v_k0, do_k0 + st_a * (kStepBytes >> 4));
+            tc_commit(&bars->sp_full[buf_a]);
+            if (left_a == 1) tc_commit(&bars->v_empty);  // the item's last step
+        }
+        __syncwarp();
+        --left_a;
+        ++ahead;
+        if (++st_a == kQStages) {
+            st_a = 0;
+            ph_a ^= 1;
+        }
+        buf_a ^= 1;
+    };
+
+    for (;;) {
+        while (ahead < kBufs && probe()) issue_sp();
         if (!ok || ahead == 0) break;  // given up, or no items left
+        // The loads of the step that takes over the buffer of the oldest one are looked for before that one is waited
+        // for: nothing then stands between its dV and dK and the next S^T and dP^T (worth 20 %: the tensor pipe idles
+        // while its issuer waits).
+        const bool next_there = ahead == kBufs && probe();
+        if (!ok) break;
         // ---- dV and dK of the oldest step
         ok = mbar_wait(&bars->ready[buf_c], rdy_ph, abort_flag);
         // the previous item's dV and dK must have been read out of TMEM before they are overwritten
@@ -255,6 +278,7 @@ __device__ __forceinline__ void kv_mma(uint8_t* smem, KvBars* bars, uint32_t tme
             if (last) tc_commit(&bars->dkv_full);
         }
         __syncwarp();
+        if (next_there) issue_sp();
         --ahead;
         if (++st_c == kQStages) st_c = 0;
         rdy_ph ^= buf_c;  // after the second buffer
@@ -318,21 +342,18 @@ __device__ __forceinline__ void kv_row_loader(KvBars* bars, float* row_buf, cons
 }
 
 // Compute group `grp` (steps g with g % 2 == grp, which are those of buffer `grp`), warp `cwarp` of it.
-template <bool kCausal, bool kStrided>
-__device__ __forceinline__ void kv_compute(uint8_t* smem, KvBars* bars, uint32_t tmem_base, const CUtensorMap* tmdK,
-                                           const CUtensorMap* tmdV, float scale, const KvWork& wk, int grp, int cwarp,
-                                           int lane) {
+template <bool kCausal>
+__device__ __forceinline__ void kv_compute(const uint8_t* smem, KvBars* bars, uint32_t tmem_base, float scale,
+                                           const KvWork& wk, int grp, int cwarp, int lane) {
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * cwarp;
     const int r = lane_base + lane;  // local key row
-    const bool leader = (cwarp == 0 && lane == 0);
     const float c = scale * kLog2e;
     const uint64_t c2 = f32x2_pack(c, c);
     const float* row_buf = reinterpret_cast<const float*>(smem + kOffRow);
     const uint32_t t_s = tmem_addr(tmem_base, lane_base, kColBuf + 128 * grp), t_dp = t_s + 64;
     bool ok = true;
-    int g = 0;             // steps of all items so far
-    int pending_ks = -1;   // K/V stage whose store was issued at the end of the previous item
+    int g = 0;  // steps of all items so far
 
     for (int w = 0;; ++w) {
         const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
@@ -402,70 +423,100 @@ __device__ __forceinline__ void kv_compute(uint8_t* smem, KvBars* bars, uint32_t
                 mbar_arrive(&bars->ready[grp]);
                 mbar_arrive(&bars->row_empty[rb]);
             }
-            if (pending_ks >= 0) {  // the copy engine has long read what was staged at the end of the previous item
-                if (leader) {
-                    bulk_wait_group_read<0>();
-                    mbar_arrive(&bars->kv_empty[pending_ks]);
-                }
-                pending_ks = -1;
-                __syncwarp();
-            }
         }
         if (!ok) break;
-        // ---- end of the item: dV (group 0) or dK * scale (group 1) as bf16 into the item's V or K buffer
+        g += n;
+    }
+}
+
+// 128 bf16 numbers of key row r into a tile's two boxes, 128-byte swizzle.
+__device__ __forceinline__ void kv_stage_row(uint8_t* stage, int r, const uint32_t (&pk)[D / 2]) {
+#pragma unroll
+    for (int x = 0; x < D / 8; ++x)
+        *reinterpret_cast<uint4*>(stage + (x / 8) * kHalfTileBytes + r * 128 + (((x % 8) ^ (r & 7)) << 4)) =
+            make_uint4(pk[4 * x], pk[4 * x + 1], pk[4 * x + 2], pk[4 * x + 3]);
+}
+
+// Write-out warps (warp `owarp` of four, thread = key row): dV, then dK * scale, of a finished item as bf16 into the item's K
+// buffer and out with TMA stores, while the compute warps are in the next item.
+template <bool kStrided>
+__device__ __forceinline__ void kv_write_out(uint8_t* smem, KvBars* bars, uint32_t tmem_base, const CUtensorMap* tmdK,
+                                             const CUtensorMap* tmdV, float scale, const KvWork& wk, int owarp, int lane) {
+    volatile int* abort_flag = &bars->abort_flag;
+    const uint32_t lane_base = 32u * owarp;
+    const int r = lane_base + lane;
+    const bool leader = (owarp == 0 && lane == 0);
+    bool ok = true;
+    for (int w = 0;; ++w) {
+        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
+        if (item < 0) break;
+        int kt, bh, s0, n;
+        wk.get(item, &kt, &bh, &s0, &n);
         const int ks = w & 1;
         ok = mbar_wait(&bars->dkv_full, w & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t t_o = tmem_addr(tmem_base, lane_base, grp ? kColdK : kColdV);
-        const float f = grp ? scale : 1.0f;
-        uint8_t* stage = smem + (grp ? kOffK : kOffV) + ks * kTileBytes;
+        // Both go through the item's K buffer, dV first; dK waits in registers (64 of packed bf16) meanwhile, so that the
+        // accumulators are free for the next item at once.
+        const int hh = kStrided ? bh % wk.H : 0, bb = kStrided ? bh / wk.H : 0;
+        uint8_t* stage = smem + kOffK + ks * kTileBytes;
+        uint32_t pk[2][D / 2];
 #pragma unroll
-        for (int cb = 0; cb < D; cb += 32) {
-            uint32_t a[32];
-            tmem_ld_x32(t_o + cb, a);
-            tmem_wait_ld();
-            uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + r * 128;
+        for (int which = 0; which < 2; ++which) {
+            const uint32_t t_o = tmem_addr(tmem_base, lane_base, which ? kColdK : kColdV);
+            const float f = which ? scale : 1.0f;
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
-                uint4 v;
-                v.x = pack_bf16x2(__uint_as_float(a[8 * x + 0]) * f, __uint_as_float(a[8 * x + 1]) * f);
-                v.y = pack_bf16x2(__uint_as_float(a[8 * x + 2]) * f, __uint_as_float(a[8 * x + 3]) * f);
-                v.z = pack_bf16x2(__uint_as_float(a[8 * x + 4]) * f, __uint_as_float(a[8 * x + 5]) * f);
-                v.w = pack_bf16x2(__uint_as_float(a[8 * x + 6]) * f, __uint_as_float(a[8 * x + 7]) * f);
-                *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (r & 7)) << 4)) = v;
+            for (int cb = 0; cb < D; cb += 32) {
+                uint32_t a[32];
+                tmem_ld_x32(t_o + cb, a);
+                tmem_wait_ld();
+#pragma unroll
+                for (int x = 0; x < 16; ++x)
+                    pk[which][cb / 2 + x] = pack_bf16x2(__uint_as_float(a[2 * x]) * f, __uint_as_float(a[2 * x + 1]) * f);
             }
+            if (which == 0) kv_stage_row(stage, r, pk[0]);
         }
         tc_fence_before();
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
             mbar_arrive(&bars->dkv_free);
-            mbar_arrive(&bars->staged[grp]);
+            mbar_arrive(&bars->staged);
         }
         bool leader_ok = true;
         if (leader) {
-            // a group that had no step of this item has not handed the previous item's buffer back yet
-            if (pending_ks >= 0) {
-                bulk_wait_group_read<0>();
-                mbar_arrive(&bars->kv_empty[pending_ks]);
-            }
-            leader_ok = mbar_wait(&bars->staged[grp], w & 1, abort_flag);
+            leader_ok = mbar_wait(&bars->staged, 0, abort_flag);
             if (leader_ok) {
-                const CUtensorMap* tm = grp ? tmdK : tmdV;
-                const int order = grp ? (wk.orders >> 16) & 15 : (wk.orders >> 20) & 15;
 #pragma unroll
                 for (int h = 0; h < kHalves; ++h)
-                    tma_store_tile<kStrided>(tm, stage + h * kHalfTileBytes, order, h * kBoxCols, kt * kBlockK,
-                                             kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
+                    tma_store_tile<kStrided>(tmdV, stage + h * kHalfTileBytes, (wk.orders >> 20) & 15, h * kBoxCols,
+                                             kt * kBlockK, hh, bb, bh);
                 bulk_commit_group();
+                bulk_wait_group_read<0>();
+                mbar_arrive(&bars->stage_free);
             }
         }
-        pending_ks = ks;
+        ok = __all_sync(0xffffffffu, leader_ok);
+        if (ok) ok = mbar_wait(&bars->stage_free, w & 1, abort_flag);
+        if (!ok) break;
+        kv_stage_row(stage, r, pk[1]);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->staged);
+        if (leader) {
+            leader_ok = mbar_wait(&bars->staged, 1, abort_flag);
+            if (leader_ok) {
+#pragma unroll
+                for (int h = 0; h < kHalves; ++h)
+                    tma_store_tile<kStrided>(tmdK, stage + h * kHalfTileBytes, (wk.orders >> 16) & 15, h * kBoxCols,
+                                             kt * kBlockK, hh, bb, bh);
+                bulk_commit_group();
+                bulk_wait_group_read<0>();
+                mbar_arrive(&bars->k_empty[ks]);
+            }
+        }
         ok = __all_sync(0xffffffffu, leader_ok);
         if (!ok) break;
-        g += n;
     }
     if (leader) bulk_wait_group<0>();  // dV and dK must be complete before the kernel ends
 }
@@ -492,9 +543,8 @@ attn_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
-            mbar_init(&bars->kv_full[s], 1);
-            mbar_init(&bars->kv_empty[s], 2);  // the leaders of the two groups
-            mbar_init(&bars->staged[s], 4);
+            mbar_init(&bars->k_full[s], 1);
+            mbar_init(&bars->k_empty[s], 1);
             mbar_init(&bars->sp_full[s], 1);
             mbar_init(&bars->ready[s], 4);
         }
@@ -507,7 +557,11 @@ attn_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             mbar_init(&bars->row_empty[s], 4);
         }
         mbar_init(&bars->dkv_full, 1);
-        mbar_init(&bars->dkv_free, 8);
+        mbar_init(&bars->dkv_free, 4);
+        mbar_init(&bars->v_full, 1);
+        mbar_init(&bars->v_empty, 1);
+        mbar_init(&bars->staged, 4);
+        mbar_init(&bars->stage_free, 1);
         mbar_init(&bars->drain, 1);
         bars->ring.init(kWorkConsumers);
         bars->abort_flag = 0;
@@ -536,8 +590,10 @@ attn_dkdv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         kv_mma(smem, bars, tmem_base, wk);
     } else if (warp == 2) {
         kv_row_loader(bars, reinterpret_cast<float*>(smem + kOffRow), LSE, Delta, wk, lane);
+    } else if (warp >= 12) {
+        kv_write_out<kStrided>(smem, bars, tmem_base, &tmdK, &tmdV, scale, wk, warp & 3, lane);
     } else if (warp >= 4) {
-        kv_compute<kCausal, kStrided>(smem, bars, tmem_base, &tmdK, &tmdV, scale, wk, (warp - 4) >> 2, warp & 3, lane);
+        kv_compute<kCausal>(smem, bars, tmem_base, scale, wk, (warp - 4) >> 2, warp & 3, lane);
     }
 
     tc_fence_before();
