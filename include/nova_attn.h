@@ -109,10 +109,12 @@ size_t nova_attn_bwd_workspace_bytes(int B, int H, int T, int D);
  *   LSE, Delta  : in, fp32 [B,H,T] from nova_attn_fwd / nova_attn_bwd_preprocess
  *   dQ, dK, dV  : out, bf16 [B,H,T,D]; gradient of sum(O * dO) with respect to Q, K, V
  *   workspace   : device scratch of at least nova_attn_bwd_workspace_bytes(B,H,T,D) bytes, 16-byte
- *                 aligned; zeroed by the call itself on `stream`; contents afterwards unspecified.
+ *                 aligned; zeroed by the call itself on `stream` where it is used; contents afterwards
+ *                 unspecified.
  * dQ is accumulated in fp32 across key tiles with floating-point reduce-adds whose order is not fixed,
  * so its low-order bits may differ from run to run; dK and dV are deterministic.  A final pass scales
- * the accumulator, rounds it once to bf16 and writes dQ.
+ * the accumulator, rounds it once to bf16 and writes dQ.  Where it is faster (a single key tile, T <= 128;
+ * most shapes of D = 128 that fill the GPU) dQ is summed in a fixed order without the accumulator.
  */
 int nova_attn_bwd(const void* Q, const void* K, const void* V, const void* O, const void* dO,
                   const float* LSE, const float* Delta, void* dQ, void* dK, void* dV,
@@ -125,8 +127,8 @@ int nova_attn_bwd(const void* Q, const void* K, const void* V, const void* O, co
  *   NOVA_ATTN_BWD_STEP_ZERO     clear the fp32 dQ accumulator in `workspace`
  *   NOVA_ATTN_BWD_STEP_MAIN     the fused backward kernel: writes dK, dV, accumulates unscaled dQ
  *   NOVA_ATTN_BWD_STEP_CONVERT  dQ = bf16(scale * accumulator)
- * All three, in this order, are what nova_attn_bwd does; any other combination leaves sequencing to
- * the caller.  Arguments, validation and errors are those of nova_attn_bwd.
+ * All three, in this order, give what nova_attn_bwd gives (which for some shapes uses kernels that write
+ * dQ without the accumulator); any other combination leaves sequencing to the caller.  Arguments, validation and errors are those of nova_attn_bwd.
  */
 #define NOVA_ATTN_BWD_STEP_ZERO 1
 #define NOVA_ATTN_BWD_STEP_MAIN 2

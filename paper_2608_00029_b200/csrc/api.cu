@@ -385,6 +385,53 @@ size_t nova_attn_bwd_workspace_bytes(int B, int H, int T, int D) {
 }
 
 namespace {
+// Does the two-kernel backward pay at D=128?  The fused kernel is bound there by the stream of fp32 partial sums of dQ (64
+// KB per 128 x 128 tile) and clears and converts 4 bytes of accumulator per element besides; the two kernels recompute S
+// and dP instead.  Whole backward, fused against two kernels: B=4, H=32, T=1000: 175 -> 143 us; B=16, H=32, T=1024: 711
+// -> 605 us; B=4, H=32, T=512: 68 -> 61 us; B=4, H=16, T=2048 without the mask: 505 -> 440 us; B=2, H=16, T=4096: 480 ->
+// 460 us; but B=2, H=12, T=8192: 1290 -> 1340 us (the card's power limit, and two contractions more).  And they
+// need the SMs filled: each is half the work in as long chains (B=1, H=32, T=1024, 128 blocks of 256 rows: 47 -> 55
+// us; B=2, H=32, T=640, 192 blocks: 49 us both).
+bool two_kernels_pay(long long BH, int T, int D, int num_sms) {
+    return D == 128 && T <= 4096 && BH * ((T + 255) / 256) * 2 >= 3ll * num_sms;
+}
+
+// dQ, dK and dV by the two-kernel backward. 
+int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO, const float* LSE, const float* Delta,
+                    void* dQ, void* dK, void* dV, const AttnShape& s, const TensorStrides& sq, const TensorStrides& sk,
+                    const TensorStrides& sv, const TensorStrides& sdo, const TensorStrides& sdq, const TensorStrides& sdk,
+                    const TensorStrides& sdv, const DeviceState& st, cudaStream_t cs) {
+    const bool strided = !(merges(s, sq) && merges(s, sk) && merges(s, sv) && merges(s, sdo) && merges(s, sdq) &&
+                           merges(s, sdk) && merges(s, sdv));
+    // Each kernel takes what it streams in boxes of kKeyStep rows and what it holds in boxes of 128.
+    CUtensorMap tmQ, tmK, tmV, tmdO, tmQs, tmKs, tmVs, tmdOs, tmdQ, tmdK, tmdV;
+    uint32_t oq, ok, ov, odo, odq, odk, odv;
+    if (int rc = get_bf16_map(Q, s, sq, strided, &tmQ, &oq)) return rc;
+    if (int rc = get_bf16_map(K, s, sk, strided, &tmK, &ok)) return rc;
+    if (int rc = get_bf16_map(V, s, sv, strided, &tmV, &ov)) return rc;
+    if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdO, &odo)) return rc;
+    if (int rc = get_bf16_map(K, s, sk, strided, &tmKs, &ok, kKeyStep)) return rc;
+    if (int rc = get_bf16_map(V, s, sv, strided, &tmVs, &ov, kKeyStep)) return rc;
+    if (int rc = get_bf16_map(dQ, s, sdq, strided, &tmdQ, &odq)) return rc;
+    if (int rc = get_bf16_map(dK, s, sdk, strided, &tmdK, &odk)) return rc;
+    if (int rc = get_bf16_map(dV, s, sdv, strided, &tmdV, &odv)) return rc;
+    const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12);
+    cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders | (odq << 16), LSE, Delta, s, st.dev_status, cs);
+    if (e != cudaSuccess) return fail_cuda(e);
+    if (s.D == 128) {
+        if (int rc = get_bf16_map(Q, s, sq, strided, &tmQs, &oq, kKeyStep)) return rc;
+        if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdOs, &odo, kKeyStep)) return rc;
+        e = launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders | (odk << 16) | (odv << 20), LSE, Delta, s,
+                             st.num_sms, st.dev_status, cs);
+    } else {
+        // the fused kernel without its dQ product (the accumulator map is never used: any map will do)
+        e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmQ, tmdK, tmdV, strided, orders | (odk << 16) | (odv << 20), DqMode::kNone,
+                            LSE, Delta, static_cast<__nv_bfloat16*>(dK), static_cast<__nv_bfloat16*>(dV), sdk, sdv, s,
+                            st.num_sms, st.dev_status, cs);
+    }
+    return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
+}
+
 // The three steps of the backward on strided bf16 tensors; `steps` as in nova_attn_bwd_steps.
 int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const float* LSE, const float* Delta, void* dQ,
              void* dK, void* dV, int B, int H, int T, int D, const TensorStrides& sq, const TensorStrides& sk,
@@ -405,7 +452,10 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
     // One key tile per head (T <= 128): every dQ tile receives a single contribution, so the main kernel writes dQ itself
     // and the accumulator's clear and conversion fall away (B=1, H=2, T=64: 9.0 -> 6.2 us;
     // B=8, H=32, T=100, D=128: 24.9 -> 16.5 us).
-    const bool direct = T <= kBlockK && steps == (NOVA_ATTN_BWD_STEP_ZERO | NOVA_ATTN_BWD_STEP_MAIN | NOVA_ATTN_BWD_STEP_CONVERT);
+    const bool whole = steps == (NOVA_ATTN_BWD_STEP_ZERO | NOVA_ATTN_BWD_STEP_MAIN | NOVA_ATTN_BWD_STEP_CONVERT);
+    const bool direct = T <= kBlockK && whole;
+    if (whole && !direct && two_kernels_pay(BH, T, D, st->num_sms))
+        return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv, *st, cs);
     if ((steps & NOVA_ATTN_BWD_STEP_ZERO) && !direct) {
         e = launch_zero(acc, need, st->num_sms, cs);
         if (e != cudaSuccess) return fail_cuda(e);
@@ -467,34 +517,19 @@ int nova_attn_bwd_deterministic(const void* Q, const void* K, const void* V, con
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const TensorStrides c = contiguous_strides(H, T, D);
-    CUtensorMap tmQ, tmK, tmV, tmKs, tmVs, tmdO, tmdQ, tmdK, tmdV;
+    if (T > kBlockK) return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, c, c, c, c, c, c, c, *st, cs);
+    // one key tile per head: nothing is summed across blocks, the fused kernel is deterministic too
+    CUtensorMap tmQ, tmK, tmV, tmdO, tmdQ, tmdK, tmdV;
     if (int rc = get_tensor_map(Q, D, T, BH, &tmQ)) return rc;
     if (int rc = get_tensor_map(K, D, T, BH, &tmK)) return rc;
     if (int rc = get_tensor_map(V, D, T, BH, &tmV)) return rc;
     if (int rc = get_tensor_map(dO, D, T, BH, &tmdO)) return rc;
+    if (int rc = get_tensor_map(dQ, D, T, BH, &tmdQ)) return rc;
     if (int rc = get_tensor_map(dK, D, T, BH, &tmdK)) return rc;
     if (int rc = get_tensor_map(dV, D, T, BH, &tmdV)) return rc;
-    if (int rc = get_tensor_map(dQ, D, T, BH, &tmdQ)) return rc;
-    if (T <= kBlockK) {  // one key tile per head: nothing is summed across blocks, the fused kernel is deterministic too
-        const cudaError_t e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmdQ, tmdK, tmdV, false, 0u, DqMode::kDirect, LSE, Delta,
-                                              static_cast<__nv_bfloat16*>(dK), static_cast<__nv_bfloat16*>(dV), c, c, s,
-                                              st->num_sms, st->dev_status, cs);
-        return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
-    }
-    if (int rc = get_tensor_map(K, D, T, BH, &tmKs, 2, 0, 0, kKeyStep)) return rc;
-    if (int rc = get_tensor_map(V, D, T, BH, &tmVs, 2, 0, 0, kKeyStep)) return rc;
-    cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, false, 0u, LSE, Delta, s, st->dev_status, cs);
-    if (e != cudaSuccess) return fail_cuda(e);
-    if (D == 128) {
-        CUtensorMap tmQs, tmdOs;
-        if (int rc = get_tensor_map(Q, D, T, BH, &tmQs, 2, 0, 0, kKeyStep)) return rc;
-        if (int rc = get_tensor_map(dO, D, T, BH, &tmdOs, 2, 0, 0, kKeyStep)) return rc;
-        e = launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, false, 0u, LSE, Delta, s, st->num_sms, st->dev_status, cs);
-        return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
-    }
-    // the dK/dV half: the fused kernel without its dQ product (the accumulator map is never used: any map will do)
-    e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmQ, tmdK, tmdV, false, 0u, DqMode::kNone, LSE, Delta, static_cast<__nv_bfloat16*>(dK),
-                        static_cast<__nv_bfloat16*>(dV), c, c, s, st->num_sms, st->dev_status, cs);
+    const cudaError_t e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmdQ, tmdK, tmdV, false, 0u, DqMode::kDirect, LSE, Delta,
+                                          static_cast<__nv_bfloat16*>(dK), static_cast<__nv_bfloat16*>(dV), c, c, s,
+                                          st->num_sms, st->dev_status, cs);
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 

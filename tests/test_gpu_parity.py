@@ -445,6 +445,44 @@ def test_scales_far_from_ordinary(scale, qk, T):
     h.compare(h.select_heads(got, None), ref, label=f"scale={scale}: ", dO=ref["dO_in"], rms=scale > 1)
 
 
+# D=128: B*H*ceil(T/256) >= 222 takes the two-kernel backward, fewer blocks the fused kernel (one case on that side);
+# lengths around a step of 64, a tile of 128 and a pair of tiles, single-step items, more items than SMs.
+TWO_KERNELS = [(8, 30, 129, True), (8, 30, 191, False), (8, 30, 256, True), (8, 14, 257, True), (5, 25, 449, False),
+               (10, 8, 700, True), (4, 32, 1000, True), (7, 30, 200, True)]
+
+
+@pytest.mark.parametrize("B,H,T,causal", TWO_KERNELS)
+def test_wide_heads_backward_routes(B, H, T, causal):
+    """nova_attn_bwd at D=128 where it goes through the dQ and the dK/dV kernel: the same dK and dV as the fused kernel's
+    (its steps issued one by one), on the plain and on the fused-projection layout, and everything against the oracle."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("wide", B=B, H=H, T=T, D=128, seed=40 + T, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    got = h.run_gpu(Q, K, V, dO, cfg.scale, causal)
+    q, k, v, do = (x.to(dev) for x in (Q, K, V, dO))
+    o, lse, delta = got["O"].to(dev), got["LSE"].to(dev), got["Delta"].to(dev)
+    ws = torch.empty(nova_attn.nova_attn_bwd_workspace_bytes(B, H, T, 128), dtype=torch.uint8, device=dev)
+    fused = [torch.full_like(q, 7.0) for _ in range(3)]
+    for step in (nova_attn.BWD_STEP_ZERO, nova_attn.BWD_STEP_MAIN, nova_attn.BWD_STEP_CONVERT):
+        nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *fused, cfg.scale, causal, ws, steps=step)
+    qkv = torch.stack([x.transpose(1, 2) for x in (q, k, v)], 2)
+    dqkv = torch.full_like(qkv, 7.0)
+    views, grads = ([t[:, :, i].permute(0, 2, 1, 3) for i in range(3)] for t in (qkv, dqkv))
+    nova_attn.nova_attn_bwd_strided(*views, do.transpose(1, 2).contiguous().transpose(1, 2), lse, delta, *grads, cfg.scale,
+                                    causal, ws)
+    nova_attn.nova_attn_poll_device_status()
+    for name, a, b in (("dK", fused[1], grads[1]), ("dV", fused[2], grads[2])):
+        assert torch.equal(a.cpu(), got[name]) and torch.equal(b.cpu(), got[name]), name
+    for other in (fused[0], grads[0]):
+        d = (other.cpu().float() - got["dQ"].float()).abs().max()
+        assert d <= 1e-2 * got["dQ"].float().abs().max()
+    heads = [(0, 0), (B - 1, H - 1)]
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal, heads=heads)
+    h.compare(h.select_heads(got, heads), ref, label=f"wide T={T}: ", dO=ref["dO_in"])
+
+
 DETERMINISTIC = [  # (B, H, T, D, causal)
     (1, 2, 64, 64, True),
     (2, 3, 300, 64, True),
