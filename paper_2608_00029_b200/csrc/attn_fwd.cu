@@ -47,7 +47,14 @@ struct FwdCfg {
     static constexpr int kOffQ = 0;                                    // [kQStages][2 tiles]
     static constexpr int kOffK = kQStages * 2 * kTileBytes;            // [kKVStages]
     static constexpr int kOffV = kOffK + kKVStages * kTileBytes;       // [kKVStages]
-    static constexpr int kOffBar = kOffV + kKVStages * kTileBytes;
+    // Where O goes on its way out.  D=64: into the tile's Q buffer of the item, which has a second stage.  D=128: through
+    // 16 KB per tile of its own, half of the columns at a time, so that the one Q stage can take the next item's Q as
+    // soon as the last Q K^T has read it instead of after the item's O has left: 207 -> 188 us at B=16, H=32, T=1024, 66
+    // -> 59 us at B=4, H=32, T=1000, 33 -> 28 us at B=64, H=12, T=100.  Items of a single tile, as a rule the only one of
+    // their CTA, keep to the Q buffer (18.5 against 21 us at B=1, H=16, T=1024 without the mask).
+    static constexpr bool kOwnStage = (kQStages == 1);
+    static constexpr int kOffO = kOffV + kKVStages * kTileBytes;      // kOwnStage: [2 tiles]
+    static constexpr int kOffBar = kOffO + (kOwnStage ? 2 * kHalfTileBytes : 0);
     static constexpr int kSmemBytes = kOffBar + 512 + 1024;
     static constexpr int kColS = 0;      // + 128 * tile
     static constexpr int kColO = 256;    // + D * tile
@@ -61,7 +68,7 @@ struct FwdCfg {
 struct FwdBars {
     uint64_t q_full[2], q_empty[2];
     uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2];
-    uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2], o_free[2], o_staged[2];  // per query tile
+    uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2], o_free[2], o_staged[2], o_sent[2];  // per query tile
     uint64_t drain;
     WorkRing ring;  // item numbers: producer -> UMMA issuer and softmax warps
     uint32_t tmem_base;
@@ -74,6 +81,8 @@ template <bool kSingle>
 struct FwdWork {
     static constexpr int kRows = kSingle ? kBlockQ : kBlockRows;
     static constexpr int kTiles = kRows / kBlockQ;
+    template <typename Cfg>
+    static constexpr bool own_stage = Cfg::kOwnStage && !kSingle;
     int n_items, BH, n_blocks, n_kv_all, T, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, O tensor maps, four bits each
     bool causal;
@@ -172,6 +181,7 @@ template <int D, typename Work>
 __device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const Work& wk,
                                         long long limit) {
     using Cfg = FwdCfg<D>;
+    constexpr bool kOwnStage = Work::template own_stage<Cfg>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescQK = umma_idesc_bf16(128, 128, 0, 0);
     constexpr uint32_t kIdescPV = umma_idesc_bf16(128, D, 0, 1);
@@ -244,7 +254,10 @@ __device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t t
             if (n_a > 0) issue_qk(0, g, q_k[0]);
             if (n_b > 0 && ok) issue_qk(1, g, q_k[1]);
             if (!ok) break;
-            if (el) tc_commit(&bars->k_empty[g & 1]);  // K tile 0 is no longer read once these have run
+            if (el) {
+                tc_commit(&bars->k_empty[g & 1]);  // K tile 0 is no longer read once these have run
+                if (kOwnStage && n == 1) tc_commit(&bars->q_empty[qs]);
+            }
             __syncwarp();
         }
         first_queued = false;
@@ -329,6 +342,7 @@ __device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t t
             if (el) {
                 tc_commit(&bars->v_empty[st]);                    // V tile j is no longer read
                 if (j + 1 < n) tc_commit(&bars->k_empty[st ^ 1]);  // nor K tile j+1 (both Q K^T are queued)
+                if (kOwnStage && j + 2 == n) tc_commit(&bars->q_empty[qs]);  // nor Q: that was its last Q K^T
             }
             __syncwarp();
         }
@@ -351,6 +365,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                                             float* __restrict__ LSE, float scale, const Work& wk, int t, int swarp,
                                             int lane, long long limit) {
     using Cfg = FwdCfg<D>;
+    constexpr bool kOwnStage = Work::template own_stage<Cfg>;
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * (swarp & 3);
     const int row_local = lane_base + lane;
@@ -381,7 +396,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
             // Tile entirely past the end of the sequence: only release the Q stage, and only once it
             // has been filled, so that this warpgroup never runs ahead of the ring.
             bool leader_ok = true;
-            if (leader) {
+            if (leader && !kOwnStage) {
                 if (pending_qs >= 0) {
                     bulk_wait_group_read<0>();
                     mbar_arrive(&bars->q_empty[pending_qs]);
@@ -389,7 +404,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                 leader_ok = mbar_wait(&bars->q_full[qs], (w / Cfg::kQStages) & 1, abort_flag, limit);
                 if (leader_ok) mbar_arrive(&bars->q_empty[qs]);
             }
-            pending_qs = -1;
+            if (!kOwnStage) pending_qs = -1;
             ok = __all_sync(0xffffffffu, leader_ok);
             if (!ok) break;
             ++w;
@@ -501,7 +516,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
             if (pending_qs >= 0) {
                 if (leader) {
                     bulk_wait_group_read<0>();
-                    mbar_arrive(&bars->q_empty[pending_qs]);
+                    mbar_arrive(kOwnStage ? &bars->o_sent[t] : &bars->q_empty[pending_qs]);
                 }
                 pending_qs = -1;
                 __syncwarp();
@@ -515,50 +530,101 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
         if (!ok) break;
         tc_fence_after();
         const float inv_l = 1.0f / l;
-#pragma unroll
-        for (int cb = 0; cb < D; cb += 32) {
-            uint32_t o[32];
-            tmem_ld_x32(t_o + cb, o);
-            tmem_wait_ld();
-            uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + row_local * 128;
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
-                uint4 v;
-                v.x = pack_bf16x2(__uint_as_float(o[8 * x + 0]) * inv_l, __uint_as_float(o[8 * x + 1]) * inv_l);
-                v.y = pack_bf16x2(__uint_as_float(o[8 * x + 2]) * inv_l, __uint_as_float(o[8 * x + 3]) * inv_l);
-                v.z = pack_bf16x2(__uint_as_float(o[8 * x + 4]) * inv_l, __uint_as_float(o[8 * x + 5]) * inv_l);
-                v.w = pack_bf16x2(__uint_as_float(o[8 * x + 6]) * inv_l, __uint_as_float(o[8 * x + 7]) * inv_l);
-                *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (row_local & 7)) << 4)) = v;
-            }
-        }
-        tc_fence_before();
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-            mbar_arrive(&bars->o_free[t]);    // O_t has been read out of TMEM
-            mbar_arrive(&bars->o_staged[t]);  // and this warp's rows are staged
-        }
-        if (row < T) LSE[static_cast<size_t>(bh) * T + row] = m_ref * scale + logf(l);
         bool leader_ok = true;
-        if (leader) {
-            leader_ok = mbar_wait(&bars->o_staged[t], wt & 1, abort_flag, limit);
-            if (leader_ok) {
+        if constexpr (kOwnStage) {
+            // 64 columns to the staging box and out, the other 64 packed in registers meanwhile
+            uint8_t* row_ptr = smem + Cfg::kOffO + t * kHalfTileBytes + row_local * 128;
+            uint32_t pk[2][32];
 #pragma unroll
-                for (int h = 0; h < Cfg::kHalves; ++h)
-                    tma_store_tile<kStrided>(tmO, stage + h * kHalfTileBytes, (wk.orders >> 12) & 15, h * kBoxCols,
-                                             qt * kBlockQ, kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
-                bulk_commit_group();
-                if (Cfg::kQStages == 1) {  // the next item's Q tile needs this very buffer
-                    bulk_wait_group_read<0>();
-                    mbar_arrive(&bars->q_empty[qs]);
+            for (int cb = 0; cb < D; cb += 32) {
+                uint32_t o[32];
+                tmem_ld_x32(t_o + cb, o);
+                tmem_wait_ld();
+#pragma unroll
+                for (int x = 0; x < 16; ++x)
+                    pk[cb / 64][(cb % 64) / 2 + x] =
+                        pack_bf16x2(__uint_as_float(o[2 * x]) * inv_l, __uint_as_float(o[2 * x + 1]) * inv_l);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->o_free[t]);  // O_t has been read out of TMEM
+            if (row < T) LSE[static_cast<size_t>(bh) * T + row] = m_ref * scale + logf(l);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                // the box is free once what was sent from it last has been read (the second half of the previous item
+                // is handed back after this item's first key tile, as in D=64)
+                const int u = 2 * wt + h;
+                if (u > 0) ok = mbar_wait(&bars->o_sent[t], (u - 1) & 1, abort_flag, limit);
+                if (!ok) break;
+#pragma unroll
+                for (int ch = 0; ch < 8; ++ch)
+                    *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (row_local & 7)) << 4)) =
+                        make_uint4(pk[h][4 * ch], pk[h][4 * ch + 1], pk[h][4 * ch + 2], pk[h][4 * ch + 3]);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars->o_staged[t]);
+                if (leader) {
+                    leader_ok = mbar_wait(&bars->o_staged[t], h, abort_flag, limit);
+                    if (leader_ok) {
+                        tma_store_tile<kStrided>(tmO, smem + Cfg::kOffO + t * kHalfTileBytes, (wk.orders >> 12) & 15,
+                                                 h * kBoxCols, qt * kBlockQ, kStrided ? bh % wk.H : 0,
+                                                 kStrided ? bh / wk.H : 0, bh);
+                        bulk_commit_group();
+                        if (h == 0) {
+                            bulk_wait_group_read<0>();
+                            mbar_arrive(&bars->o_sent[t]);
+                        }
+                    }
+                }
+                leader_ok = __all_sync(0xffffffffu, leader_ok);
+                if (!leader_ok) break;
+            }
+            if (!ok) break;
+        } else {
+#pragma unroll
+            for (int cb = 0; cb < D; cb += 32) {
+                uint32_t o[32];
+                tmem_ld_x32(t_o + cb, o);
+                tmem_wait_ld();
+                uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + row_local * 128;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
+                    uint4 v;
+                    v.x = pack_bf16x2(__uint_as_float(o[8 * x + 0]) * inv_l, __uint_as_float(o[8 * x + 1]) * inv_l);
+                    v.y = pack_bf16x2(__uint_as_float(o[8 * x + 2]) * inv_l, __uint_as_float(o[8 * x + 3]) * inv_l);
+                    v.z = pack_bf16x2(__uint_as_float(o[8 * x + 4]) * inv_l, __uint_as_float(o[8 * x + 5]) * inv_l);
+                    v.w = pack_bf16x2(__uint_as_float(o[8 * x + 6]) * inv_l, __uint_as_float(o[8 * x + 7]) * inv_l);
+                    *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (row_local & 7)) << 4)) = v;
+                }
+            }
+            tc_fence_before();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&bars->o_free[t]);    // O_t has been read out of TMEM
+                mbar_arrive(&bars->o_staged[t]);  // and this warp's rows are staged
+            }
+            if (row < T) LSE[static_cast<size_t>(bh) * T + row] = m_ref * scale + logf(l);
+            if (leader) {
+                leader_ok = mbar_wait(&bars->o_staged[t], wt & 1, abort_flag, limit);
+                if (leader_ok) {
+#pragma unroll
+                    for (int h = 0; h < Cfg::kHalves; ++h)
+                        tma_store_tile<kStrided>(tmO, stage + h * kHalfTileBytes, (wk.orders >> 12) & 15, h * kBoxCols,
+                                                 qt * kBlockQ, kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
+                    bulk_commit_group();
+                    if (Cfg::kQStages == 1) {  // the next item's Q tile needs this very buffer
+                        bulk_wait_group_read<0>();
+                        mbar_arrive(&bars->q_empty[qs]);
+                    }
                 }
             }
         }
         // With two Q stages the buffer is only needed for the item after next: it is handed back after the next
         // item's first key tile, when the store has long read it, instead of holding this warp up now (worth 7 %
         // at B=8, H=12, T=1024; a separate store thread that waits in the softmax warps' stead was slower).
-        if (Cfg::kQStages > 1) pending_qs = qs;
+        if (Cfg::kQStages > 1 || kOwnStage) pending_qs = qs;
         // Brings the leader back together with the rest of its warp before the next warp-wide TMEM
         // load, and makes a failed wait of the leader a failure of the whole warp.
         ok = __all_sync(0xffffffffu, leader_ok);
@@ -586,7 +652,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(&bars->q_full[s], 1);
-            mbar_init(&bars->q_empty[s], 2);  // the store leaders of the two query tiles
+            // the store leaders of the two query tiles, or the UMMA issuer where O has buffers of its own
+            mbar_init(&bars->q_empty[s], Work::template own_stage<Cfg> ? 1 : 2);
+            mbar_init(&bars->o_sent[s], 1);
             mbar_init(&bars->k_full[s], 1);
             mbar_init(&bars->k_empty[s], 1);
             mbar_init(&bars->v_full[s], 1);
