@@ -375,7 +375,7 @@ int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, 
     if (int rc = get_tensor_map(dO, D, T, BH, &tmdO)) return rc;
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const cudaError_t e =
-        launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->dev_status, static_cast<cudaStream_t>(stream));
+        launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 
@@ -416,7 +416,8 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     if (int rc = get_bf16_map(dK, s, sdk, strided, &tmdK, &odk)) return rc;
     if (int rc = get_bf16_map(dV, s, sdv, strided, &tmdV, &odv)) return rc;
     const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12);
-    cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders | (odq << 16), LSE, Delta, s, st.dev_status, cs);
+    cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders | (odq << 16), LSE, Delta, s, st.num_sms,
+                                   st.dev_status, cs);
     if (e != cudaSuccess) return fail_cuda(e);
     if (s.D == 128) {
         if (int rc = get_bf16_map(Q, s, sq, strided, &tmQs, &oq, kKeyStep)) return rc;

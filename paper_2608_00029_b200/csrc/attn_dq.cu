@@ -73,15 +73,28 @@ struct DqBars {
 };
 static_assert(sizeof(DqBars) <= 512, "barrier block");
 
-// Work items: 256-row query blocks, heaviest first (the last block of a causal problem sees every key).
+// Work items: 256-row query blocks, heaviest first (the last block of a causal problem sees every key).  D=128: within
+// chunks of heads whose tensors stay in L2 together (the exact Delta at B=16, H=32, T=1024 175 -> 157 us, the
+// deterministic backward 650 -> 627 us); at D=64 a head's K and V are half as large and the longer arithmetic costs
+// 1 % where there is nothing to gain.
+template <int D>
 struct DqWork {
-    int BH, n_blocks, T, H;
+    int BH, n_blocks, chunk, T, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, dO, dQ tensor maps, four bits each
     bool causal;
     // Block index, head, and the number of key steps each tile visits (0: the tile lies past the end of the sequence).
     __device__ __forceinline__ void get(int idx, int* blk, int* bh, int* n_a, int* n_b) const {
-        *blk = n_blocks - 1 - idx / BH;
-        *bh = idx % BH;
+        if constexpr (D == 128) {
+            const int per_chunk = chunk * n_blocks;
+            const int ck = idx / per_chunk, in = idx - ck * per_chunk;
+            const int heads = min(chunk, BH - ck * chunk);
+            const int order = in / heads;
+            *blk = n_blocks - 1 - order;
+            *bh = ck * chunk + in - order * heads;
+        } else {
+            *blk = n_blocks - 1 - idx / BH;
+            *bh = idx % BH;
+        }
         const int n_all = (T + kStep - 1) / kStep;
         const int qt_a = 2 * (*blk), qt_b = qt_a + 1;
         *n_a = causal ? min((qt_a + 1) * (kBlockQ / kStep), n_all) : n_all;
@@ -91,7 +104,7 @@ struct DqWork {
 
 template <int D, bool kStrided>
 __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork& wk) {
+                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork<D>& wk) {
     using Cfg = DqCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr long long limit = kWaitLimitCycles;
@@ -170,7 +183,7 @@ __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtens
 
 // The issuer of query tile t: the whole warp in uniform control flow, one elected lane issues.
 template <int D, bool kDelta>
-__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork& wk, int t) {
+__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork<D>& wk, int t) {
     using Cfg = DqCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescT = umma_idesc_bf16(128, kStep, 0, 0);  // S, dP
@@ -326,7 +339,7 @@ __device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tme
 template <int D, bool kCausal, bool kStrided, bool kDelta>
 __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const CUtensorMap* tmdQ,
                                         const float* __restrict__ LSE, const float* __restrict__ Delta,
-                                        float* __restrict__ Delta_out, float scale, const DqWork& wk, int t, int rwarp,
+                                        float* __restrict__ Delta_out, float scale, const DqWork<D>& wk, int t, int rwarp,
                                         int lane) {
     using Cfg = DqCfg<D>;
     volatile int* abort_flag = &bars->abort_flag;
@@ -503,7 +516,7 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
 template <int D, bool kCausal, bool kStrided, bool kDelta>
 __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
                                         const CUtensorMap* tmdO, const CUtensorMap* tmdQ, const float* __restrict__ LSE,
-                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork& wk,
+                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork<D>& wk,
                                         float scale, int* __restrict__ dev_status) {
     using Cfg = DqCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -569,22 +582,23 @@ __global__ void __launch_bounds__(kThreads, 1)
 attn_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                const __grid_constant__ CUtensorMap tmdQ, const float* __restrict__ LSE, const float* __restrict__ Delta,
-               int T, int BH, int H, uint32_t orders, int n_blocks, float scale, int* __restrict__ dev_status) {
+               int T, int BH, int H, uint32_t orders, int n_blocks, int chunk, float scale, int* __restrict__ dev_status) {
     dq_body<D, kCausal, kStrided, false>(&tmQ, &tmK, &tmV, &tmdO, &tmdQ, LSE, Delta, nullptr,
-                                         DqWork{BH, n_blocks, T, H, orders, kCausal}, scale, dev_status);
+                                         DqWork<D>{BH, n_blocks, chunk, T, H, orders, kCausal}, scale, dev_status);
 }
 
 template <int D, bool kCausal>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
-                  const float* __restrict__ LSE, float* __restrict__ Delta, int T, int BH, int n_blocks, float scale,
+                  const float* __restrict__ LSE, float* __restrict__ Delta, int T, int BH, int n_blocks, int chunk, float scale,
                   int* __restrict__ dev_status) {
     dq_body<D, kCausal, false, true>(&tmQ, &tmK, &tmV, &tmdO, nullptr, LSE, nullptr, Delta,
-                                     DqWork{BH, n_blocks, T, 1, 0u, kCausal}, scale, dev_status);
+                                     DqWork<D>{BH, n_blocks, chunk, T, 1, 0u, kCausal}, scale, dev_status);
 }
 
 int n_blocks_of(const AttnShape& s) { return (s.T + kBlockRows - 1) / kBlockRows; }
+int chunk_of(const AttnShape& s, int num_sms) { return heads_per_chunk(s.B * s.H, n_blocks_of(s), s.T, s.D, num_sms); }
 // One CTA per item; those that do not start at once are taken over by those that did.
 dim3 grid_of(const AttnShape& s) { return dim3(static_cast<unsigned>(n_blocks_of(s)) * s.B * s.H); }
 
@@ -620,14 +634,14 @@ cudaError_t configure_attn_dq() {
 
 cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                            const CUtensorMap& tmdO, const CUtensorMap& tmdQ, bool strided, uint32_t orders,
-                           const float* LSE, const float* Delta, const AttnShape& s, int* dev_status,
+                           const float* LSE, const float* Delta, const AttnShape& s, int num_sms, int* dev_status,
                            cudaStream_t stream) {
     return dispatch(s, [&](auto d, auto causal) {
         constexpr int D = decltype(d)::value;
         constexpr bool kCausal = decltype(causal)::value;
         auto go = [&](auto kernel) {
             return launch_overlapped(kernel, grid_of(s), dim3(kThreads), DqCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO,
-                                     tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, n_blocks_of(s), s.scale, dev_status);
+                                     tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, n_blocks_of(s), chunk_of(s, num_sms), s.scale, dev_status);
         };
         return strided ? go(attn_dq_kernel<D, kCausal, true>) : go(attn_dq_kernel<D, kCausal, false>);
     });
@@ -635,12 +649,12 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
 
 cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                               const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s,
-                              int* dev_status, cudaStream_t stream) {
+                              int num_sms, int* dev_status, cudaStream_t stream) {
     return dispatch(s, [&](auto d, auto causal) {
         constexpr int D = decltype(d)::value;
         constexpr bool kCausal = decltype(causal)::value;
         return launch_overlapped(attn_delta_kernel<D, kCausal>, grid_of(s), dim3(kThreads), DqCfg<D>::kSmemBytes, stream, tmQ,
-                                 tmK, tmV, tmdO, LSE, Delta, s.T, s.B * s.H, n_blocks_of(s), s.scale, dev_status);
+                                 tmK, tmV, tmdO, LSE, Delta, s.T, s.B * s.H, n_blocks_of(s), chunk_of(s, num_sms), s.scale, dev_status);
     });
 }
 

@@ -74,13 +74,13 @@ constexpr int kKeyStep = 64;
 // Exact Delta_i = sum_j P_ij (dO_i . V_j) with P rebuilt from LSE (two contractions + exp2 per tile).
 cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                               const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s,
-                              int* dev_status, cudaStream_t stream);
+                              int num_sms, int* dev_status, cudaStream_t stream);
 // Deterministic dQ (the dQ half of the paper's two-kernel backward): one CTA per pair of 128-row query tiles walks
 // the keys in order and writes dQ = bf16(scale * sum_j dS_j K_j) through `tmdQ`.  `strided`, `orders`: as in the
 // forward, for Q, K, V, dO, dQ.
 cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                            const CUtensorMap& tmdO, const CUtensorMap& tmdQ, bool strided, uint32_t orders,
-                           const float* LSE, const float* Delta, const AttnShape& s, int* dev_status,
+                           const float* LSE, const float* Delta, const AttnShape& s, int num_sms, int* dev_status,
                            cudaStream_t stream);
 cudaError_t configure_attn_dq();
 
