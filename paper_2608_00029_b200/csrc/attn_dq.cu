@@ -85,12 +85,16 @@ struct DqWork {
     // Block index, head, and the number of key steps each tile visits (0: the tile lies past the end of the sequence).
     __device__ __forceinline__ void get(int idx, int* blk, int* bh, int* n_a, int* n_b) const {
         if constexpr (D == 128) {
-            const int per_chunk = chunk * n_blocks;
-            const int ck = idx / per_chunk, in = idx - ck * per_chunk;
-            const int heads = min(chunk, BH - ck * chunk);
+            int first = 0, in = idx, heads = BH;  // first head of the chunk, item within it, its heads
+            if (chunk < BH) {
+                const int per_chunk = chunk * n_blocks, ck = idx / per_chunk;
+                first = ck * chunk;
+                in = idx - ck * per_chunk;
+                heads = min(chunk, BH - first);
+            }
             const int order = in / heads;
             *blk = n_blocks - 1 - order;
-            *bh = ck * chunk + in - order * heads;
+            *bh = first + in - order * heads;
         } else {
             *blk = n_blocks - 1 - idx / BH;
             *bh = idx % BH;

@@ -76,21 +76,37 @@ struct FwdBars {
 };
 constexpr int kWorkConsumers = 1 + 8;  // UMMA issuer warp + 8 softmax warps
 
-// Work items: 256-row query blocks, numbered heaviest first.  kSingle: 128-row blocks, tile A alone.
-template <bool kSingle>
+// Work items: 256-row query blocks, numbered heaviest first; at D=128 within chunks of heads whose K and V stay in L2 from
+// one block to the next (184 -> 171 us at B=16, H=32, T=1024, 150 -> 139 us at B=2, H=16, T=4096; D=64, with half the
+// bytes per head, gained nothing).  kSingle: 128-row blocks, tile A alone.
+template <int D, bool kSingle>
 struct FwdWork {
+    static constexpr bool kChunks = (D == 128) && !kSingle;
     static constexpr int kRows = kSingle ? kBlockQ : kBlockRows;
     static constexpr int kTiles = kRows / kBlockQ;
     template <typename Cfg>
     static constexpr bool own_stage = Cfg::kOwnStage && !kSingle;
-    int n_items, BH, n_blocks, n_kv_all, T, H;
+    int n_items, BH, n_blocks, n_kv_all, T, H, chunk;
     uint32_t orders;  // coordinate orders of the Q, K, V, O tensor maps, four bits each
     bool causal;
     // Item `idx`: block index, head, and the number of key tiles each query tile visits
     // (0 if the tile lies entirely past the end of the sequence).
     __device__ __forceinline__ void get(int idx, int* blk, int* bh, int* n_a, int* n_b) const {
-        *blk = n_blocks - 1 - idx / BH;
-        *bh = idx % BH;
+        if constexpr (kChunks) {
+            int first = 0, in = idx, heads = BH;  // first head of the chunk, item within it, its heads
+            if (chunk < BH) {
+                const int per_chunk = chunk * n_blocks, ck = idx / per_chunk;
+                first = ck * chunk;
+                in = idx - ck * per_chunk;
+                heads = min(chunk, BH - first);
+            }
+            const int order = in / heads;
+            *blk = n_blocks - 1 - order;
+            *bh = first + in - order * heads;
+        } else {
+            *blk = n_blocks - 1 - idx / BH;
+            *bh = idx % BH;
+        }
         const int qt_a = kTiles * (*blk), qt_b = qt_a + 1;
         // causal clamp of the key loop: tile qt visits key tiles 0..qt
         *n_a = causal ? min(qt_a + 1, n_kv_all) : n_kv_all;
@@ -639,15 +655,15 @@ template <int D, bool kCausal, bool kStrided, bool kSingle>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
-                float* __restrict__ LSE, int T, int BH, int H, uint32_t orders, int n_blocks, float scale,
+                float* __restrict__ LSE, int T, int BH, int H, uint32_t orders, int n_blocks, int chunk, float scale,
                 long long limit, int inject, int* __restrict__ dev_status) {
     using Cfg = FwdCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     FwdBars* bars = reinterpret_cast<FwdBars*>(smem + Cfg::kOffBar);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    using Work = FwdWork<kSingle>;
-    const Work wk{n_blocks * BH, BH, n_blocks, (T + kBlockK - 1) / kBlockK, T, H, orders, kCausal};
+    using Work = FwdWork<D, kSingle>;
+    const Work wk{n_blocks * BH, BH, n_blocks, (T + kBlockK - 1) / kBlockK, T, H, chunk, orders, kCausal};
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -728,10 +744,11 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     // B=1, H=16, T=1024 without the mask: 20.9 -> 18.1 us.
     const bool single = static_cast<long long>(n_tiles) * BH <= num_sms;
     const int n_blocks = single ? n_tiles : (n_tiles + 1) / 2;
+    const int chunk = D == 128 ? heads_per_chunk(BH, n_blocks, s.T, D, num_sms) : BH;
     const dim3 grid(static_cast<unsigned>(n_blocks) * BH);  // one CTA per item; those that do not start at once are taken over
     auto go = [&](auto kernel) {
         return launch_overlapped(kernel, grid, dim3(kFwdThreads), FwdCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmO, LSE, s.T,
-                                 BH, s.H, orders, n_blocks, s.scale, wait_limit, inject, dev_status);
+                                 BH, s.H, orders, n_blocks, chunk, s.scale, wait_limit, inject, dev_status);
     };
     if (single)
         return strided ? go(attn_fwd_kernel<D, kCausal, true, true>) : go(attn_fwd_kernel<D, kCausal, false, true>);
