@@ -50,8 +50,7 @@ struct FwdCfg {
     // Where O goes on its way out.  D=64: into the tile's Q buffer of the item, which has a second stage.  D=128: through
     // 16 KB per tile of its own, half of the columns at a time, so that the one Q stage can take the next item's Q as
     // soon as the last Q K^T has read it instead of after the item's O has left: 207 -> 188 us at B=16, H=32, T=1024, 66
-    // -> 59 us at B=4, H=32, T=1000, 33 -> 28 us at B=64, H=12, T=100.  Items of a single tile, as a rule the only one of
-    // their CTA, keep to the Q buffer (18.5 against 21 us at B=1, H=16, T=1024 without the mask).
+    // -> 59 us at B=4, H=32, T=1000, 33 -> 28 us at B=64, H=12, T=100. 
     static constexpr bool kOwnStage = (kQStages == 1);
     static constexpr int kOffO = kOffV + kKVStages * kTileBytes;      // kOwnStage: [2 tiles]
     static constexpr int kOffBar = kOffO + (kOwnStage ? 2 * kHalfTileBytes : 0);
@@ -69,6 +68,7 @@ struct FwdBars {
     uint64_t q_full[2], q_empty[2];
     uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2];
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2], o_free[2], o_staged[2], o_sent[2];  // per query tile
+    uint64_t half_ready[2][2], sums_ready;  // kSingle: [key half][S buffer]; the second half's sums are in shared memory
     uint64_t drain;
     WorkRing ring;  // item numbers: producer -> UMMA issuer and softmax warps
     uint32_t tmem_base;
@@ -84,8 +84,6 @@ struct FwdWork {
     static constexpr bool kChunks = (D == 128) && !kSingle;
     static constexpr int kRows = kSingle ? kBlockQ : kBlockRows;
     static constexpr int kTiles = kRows / kBlockQ;
-    template <typename Cfg>
-    static constexpr bool own_stage = Cfg::kOwnStage && !kSingle;
     int n_items, BH, n_blocks, n_kv_all, T, H, chunk;
     uint32_t orders;  // coordinate orders of the Q, K, V, O tensor maps, four bits each
     bool causal;
@@ -197,7 +195,7 @@ template <int D, typename Work>
 __device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const Work& wk,
                                         long long limit) {
     using Cfg = FwdCfg<D>;
-    constexpr bool kOwnStage = Work::template own_stage<Cfg>;
+    constexpr bool kOwnStage = Cfg::kOwnStage;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescQK = umma_idesc_bf16(128, 128, 0, 0);
     constexpr uint32_t kIdescPV = umma_idesc_bf16(128, D, 0, 1);
@@ -381,7 +379,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                                             float* __restrict__ LSE, float scale, const Work& wk, int t, int swarp,
                                             int lane, long long limit) {
     using Cfg = FwdCfg<D>;
-    constexpr bool kOwnStage = Work::template own_stage<Cfg>;
+    constexpr bool kOwnStage = Cfg::kOwnStage;
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * (swarp & 3);
     const int row_local = lane_base + lane;
@@ -630,23 +628,273 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                         tma_store_tile<kStrided>(tmO, stage + h * kHalfTileBytes, (wk.orders >> 12) & 15, h * kBoxCols,
                                                  qt * kBlockQ, kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
                     bulk_commit_group();
-                    if (Cfg::kQStages == 1) {  // the next item's Q tile needs this very buffer
-                        bulk_wait_group_read<0>();
-                        mbar_arrive(&bars->q_empty[qs]);
-                    }
                 }
             }
         }
         // With two Q stages the buffer is only needed for the item after next: it is handed back after the next
         // item's first key tile, when the store has long read it, instead of holding this warp up now (worth 7 %
         // at B=8, H=12, T=1024; a separate store thread that waits in the softmax warps' stead was slower).
-        if (Cfg::kQStages > 1 || kOwnStage) pending_qs = qs;
+        pending_qs = qs;
         // Brings the leader back together with the rest of its warp before the next warp-wide TMEM
         // load, and makes a failed wait of the leader a failure of the whole warp.
         ok = __all_sync(0xffffffffu, leader_ok);
         if (!ok) break;
         ++w;
         ++wt;
+    }
+    if (leader) bulk_wait_group<0>();  // O must be complete before the kernel ends
+}
+
+// ---- Items of a single query tile (small problems): the softmax warpgroups share the tile.  Group t takes keys 64t to
+// 64t + 63 of every key tile, with a running maximum, a sum and an accumulator O_t of its own (keys split as between two
+// CTAs), so that they never wait for each other; at the end of the item group 0 reads both accumulators out of
+// TMEM and brings them to a common maximum.  Against one group with the whole row a key tile takes 64 exponentials a
+// thread instead of 128, which is the chain that bounds these problems.  TMEM: two buffers of S, columns 0-127 and
+// 128-255, each half with its own bf16 P over its first 32 columns, so that Q K^T runs two tiles ahead; O_t as above.
+template <int D, typename Work>
+__device__ __forceinline__ void fwd_mma_single(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const Work& wk,
+                                               long long limit) {
+    using Cfg = FwdCfg<D>;
+    volatile int* abort_flag = &bars->abort_flag;
+    constexpr uint32_t kIdescQK = umma_idesc_bf16(128, 128, 0, 0);
+    constexpr uint32_t kIdescPV = umma_idesc_bf16(128, D, 0, 1);
+    const uint32_t hi = umma_desc_hi_sw128(1024);
+    const uint32_t k_k0 = umma_desc_lo(smem_u32(smem + Cfg::kOffK), 16);
+    const uint32_t v_m0 = umma_desc_lo(smem_u32(smem + Cfg::kOffV), kHalfTileBytes);
+    constexpr uint32_t kStageStep = Cfg::kTileBytes >> 4;
+    const bool el = elect_one();
+    const int lane = threadIdx.x & 31;
+    bool ok = true;
+    int w = 0, g = 0;  // items, key tiles of all items
+    // S = Q K^T for key tile gk into buffer gk & 1; what that buffer held was consumed by P V products queued earlier
+    auto issue_qk = [&](int gk, uint32_t q_desc) {
+        ok = mbar_wait(&bars->k_full[gk & 1], (gk >> 1) & 1, abort_flag, limit);
+        if (!ok) return;
+        tc_fence_after();
+        if (el) {
+            const uint32_t b = k_k0 + (gk & 1) * kStageStep;
+#pragma unroll
+            for (int k = 0; k < D / 16; ++k) {
+                const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
+                umma_ss(tmem_base + 128 * (gk & 1), umma_desc_join(q_desc + off, hi), umma_desc_join(b + off, hi), kIdescQK,
+                        k > 0 ? 1u : 0u);
+            }
+            tc_commit(&bars->s_full[gk & 1]);
+            tc_commit(&bars->k_empty[gk & 1]);
+        }
+        __syncwarp();
+    };
+    for (;;) {
+        const int item = bars->ring.take(w, lane, abort_flag, limit);
+        if (item < 0) {
+            ok = (item == -1);
+            break;
+        }
+        int blk, bh, n, n_b;
+        wk.get(item, &blk, &bh, &n, &n_b);
+        const int qs = w % Cfg::kQStages;
+        const uint32_t q_k = umma_desc_lo(smem_u32(smem + Cfg::kOffQ + qs * 2 * Cfg::kTileBytes), 16);
+        ok = mbar_wait(&bars->q_full[qs], (w / Cfg::kQStages) & 1, abort_flag, limit);
+        if (ok) issue_qk(g, q_k);
+        if (ok && n > 1) issue_qk(g + 1, q_k);
+        for (int j = 0; j < n && ok; ++j, ++g) {
+            const int st = g & 1;
+            ok = mbar_wait(&bars->v_full[st], (g >> 1) & 1, abort_flag, limit);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (ok) ok = mbar_wait(&bars->half_ready[t][st], (g >> 1) & 1, abort_flag, limit);
+                // the previous item's O_t must have been read out of TMEM before it is overwritten
+                if (ok && j == 0 && w > 0) ok = mbar_wait(&bars->o_free[t], (w - 1) & 1, abort_flag, limit);
+                if (!ok) break;
+                tc_fence_after();
+                // O_t += P V over the 64 keys of half t: V rows 64t on (128 bytes each), MN-major
+                if (el) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        umma_ts(tmem_base + Cfg::kColO + D * t, tmem_base + 128 * st + 64 * t + 8 * k,
+                                umma_desc_join(v_m0 + st * kStageStep + ((64 * 128 * t) >> 4) + k * 128, hi), kIdescPV,
+                                (j > 0 || k > 0) ? 1u : 0u);
+                    tc_commit(&bars->pv_done[t]);
+                }
+                __syncwarp();
+            }
+            if (!ok) break;
+            if (el) tc_commit(&bars->v_empty[st]);
+            __syncwarp();
+            if (j + 2 < n) issue_qk(g + 2, q_k);
+        }
+        if (!ok) break;
+        ++w;
+    }
+    if (!ok) {
+        int none = 0;
+        if (el) tc_commit(&bars->drain);
+        __syncwarp();
+        (void)mbar_wait(&bars->drain, 0, &none);
+    }
+}
+
+template <int D, bool kCausal, bool kStrided, typename Work>
+__device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const CUtensorMap* tmO,
+                                                   float* __restrict__ LSE, float scale, const Work& wk, int t, int swarp,
+                                                   int lane, long long limit) {
+    using Cfg = FwdCfg<D>;
+    volatile int* abort_flag = &bars->abort_flag;
+    const uint32_t lane_base = 32u * (swarp & 3);
+    const int row_local = lane_base + lane;
+    const bool leader = (t == 0 && swarp == 0 && lane == 0);
+    const uint32_t t_o = tmem_addr(tmem_base, lane_base, Cfg::kColO + D * t);
+    float2* sums = reinterpret_cast<float2*>(smem + Cfg::kOffQ + Cfg::kTileBytes);  // the unused Q buffer of tile B
+    const float c = scale * kLog2e;
+    const uint64_t c2 = f32x2_pack(c, c);
+    const int T = wk.T;
+    bool ok = true;
+    int w = 0, cnt = 0;  // items, key tiles of all items
+    for (;;) {
+        const int item = bars->ring.take(w, lane, abort_flag, limit);
+        if (item < 0) {
+            ok = (item == -1);
+            break;
+        }
+        int blk, bh, n, n_b;
+        wk.get(item, &blk, &bh, &n, &n_b);
+        const int row = blk * kBlockQ + row_local;
+        float m_ref = -INFINITY, l = 0.f;  // -inf while the half has had no key that the row keeps
+        for (int j = 0; j < n; ++j, ++cnt) {
+            const int buf = cnt & 1;
+            ok = mbar_wait(&bars->s_full[buf], (cnt >> 1) & 1, abort_flag, limit);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t t_s = tmem_addr(tmem_base, lane_base, 128 * buf + 64 * t);
+            uint32_t sr[64];
+            tmem_ld_x32(t_s, sr);
+            tmem_ld_x32(t_s + 32, sr + 32);
+            tmem_wait_ld();
+            const bool diag = kCausal && (j == blk);
+            const int keys_left = T - j * kBlockK;
+            if (diag || keys_left < kBlockK) {
+                const int lim = (diag ? min(row_local, keys_left - 1) : keys_left - 1) - 64 * t;
+#pragma unroll
+                for (int i = 0; i < 64; ++i)
+                    if (i > lim) sr[i] = 0xff800000u;  // -inf
+            }
+            float mx0 = fmaxf(__uint_as_float(sr[0]), __uint_as_float(sr[1]));
+            float mx1 = fmaxf(__uint_as_float(sr[2]), __uint_as_float(sr[3]));
+#pragma unroll
+            for (int i = 4; i < 64; i += 4) {
+                mx0 = fmax3(mx0, __uint_as_float(sr[i + 0]), __uint_as_float(sr[i + 1]));
+                mx1 = fmax3(mx1, __uint_as_float(sr[i + 2]), __uint_as_float(sr[i + 3]));
+            }
+            const float m_new = fmaxf(m_ref, fmaxf(mx0, mx1));
+            if (j == 0) {
+                m_ref = m_new;
+            } else if (__any_sync(0xffffffffu, (m_new - m_ref) * c > kRescaleThreshold)) {  // (-inf against -inf: no)
+                const float f = m_new > m_ref ? ex2_approx((m_ref - m_new) * c) : 1.f;  // 0 from -inf
+                m_ref = m_new;
+                l *= f;
+                ok = mbar_wait(&bars->pv_done[t], (cnt - 1) & 1, abort_flag, limit);
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll 1
+                for (int cb = 0; cb < D; cb += 16) {
+                    uint32_t o[16];
+                    tmem_ld_x16(t_o + cb, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+                    tmem_st_x16(t_o + cb, o);
+                }
+            }
+            const float mc = m_ref == -INFINITY ? 0.f : m_ref * c;
+            const uint64_t nmc2 = f32x2_pack(-mc, -mc);
+            uint64_t acc0 = 0, acc1 = 0;
+            uint32_t pk[32];
+#pragma unroll
+            for (int i = 0; i < 64; i += 4) {
+                float x0, x1, x2, x3;
+                f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sr[i + 0]), __uint_as_float(sr[i + 1])), c2, nmc2), x0, x1);
+                f32x2_unpack(f32x2_fma(f32x2_pack(__uint_as_float(sr[i + 2]), __uint_as_float(sr[i + 3])), c2, nmc2), x2, x3);
+                const float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
+                acc0 = f32x2_add(acc0, f32x2_pack(p0, p1));
+                acc1 = f32x2_add(acc1, f32x2_pack(p2, p3));
+                pk[i / 2] = pack_bf16x2(p0, p1);
+                pk[i / 2 + 1] = pack_bf16x2(p2, p3);
+            }
+            tmem_st_x32(t_s, pk);
+            float a0, a1, a2, a3;
+            f32x2_unpack(acc0, a0, a1);
+            f32x2_unpack(acc1, a2, a3);
+            l += (a0 + a1) + (a2 + a3);
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->half_ready[t][buf]);
+        }
+        if (!ok) break;
+        if (t == 1) {
+            // The other group reads O_1 from TMEM itself.  The sums are not overwritten too early: the next item gets no
+            // further than its second tile without that group.
+            sums[row_local] = make_float2(m_ref, l);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->sums_ready);
+            ++w;
+            continue;
+        }
+        const int qs = w % Cfg::kQStages;
+        uint8_t* stage = smem + Cfg::kOffQ + qs * 2 * Cfg::kTileBytes;  // no longer read: every Q K^T has completed
+        ok = mbar_wait(&bars->pv_done[0], (cnt - 1) & 1, abort_flag, limit);
+        if (ok) ok = mbar_wait(&bars->pv_done[1], (cnt - 1) & 1, abort_flag, limit);
+        if (ok) ok = mbar_wait(&bars->sums_ready, w & 1, abort_flag, limit);
+        if (!ok) break;
+        tc_fence_after();
+        const float2 other = sums[row_local];
+        const float m = fmaxf(m_ref, other.x);  // finite: key 0 is in this half and every row keeps it
+        const float fa = ex2_approx((m_ref - m) * c), fb = ex2_approx((other.x - m) * c);  // 2^-inf = 0
+        l = l * fa + other.y * fb;
+        const float ia = fa / l, ib = fb / l;
+#pragma unroll
+        for (int cb = 0; cb < D; cb += 32) {
+            uint32_t a[32], b[32];
+            tmem_ld_x32(t_o + cb, a);
+            tmem_ld_x32(t_o + D + cb, b);
+            tmem_wait_ld();
+            uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + row_local * 128;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
+                uint32_t v[4];
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    v[y] = pack_bf16x2(fmaf(__uint_as_float(a[8 * x + 2 * y]), ia, __uint_as_float(b[8 * x + 2 * y]) * ib),
+                                       fmaf(__uint_as_float(a[8 * x + 2 * y + 1]), ia, __uint_as_float(b[8 * x + 2 * y + 1]) * ib));
+                *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (row_local & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
+            }
+        }
+        tc_fence_before();
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+            mbar_arrive(&bars->o_free[0]);
+            mbar_arrive(&bars->o_free[1]);
+            mbar_arrive(&bars->o_staged[0]);
+        }
+        if (row < T) LSE[static_cast<size_t>(bh) * T + row] = m * scale + logf(l);
+        bool leader_ok = true;
+        if (leader) {
+            leader_ok = mbar_wait(&bars->o_staged[0], w & 1, abort_flag, limit);
+            if (leader_ok) {
+#pragma unroll
+                for (int h = 0; h < Cfg::kHalves; ++h)
+                    tma_store_tile<kStrided>(tmO, stage + h * kHalfTileBytes, (wk.orders >> 12) & 15, h * kBoxCols,
+                                             blk * kBlockQ, kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
+                bulk_commit_group();
+                bulk_wait_group_read<0>();
+                mbar_arrive(&bars->q_empty[qs]);
+            }
+        }
+        ok = __all_sync(0xffffffffu, leader_ok);
+        if (!ok) break;
+        ++w;
     }
     if (leader) bulk_wait_group<0>();  // O must be complete before the kernel ends
 }
@@ -669,7 +917,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int s = 0; s < 2; ++s) {
             mbar_init(&bars->q_full[s], 1);
             // the store leaders of the two query tiles, or the UMMA issuer where O has buffers of its own
-            mbar_init(&bars->q_empty[s], Work::template own_stage<Cfg> ? 1 : 2);
+            mbar_init(&bars->q_empty[s], kSingle || Cfg::kOwnStage ? 1 : 2);
             mbar_init(&bars->o_sent[s], 1);
             mbar_init(&bars->k_full[s], 1);
             mbar_init(&bars->k_empty[s], 1);
@@ -681,7 +929,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             mbar_init(&bars->pv_done[s], 1);
             mbar_init(&bars->o_free[s], 4);
             mbar_init(&bars->o_staged[s], 4);
+            mbar_init(&bars->half_ready[s][0], 4);
+            mbar_init(&bars->half_ready[s][1], 4);
         }
+        mbar_init(&bars->sums_ready, 4);
         mbar_init(&bars->drain, 1);
         bars->ring.init(kWorkConsumers);
         bars->abort_flag = 0;
@@ -720,10 +971,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (warp == 0) {
         if (lane == 0) fwd_producer<D, kStrided>(&tmQ, &tmK, &tmV, smem, bars, wk, limit, inject);
     } else if (warp == 1) {
-        fwd_mma<D>(smem, bars, tmem_base, wk, limit);
+        if constexpr (kSingle) fwd_mma_single<D>(smem, bars, tmem_base, wk, limit);
+        else fwd_mma<D>(smem, bars, tmem_base, wk, limit);
     } else if (warp >= 4) {
         const int t = (warp - 4) >> 2;
-        fwd_softmax<D, kCausal, kStrided>(smem, bars, tmem_base, &tmO, LSE, scale, wk, t, (warp - 4) & 3, lane, limit);
+        if constexpr (kSingle)
+            fwd_softmax_single<D, kCausal, kStrided>(smem, bars, tmem_base, &tmO, LSE, scale, wk, t, (warp - 4) & 3, lane, limit);
+        else
+            fwd_softmax<D, kCausal, kStrided>(smem, bars, tmem_base, &tmO, LSE, scale, wk, t, (warp - 4) & 3, lane, limit);
     }
 
     tc_fence_before();
@@ -739,9 +994,8 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     const int BH = s.B * s.H;
     const int n_tiles = (s.T + kBlockQ - 1) / kBlockQ;
     // Pairs of query tiles share their K and V tiles and fill each other's gaps; but if every tile can have an SM of its
-    // own, a tile is done sooner alone (softmax of one tile: 1450 clocks, of two at a time 2300).  D=64, pairs against
-    // single tiles: B=1, H=12, T=777: 13.6 -> 12.1 us, T=1500: 23.4 -> 18.0 us; H=1, T=8192: 99.5 -> 76.8 us; D=128,
-    // B=1, H=16, T=1024 without the mask: 20.9 -> 18.1 us.
+    // own, a tile is done sooner alone, with both softmax groups on it.  Pairs, single tiles: D=64, B=1, H=12, T=777: 13.6,
+    // 10.0 us; T=1500: 23.4, 14.7 us; H=1, T=8192: 99.5, 56.5 us; D=128, B=1, H=16, T=1024 without the mask: 20.9, 12.9 us.
     const bool single = static_cast<long long>(n_tiles) * BH <= num_sms;
     const int n_blocks = single ? n_tiles : (n_tiles + 1) / 2;
     const int chunk = D == 128 ? heads_per_chunk(BH, n_blocks, s.T, D, num_sms) : BH;
