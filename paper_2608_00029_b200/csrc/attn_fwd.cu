@@ -68,7 +68,7 @@ struct FwdBars {
     uint64_t q_full[2], q_empty[2];
     uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2];
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2], o_free[2], o_staged[2], o_sent[2];  // per query tile
-    uint64_t half_ready[2][2], sums_ready;  // kSingle: [key half][S buffer]; the second half's sums are in shared memory
+    uint64_t half_ready[2][2], sums_ready, o_done;  // kSingle: [key half][S buffer]; the second half's sums are in shared memory
     uint64_t drain;
     WorkRing ring;  // item numbers: producer -> UMMA issuer and softmax warps
     uint32_t tmem_base;
@@ -719,7 +719,10 @@ __device__ __forceinline__ void fwd_mma_single(uint8_t* smem, FwdBars* bars, uin
                 __syncwarp();
             }
             if (!ok) break;
-            if (el) tc_commit(&bars->v_empty[st]);
+            if (el) {
+                tc_commit(&bars->v_empty[st]);
+                if (j + 1 == n) tc_commit(&bars->o_done);
+            }
             __syncwarp();
             if (j + 2 < n) issue_qk(g + 2, q_k);
         }
@@ -842,8 +845,9 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
         }
         const int qs = w % Cfg::kQStages;
         uint8_t* stage = smem + Cfg::kOffQ + qs * 2 * Cfg::kTileBytes;  // no longer read: every Q K^T has completed
-        ok = mbar_wait(&bars->pv_done[0], (cnt - 1) & 1, abort_flag, limit);
-        if (ok) ok = mbar_wait(&bars->pv_done[1], (cnt - 1) & 1, abort_flag, limit);
+        // Not pv_done: of the tile before the last, P V may be outstanding still (S runs two tiles ahead, and the other group
+        // may be a tile behind), and a wait two phases on would pass at once.
+        ok = mbar_wait(&bars->o_done, w & 1, abort_flag, limit);
         if (ok) ok = mbar_wait(&bars->sums_ready, w & 1, abort_flag, limit);
         if (!ok) break;
         tc_fence_after();
@@ -933,6 +937,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             mbar_init(&bars->half_ready[s][1], 4);
         }
         mbar_init(&bars->sums_ready, 4);
+        mbar_init(&bars->o_done, 1);
         mbar_init(&bars->drain, 1);
         bars->ring.init(kWorkConsumers);
         bars->abort_flag = 0;
