@@ -68,7 +68,7 @@ struct FwdBars {
     uint64_t q_full[2], q_empty[2];
     uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2];
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2], o_free[2], o_staged[2], o_sent[2];  // per query tile
-    uint64_t half_ready[2][2], sums_ready, o_done;  // kSingle: [key half][S buffer]; the second half's sums are in shared memory
+    uint64_t half_ready[2][2], sums_ready, o_done;  // kSingle: [key half][S buffer]; the groups' sums are in shared memory
     uint64_t drain;
     WorkRing ring;  // item numbers: producer -> UMMA issuer and softmax warps
     uint32_t tmem_base;
@@ -647,8 +647,8 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
 
 // ---- Items of a single query tile (small problems): the softmax warpgroups share the tile.  Group t takes keys 64t to
 // 64t + 63 of every key tile, with a running maximum, a sum and an accumulator O_t of its own (keys split as between two
-// CTAs), so that they never wait for each other; at the end of the item group 0 reads both accumulators out of
-// TMEM and brings them to a common maximum.  Against one group with the whole row a key tile takes 64 exponentials a
+// CTAs), so that they never wait for each other; at the end of the item both read the accumulators out of TMEM, half of the
+// columns each, and bring them to a common maximum.  Against one group with the whole row a key tile takes 64 exponentials a
 // thread instead of 128, which is the chain that bounds these problems.  TMEM: two buffers of S, columns 0-127 and
 // 128-255, each half with its own bf16 P over its first 32 columns, so that Q K^T runs two tiles ahead; O_t as above.
 template <int D, typename Work>
@@ -684,8 +684,13 @@ __device__ __forceinline__ void fwd_mma_single(uint8_t* smem, FwdBars* bars, uin
         }
         __syncwarp();
     };
+    constexpr int kNotPeeked = -3;
+    int peeked = kNotPeeked;    // the next item's number, if it was looked at from inside the current item
+    bool first_queued = false;  // ... and its first Q K^T was queued from there
+    auto q_desc_of = [&](int stage) { return umma_desc_lo(smem_u32(smem + Cfg::kOffQ + stage * 2 * Cfg::kTileBytes), 16); };
     for (;;) {
-        const int item = bars->ring.take(w, lane, abort_flag, limit);
+        const int item = (peeked != kNotPeeked) ? peeked : bars->ring.take(w, lane, abort_flag, limit);
+        peeked = kNotPeeked;
         if (item < 0) {
             ok = (item == -1);
             break;
@@ -693,18 +698,35 @@ __device__ __forceinline__ void fwd_mma_single(uint8_t* smem, FwdBars* bars, uin
         int blk, bh, n, n_b;
         wk.get(item, &blk, &bh, &n, &n_b);
         const int qs = w % Cfg::kQStages;
-        const uint32_t q_k = umma_desc_lo(smem_u32(smem + Cfg::kOffQ + qs * 2 * Cfg::kTileBytes), 16);
-        ok = mbar_wait(&bars->q_full[qs], (w / Cfg::kQStages) & 1, abort_flag, limit);
-        if (ok) issue_qk(g, q_k);
+        const uint32_t q_k = q_desc_of(qs);
+        if (!first_queued) {
+            ok = mbar_wait(&bars->q_full[qs], (w / Cfg::kQStages) & 1, abort_flag, limit);
+            if (ok) issue_qk(g, q_k);
+        }
+        first_queued = false;
         if (ok && n > 1) issue_qk(g + 1, q_k);
         for (int j = 0; j < n && ok; ++j, ++g) {
             const int st = g & 1;
-            ok = mbar_wait(&bars->v_full[st], (g >> 1) & 1, abort_flag, limit);
+            if (Cfg::kQStages > 1 && j + 1 == n && bars->ring.published(w + 1)) {
+                // Last key tile: the first Q K^T of the next item, if its Q and K have landed, so that neither softmax group
+                // waits at the item boundary.
+                peeked = bars->ring.take(w + 1, lane, abort_flag, limit);
+                if (peeked >= 0) {
+                    const int qs2 = (w + 1) % Cfg::kQStages;
+                    const bool there = mbar_test(&bars->q_full[qs2], ((w + 1) / Cfg::kQStages) & 1) &&
+                                       mbar_test(&bars->k_full[st ^ 1], ((g + 1) >> 1) & 1);
+                    if (__all_sync(0xffffffffu, there)) {
+                        issue_qk(g + 1, q_desc_of(qs2));
+                        first_queued = true;
+                    }
+                }
+            }
+            if (ok) ok = mbar_wait(&bars->v_full[st], (g >> 1) & 1, abort_flag, limit);
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
                 if (ok) ok = mbar_wait(&bars->half_ready[t][st], (g >> 1) & 1, abort_flag, limit);
                 // the previous item's O_t must have been read out of TMEM before it is overwritten
-                if (ok && j == 0 && w > 0) ok = mbar_wait(&bars->o_free[t], (w - 1) & 1, abort_flag, limit);
+                if (ok && j == 0 && w > 0 && t == 0) ok = mbar_wait(&bars->o_free[0], (w - 1) & 1, abort_flag, limit);
                 if (!ok) break;
                 tc_fence_after();
                 // O_t += P V over the 64 keys of half t: V rows 64t on (128 bytes each), MN-major
@@ -747,12 +769,16 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
     const int row_local = lane_base + lane;
     const bool leader = (t == 0 && swarp == 0 && lane == 0);
     const uint32_t t_o = tmem_addr(tmem_base, lane_base, Cfg::kColO + D * t);
-    float2* sums = reinterpret_cast<float2*>(smem + Cfg::kOffQ + Cfg::kTileBytes);  // the unused Q buffer of tile B
+    const uint32_t t_o_half = tmem_addr(tmem_base, lane_base, Cfg::kColO + D / 2 * t);
+    // [item & 1][group][row], in the unused Q buffer of tile B.  Two items' worth: a group may be through the tiles of
+    // the next item (if there are no more than two) before the other has read the sums of this one.
+    float2* sums = reinterpret_cast<float2*>(smem + Cfg::kOffQ + Cfg::kTileBytes);
     const float c = scale * kLog2e;
     const uint64_t c2 = f32x2_pack(c, c);
     const int T = wk.T;
     bool ok = true;
-    int w = 0, cnt = 0;  // items, key tiles of all items
+    int w = 0, cnt = 0;   // items, key tiles of all items
+    int pending_qs = -1;  // Q stage whose O store was issued at the end of the previous item
     for (;;) {
         const int item = bars->ring.take(w, lane, abort_flag, limit);
         if (item < 0) {
@@ -832,45 +858,50 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars->half_ready[t][buf]);
+            if (pending_qs >= 0) {
+                if (leader) {
+                    bulk_wait_group_read<0>();
+                    mbar_arrive(&bars->q_empty[pending_qs]);
+                }
+                pending_qs = -1;
+                __syncwarp();
+            }
         }
         if (!ok) break;
-        if (t == 1) {
-            // The other group reads O_1 from TMEM itself.  The sums are not overwritten too early: the next item gets no
-            // further than its second tile without that group.
-            sums[row_local] = make_float2(m_ref, l);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars->sums_ready);
-            ++w;
-            continue;
-        }
+        // ---- end of the item: both groups read both accumulators, D/2 columns each, and bring them to one maximum
+        float2* const s_w = sums + (w & 1) * 2 * kBlockQ;
+        s_w[t * kBlockQ + row_local] = make_float2(m_ref, l);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->sums_ready);
         const int qs = w % Cfg::kQStages;
         uint8_t* stage = smem + Cfg::kOffQ + qs * 2 * Cfg::kTileBytes;  // no longer read: every Q K^T has completed
+        ok = mbar_wait(&bars->sums_ready, w & 1, abort_flag, limit);
         // Not pv_done: of the tile before the last, P V may be outstanding still (S runs two tiles ahead, and the other group
         // may be a tile behind), and a wait two phases on would pass at once.
-        ok = mbar_wait(&bars->o_done, w & 1, abort_flag, limit);
-        if (ok) ok = mbar_wait(&bars->sums_ready, w & 1, abort_flag, limit);
+        if (ok) ok = mbar_wait(&bars->o_done, w & 1, abort_flag, limit);
         if (!ok) break;
         tc_fence_after();
-        const float2 other = sums[row_local];
-        const float m = fmaxf(m_ref, other.x);  // finite: key 0 is in this half and every row keeps it
-        const float fa = ex2_approx((m_ref - m) * c), fb = ex2_approx((other.x - m) * c);  // 2^-inf = 0
-        l = l * fa + other.y * fb;
-        const float ia = fa / l, ib = fb / l;
+        const float2 s0 = s_w[row_local], s1 = s_w[kBlockQ + row_local];
+        const float m = fmaxf(s0.x, s1.x);  // finite: key 0 is in the first half and every row keeps it
+        const float f0 = ex2_approx((s0.x - m) * c), f1 = ex2_approx((s1.x - m) * c);  // 2^-inf = 0
+        l = s0.y * f0 + s1.y * f1;
+        const float i0 = f0 / l, i1 = f1 / l;
 #pragma unroll
-        for (int cb = 0; cb < D; cb += 32) {
+        for (int cb = 0; cb < D / 2; cb += 32) {
             uint32_t a[32], b[32];
-            tmem_ld_x32(t_o + cb, a);
-            tmem_ld_x32(t_o + D + cb, b);
+            tmem_ld_x32(t_o_half + cb, a);
+            tmem_ld_x32(t_o_half + D + cb, b);
             tmem_wait_ld();
-            uint8_t* row_ptr = stage + (cb / 64) * kHalfTileBytes + row_local * 128;
+            const int col = D / 2 * t + cb;
+            uint8_t* row_ptr = stage + (col / 64) * kHalfTileBytes + row_local * 128;
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
-                const int ch = (cb % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
+                const int ch = (col % 64) / 8 + x;  // 16-byte chunk of the 128-byte swizzled row
                 uint32_t v[4];
 #pragma unroll
                 for (int y = 0; y < 4; ++y)
-                    v[y] = pack_bf16x2(fmaf(__uint_as_float(a[8 * x + 2 * y]), ia, __uint_as_float(b[8 * x + 2 * y]) * ib),
-                                       fmaf(__uint_as_float(a[8 * x + 2 * y + 1]), ia, __uint_as_float(b[8 * x + 2 * y + 1]) * ib));
+                    v[y] = pack_bf16x2(fmaf(__uint_as_float(a[8 * x + 2 * y]), i0, __uint_as_float(b[8 * x + 2 * y]) * i1),
+                                       fmaf(__uint_as_float(a[8 * x + 2 * y + 1]), i0, __uint_as_float(b[8 * x + 2 * y + 1]) * i1));
                 *reinterpret_cast<uint4*>(row_ptr + ((ch ^ (row_local & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
             }
         }
@@ -879,10 +910,9 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
         __syncwarp();
         if (lane == 0) {
             mbar_arrive(&bars->o_free[0]);
-            mbar_arrive(&bars->o_free[1]);
             mbar_arrive(&bars->o_staged[0]);
         }
-        if (row < T) LSE[static_cast<size_t>(bh) * T + row] = m * scale + logf(l);
+        if (t == 0 && row < T) LSE[static_cast<size_t>(bh) * T + row] = m * scale + logf(l);
         bool leader_ok = true;
         if (leader) {
             leader_ok = mbar_wait(&bars->o_staged[0], w & 1, abort_flag, limit);
@@ -892,10 +922,13 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
                     tma_store_tile<kStrided>(tmO, stage + h * kHalfTileBytes, (wk.orders >> 12) & 15, h * kBoxCols,
                                              blk * kBlockQ, kStrided ? bh % wk.H : 0, kStrided ? bh / wk.H : 0, bh);
                 bulk_commit_group();
-                bulk_wait_group_read<0>();
-                mbar_arrive(&bars->q_empty[qs]);
+                if (Cfg::kQStages == 1) {  // the next item's Q tile needs this very buffer
+                    bulk_wait_group_read<0>();
+                    mbar_arrive(&bars->q_empty[qs]);
+                }
             }
         }
+        if (Cfg::kQStages > 1) pending_qs = qs;  // handed back after the next item's first tile, as with pairs
         ok = __all_sync(0xffffffffu, leader_ok);
         if (!ok) break;
         ++w;
@@ -931,12 +964,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             mbar_init(&bars->s_free[s], 4);
             mbar_init(&bars->p_ready[s], 4);
             mbar_init(&bars->pv_done[s], 1);
-            mbar_init(&bars->o_free[s], 4);
-            mbar_init(&bars->o_staged[s], 4);
+            mbar_init(&bars->o_free[s], kSingle ? 8 : 4);
+            mbar_init(&bars->o_staged[s], kSingle ? 8 : 4);
             mbar_init(&bars->half_ready[s][0], 4);
             mbar_init(&bars->half_ready[s][1], 4);
         }
-        mbar_init(&bars->sums_ready, 4);
+        mbar_init(&bars->sums_ready, 8);
         mbar_init(&bars->o_done, 1);
         mbar_init(&bars->drain, 1);
         bars->ring.init(kWorkConsumers);
@@ -1001,7 +1034,10 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     // Pairs of query tiles share their K and V tiles and fill each other's gaps; but if every tile can have an SM of its
     // own, a tile is done sooner alone, with both softmax groups on it.  Pairs, single tiles: D=64, B=1, H=12, T=777: 13.6,
     // 10.0 us; T=1500: 23.4, 14.7 us; H=1, T=8192: 99.5, 56.5 us; D=128, B=1, H=16, T=1024 without the mask: 20.9, 12.9 us.
-    const bool single = static_cast<long long>(n_tiles) * BH <= num_sms;
+    // With T <= 128 a pair has no second tile and one softmax group would be idle.  At D=64 that alone decides: B=64, H=12,
+    // T=100: 20.1, 17.4 us; B=50, T=17: 16.1, 14.2 us.  At D=128 O and the next Q tile share a buffer in this form, and
+    // items follow each other sooner in the other: B=64, H=12, T=100: 25.1, 29.8 us; B=8, H=32, T=128: 10.7, 12.0 us.
+    const bool single = static_cast<long long>(n_tiles) * BH <= num_sms || (D == 64 && n_tiles == 1);
     const int n_blocks = single ? n_tiles : (n_tiles + 1) / 2;
     const int chunk = D == 128 ? heads_per_chunk(BH, n_blocks, s.T, D, num_sms) : BH;
     const dim3 grid(static_cast<unsigned>(n_blocks) * BH);  // one CTA per item; those that do not start at once are taken over
