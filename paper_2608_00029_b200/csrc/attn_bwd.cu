@@ -52,6 +52,8 @@ namespace {
 constexpr int kBwdTmemCols = 512;
 // LSE/scale has to be finite.  Below this scale the scores add nothing to P (|s| < 1e6 at most), with it or without.
 constexpr float kLeastScale = 1e-30f;
+// Largest |LSE/scale| (bf16 ends at 3.39e38): times kLeastScale it is still far past where 2^x becomes 0 or infinite.
+constexpr float kMostLse = 3e38f;
 
 template <int D>
 struct BwdCfg {
@@ -74,15 +76,19 @@ struct BwdCfg {
     static constexpr bool kBulkdQ = (D == 64);
     static constexpr int kStageBytes = 2 * kHalfTileBytes;
     // At D=64 the row terms enter S^T and dP^T through the tensor core: one more instruction per product multiplies a
-    // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale and -Delta, each as three bf16 numbers
-    // that add up to it exactly to 24 bits.  The compute warps then read no rows from shared memory (512 broadcasts of
+    // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale or -Delta, each as three bf16 numbers
+    // that add up to it exactly to 24 bits.  The two terms lie in tiles of their own, so that a Delta that is not finite
+    // does not reach S (0 * inf).  The compute warps then read no rows from shared memory (512 broadcasts of
     // 16 bytes a tile, some 600 clocks of its one port, which the operands of the products need as well) and have an
     // fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at B=32, 337 -> 321 us at
     // B=1, T=8192, 214 -> 182 us at B=4, T=2048 without the mask.  D=128 has no shared memory left for the tiles.
     static constexpr bool kFold = (D == 64);
-    static constexpr int kExtBytes = 128 * 16 * 2;
-    static constexpr int kOffExt = kOffRow;                           // kFold: 2 stages, then the constants for S^T and dP^T
-    static constexpr int kOffStage = kOffRow + (kFold ? 4 * kExtBytes : 2 * 2 * 128 * 4);
+    // An operand of 128 rows x 16 columns is two planes of 128 x 8: in order -LSE/scale (two stages), -Delta (two
+    // stages), ones in columns 0-2, zeros; the last is the second plane of all the others.
+    static constexpr int kExtPlane = 128 * 8 * 2;
+    static constexpr int kExtOnes = 4, kExtZeros = 5, kExtPlanes = 6;
+    static constexpr int kOffExt = kOffRow;                           // kFold: kExtPlanes planes
+    static constexpr int kOffStage = kOffRow + (kFold ? kExtPlanes * kExtPlane : 2 * 2 * 128 * 4);
     static constexpr int kOffBar = kOffStage + kStageBytes;
     // At D=128 the tiles fill the 227 KB a CTA can have to within 512 bytes, so there is no room for
     // the padding that would let the kernel align its window itself: the kernel checks that the window
@@ -221,18 +227,19 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     // The whole warp runs this role in uniform control flow; one elected lane issues.
     const bool el = elect_one();
 
-    // The row terms of tile gq: unswizzled tiles, 8 x 16-byte core matrices 128 bytes apart along K, 256 along M and N.
-    const uint32_t ext_hi = umma_desc_hi_plain(256);
-    const uint32_t ext_b = umma_desc_lo(smem_u32(smem + Cfg::kOffExt), 128);
-    constexpr uint32_t kExtStep = Cfg::kExtBytes >> 4;
-    (void)ext_hi, (void)ext_b;
+    // The row terms of tile gq: unswizzled, 8 x 16-byte core matrices 128 bytes apart along M and N; along K the second one
+    // lies in the plane of zeros.  From one plane to the next the address grows by what that distance shrinks by.
+    const uint32_t ext_hi = umma_desc_hi_plain(128);
+    const uint32_t ext_0 = umma_desc_lo(smem_u32(smem + Cfg::kOffExt), Cfg::kExtZeros * Cfg::kExtPlane);
+    constexpr uint32_t kExtStep = (Cfg::kExtPlane >> 4) - ((Cfg::kExtPlane >> 4) << 16);
+    const uint32_t ext_ones = ext_0 + Cfg::kExtOnes * kExtStep;
+    (void)ext_hi, (void)ext_ones;
 
     auto issue_st = [&](int gq, uint32_t kd) {  // S^T = K Q^T: K tile `kd`, query tile in Q stage gq % kQStages
         const uint32_t b = q_k0 + (gq % Cfg::kQStages) * kQStageStep;
         if (el) {
             if (Cfg::kFold)
-                umma_ss(t_s, umma_desc_join(ext_b + 2 * kExtStep, ext_hi), umma_desc_join(ext_b + (gq & 1) * kExtStep, ext_hi),
-                        kIdescT, 0u);
+                umma_ss(t_s, umma_desc_join(ext_ones, ext_hi), umma_desc_join(ext_0 + (gq & 1) * kExtStep, ext_hi), kIdescT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
                 const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
@@ -246,7 +253,7 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
         const uint32_t b = do_k[gq % Cfg::kdOStages];
         if (el) {
             if (Cfg::kFold)
-                umma_ss(t_dp, umma_desc_join(ext_b + 3 * kExtStep, ext_hi), umma_desc_join(ext_b + (gq & 1) * kExtStep, ext_hi),
+                umma_ss(t_dp, umma_desc_join(ext_ones, ext_hi), umma_desc_join(ext_0 + (2 + (gq & 1)) * kExtStep, ext_hi),
                         kIdescT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
@@ -413,19 +420,20 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     }
 }
 
-// Three bf16 numbers that add up to v (to 24 bits), as the lower 16 bits of three words.
-__device__ __forceinline__ void split_bf16x3(float v, uint32_t* hi, uint32_t* mid, uint32_t* lo) {
+// Three bf16 numbers that add up to v (to 24 bits), packed as columns 0-2 of a row of 8; an infinite or NaN v is itself.
+__device__ __forceinline__ uint4 split_bf16x3(float v) {
     const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const float r = v - __bfloat162float(h);
+    const float r = isinf(v) ? 0.f : v - __bfloat162float(h);
     const __nv_bfloat16 m = __float2bfloat16_rn(r);
     const __nv_bfloat16 l = __float2bfloat16_rn(r - __bfloat162float(m));
-    *hi = __bfloat16_as_ushort(h);
-    *mid = __bfloat16_as_ushort(m);
-    *lo = __bfloat16_as_ushort(l);
+    return make_uint4(__bfloat16_as_ushort(h) | (static_cast<uint32_t>(__bfloat16_as_ushort(m)) << 16),
+                      __bfloat16_as_ushort(l), 0u, 0u);
 }
 
-// Row loader where the row terms go through the tensor core (kFold): one row of the (queries x 16) tile per query, 16
-// bytes: -LSE/scale in columns 0-2, -Delta in 3-5.  Queries past the end of the sequence get -1e30, so that their P is 0.
+// Row loader where the row terms go through the tensor core (kFold): one row of 8 columns per query in the plane of
+// -LSE/scale and in that of -Delta.  LSE/scale is held below kMostLse, which keeps what an infinite LSE means (P = 0 for
+// +inf, P = inf for -inf) without an infinity that would meet another in the sum; queries past the end of the sequence get
+// the same value, so that their P is 0.
 __device__ __forceinline__ void bwd_rows_folded(BwdBars* bars, uint8_t* ext, const float* __restrict__ LSE,
                                                 const float* __restrict__ Delta, int T, float inv_scale,
                                                 const WorkList& wl, int tid64) {
@@ -437,22 +445,21 @@ __device__ __forceinline__ void bwd_rows_folded(BwdBars* bars, uint8_t* ext, con
         const size_t row_base = static_cast<size_t>(bh) * T;
         for (int it = 0; it < n_it; ++it, ++g) {
             const int b = g & 1;
-            uint4 v[2];
+            uint4 vl[2], vd[2];
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
                 const int q = (i0 + it) * kBlockQ + tid64 + 64 * x;
-                const float l = (q < T) ? -LSE[row_base + q] * inv_scale : -1e30f;
-                const float d = (q < T) ? -Delta[row_base + q] : 0.f;
-                uint32_t w[6];
-                split_bf16x3(l, w + 0, w + 1, w + 2);
-                split_bf16x3(d, w + 3, w + 4, w + 5);
-                v[x] = make_uint4(w[0] | (w[1] << 16), w[2] | (w[3] << 16), w[4] | (w[5] << 16), 0u);
+                float l = (q < T) ? -LSE[row_base + q] * inv_scale : -kMostLse;
+                if (fabsf(l) > kMostLse) l = copysignf(kMostLse, l);  // (a NaN stays)
+                vl[x] = split_bf16x3(l);
+                vd[x] = split_bf16x3((q < T) ? -Delta[row_base + q] : 0.f);
             }
             if (!mbar_wait(&bars->row_empty[b], ((g >> 1) & 1) ^ 1, abort_flag)) return;
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
-                const int rl = tid64 + 64 * x;
-                *reinterpret_cast<uint4*>(ext + b * BwdCfg<64>::kExtBytes + (rl >> 3) * 256 + (rl & 7) * 16) = v[x];
+                uint8_t* row = ext + b * BwdCfg<64>::kExtPlane + (tid64 + 64 * x) * 16;
+                *reinterpret_cast<uint4*>(row) = vl[x];
+                *reinterpret_cast<uint4*>(row + 2 * BwdCfg<64>::kExtPlane) = vd[x];
             }
             fence_proxy_async_smem();
             __syncwarp();
@@ -1072,15 +1079,10 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         tma_prefetch_desc(&tmdV);
     }
     if constexpr (Cfg::kFold) {
-        // zeros in the stages, ones in columns 0-2 and 3-5 of the two tiles of constants
-        for (int i = threadIdx.x; i < 4 * Cfg::kExtBytes / 16; i += Cfg::kThreads) {
-            const int tile = i / (Cfg::kExtBytes / 16);
-            const bool first_half = ((i >> 3) & 1) == 0;  // core matrix of columns 0-7
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (first_half && tile == 2) v = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
-            if (first_half && tile == 3) v = make_uint4(0u, 0x3f800000u, 0x3f803f80u, 0u);
-            *reinterpret_cast<uint4*>(smem + Cfg::kOffExt + 16 * i) = v;
-        }
+        // the planes of constants (the stages are written whole)
+        for (int i = threadIdx.x; i < 2 * Cfg::kExtPlane / 16; i += Cfg::kThreads)
+            *reinterpret_cast<uint4*>(smem + Cfg::kOffExt + Cfg::kExtOnes * Cfg::kExtPlane + 16 * i) =
+                i < Cfg::kExtPlane / 16 ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
         fence_proxy_async_smem();
     }
     if (warp == 1) {

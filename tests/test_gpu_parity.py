@@ -486,6 +486,57 @@ def test_wide_heads_backward_routes(B, H, T, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"wide T={T}: ", dO=ref["dO_in"])
 
 
+# One of each backward kernel: the fused one (single key tile, several), with more heads than SMs.
+NOT_FINITE = [(1, 2, 100, 64), (1, 2, 300, 64), (8, 30, 300, 64)]
+
+
+@pytest.mark.parametrize("B,H,T,D", NOT_FINITE)
+@pytest.mark.parametrize("entry", ["plain", "deterministic"])
+@pytest.mark.parametrize("row", [3, 70, 90])
+def test_a_query_that_is_not_finite_stays_in_its_place(B, H, T, D, entry, row):
+    """What one query's Delta, LSE or dO may spoil.  Delta does not enter dV; LSE = +inf means P = 0, i.e. the row takes no
+    part; a NaN LSE ends at the diagonal, as far as dV is concerned; a dO that is not finite reaches its own column of dV.
+    The outputs that are not concerned have the bits of the run without it."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("place", B=B, H=H, T=T, D=D, seed=60 + T + D, causal=True)
+    Q, K, V, dO = W.make_inputs(cfg)
+    fwd = h.run_gpu(Q, K, V, dO, cfg.scale, True)
+    q, k, v, do = (x.to(dev) for x in (Q, K, V, dO))
+
+    def backward(lse, delta, do):
+        g = [torch.full_like(q, 7.0) for _ in range(3)]
+        if entry == "plain":
+            nova_attn.nova_attn_bwd(q, k, v, q, do, lse, delta, *g, cfg.scale, True)
+        else:
+            nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *g, cfg.scale, True)
+        nova_attn.nova_attn_poll_device_status()
+        return [x.float() for x in g]
+
+    def poked(t, value, *at):
+        t = t.clone()
+        t[(0, 1, row) + at] = value
+        return t
+
+    lse, delta = fwd["LSE"].to(dev), fwd["Delta"].to(dev)
+    dq0, dk0, dv0 = backward(lse, delta, do)
+    for value in (float("inf"), float("-inf"), float("nan")):
+        dq, dk, dv = backward(lse, poked(delta, value), do)
+        assert torch.equal(dv, dv0), f"Delta = {value} reached dV"
+        assert not torch.isfinite(dq[0, 1, row]).any() and not torch.isfinite(dk[0, 1, 0]).any()
+        dv = backward(lse, delta, poked(do, value, 5))[2]
+        keep = torch.arange(D, device=dev) != 5
+        assert torch.equal(dv[..., keep], dv0[..., keep]), f"dO = {value} reached other columns of dV"
+    _, dk0, dv0 = backward(poked(lse, 1e4), delta, do)  # 2^-14000: P = 0
+    for value in (3e38, float("inf")):
+        dq, dk, dv = backward(poked(lse, value), delta, do)
+        assert torch.equal(dk, dk0) and torch.equal(dv, dv0) and bool((dq[0, 1, row] == 0).all()), f"LSE = {value}"
+        assert torch.isfinite(dq).all()
+    dv = backward(poked(lse, float("nan")), delta, do)[2]
+    assert torch.equal(dv[0, 1, row + 1:], dv0[0, 1, row + 1:]) and not torch.isfinite(dv[0, 1, : row + 1]).any()
+
+
 DETERMINISTIC = [  # (B, H, T, D, causal)
     (1, 2, 64, 64, True),
     (2, 3, 300, 64, True),
