@@ -299,8 +299,11 @@ __device__ __forceinline__ void kv_mma(uint8_t* smem, KvBars* bars, uint32_t tme
 }
 
 // Row loader (one warp): -LSE*log2e and -Delta of each step, negated so that the compute warps fold them in with a packed
-// fma / add.  Queries past the end of the sequence get -inf, so that their P is exactly 0.  The loads of four steps are
-// in flight together.
+// fma / add.  Queries past the end of the sequence get -inf, so that their P is exactly 0.  A NaN (or + inf) becomes 3e38:
+// P of that query is infinite where it is kept, as unusable as NaN, but 0 where the causal mask puts -inf in front of the
+// sum, so that it reaches no key behind it.  (Making what is masked zero in the compute warps, per packed word or in a
+// branch that is not taken, cost 0.8 to 1.5 % of the training pass at B=4, H=32, T=1000.)  The loads of four steps are in
+// flight together.
 __device__ __forceinline__ void kv_row_loader(KvBars* bars, float* row_buf, const float* __restrict__ LSE,
                                               const float* __restrict__ Delta, const KvWork& wk, int lane) {
     volatile int* abort_flag = &bars->abort_flag;
@@ -330,7 +333,8 @@ __device__ __forceinline__ void kv_row_loader(KvBars* bars, float* row_buf, cons
                 float* r = row_buf + b * 2 * kStep;
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    r[lane + 32 * x] = -l[u][x] * kLog2e;
+                    const float nl = -l[u][x] * kLog2e;
+                    r[lane + 32 * x] = nl < 3e38f ? nl : 3e38f;
                     r[kStep + lane + 32 * x] = -d[u][x];
                 }
                 __syncwarp();

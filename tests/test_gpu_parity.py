@@ -486,8 +486,9 @@ def test_wide_heads_backward_routes(B, H, T, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"wide T={T}: ", dO=ref["dO_in"])
 
 
-# One of each backward kernel: the fused one (single key tile, several), with more heads than SMs.
-NOT_FINITE = [(1, 2, 100, 64), (1, 2, 300, 64), (8, 30, 300, 64)]
+# One of each backward kernel: the fused one (single key tile, several), with more heads than SMs, and at D=128 the pair of
+# kernels (which the deterministic entry point takes at every T > 128).
+NOT_FINITE = [(1, 2, 100, 64), (1, 2, 300, 64), (8, 30, 300, 64), (1, 2, 100, 128), (1, 2, 300, 128), (8, 30, 300, 128)]
 
 
 @pytest.mark.parametrize("B,H,T,D", NOT_FINITE)
