@@ -432,6 +432,31 @@ def test_forward_alone_and_in_a_crowd(T, D, causal):
         tol.assert_close(W.widen(lse[:1, :1]), ref["LSE"], tol.FWD_ATOL, tol.FWD_RTOL, "LSE", tol.FWD_REL_RMS)
 
 
+@pytest.mark.parametrize("T", [128, 200, 500])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("first", [0, 64])
+def test_forward_with_half_a_tile_of_lowest_scores(T, D, first):
+    """One query tile per CTA splits its keys in halves of 64.  Keys whose scores are around -1e37, as masks of the lowest
+    value make them, have no weight beside ordinary ones, whichever half they fill: the same bits as with scores of -1e4,
+    where 2^x is 0 as well."""
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("lowest", B=1, H=2, T=T, D=D, seed=11 + T)
+    Q, K, V, _ = (x.to(dev) for x in W.make_inputs(cfg))
+    Q[..., 0] = 1.0
+    out = []
+    for low in (-1e37, -1e4 / cfg.scale):
+        k = K.clone()
+        k[:, :, first : first + 64] = 0
+        k[:, :, first : first + 64, 0] = low
+        o, lse = torch.empty_like(Q), torch.empty((1, 2, T), device=dev)
+        nova_attn.nova_attn_fwd(Q, k, V, o, lse, cfg.scale, False)
+        nova_attn.nova_attn_poll_device_status()
+        out.append((o, lse))
+    assert torch.isfinite(out[0][1]).all() and torch.isfinite(out[0][0].float()).all()
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("scale,qk", [(1e-36, 1.0), (1e-20, 1.0), (12.5, 0.01)])
 @pytest.mark.parametrize("T", [100, 300])
 def test_scales_far_from_ordinary(scale, qk, T):
