@@ -248,9 +248,10 @@ lmhead_rows_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
         if (et < M && ok) {
             float m = -INFINITY, s = 0.f;
             for (int w = 0; w < kEpiWarps; ++w) m = fmaxf(m, stat[w * kLmHeadFewRows + et].x);
+            const float ref = (m == -INFINITY) ? 0.f : m;  // -inf: every logit of the CTA is (a masked stretch of the vocabulary)
             for (int w = 0; w < kEpiWarps; ++w) {
                 const float2 p = stat[w * kLmHeadFewRows + et];
-                s += p.y * ex2_approx(p.x - m);  // m is finite: the CTA has at least one entry
+                s += p.y * ex2_approx(p.x - ref);
             }
             partials[static_cast<size_t>(et) * gridDim.x + blockIdx.x] = make_float2(m, s);
         }
@@ -284,9 +285,10 @@ lmhead_rows_merge_kernel(const float2* __restrict__ partials, const float* __res
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    const float ref = (m == -INFINITY) ? 0.f : m;
     float s = 0.f;
 #pragma unroll
-    for (int k = 0; k < kMergeSteps; ++k) s += p[k].y * ex2_approx(p[k].x - m);
+    for (int k = 0; k < kMergeSteps; ++k) s += p[k].y * ex2_approx(p[k].x - ref);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if (lane == 0) {

@@ -83,6 +83,36 @@ def test_few_rows(M, N, K):
     _check(cfg, X, Wm, t, want_logits=False)
 
 
+def _masked(M, N, K, low, stretches):
+    """Logits of which whole stretches of the vocabulary are `low`, through a constant 1 in X and `low` in W."""
+    cfg = W.LmHeadConfig("masked", M=M, N=N, K=K, seed=3 + M + N, w_factor=0.3)
+    X, Wm, t = W.make_lmhead_inputs(cfg)
+    X[:, 0] = 1.0
+    Wm[:, 0] = 0.0
+    keep = torch.ones(N, dtype=torch.bool)
+    for lo, hi in stretches:
+        keep[lo:hi] = False
+        Wm[lo:hi] = 0.0
+        Wm[lo:hi, 0] = low
+    _, lse, loss = _run(cfg, X, Wm, t, want_logits=False)
+    z = X.double() @ Wm.double().T
+    return lse, loss, torch.logsumexp(z[:, keep], dim=1) if bool(keep.any()) else None
+
+
+# The first two stretches are all that one CTA has (tiles of 72 entries, 264 of them on 148 CTAs), the third a tile of its own.
+MASKED = [(18952, [(9000, 9072), (9072, 9144)]), (1000, [(128, 256)]), (50304, [(50257, 50304)]), (2048, [(0, 2000)])]
+
+
+@pytest.mark.parametrize("M", [1, 24, 64])
+@pytest.mark.parametrize("low", [float("-inf"), -3.3e38])
+@pytest.mark.parametrize("N,stretches", MASKED)
+def test_masked_stretches_of_the_vocabulary(M, low, N, stretches):
+    """Entries without weight (logit -inf, or so low that it is in base 2) change nothing, also where a thread, a tile or a
+    thread block sees no others."""
+    lse, _, ref = _masked(M, N, 64, low, stretches)
+    assert (lse.double().cpu() - ref).abs().max() <= 1e-5 * max(1.0, float(ref.abs().max()))
+
+
 def test_without_logits_and_run_to_run_determinism():
     cfg = W.LmHeadConfig("nolog", M=384, N=3000 // 8 * 8, K=256, seed=5, w_factor=0.1)
     X, Wm, t = W.make_lmhead_inputs(cfg)
