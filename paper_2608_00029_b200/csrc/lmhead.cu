@@ -238,11 +238,12 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ C
                     mx0 = fmax3(mx0, __uint_as_float(z[i + 0]), __uint_as_float(z[i + 1]));
                     mx1 = fmax3(mx1, __uint_as_float(z[i + 2]), __uint_as_float(z[i + 3]));
                 }
-                const float m_new = fmaxf(m2, fmaxf(mx0, mx1) * kLog2e);  // finite: the chunk has a valid entry
-                l *= ex2_approx(m2 - m_new);                               // 0 the first time (m2 = -inf)
+                const float m_new = fmaxf(m2, fmaxf(mx0, mx1) * kLog2e);
+                const float ref = (m_new == -INFINITY) ? 0.f : m_new;  // -inf: nothing but masked entries so far
+                l *= ex2_approx(m2 - ref);                             // 0 the first time (m2 = -inf)
                 m2 = m_new;
                 const uint64_t c2 = f32x2_pack(kLog2e, kLog2e);
-                const uint64_t nm2 = f32x2_pack(-m_new, -m_new);
+                const uint64_t nm2 = f32x2_pack(-ref, -ref);
                 uint64_t acc0 = 0, acc1 = 0;
 #pragma unroll
                 for (int i = 0; i < 32; i += 4) {
@@ -577,10 +578,11 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
                     mx1 = fmax3(mx1, __uint_as_float(z[i + 2]), __uint_as_float(z[i + 3]));
                 }
                 const float m_new = fmaxf(m2, fmaxf(mx0, mx1) * kLog2e);
-                l *= ex2_approx(m2 - m_new);
+                const float ref = (m_new == -INFINITY) ? 0.f : m_new;
+                l *= ex2_approx(m2 - ref);
                 m2 = m_new;
                 const uint64_t c2 = f32x2_pack(kLog2e, kLog2e);
-                const uint64_t nm2 = f32x2_pack(-m_new, -m_new);
+                const uint64_t nm2 = f32x2_pack(-ref, -ref);
                 uint64_t acc0 = 0, acc1 = 0;
 #pragma unroll
                 for (int i = 0; i < 32; i += 4) {
@@ -623,7 +625,7 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constan
 constexpr int kMergeRows = 32, kMergeSlices = 8;
 
 __device__ __forceinline__ void merge_pair(float& m, float& l, float m2, float l2) {
-    if (l2 > 0.f) {
+    if (!(l2 == 0.f)) {  // 0: nothing but masked entries; NaN has to get through
         if (m2 > m) {
             l = l * __expf(m - m2) + l2;  // exp(-inf) = 0 while nothing has been merged yet
             m = m2;

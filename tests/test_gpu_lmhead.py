@@ -103,7 +103,7 @@ def _masked(M, N, K, low, stretches):
 MASKED = [(18952, [(9000, 9072), (9072, 9144)]), (1000, [(128, 256)]), (50304, [(50257, 50304)]), (2048, [(0, 2000)])]
 
 
-@pytest.mark.parametrize("M", [1, 24, 64])
+@pytest.mark.parametrize("M", [1, 24, 64, 100, 300])  # the three kernels
 @pytest.mark.parametrize("low", [float("-inf"), -3.3e38])
 @pytest.mark.parametrize("N,stretches", MASKED)
 def test_masked_stretches_of_the_vocabulary(M, low, N, stretches):
@@ -111,6 +111,16 @@ def test_masked_stretches_of_the_vocabulary(M, low, N, stretches):
     thread block sees no others."""
     lse, _, ref = _masked(M, N, 64, low, stretches)
     assert (lse.double().cpu() - ref).abs().max() <= 1e-5 * max(1.0, float(ref.abs().max()))
+
+
+@pytest.mark.parametrize("M", [24, 100, 300])
+def test_a_logit_that_is_nan_shows_in_its_row(M):
+    cfg = W.LmHeadConfig("nan", M=M, N=1000, K=64, seed=8, w_factor=0.3)
+    X, Wm, t = W.make_lmhead_inputs(cfg)
+    X[7, 3] = float("nan")
+    _, lse, loss = _run(cfg, X, Wm, t)
+    rows = torch.arange(M) != 7
+    assert bool(torch.isnan(lse[7])) and bool(torch.isfinite(lse[rows]).all()) and bool(torch.isfinite(loss[rows]).all())
 
 
 def test_without_logits_and_run_to_run_determinism():
