@@ -106,7 +106,7 @@ void* stream(PyObject* o) {
     return p;
 }
 
-// The caller's workspace, or one of `need` bytes allocated for this call.
+// The caller's workspace (any type: a span of bytes on the GPU), or one of `need` bytes allocated for this call.
 struct Workspace {
     at::Tensor own;
     void* ptr;
@@ -117,6 +117,8 @@ struct Workspace {
             own = at::empty({static_cast<int64_t>(need)}, tensor(like, "tensor").options().dtype(at::kByte));
         else
             t = &tensor(o, "workspace");
+        if (!t->is_cuda() || !t->is_non_overlapping_and_dense())
+            raise(PyExc_TypeError, "workspace must be a CUDA tensor without gaps");
         ptr = data(*t);
         bytes = t->nbytes();
     }
@@ -293,8 +295,8 @@ int lmhead_fwd(Args a) {  // X W targets logits lse loss workspace stream
     const int64_t M = X.size(0), K = X.size(1), N = W.size(0);
     if (W.size(1) != K) raise(PyExc_ValueError, "X [M,K] and W [N,K] must agree in K");
     const at::Tensor& tg = tensor(a[2], "targets");
-    if (tg.scalar_type() != at::kInt || !tg.is_cuda() || tg.sizes() != at::IntArrayRef({M}))
-        raise(PyExc_TypeError, "targets must be a CUDA int32 tensor [M]");
+    if (tg.scalar_type() != at::kInt || !tg.is_cuda() || !tg.is_contiguous() || tg.sizes() != at::IntArrayRef({M}))
+        raise(PyExc_TypeError, "targets must be a contiguous CUDA int32 tensor [M]");
     void* logits = nullptr;
     if (a[3] != Py_None) {
         const at::Tensor& t = tensor(a[3], "logits");
@@ -306,8 +308,8 @@ int lmhead_fwd(Args a) {  // X W targets logits lse loss workspace stream
     for (int i = 0; i < 2; ++i) {
         const char* name = i ? "loss" : "lse";
         const at::Tensor& t = tensor(a[4 + i], name);
-        if (t.scalar_type() != at::kFloat || !t.is_cuda() || t.sizes() != at::IntArrayRef({M}))
-            raise(PyExc_TypeError, std::string(name) + " must be a CUDA fp32 tensor [M]");
+        if (t.scalar_type() != at::kFloat || !t.is_cuda() || !t.is_contiguous() || t.sizes() != at::IntArrayRef({M}))
+            raise(PyExc_TypeError, std::string(name) + " must be a contiguous CUDA fp32 tensor [M]");
         stat[i] = static_cast<float*>(data(t));
     }
     const int m = static_cast<int>(M), n = static_cast<int>(N), k = static_cast<int>(K);

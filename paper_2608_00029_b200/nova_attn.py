@@ -137,7 +137,7 @@ BWD_STEP_ALL = 7
 
 def nova_attn_bwd(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: bool = True, workspace=None,
                   stream=None, steps: int = BWD_STEP_ALL) -> None:
-    """dQ, dK, dV <- gradients of sum(O*dO); `workspace` is a CUDA byte/float tensor of at least
+    """dQ, dK, dV <- gradients of sum(O*dO); `workspace` is a CUDA byte/float tensor without gaps of at least
     nova_attn_bwd_workspace_bytes(B,H,T,D) bytes (allocated here if omitted).  `steps` other than
     BWD_STEP_ALL goes through nova_attn_bwd_steps (a timing aid)."""
     rc = _binding().bwd(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale, causal, workspace, stream, steps)

@@ -28,8 +28,8 @@ def nova_lmhead_workspace_bytes(M: int, N: int, K: int) -> int:
 
 def nova_lmhead_fwd(X, W, targets, logits, lse, loss, workspace=None, stream=None) -> None:
     """lse, loss (and logits unless None) <- loss head of X [M,K] against W [N,K] with int32 targets [M].
-    X, W, logits are contiguous CUDA bf16 tensors, lse and loss fp32 [M]; `workspace` is a CUDA byte tensor of
-    at least nova_lmhead_workspace_bytes(M, N, K) bytes (allocated here if omitted)."""
+    X, W, logits are contiguous CUDA bf16 tensors, targets, lse and loss contiguous [M]; `workspace` is a
+    CUDA tensor without gaps of at least nova_lmhead_workspace_bytes(M, N, K) bytes (allocated here if omitted)."""
     rc = _na._binding().lmhead_fwd(X, W, targets, logits, lse, loss, workspace, stream)
     if rc != _na.OK:
         raise _na.NovaAttnError(rc, "nova_lmhead_fwd")

@@ -192,3 +192,25 @@ def test_both_kernels_agree_and_cuda_graph_replay():
         torch.cuda.synchronize()
         na.nova_attn_poll_device_status()
         assert torch.equal(lse2, lse) and torch.equal(loss2, loss) and torch.equal(logits2, logits)
+
+
+@pytest.mark.parametrize("what", ["targets", "lse", "loss", "workspace on the CPU", "strided workspace"])
+def test_binding_refuses_what_the_kernels_could_not_address(what):
+    """The kernels see addresses only: a column of a matrix would be read and written as if it were dense, a host tensor
+    through an address the GPU may not have.  Refused before anything is launched."""
+    from paper_2608_00029_b200 import nova_lmhead as lm
+    dev = torch.device("cuda:0")
+    M, N, K = 4, 64, 64
+    x, w = torch.zeros((M, K), dtype=torch.bfloat16, device=dev), torch.zeros((N, K), dtype=torch.bfloat16, device=dev)
+    column = lambda dtype: torch.full((M, 3), 7, dtype=dtype, device=dev)  # noqa: E731
+    bufs = {"targets": column(torch.int32), "lse": column(torch.float32), "loss": column(torch.float32)}
+    args = {n: b[:, 0] if n == what else b[:, 0].contiguous() for n, b in bufs.items()}
+    ws = torch.empty(lm.nova_lmhead_workspace_bytes(M, N, K), dtype=torch.uint8, device=dev)
+    if what == "workspace on the CPU":
+        ws = ws.cpu()
+    elif what == "strided workspace":
+        ws = torch.empty((ws.numel(), 2), dtype=torch.uint8, device=dev)[:, 0]
+    with pytest.raises(TypeError, match=what.split()[0] if "strided" not in what else "workspace"):
+        lm.nova_lmhead_fwd(x, w, args["targets"], None, args["lse"], args["loss"], ws)
+    torch.cuda.synchronize()
+    assert all(bool((b == 7).all()) for b in bufs.values())

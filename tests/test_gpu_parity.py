@@ -677,6 +677,26 @@ def test_random_shapes_and_entry_points(chunk):
         h.compare(h.select_heads(got, heads), ref, label=label, dO=ref["dO_in"], rms=(T >= 64))
 
 
+@pytest.mark.parametrize("strided", [False, True])
+@pytest.mark.parametrize("kind", ["on the CPU", "strided"])
+def test_backward_refuses_a_workspace_the_kernels_could_not_address(strided, kind):
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    x = torch.zeros((1, 1, 130, 64), dtype=torch.bfloat16, device=dev)
+    row = torch.zeros((1, 1, 130), device=dev)
+    need = nova_attn.nova_attn_bwd_workspace_bytes(1, 1, 130, 64)
+    ws = (torch.empty(need, dtype=torch.uint8) if kind == "on the CPU"
+          else torch.empty((need, 2), dtype=torch.uint8, device=dev)[:, 0])
+    grads = [torch.full_like(x, 7.0) for _ in range(3)]
+    with pytest.raises(TypeError, match="workspace"):
+        if strided:
+            nova_attn.nova_attn_bwd_strided(x, x, x, x, row, row, *grads, 0.125, True, ws)
+        else:
+            nova_attn.nova_attn_bwd(x, x, x, x, x, row, row, *grads, 0.125, True, ws)
+    torch.cuda.synchronize()
+    assert all(bool((g == 7.0).all()) for g in grads)
+
+
 def test_two_host_threads_two_streams():
     """Two host threads drive the library at once, each on its own stream and buffers (different shapes
     and head dimensions): the calls take the library's lock for the map cache only, the kernels of the
