@@ -11,6 +11,7 @@
 
 #include <ATen/core/Tensor.h>
 #include <ATen/ops/empty.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -106,17 +107,23 @@ void* stream(PyObject* o) {
     return p;
 }
 
-// The caller's workspace (any type: a span of bytes on the GPU), or one of `need` bytes allocated for this call.
+// The caller's workspace (any type: a span of bytes on the GPU), or one of `need` bytes allocated for this call.  That one is
+// given back when the call returns, before its kernels have run, so it has to come from the memory of the stream that they
+// run on: what is allocated on that stream next is ordered behind them.
 struct Workspace {
     at::Tensor own;
     void* ptr;
     size_t bytes;
-    Workspace(PyObject* o, size_t need, PyObject* like) {
+    Workspace(PyObject* o, size_t need, PyObject* like, void* stream) {
         const at::Tensor* t = &own;
-        if (o == Py_None)
-            own = at::empty({static_cast<int64_t>(need)}, tensor(like, "tensor").options().dtype(at::kByte));
-        else
+        if (o == Py_None) {
+            const at::Tensor& l = tensor(like, "tensor");
+            c10::cuda::CUDAStreamGuard guard(
+                c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), l.device().index()));
+            own = at::empty({static_cast<int64_t>(need)}, l.options().dtype(at::kByte));
+        } else {
             t = &tensor(o, "workspace");
+        }
         if (!t->is_cuda() || !t->is_non_overlapping_and_dense())
             raise(PyExc_TypeError, "workspace must be a CUDA tensor without gaps");
         ptr = data(*t);
@@ -231,8 +238,8 @@ int bwd(Args a) {  // Q K V O dO LSE Delta dQ dK dV scale causal workspace strea
     const Dims& d = t.d;
     const float scale = real(a[10]);
     const int causal = truth(a[11]);
-    const Workspace ws(a[12], nova_attn_bwd_workspace_bytes(d.B, d.H, d.T, d.D), a[0]);
     void* st = stream(a[13]);
+    const Workspace ws(a[12], nova_attn_bwd_workspace_bytes(d.B, d.H, d.T, d.D), a[0], st);
     const int steps = integer(a[14]);
     return without_gil([&] {
         return nova_attn_bwd_steps(t.q, t.k, t.v, t.o, t.dO, t.lse, t.delta, t.dq, t.dk, t.dv, d.B, d.H, d.T, d.D, scale,
@@ -274,8 +281,8 @@ int bwd_strided(Args a) {  // Q K V dO LSE Delta dQ dK dV scale causal workspace
     const Dims d(s);
     const float scale = real(a[9]);
     const int causal = truth(a[10]);
-    const Workspace ws(a[11], nova_attn_bwd_workspace_bytes(d.B, d.H, d.T, d.D), a[0]);
     void* st = stream(a[12]);
+    const Workspace ws(a[11], nova_attn_bwd_workspace_bytes(d.B, d.H, d.T, d.D), a[0], st);
     return without_gil([&] {
         return nova_attn_bwd_strided(q, k, v, dO, lse, delta, dq, dk, dv, d.B, d.H, d.T, d.D, &sq, &sk, &sv, &sdo, &sdq, &sdk,
                                      &sdv, scale, causal, ws.ptr, ws.bytes, st);
@@ -313,8 +320,8 @@ int lmhead_fwd(Args a) {  // X W targets logits lse loss workspace stream
         stat[i] = static_cast<float*>(data(t));
     }
     const int m = static_cast<int>(M), n = static_cast<int>(N), k = static_cast<int>(K);
-    const Workspace ws(a[6], nova_lmhead_workspace_bytes(m, n, k), a[0]);
     void* st = stream(a[7]);
+    const Workspace ws(a[6], nova_lmhead_workspace_bytes(m, n, k), a[0], st);
     const int* targets = static_cast<const int*>(data(tg));
     return without_gil(
         [&] { return nova_lmhead_fwd(xw[0], xw[1], targets, logits, stat[0], stat[1], m, n, k, ws.ptr, ws.bytes, st); });

@@ -697,6 +697,36 @@ def test_backward_refuses_a_workspace_the_kernels_could_not_address(strided, kin
     assert all(bool((g == 7.0).all()) for g in grads)
 
 
+def test_workspace_of_the_call_belongs_to_its_stream():
+    """A call without a workspace allocates one and gives it back before its kernels have run.  On a stream other than the
+    current one that memory must not go to the next tensor of the current stream: here the call waits behind a copy
+    that keeps its stream busy, and a tensor of the same size, made meanwhile, keeps its values."""
+    from paper_2608_00029_b200 import nova_attn, nova_lmhead
+    dev = torch.device("cuda:0")
+    shape = (2, 3, 1000, 64)
+    x = torch.randn(shape, device=dev).to(torch.bfloat16)
+    row, grads = torch.zeros(shape[:3], device=dev), [torch.empty_like(x) for _ in range(3)]
+    X, Wm = torch.zeros((512, 64), dtype=torch.bfloat16, device=dev), torch.zeros((4096, 64), dtype=torch.bfloat16, device=dev)
+    t, lse, loss = torch.zeros(512, dtype=torch.int32, device=dev), torch.empty(512, device=dev), torch.empty(512, device=dev)
+    side, big = torch.cuda.Stream(device=dev), torch.empty(1 << 30, dtype=torch.uint8, device=dev)
+    calls = [(nova_attn.nova_attn_bwd_workspace_bytes(*shape),
+              lambda: nova_attn.nova_attn_bwd(x, x, x, x, x, row, row, *grads, 0.125, True, stream=side)),
+             (nova_attn.nova_attn_bwd_workspace_bytes(*shape),
+              lambda: nova_attn.nova_attn_bwd_strided(x, x, x, x, row, row, *grads, 0.125, True, stream=side)),
+             (nova_lmhead.nova_lmhead_workspace_bytes(512, 4096, 64),
+              lambda: nova_lmhead.nova_lmhead_fwd(X, Wm, t, None, lse, loss, stream=side))]
+    for need, call in calls:
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            for _ in range(40):
+                big.fill_(1)
+        call()
+        mine = torch.full((need,), 7, dtype=torch.uint8, device=dev)
+        torch.cuda.synchronize()
+        nova_attn.nova_attn_poll_device_status()
+        assert bool((mine == 7).all())
+
+
 def test_two_host_threads_two_streams():
     """Two host threads drive the library at once, each on its own stream and buffers (different shapes
     and head dimensions): the calls take the library's lock for the map cache only, the kernels of the
