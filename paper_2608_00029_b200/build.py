@@ -20,9 +20,17 @@ def _sources():
     return [os.path.join(CSRC, s) for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
 
 
+def _built_for() -> str:
+    import torch
+    return f"torch {torch.__version__}, Python {sys.version_info.major}.{sys.version_info.minor}"
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
+    with open(BINDING, "rb") as f:
+        if f"nova binding for {_built_for()}\0".encode() not in f.read():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh", ".cpp"))]
     deps.append(os.path.join(os.path.dirname(HERE), "include", "nova_attn.h"))
@@ -40,7 +48,7 @@ def _build_binding() -> None:
     tmp = BINDING + f".tmp{os.getpid()}"
     subprocess.check_call(
         [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + [f"-I{p}" for p in inc] +
+         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DNOVA_BUILT_FOR="{_built_for()}"'] + [f"-I{p}" for p in inc] +
         ["-o", tmp, os.path.join(CSRC, "binding.cpp"), LIB, f"-L{lib}", "-lc10", "-lc10_cuda", "-ltorch_cpu",
          "-ltorch_python", "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{lib}"])
     os.replace(tmp, BINDING)

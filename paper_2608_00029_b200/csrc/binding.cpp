@@ -359,6 +359,25 @@ PyMethodDef methods[] = {
 };
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
+// What this module was compiled against.  It reads tensors through torch's C++ classes, whose layout belongs to one version:
+// with another it must not load (the build looks for the same text in the file to see whether it is out of date).
+const char kBuiltFor[] = "nova binding for " NOVA_BUILT_FOR;
+
+bool runs_with_what_it_was_built_for() {
+    PyObject* torch = PyImport_ImportModule("torch");
+    PyObject* version = torch ? PyObject_GetAttrString(torch, "__version__") : nullptr;
+    PyObject* now = version ? PyUnicode_FromFormat("nova binding for torch %S, Python %d.%d", version, PY_MAJOR_VERSION,
+                                                   PY_MINOR_VERSION) : nullptr;
+    const bool same = now && PyUnicode_CompareWithASCIIString(now, kBuiltFor) == 0;
+    if (now && !same)
+        PyErr_Format(PyExc_ImportError, "this is the %s, loaded with torch %S: run python -m paper_2608_00029_b200.build",
+                     kBuiltFor, version);
+    Py_XDECREF(now);
+    Py_XDECREF(version);
+    Py_XDECREF(torch);
+    return same;
+}
+
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__binding(void) { return runs_with_what_it_was_built_for() ? PyModule_Create(&module) : nullptr; }

@@ -169,6 +169,23 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
         na.load()
 
 
+def test_binding_of_another_torch_is_rebuilt_and_does_not_load(lib, monkeypatch):
+    """The native binding is compiled against one torch: with another the build is out of date whatever the file times
+    say, and the module refuses to load."""
+    import subprocess
+    import sys
+
+    import torch
+    from paper_2608_00029_b200 import build
+    monkeypatch.setattr(build.os.path, "getmtime", lambda p: 0.0)
+    assert not build._stale()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert build._stale()
+    code = "import torch; torch.__version__ = '0.0.1'; from paper_2608_00029_b200 import _binding"
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode != 0 and "ImportError" in r.stderr and "torch 0.0.1" in r.stderr
+
+
 @pytest.mark.parametrize("bad", ["device", "dtype", "not a tensor"])
 def test_binding_rejects_wrong_tensors(bad):
     """The native binding raises before anything is called (no GPU involved)."""
