@@ -78,9 +78,12 @@ float* f32(PyObject* o, const char* name, at::IntArrayRef want) {
     return static_cast<float*>(data(t));
 }
 
+// As float(o) and int(o) read them: text and numbers of other types are fine.
 float real(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw Failed{};
+    PyObject* f = PyNumber_Float(o);
+    if (!f) throw Failed{};
+    const double v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
     return static_cast<float>(v);
 }
 
@@ -91,7 +94,10 @@ int truth(PyObject* o) {
 }
 
 int integer(PyObject* o) {
-    const long v = PyLong_AsLong(o);
+    PyObject* i = PyNumber_Long(o);
+    if (!i) throw Failed{};
+    const long v = PyLong_AsLong(i);
+    Py_DECREF(i);
     if (v == -1 && PyErr_Occurred()) throw Failed{};
     return static_cast<int>(v);
 }

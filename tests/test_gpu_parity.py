@@ -677,6 +677,24 @@ def test_random_shapes_and_entry_points(chunk):
         h.compare(h.select_heads(got, heads), ref, label=label, dO=ref["dO_in"], rms=(T >= 64))
 
 
+def test_binding_takes_numbers_as_python_does():
+    """scale and steps are read as float() and int() read them."""
+    from decimal import Decimal
+
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    x = torch.randn((1, 2, 100, 64), device=dev).to(torch.bfloat16)
+    row = torch.zeros((1, 2, 100), device=dev)
+    out = []
+    for scale, steps in ((0.125, 7), ("0.125", "7"), (Decimal("0.125"), 7.0), (np.float32(0.125), np.int64(7)),
+                         (torch.tensor(0.125), torch.tensor(7))):
+        o, lse, grads = torch.empty_like(x), torch.empty_like(row), [torch.empty_like(x) for _ in range(3)]
+        nova_attn.nova_attn_fwd(x, x, x, o, lse, scale)
+        nova_attn.nova_attn_bwd(x, x, x, o, x, lse, row, *grads, scale, steps=steps)
+        out.append(torch.stack([o] + grads))
+    assert all(torch.equal(t, out[0]) for t in out)
+
+
 @pytest.mark.parametrize("strided", [False, True])
 @pytest.mark.parametrize("kind", ["on the CPU", "strided"])
 def test_backward_refuses_a_workspace_the_kernels_could_not_address(strided, kind):
