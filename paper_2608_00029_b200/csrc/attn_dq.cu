@@ -9,19 +9,21 @@
 // one kernel.
 //
 // A work item is a block of 256 query rows of one head: two 128-row tiles, A and B, that share every K and V tile
-// they both need.  The keys go by in steps of 64.  Items are handed out dynamically, heaviest first, as in the
-// forward (WorkRing).  384 threads:
+// they both need; in small problems one tile (plan_of).  The keys go by in steps of 64.  Items are handed out dynamically,
+// heaviest first, as in the forward (WorkRing).  384 threads:
 //   warp 0      TMA producer: Q and dO per tile of an item, K and V through a ring of 64-key stages
 //   warps 1, 3  UMMA issuers, one per query tile, so that neither tile waits for the other's products and A may be in
 //               the next item while B finishes this one
 //   warps 4-7   rows of tile A, warps 8-11 rows of tile B: one thread per query row takes 64 keys of S and dP out of
 //               tensor memory and writes dS back as bf16 (or adds P*dP into its Delta)
+// (with single tiles, tile B's warps have nothing to do)
 //
 // What bounds it: one tile in flight is a serial chain (products -> tensor memory -> arithmetic -> tensor memory ->
 // product), during which the tensor cores idle; two tiles fill each other's gaps.  64 keys per step is what tensor memory
 // allows two tiles at D=128: dQ takes 128 of a tile's 256 columns, S and dP 64 each.  A product of N=64 with both
 // operands in shared memory costs 49 clocks per 16 k elements against 65 for twice the keys, so a 128 x 128 block takes
 // 2100 clocks of tensor time at D=128 (1560 with N=128).
+#include <algorithm>
 #include <type_traits>
 
 #include "kernels.h"
@@ -33,29 +35,31 @@ namespace {
 constexpr int kThreads = 384;
 constexpr int kTmemCols = 512;
 constexpr int kStep = kKeyStep;                  // keys per step
-constexpr int kBlockRows = 2 * kBlockQ;          // query rows per work item
 constexpr int kHalfStepBytes = kStep * 128;      // one [64 keys x 64 bf16] box
-constexpr int kWorkConsumers = 2 + 8;            // issuers + row warps
 
-template <int D>
+// kTiles: query tiles of a work item (see plan_of).
+template <int D, int kTiles>
 struct DqCfg {
+    static constexpr int kBlockRows = kTiles * kBlockQ;   // query rows per work item
+    static constexpr int kWorkConsumers = kTiles * 5;     // an issuer and four row warps per tile
     static constexpr int kHalves = D / kBoxCols;
     static constexpr int kTileBytes = kHalves * kHalfTileBytes;
     static constexpr int kStepBytes = kHalves * kHalfStepBytes;
-    static constexpr int kQStages = (D == 64) ? 2 : 1;  // Q and dO of an item
+    static constexpr int kQStages = (D == 64 || kTiles == 1) ? 2 : 1;  // Q and dO of an item
     static constexpr int kKVStages = (D == 64) ? 5 : 3;
-    static constexpr int kOffQ = 0;                                     // [kQStages][2 tiles] of Q, then of dO
-    static constexpr int kOffdO = kQStages * 2 * kTileBytes;
+    static constexpr int kOffQ = 0;                                     // [kQStages][kTiles] of Q, then of dO
+    static constexpr int kOffdO = kQStages * kTiles * kTileBytes;
     static constexpr int kOffK = 2 * kOffdO;                            // [kKVStages] of K, then of V
     static constexpr int kOffV = kOffK + kKVStages * kStepBytes;
     static constexpr int kOffBar = kOffV + kKVStages * kStepBytes;
     static constexpr int kSmemBytes = kOffBar + 512 + 1024;
     static_assert(kSmemBytes <= 232448, "exceeds the shared memory of one CTA");
-    // Columns of a tile (256 per tile).  dQ first.  D=64: S, dP, and two buffers of dS (32 columns each), so that S and
-    // dP of the next step are queued as soon as the row warps have read them.  D=128: S and dP, and dS lies over S.
-    static constexpr bool kSepdS = (D == 64);
+    // Columns of a tile (256 per tile of a pair).  dQ first, then S and dP.  Where there is room two buffers of dS (32
+    // columns each), so that S and dP of the next step are queued as soon as the row warps have read them; with two tiles
+    // at D=128 dS lies over S.
+    static constexpr bool kSepdS = (D == 64 || kTiles == 1);
     static constexpr int kColS = D, kColdP = D + 64;
-    static constexpr int kColdS = kSepdS ? 192 : kColS;
+    static constexpr int kColdS = kSepdS ? D + 128 : kColS;
 };
 
 struct DqBars {
@@ -73,11 +77,11 @@ struct DqBars {
 };
 static_assert(sizeof(DqBars) <= 512, "barrier block");
 
-// Work items: 256-row query blocks, heaviest first (the last block of a causal problem sees every key).  D=128: within
+// Work items: blocks of kTiles query tiles, heaviest first (the last block of a causal problem sees every key).  D=128: within
 // chunks of heads whose tensors stay in L2 together (the exact Delta at B=16, H=32, T=1024 175 -> 157 us, the
 // deterministic backward 650 -> 627 us); at D=64 a head's K and V are half as large and the longer arithmetic costs
 // 1 % where there is nothing to gain.
-template <int D>
+template <int D, int kTiles>
 struct DqWork {
     int BH, n_blocks, chunk, T, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, dO, dQ tensor maps, four bits each
@@ -100,16 +104,16 @@ struct DqWork {
             *bh = idx % BH;
         }
         const int n_all = (T + kStep - 1) / kStep;
-        const int qt_a = 2 * (*blk), qt_b = qt_a + 1;
+        const int qt_a = kTiles * (*blk), qt_b = qt_a + 1;
         *n_a = causal ? min((qt_a + 1) * (kBlockQ / kStep), n_all) : n_all;
-        *n_b = (qt_b * kBlockQ < T) ? (causal ? min((qt_b + 1) * (kBlockQ / kStep), n_all) : n_all) : 0;
+        *n_b = (kTiles == 2 && qt_b * kBlockQ < T) ? (causal ? min((qt_b + 1) * (kBlockQ / kStep), n_all) : n_all) : 0;
     }
 };
 
-template <int D, bool kStrided>
+template <int D, int kTiles, bool kStrided>
 __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork<D>& wk) {
-    using Cfg = DqCfg<D>;
+                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork<D, kTiles>& wk) {
+    using Cfg = DqCfg<D, kTiles>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr long long limit = kWaitLimitCycles;
     int armed_q[2][2] = {{-1, -1}, {-1, -1}}, armed_kv[Cfg::kKVStages];
@@ -134,11 +138,11 @@ __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtens
             armed_q[qs][t] = qph;
 #pragma unroll
             for (int h = 0; h < Cfg::kHalves; ++h) {
-                const int off = (qs * 2 + t) * Cfg::kTileBytes + h * kHalfTileBytes;
+                const int off = (qs * kTiles + t) * Cfg::kTileBytes + h * kHalfTileBytes;
                 tma_load_tile<kStrided>(smem + Cfg::kOffQ + off, tmQ, &bars->q_full[qs][t], wk.orders & 15, h * kBoxCols,
-                                        blk * kBlockRows + t * kBlockQ, head, batch, bh);
+                                        blk * Cfg::kBlockRows + t * kBlockQ, head, batch, bh);
                 tma_load_tile<kStrided>(smem + Cfg::kOffdO + off, tmdO, &bars->q_full[qs][t], (wk.orders >> 12) & 15,
-                                        h * kBoxCols, blk * kBlockRows + t * kBlockQ, head, batch, bh);
+                                        h * kBoxCols, blk * Cfg::kBlockRows + t * kBlockQ, head, batch, bh);
             }
             return true;
         };
@@ -160,7 +164,7 @@ __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtens
                 st = 0;
                 ph ^= 1;
             }
-            if (j == 0) {
+            if (kTiles == 2 && j == 0) {
                 ok = load_q(1);
                 if (!ok) break;
             }
@@ -178,7 +182,7 @@ __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtens
         int none = 0;
         if (clc_pending) (void)mbar_wait(&bars->ring.answer_bar, w & 1, &none);
         for (int s = 0; s < 2; ++s)
-            for (int t = 0; t < 2; ++t)
+            for (int t = 0; t < kTiles; ++t)
                 if (armed_q[s][t] >= 0) (void)mbar_wait(&bars->q_full[s][t], armed_q[s][t], &none);
         for (int s = 0; s < Cfg::kKVStages; ++s)
             if (armed_kv[s] >= 0) (void)mbar_wait(&bars->kv_full[s], armed_kv[s], &none);
@@ -186,9 +190,9 @@ __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtens
 }
 
 // The issuer of query tile t: the whole warp in uniform control flow, one elected lane issues.
-template <int D, bool kDelta>
-__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork<D>& wk, int t) {
-    using Cfg = DqCfg<D>;
+template <int D, int kTiles, bool kDelta>
+__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork<D, kTiles>& wk, int t) {
+    using Cfg = DqCfg<D, kTiles>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescT = umma_idesc_bf16(128, kStep, 0, 0);  // S, dP
     constexpr uint32_t kIdescdQ = umma_idesc_bf16(128, D, 0, 1);     // dQ: A from TMEM, B (K) MN-major
@@ -230,8 +234,8 @@ __device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tme
         wk.get(item, &blk, &bh, &n_a, &n_b);
         const int n_t = t == 0 ? n_a : n_b, n = max(n_a, n_b);
         const int qs = w % Cfg::kQStages;
-        q_k = umma_desc_lo(smem_u32(smem + Cfg::kOffQ + (qs * 2 + t) * Cfg::kTileBytes), 16);
-        do_k = umma_desc_lo(smem_u32(smem + Cfg::kOffdO + (qs * 2 + t) * Cfg::kTileBytes), 16);
+        q_k = umma_desc_lo(smem_u32(smem + Cfg::kOffQ + (qs * kTiles + t) * Cfg::kTileBytes), 16);
+        do_k = umma_desc_lo(smem_u32(smem + Cfg::kOffdO + (qs * kTiles + t) * Cfg::kTileBytes), 16);
         if (n_t > 0) {
             ok = mbar_wait(&bars->q_full[qs][t], (w / Cfg::kQStages) & 1, abort_flag);
             if (!ok) break;
@@ -340,12 +344,12 @@ __device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tme
 }
 
 // The row warps of query tile t.
-template <int D, bool kCausal, bool kStrided, bool kDelta>
+template <int D, int kTiles, bool kCausal, bool kStrided, bool kDelta>
 __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const CUtensorMap* tmdQ,
                                         const float* __restrict__ LSE, const float* __restrict__ Delta,
-                                        float* __restrict__ Delta_out, float scale, const DqWork<D>& wk, int t, int rwarp,
+                                        float* __restrict__ Delta_out, float scale, const DqWork<D, kTiles>& wk, int t, int rwarp,
                                         int lane) {
-    using Cfg = DqCfg<D>;
+    using Cfg = DqCfg<D, kTiles>;
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * rwarp;
     const int row_local = lane_base + lane;
@@ -367,7 +371,7 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
         int blk, bh, n_a, n_b;
         wk.get(item, &blk, &bh, &n_a, &n_b);
         const int n_t = (t == 0) ? n_a : n_b;
-        const int qt = 2 * blk + t;
+        const int qt = kTiles * blk + t;
         const int row = qt * kBlockQ + row_local;
         const size_t idx = static_cast<size_t>(bh) * T + row;
         const int qs = w % Cfg::kQStages;
@@ -466,7 +470,7 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
             ok = mbar_wait(&bars->dq_done[t], wt & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
-            uint8_t* stage = smem + Cfg::kOffQ + (qs * 2 + t) * Cfg::kTileBytes;
+            uint8_t* stage = smem + Cfg::kOffQ + (qs * kTiles + t) * Cfg::kTileBytes;
 #pragma unroll
             for (int cb = 0; cb < D; cb += 32) {
                 uint32_t a[32];
@@ -517,12 +521,12 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
 }
 
 // Set-up and roles, shared by the two builds below.
-template <int D, bool kCausal, bool kStrided, bool kDelta>
+template <int D, int kTiles, bool kCausal, bool kStrided, bool kDelta>
 __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
                                         const CUtensorMap* tmdO, const CUtensorMap* tmdQ, const float* __restrict__ LSE,
-                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork<D>& wk,
+                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork<D, kTiles>& wk,
                                         float scale, int* __restrict__ dev_status) {
-    using Cfg = DqCfg<D>;
+    using Cfg = DqCfg<D, kTiles>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     DqBars* bars = reinterpret_cast<DqBars*>(smem + Cfg::kOffBar);
@@ -544,9 +548,9 @@ __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMa
         }
         for (int s = 0; s < Cfg::kKVStages; ++s) {
             mbar_init(&bars->kv_full[s], 1);
-            mbar_init(&bars->kv_empty[s], 2);  // the two issuers
+            mbar_init(&bars->kv_empty[s], kTiles);  // the issuers
         }
-        bars->ring.init(kWorkConsumers);
+        bars->ring.init(Cfg::kWorkConsumers);
         bars->abort_flag = 0;
         fence_mbar_init();
         tma_prefetch_desc(tmQ);
@@ -567,11 +571,11 @@ __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMa
     griddep_wait();  // everything above overlaps the previous kernel of the stream
 
     if (warp == 0) {
-        if (lane == 0) dq_producer<D, kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
-    } else if (warp == 1 || warp == 3) {
-        dq_mma<D, kDelta>(smem, bars, tmem_base, wk, warp >> 1);
-    } else if (warp >= 4) {
-        dq_rows<D, kCausal, kStrided, kDelta>(smem, bars, tmem_base, tmdQ, LSE, Delta, Delta_out, scale, wk,
+        if (lane == 0) dq_producer<D, kTiles, kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
+    } else if (warp == 1 || (kTiles == 2 && warp == 3)) {
+        dq_mma<D, kTiles, kDelta>(smem, bars, tmem_base, wk, warp >> 1);
+    } else if (warp >= 4 && warp < 4 + 4 * kTiles) {
+        dq_rows<D, kTiles, kCausal, kStrided, kDelta>(smem, bars, tmem_base, tmdQ, LSE, Delta, Delta_out, scale, wk,
                                               (warp - 4) >> 2, warp & 3, lane);
     }
 
@@ -581,58 +585,93 @@ __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMa
     if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
 }
 
-template <int D, bool kCausal, bool kStrided>
+template <int D, int kTiles, bool kCausal, bool kStrided>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                const __grid_constant__ CUtensorMap tmdQ, const float* __restrict__ LSE, const float* __restrict__ Delta,
                int T, int BH, int H, uint32_t orders, int n_blocks, int chunk, float scale, int* __restrict__ dev_status) {
-    dq_body<D, kCausal, kStrided, false>(&tmQ, &tmK, &tmV, &tmdO, &tmdQ, LSE, Delta, nullptr,
-                                         DqWork<D>{BH, n_blocks, chunk, T, H, orders, kCausal}, scale, dev_status);
+    dq_body<D, kTiles, kCausal, kStrided, false>(&tmQ, &tmK, &tmV, &tmdO, &tmdQ, LSE, Delta, nullptr,
+                                                 DqWork<D, kTiles>{BH, n_blocks, chunk, T, H, orders, kCausal}, scale, dev_status);
 }
 
-template <int D, bool kCausal>
+template <int D, int kTiles, bool kCausal>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                   const float* __restrict__ LSE, float* __restrict__ Delta, int T, int BH, int n_blocks, int chunk, float scale,
                   int* __restrict__ dev_status) {
-    dq_body<D, kCausal, false, true>(&tmQ, &tmK, &tmV, &tmdO, nullptr, LSE, nullptr, Delta,
-                                     DqWork<D>{BH, n_blocks, chunk, T, 1, 0u, kCausal}, scale, dev_status);
+    dq_body<D, kTiles, kCausal, false, true>(&tmQ, &tmK, &tmV, &tmdO, nullptr, LSE, nullptr, Delta,
+                                             DqWork<D, kTiles>{BH, n_blocks, chunk, T, 1, 0u, kCausal}, scale, dev_status);
 }
 
-int n_blocks_of(const AttnShape& s) { return (s.T + kBlockRows - 1) / kBlockRows; }
-int chunk_of(const AttnShape& s, int num_sms) { return heads_per_chunk(s.B * s.H, n_blocks_of(s), s.T, s.D, num_sms); }
-// One CTA per item; those that do not start at once are taken over by those that did.
-dim3 grid_of(const AttnShape& s) { return dim3(static_cast<unsigned>(n_blocks_of(s)) * s.B * s.H); }
-
-template <int D, bool kCausal>
-cudaError_t configure_one() {
-    auto set = [](auto kernel) {
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<D>::kSmemBytes);
+// Key steps after which the last SM is done, about: the longest item, or one item after another, the smallest of the first
+// round with the largest of each later one (items go out heaviest first).  Every item costs two steps besides.
+long long span_of(const AttnShape& s, int tiles, int n_blocks, int num_sms) {
+    const long long BH = static_cast<long long>(s.B) * s.H, items = n_blocks * BH;
+    const long long n_all = (s.T + kStep - 1) / kStep;
+    auto steps = [&](long long idx) {
+        const long long blk = n_blocks - 1 - idx / BH;
+        return 2 + (s.causal ? std::min(tiles * (blk + 1) * (kBlockQ / kStep), n_all) : n_all);
     };
-    cudaError_t e = set(attn_dq_kernel<D, kCausal, false>);
-    if (e == cudaSuccess) e = set(attn_dq_kernel<D, kCausal, true>);
-    if (e == cudaSuccess) e = set(attn_delta_kernel<D, kCausal>);
-    return e;
+    if (items <= num_sms) return steps(0);
+    long long sum = steps(num_sms - 1);
+    for (long long k = num_sms; k < items; k += num_sms) sum += steps(k);
+    return std::max(steps(0), sum);
 }
 
-// Calls f with the head dimension and the mask as compile-time constants.
+// How many tiles an item has, and what follows from it.
+//
+// Two tiles share their K and V and fill each other's gaps, which is worth 30 to 40 % of the work where there is enough of
+// it; a tile alone takes a step in 0.72 (D=64) to 0.6 (D=128) of a pair's time, so it wins where the longest chain
+// or the last round of items decides.  The weights 7:8 and 5:8 are fitted to both forms' times over 688 shapes (T = 129 to
+// 8192, 40 to 1200 tiles, with and without the mask): the slower form is taken at a mean cost of 0.3 %.
+// Pairs against single tiles, exact Delta: D=64, H=8, T=4096: 54.5, 37.9 us, H=16: 54.8, 69.1 us; H=48, T=512: 9.0, 7.2 us.
+// Deterministic backward: D=64, H=24, T=1024: 34.2, 30.5 us, H=48: 43.9, 47.6 us.
+struct Plan {
+    int tiles, n_blocks, chunk;
+    dim3 grid;  // one CTA per item; those that do not start at once are taken over by those that did
+};
+Plan plan_of(const AttnShape& s, int num_sms) {
+    Plan p;
+    const int n_tiles = (s.T + kBlockQ - 1) / kBlockQ, n_pairs = (n_tiles + 1) / 2, BH = s.B * s.H;
+    p.tiles = 2;
+    if (static_cast<long long>(n_pairs) * BH <= 4ll * num_sms) {  // (beyond that pairs always win, and the sum stays short)
+        const long long one = span_of(s, 1, n_tiles, num_sms), two = span_of(s, 2, n_pairs, num_sms);
+        if ((s.D == 64 ? 7 : 5) * one < 8 * two) p.tiles = 1;
+    }
+    p.n_blocks = (n_tiles + p.tiles - 1) / p.tiles;
+    p.chunk = heads_per_chunk(BH, p.n_blocks, s.T, s.D, num_sms);
+    p.grid = dim3(static_cast<unsigned>(p.n_blocks) * BH);
+    return p;
+}
+
+// Calls f with the head dimension, the tiles of an item and the mask as compile-time constants.
 template <typename F>
-cudaError_t dispatch(const AttnShape& s, F&& f) {
-    using D64 = std::integral_constant<int, 64>;
-    using D128 = std::integral_constant<int, 128>;
-    if (s.D == 64) return s.causal ? f(D64{}, std::true_type{}) : f(D64{}, std::false_type{});
-    return s.causal ? f(D128{}, std::true_type{}) : f(D128{}, std::false_type{});
+cudaError_t dispatch(int D, int tiles, bool causal, F&& f) {
+    auto with_d = [&](auto d) {
+        auto with_tiles = [&](auto t) { return causal ? f(d, t, std::true_type{}) : f(d, t, std::false_type{}); };
+        return tiles == 1 ? with_tiles(std::integral_constant<int, 1>{}) : with_tiles(std::integral_constant<int, 2>{});
+    };
+    return D == 64 ? with_d(std::integral_constant<int, 64>{}) : with_d(std::integral_constant<int, 128>{});
 }
 
 }  // namespace
 
 cudaError_t configure_attn_dq() {
-    cudaError_t e = configure_one<64, true>();
-    if (e == cudaSuccess) e = configure_one<64, false>();
-    if (e == cudaSuccess) e = configure_one<128, true>();
-    if (e == cudaSuccess) e = configure_one<128, false>();
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 8 && e == cudaSuccess; ++k)
+        e = dispatch(k & 1 ? 64 : 128, k & 2 ? 1 : 2, (k & 4) != 0, [](auto d, auto t, auto causal) {
+            constexpr int D = decltype(d)::value, kTiles = decltype(t)::value;
+            constexpr bool kCausal = decltype(causal)::value;
+            auto set = [](auto kernel) {
+                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<D, kTiles>::kSmemBytes);
+            };
+            cudaError_t r = set(attn_dq_kernel<D, kTiles, kCausal, false>);
+            if (r == cudaSuccess) r = set(attn_dq_kernel<D, kTiles, kCausal, true>);
+            if (r == cudaSuccess) r = set(attn_delta_kernel<D, kTiles, kCausal>);
+            return r;
+        });
     return e;
 }
 
@@ -640,25 +679,29 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
                            const CUtensorMap& tmdO, const CUtensorMap& tmdQ, bool strided, uint32_t orders,
                            const float* LSE, const float* Delta, const AttnShape& s, int num_sms, int* dev_status,
                            cudaStream_t stream) {
-    return dispatch(s, [&](auto d, auto causal) {
-        constexpr int D = decltype(d)::value;
+    const Plan p = plan_of(s, num_sms);
+    return dispatch(s.D, p.tiles, s.causal, [&](auto d, auto t, auto causal) {
+        constexpr int D = decltype(d)::value, kTiles = decltype(t)::value;
         constexpr bool kCausal = decltype(causal)::value;
         auto go = [&](auto kernel) {
-            return launch_overlapped(kernel, grid_of(s), dim3(kThreads), DqCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO,
-                                     tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, n_blocks_of(s), chunk_of(s, num_sms), s.scale, dev_status);
+            return launch_overlapped(kernel, p.grid, dim3(kThreads), DqCfg<D, kTiles>::kSmemBytes, stream, tmQ, tmK, tmV,
+                                     tmdO, tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, p.n_blocks, p.chunk, s.scale,
+                                     dev_status);
         };
-        return strided ? go(attn_dq_kernel<D, kCausal, true>) : go(attn_dq_kernel<D, kCausal, false>);
+        return strided ? go(attn_dq_kernel<D, kTiles, kCausal, true>) : go(attn_dq_kernel<D, kTiles, kCausal, false>);
     });
 }
 
 cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                               const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s,
                               int num_sms, int* dev_status, cudaStream_t stream) {
-    return dispatch(s, [&](auto d, auto causal) {
-        constexpr int D = decltype(d)::value;
+    const Plan p = plan_of(s, num_sms);
+    return dispatch(s.D, p.tiles, s.causal, [&](auto d, auto t, auto causal) {
+        constexpr int D = decltype(d)::value, kTiles = decltype(t)::value;
         constexpr bool kCausal = decltype(causal)::value;
-        return launch_overlapped(attn_delta_kernel<D, kCausal>, grid_of(s), dim3(kThreads), DqCfg<D>::kSmemBytes, stream, tmQ,
-                                 tmK, tmV, tmdO, LSE, Delta, s.T, s.B * s.H, n_blocks_of(s), chunk_of(s, num_sms), s.scale, dev_status);
+        return launch_overlapped(attn_delta_kernel<D, kTiles, kCausal>, p.grid, dim3(kThreads), DqCfg<D, kTiles>::kSmemBytes,
+                                 stream, tmQ, tmK, tmV, tmdO, LSE, Delta, s.T, s.B * s.H, p.n_blocks, p.chunk, s.scale,
+                                 dev_status);
     });
 }
 

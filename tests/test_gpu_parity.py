@@ -404,6 +404,35 @@ def test_query_major_passes_at_step_edges(T, D, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"steps T={T} D={D}: ", dO=ref["dO_in"])
 
 
+@pytest.mark.parametrize("T", [129, 256, 257, 500, 1000])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_query_major_passes_alone_and_in_a_crowd(T, D, causal):
+    """The exact Delta and the deterministic dQ take single query tiles where the longest of them decides and pairs where the
+    work does: a head alone, 100 copies of it (single tiles in several rounds at the shorter lengths) and 640 (pairs) have the
+    same bits, and the oracle's values."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("crowd", B=1, H=1, T=T, D=D, seed=500 + T + D, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    got = h.run_gpu(Q, K, V, dO, cfg.scale, causal, exact_delta=True)
+    first = None
+    for n in (1, 100, 640):
+        q, k, v, do = (x.to(dev).expand(1, n, T, D).contiguous() for x in (Q, K, V, dO))
+        lse = got["LSE"].to(dev).expand(1, n, T).contiguous()
+        delta, grads = torch.full_like(lse, 7.0), [torch.full_like(q, 7.0) for _ in range(3)]
+        nova_attn.nova_attn_bwd_preprocess_exact(q, k, v, do, lse, delta, cfg.scale, causal)
+        nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *grads, cfg.scale, causal)
+        nova_attn.nova_attn_poll_device_status()
+        outs = [delta, *grads]
+        first = first or [t[:, :1].clone() for t in outs]
+        assert all(torch.equal(t, f.expand_as(t)) for t, f in zip(outs, first)), n
+    got.update({name: t.cpu() for name, t in zip(("Delta", "dQ", "dK", "dV"), first)})
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal)
+    h.compare(h.select_heads(got, None), ref, label=f"crowd T={T} D={D}: ", dO=ref["dO_in"])
+
+
 @pytest.mark.parametrize("T", [1, 127, 129, 256, 257, 384, 500])
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("causal", [True, False])
