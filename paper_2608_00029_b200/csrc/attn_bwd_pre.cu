@@ -97,19 +97,22 @@ __global__ void __launch_bounds__(256) bwd_preprocess_kernel(const uint4* __rest
     }
 }
 
-// Heads inside tokens (O and dO as [B,T,H,D] views): a block takes kTokTile tokens of kTokHeads heads, reads them in the order
+// Heads inside tokens (O and dO as [B,T,H,D] views): a block takes a tile of tokens of kTokHeads heads, reads them in the order
 // in which they lie in memory, kTokHeads * 2 * D bytes at a time, and turns the sums round in shared memory, so that
-// Delta [B,H,T] is written in lines as well.  Head by head through such a layout (128 bytes every 2 KB) reading took
-// 10.8 us at B=8, H=16, T=1024, D=64 and 18.5 us at B=4, H=32, T=1000, D=128, against 8.5 and 14.1 us here; in memory
-// order with the sums written as they come 16 and 28 us.  Tiles of 32 tokens: 7.4 to 10 and 17.6 us.
-constexpr int kTokTile = 16, kTokHeads = 8;
+// Delta [B,H,T] is written in lines as well.  Of 8, 4 and 2 heads the number that pads H least (8 alone left most lanes
+// of a model with two or three heads idle: H=2, B=32, T=2048, D=64 15.4 us against 5.5, 8.4 head by head).  A thread has
+// kBatches * 4 rows, four in flight: one batch, so that small problems have more blocks (B=1, H=12, T=1024, D=128 3.9 us with
+// two, 2.3 with one), but two at D=128 from six blocks per SM on (B=8, H=32, T=1024: 26.2 us with one, 25.1 with two).
+// Head by head through such a layout (128 bytes every 2 KB) reading took 8.4 us at B=8, H=16, T=1024, D=64 and 15.8 us at
+// B=4, H=32, T=1000, D=128, against 5.5 and 9.4 us here (inputs in L2); from DRAM 16.4 and 24.6 against 14.3 and 21.4.
+__host__ __device__ constexpr int tok_tile(int D, int heads, int batches) { return batches * 4 * (2048 / D) / heads; }
 
-template <int LPR>
+template <int LPR, int kTokHeads, int kBatches>
 __global__ void __launch_bounds__(256, 4) bwd_preprocess_tokens_kernel(const uint4* __restrict__ O, const uint4* __restrict__ dO,
                                                                     float* __restrict__ Delta, int H, int T, int t_tiles,
                                                                     int h_tiles, const TensorStrides so,
                                                                     const TensorStrides sdo) {
-    constexpr int kRowsPerPass = 256 / LPR, kPasses = kTokTile * kTokHeads / kRowsPerPass, kUnroll = 4;
+    constexpr int kRowsPerPass = 256 / LPR, kPasses = 4, kTokTile = tok_tile(8 * LPR, kTokHeads, kBatches);
     __shared__ float sums[kTokHeads][kTokTile + 1];
     griddep_launch_dependents();
     const int h0 = static_cast<int>(blockIdx.x) % h_tiles * kTokHeads;
@@ -120,10 +123,10 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_tokens_kernel(const uin
     const uint4* pd = dO + ((b * sdo.b) >> 3) + sub;
     griddep_wait();
 #pragma unroll
-    for (int p = 0; p < kPasses; p += kUnroll) {
-        uint4 x[kUnroll], y[kUnroll];
+    for (int p = 0; p < kBatches * kPasses; p += kPasses) {
+        uint4 x[kPasses], y[kPasses];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < kPasses; ++u) {
             const int r = row0 + (p + u) * kRowsPerPass, t = t0 + r / kTokHeads, h = h0 + r % kTokHeads;
             x[u] = y[u] = make_uint4(0, 0, 0, 0);
             if (t < T && h < H) {
@@ -132,7 +135,7 @@ __global__ void __launch_bounds__(256, 4) bwd_preprocess_tokens_kernel(const uin
             }
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < kPasses; ++u) {
             float acc = dot8_bf16(x[u], y[u]);
 #pragma unroll
             for (int off = LPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
@@ -232,14 +235,32 @@ cudaError_t launch_attn_bwd_preprocess(const __nv_bfloat16* O, const __nv_bfloat
     const uint4* d4 = reinterpret_cast<const uint4*>(dO);
     const dim3 grid(static_cast<unsigned>(blocks));
     const bool contiguous = is_contiguous(s, so) && is_contiguous(s, sdo);
-    const int t_tiles = (s.T + kTokTile - 1) / kTokTile, h_tiles = (s.H + kTokHeads - 1) / kTokHeads;
-    const long long token_blocks = static_cast<long long>(s.B) * t_tiles * h_tiles;
-    if (!contiguous && so.h < so.t && sdo.h < sdo.t && token_blocks <= 0x7fffffff) {
+    if (!contiguous && so.h < so.t && sdo.h < sdo.t) {
+        int heads = 8;
+        auto padded = [&](int n) { return (s.H + n - 1) / n * n; };
+        for (int n : {4, 2})
+            if (padded(n) < padded(heads)) heads = n;
+        const long long rows_padded = static_cast<long long>(s.B) * padded(heads) * s.T;
+        const int batches = (s.D == 128 && rows_padded / (128 * 6) >= num_sms) ? 2 : 1;
+        const int tile = tok_tile(s.D, heads, batches), t_tiles = (s.T + tile - 1) / tile, h_tiles = (s.H + heads - 1) / heads;
+        const long long blocks_tok = static_cast<long long>(s.B) * t_tiles * h_tiles;
         auto go = [&](auto kernel) {
-            return launch_overlapped(kernel, dim3(static_cast<unsigned>(token_blocks)), dim3(kThreads), 0, stream, o4, d4,
-                                     Delta, s.H, s.T, t_tiles, h_tiles, so, sdo);
+            return launch_overlapped(kernel, dim3(static_cast<unsigned>(blocks_tok)), dim3(kThreads), 0, stream, o4, d4, Delta,
+                                     s.H, s.T, t_tiles, h_tiles, so, sdo);
         };
-        return s.D == 64 ? go(bwd_preprocess_tokens_kernel<8>) : go(bwd_preprocess_tokens_kernel<16>);
+        if (blocks_tok <= 0x7fffffff) {
+            if (s.D == 64)
+                return heads == 8   ? go(bwd_preprocess_tokens_kernel<8, 8, 1>)
+                       : heads == 4 ? go(bwd_preprocess_tokens_kernel<8, 4, 1>)
+                                    : go(bwd_preprocess_tokens_kernel<8, 2, 1>);
+            if (batches == 1)
+                return heads == 8   ? go(bwd_preprocess_tokens_kernel<16, 8, 1>)
+                       : heads == 4 ? go(bwd_preprocess_tokens_kernel<16, 4, 1>)
+                                    : go(bwd_preprocess_tokens_kernel<16, 2, 1>);
+            return heads == 8   ? go(bwd_preprocess_tokens_kernel<16, 8, 2>)
+                   : heads == 4 ? go(bwd_preprocess_tokens_kernel<16, 4, 2>)
+                                : go(bwd_preprocess_tokens_kernel<16, 2, 2>);
+        }
     }
     auto go = [&](auto kernel) {
         return launch_overlapped(kernel, grid, dim3(kThreads), 0, stream, o4, d4, Delta, rows, split_of(s), so, sdo);

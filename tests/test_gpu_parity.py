@@ -231,7 +231,8 @@ def test_preprocess_matches_rowsum():
         torch.testing.assert_close(Delta.cpu().double(), ref, rtol=1e-5, atol=1e-5)
 
 
-@pytest.mark.parametrize("B,H,T", [(1, 1, 1), (2, 7, 33), (1, 9, 16), (3, 8, 257), (16, 12, 513), (4, 12, 1024)])
+@pytest.mark.parametrize("B,H,T", [(1, 1, 1), (2, 7, 33), (1, 9, 16), (3, 8, 257), (16, 12, 513), (4, 12, 1024), (3, 2, 129),
+                                   (2, 3, 77), (1, 6, 65), (9, 25, 700), (60, 3, 705), (60, 2, 1001)])
 @pytest.mark.parametrize("D", [64, 128])
 def test_preprocess_with_heads_inside_tokens(B, H, T, D):
     """O and dO as views of [B,T,H,D] buffers take the path that reads in memory order: tiles of tokens and heads with
