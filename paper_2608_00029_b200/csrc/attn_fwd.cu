@@ -759,12 +759,6 @@ __device__ __forceinline__ void fwd_mma_single(uint8_t* smem, FwdBars* bars, uin
     }
 }
 
-// Does a sum `l` of 64 keys, to be weighted with f, take no part at all?  Scores of a size at which the rounding of m * c
-// alone exceeds the exponent's range (masks of the type's lowest value) make P = 2^(s * c - m * c) infinite among
-// themselves, and infinity times the weight 0 would be NaN.  (A sum that is NaN itself takes part, and with l = 0 there is
-// nothing to leave out.)
-__device__ __forceinline__ bool no_part(float f, float l) { return f == 0.f && l > 0.f; }
-
 template <int D, bool kCausal, bool kStrided, typename Work>
 __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const CUtensorMap* tmO,
                                                    float* __restrict__ LSE, float scale, const Work& wk, int t, int swarp,
@@ -826,8 +820,7 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
             } else if (__any_sync(0xffffffffu, (m_new - m_ref) * c > kRescaleThreshold)) {  // (-inf against -inf: no)
                 const float f = m_new > m_ref ? ex2_approx((m_ref - m_new) * c) : 1.f;  // 0 from -inf
                 m_ref = m_new;
-                const bool none = no_part(f, l);
-                l = none ? 0.f : l * f;
+                l *= f;
                 ok = mbar_wait(&bars->pv_done[t], (cnt - 1) & 1, abort_flag, limit);
                 if (!ok) break;
                 tc_fence_after();
@@ -837,11 +830,15 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
                     tmem_ld_x16(t_o + cb, o);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) o[i] = none ? 0u : __float_as_uint(__uint_as_float(o[i]) * f);
+                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
                     tmem_st_x16(t_o + cb, o);
                 }
             }
-            const float mc = m_ref == -INFINITY ? 0.f : m_ref * c;
+            // P = 2^(s * c - m * c).  Where the rounding of m * c is as large as the exponent's range (a half whose scores are
+            // all the type's lowest value, beside ordinary ones in the other) m * c is rounded up, which keeps P <= 1: an
+            // infinite sum would be NaN times the weight 0 that it gets in the end.
+            const float mc_near = m_ref * c, mc_up = __fmul_ru(m_ref, c);
+            const float mc = m_ref == -INFINITY ? 0.f : fabsf(mc_near) > 1e9f ? mc_up : mc_near;
             const uint64_t nmc2 = f32x2_pack(-mc, -mc);
             uint64_t acc0 = 0, acc1 = 0;
             uint32_t pk[32];
@@ -891,8 +888,7 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
         const float2 s0 = s_w[row_local], s1 = s_w[kBlockQ + row_local];
         const float m = fmaxf(s0.x, s1.x);  // finite: key 0 is in the first half and every row keeps it
         const float f0 = ex2_approx((s0.x - m) * c), f1 = ex2_approx((s1.x - m) * c);  // 2^-inf = 0
-        const bool none0 = no_part(f0, s0.y), none1 = no_part(f1, s1.y), any_none = __any_sync(0xffffffffu, none0 || none1);
-        l = (none0 ? 0.f : s0.y * f0) + (none1 ? 0.f : s1.y * f1);
+        l = s0.y * f0 + s1.y * f1;
         const float i0 = f0 / l, i1 = f1 / l;
 #pragma unroll
         for (int cb = 0; cb < D / 2; cb += 32) {
@@ -900,13 +896,6 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
             tmem_ld_x32(t_o_half + cb, a);
             tmem_ld_x32(t_o_half + D + cb, b);
             tmem_wait_ld();
-            if (any_none) {
-#pragma unroll
-                for (int x = 0; x < 32; ++x) {
-                    a[x] = none0 ? 0u : a[x];
-                    b[x] = none1 ? 0u : b[x];
-                }
-            }
             const int col = D / 2 * t + cb;
             uint8_t* row_ptr = stage + (col / 64) * kHalfTileBytes + row_local * 128;
 #pragma unroll
