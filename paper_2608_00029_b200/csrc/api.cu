@@ -391,12 +391,16 @@ namespace {
 // -> 605 us; B=4, H=32, T=512: 68 -> 61 us; B=4, H=16, T=2048 without the mask: 505 -> 440 us; B=2, H=16, T=4096: 480 ->
 // 460 us; but B=2, H=12, T=8192: 1290 -> 1340 us (the card's power limit, and two contractions more).  And they
 // need the SMs filled: each is half the work in as long chains (B=1, H=32, T=1024, 128 blocks of 256 rows: 47 -> 55
-// us; B=2, H=32, T=640, 192 blocks: 49 us both).
-bool two_kernels_pay(long long BH, int T, int D, int num_sms) {
-    return D == 128 && T <= 4096 && BH * ((T + 255) / 256) * 2 >= 3ll * num_sms;
+// us; B=2, H=32, T=640, 192 blocks: 49 us both).  Without the mask every item of a head is as long as its longest, so that a
+// last round with few items costs as much as a full one: above T=2560 the two kernels then need more than three rounds of
+// blocks (H=28, T=4096: 763 -> 807 us, H=20: 539 -> 590 us; but H=32: 909 -> 843 us, H=40, T=3584: 827 -> 797 us).
+bool two_kernels_pay(long long BH, int T, int D, bool causal, int num_sms) {
+    const long long blocks = BH * ((T + 255) / 256);
+    if (D != 128 || T > 4096) return false;
+    return !causal && T > 2560 ? blocks * 3 >= 10ll * num_sms : blocks * 2 >= 3ll * num_sms;
 }
 
-// dQ, dK and dV by the two-kernel backward. 
+// dQ, dK and dV by the two-kernel backward.
 int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO, const float* LSE, const float* Delta,
                     void* dQ, void* dK, void* dV, const AttnShape& s, const TensorStrides& sq, const TensorStrides& sk,
                     const TensorStrides& sv, const TensorStrides& sdo, const TensorStrides& sdq, const TensorStrides& sdk,
@@ -455,7 +459,7 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
     // B=8, H=32, T=100, D=128: 24.9 -> 16.5 us).
     const bool whole = steps == (NOVA_ATTN_BWD_STEP_ZERO | NOVA_ATTN_BWD_STEP_MAIN | NOVA_ATTN_BWD_STEP_CONVERT);
     const bool direct = T <= kBlockK && whole;
-    if (whole && !direct && two_kernels_pay(BH, T, D, st->num_sms))
+    if (whole && !direct && two_kernels_pay(BH, T, D, causal != 0, st->num_sms))
         return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv, *st, cs);
     if ((steps & NOVA_ATTN_BWD_STEP_ZERO) && !direct) {
         e = launch_zero(acc, need, st->num_sms, cs);
