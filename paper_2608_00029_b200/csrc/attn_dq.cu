@@ -605,19 +605,13 @@ attn_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                                              DqWork<D, kTiles>{BH, n_blocks, chunk, T, 1, 0u, kCausal}, scale, dev_status);
 }
 
-// Key steps after which the last SM is done, about: the longest item, or one item after another, the smallest of the first
-// round with the largest of each later one (items go out heaviest first).  Every item costs two steps besides.
+// Key steps after which the last SM is done.  Every item costs two besides its own.
 long long span_of(const AttnShape& s, int tiles, int n_blocks, int num_sms) {
-    const long long BH = static_cast<long long>(s.B) * s.H, items = n_blocks * BH;
-    const long long n_all = (s.T + kStep - 1) / kStep;
-    auto steps = [&](long long idx) {
+    const long long BH = static_cast<long long>(s.B) * s.H, n_all = (s.T + kStep - 1) / kStep;
+    return steps_until_done(n_blocks * BH, num_sms, [&](long long idx) {
         const long long blk = n_blocks - 1 - idx / BH;
         return 2 + (s.causal ? std::min(tiles * (blk + 1) * (kBlockQ / kStep), n_all) : n_all);
-    };
-    if (items <= num_sms) return steps(0);
-    long long sum = steps(num_sms - 1);
-    for (long long k = num_sms; k < items; k += num_sms) sum += steps(k);
-    return std::max(steps(0), sum);
+    });
 }
 
 // How many tiles an item has, and what follows from it.

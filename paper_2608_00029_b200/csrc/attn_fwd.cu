@@ -1034,15 +1034,30 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
                        const CUtensorMap& tmO, bool strided, uint32_t orders, float* LSE, const AttnShape& s,
                        int num_sms, long long wait_limit, int inject, int* dev_status, cudaStream_t stream) {
     const int BH = s.B * s.H;
-    const int n_tiles = (s.T + kBlockQ - 1) / kBlockQ;
+    const int n_tiles = (s.T + kBlockQ - 1) / kBlockQ, n_pairs = (n_tiles + 1) / 2;
     // Pairs of query tiles share their K and V tiles and fill each other's gaps; but if every tile can have an SM of its
     // own, a tile is done sooner alone, with both softmax groups on it.  Pairs, single tiles: D=64, B=1, H=12, T=777: 13.6,
     // 10.0 us; T=1500: 23.4, 14.7 us; H=1, T=8192: 99.5, 56.5 us; D=128, B=1, H=16, T=1024 without the mask: 20.9, 12.9 us.
+    // With more tiles than that it depends on where the last round of items ends.  A step of a single tile takes 0.57 (D=64)
+    // or 0.66 (D=128) of a pair's and an item three steps besides; at D=128, where O and the next Q tile share a buffer in
+    // this form, single tiles have to promise more (7:9).  Fitted to both forms' times over 804 shapes (T = 64 to 8192, 60
+    // to 1000 tiles).  Pairs, single tiles: D=64, H=24, T=1024 17.3, 11.3 us; H=12, T=4096 54.8, 46.1 us; H=96, T=1024 29.4,
+    // 32.1 us; D=128, H=24, T=1024 21.1, 12.7 us; H=96, T=384 without the mask 17.8, 13.4 us; H=96, T=256 10.0, 10.9 us.
     // With T <= 128 a pair has no second tile and one softmax group would be idle.  At D=64 that alone decides: B=64, H=12,
     // T=100: 20.1, 17.4 us; B=50, T=17: 16.1, 14.2 us.  At D=128 O and the next Q tile share a buffer in this form, and
     // items follow each other sooner in the other: B=64, H=12, T=100: 25.1, 29.8 us; B=8, H=32, T=128: 10.7, 12.0 us.
-    const bool single = static_cast<long long>(n_tiles) * BH <= num_sms || (D == 64 && n_tiles == 1);
-    const int n_blocks = single ? n_tiles : (n_tiles + 1) / 2;
+    bool single = static_cast<long long>(n_tiles) * BH <= num_sms || (D == 64 && n_tiles == 1);
+    if (!single && n_tiles > 1 && static_cast<long long>(n_tiles) * BH <= 7ll * num_sms) {
+        auto span = [&](int tiles, int blocks) {
+            return steps_until_done(static_cast<long long>(blocks) * BH, num_sms, [&](long long idx) -> long long {
+                const int blk = blocks - 1 - static_cast<int>(idx / BH), last = tiles * (blk + 1);
+                return 3 + (kCausal && last < n_tiles ? last : n_tiles);
+            });
+        };
+        const long long one = span(1, n_tiles), two = span(2, n_pairs);
+        single = D == 64 ? 4 * one < 7 * two : 7 * one < 9 * two;
+    }
+    const int n_blocks = single ? n_tiles : n_pairs;
     const int chunk = D == 128 ? heads_per_chunk(BH, n_blocks, s.T, D, num_sms) : BH;
     const dim3 grid(static_cast<unsigned>(n_blocks) * BH);  // one CTA per item; those that do not start at once are taken over
     auto go = [&](auto kernel) {

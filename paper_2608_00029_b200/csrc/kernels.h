@@ -105,6 +105,17 @@ inline int heads_per_chunk(int BH, int items_per_head, long long T, int D, int n
     return static_cast<int>((BH + n - 1) / n);
 }
 
+// Steps after which the last SM is done with `items` work items that go out heaviest first, about: the longest item, or one
+// item after another, the smallest of the first round with the largest of each later one.  steps(i): those of item i, with
+// what an item costs besides.  For a few rounds of items (it adds them up).
+template <typename F>
+long long steps_until_done(long long items, int num_sms, F&& steps) {
+    if (items <= num_sms) return steps(0);
+    long long sum = steps(num_sms - 1);
+    for (long long k = num_sms; k < items; k += num_sms) sum += steps(k);
+    return steps(0) > sum ? steps(0) : sum;
+}
+
 // What the backward main kernel does with its partial tiles of dQ.
 enum class DqMode {
     kAccumulate,  // adds them, unscaled, into the fp32 accumulator

@@ -462,6 +462,29 @@ def test_forward_alone_and_in_a_crowd(T, D, causal):
         tol.assert_close(W.widen(lse[:1, :1]), ref["LSE"], tol.FWD_ATOL, tol.FWD_RTOL, "LSE", tol.FWD_REL_RMS)
 
 
+@pytest.mark.parametrize("n", [20, 60, 600])
+@pytest.mark.parametrize("T", [257, 640, 1024])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_forward_between_one_tile_per_sm_and_many_rounds(n, T, D, causal):
+    """Which of its two forms the forward takes there depends on how the last round of items ends; single tiles then also
+    follow each other on an SM.  Copies of one head, at head counts on both sides: all the same, and the oracle's values."""
+    import tolerance as tol
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("rounds", B=1, H=1, T=T, D=D, seed=800 + T + D, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal)
+    q, k, v = (x.to(dev).expand(1, n, T, D).contiguous() for x in (Q, K, V))
+    o, lse = torch.full_like(q, 7.0), torch.full((1, n, T), 7.0, device=dev)
+    nova_attn.nova_attn_fwd(q, k, v, o, lse, cfg.scale, causal)
+    nova_attn.nova_attn_poll_device_status()
+    assert torch.equal(o, o[:, :1].expand_as(o)) and torch.equal(lse, lse[:, :1].expand_as(lse))
+    tol.assert_close(W.widen(o[:, :1]), ref["O"], tol.FWD_ATOL, tol.FWD_RTOL, "O", tol.FWD_REL_RMS)
+    tol.assert_close(W.widen(lse[:, :1]), ref["LSE"], tol.FWD_ATOL, tol.FWD_RTOL, "LSE", tol.FWD_REL_RMS)
+
+
 @pytest.mark.parametrize("T", [128, 200, 500])
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("first", [0, 64])
