@@ -51,9 +51,10 @@ struct FwdCfg {
     // 16 KB per tile of its own, half of the columns at a time, so that the one Q stage can take the next item's Q as
     // soon as the last Q K^T has read it instead of after the item's O has left: 207 -> 188 us at B=16, H=32, T=1024, 66
     // -> 59 us at B=4, H=32, T=1000, 33 -> 28 us at B=64, H=12, T=100. 
-    static constexpr bool kOwnStage = (kQStages == 1);
-    static constexpr int kOffO = kOffV + kKVStages * kTileBytes;      // kOwnStage: [2 tiles]
-    static constexpr int kOffBar = kOffO + (kOwnStage ? 2 * kHalfTileBytes : 0);
+    // With an SM for every item no next Q tile is waiting, and O leaves sooner whole, through the Q buffers there too: 9.98 ->
+    // 9.67 us at B=8, H=12, T=256 without the mask.
+    static constexpr int kOffO = kOffV + kKVStages * kTileBytes;      // kOwn: [2 tiles]
+    static constexpr int kOffBar = kOffO + (kQStages == 1 ? 2 * kHalfTileBytes : 0);
     static constexpr int kSmemBytes = kOffBar + 512 + 1024;
     static constexpr int kColS = 0;      // + 128 * tile
     static constexpr int kColO = 256;    // + D * tile
@@ -79,8 +80,10 @@ constexpr int kWorkConsumers = 1 + 8;  // UMMA issuer warp + 8 softmax warps
 // Work items: 256-row query blocks, numbered heaviest first; at D=128 within chunks of heads whose K and V stay in L2 from
 // one block to the next (184 -> 171 us at B=16, H=32, T=1024, 150 -> 139 us at B=2, H=16, T=4096; D=64, with half the
 // bytes per head, gained nothing).  kSingle: 128-row blocks, tile A alone.
-template <int D, bool kSingle>
+// kOwn: O leaves through buffers of its own (D=128, pairs of tiles, more items than SMs).
+template <int D, bool kSingle, bool kOwn>
 struct FwdWork {
+    static constexpr bool kOwnStage = kOwn;
     static constexpr bool kChunks = (D == 128) && !kSingle;
     static constexpr int kRows = kSingle ? kBlockQ : kBlockRows;
     static constexpr int kTiles = kRows / kBlockQ;
@@ -195,7 +198,7 @@ template <int D, typename Work>
 __device__ __forceinline__ void fwd_mma(uint8_t* smem, FwdBars* bars, uint32_t tmem_base, const Work& wk,
                                         long long limit) {
     using Cfg = FwdCfg<D>;
-    constexpr bool kOwnStage = Cfg::kOwnStage;
+    constexpr bool kOwnStage = Work::kOwnStage;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescQK = umma_idesc_bf16(128, 128, 0, 0);
     constexpr uint32_t kIdescPV = umma_idesc_bf16(128, D, 0, 1);
@@ -379,7 +382,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                                             float* __restrict__ LSE, float scale, const Work& wk, int t, int swarp,
                                             int lane, long long limit) {
     using Cfg = FwdCfg<D>;
-    constexpr bool kOwnStage = Cfg::kOwnStage;
+    constexpr bool kOwnStage = Work::kOwnStage;
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * (swarp & 3);
     const int row_local = lane_base + lane;
@@ -631,10 +634,14 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                 }
             }
         }
+        if (Cfg::kQStages == 1 && !kOwnStage && leader && leader_ok) {  // the next item's Q tile needs this very buffer
+            bulk_wait_group_read<0>();
+            mbar_arrive(&bars->q_empty[qs]);
+        }
         // With two Q stages the buffer is only needed for the item after next: it is handed back after the next
         // item's first key tile, when the store has long read it, instead of holding this warp up now (worth 7 %
         // at B=8, H=12, T=1024; a separate store thread that waits in the softmax warps' stead was slower).
-        pending_qs = qs;
+        if (Cfg::kQStages > 1 || kOwnStage) pending_qs = qs;
         // Brings the leader back together with the rest of its warp before the next warp-wide TMEM
         // load, and makes a failed wait of the leader a failure of the whole warp.
         ok = __all_sync(0xffffffffu, leader_ok);
@@ -940,7 +947,7 @@ __device__ __forceinline__ void fwd_softmax_single(uint8_t* smem, FwdBars* bars,
     if (leader) bulk_wait_group<0>();  // O must be complete before the kernel ends
 }
 
-template <int D, bool kCausal, bool kStrided, bool kSingle>
+template <int D, bool kCausal, bool kStrided, bool kSingle, bool kOwn>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -951,14 +958,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     FwdBars* bars = reinterpret_cast<FwdBars*>(smem + Cfg::kOffBar);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    using Work = FwdWork<D, kSingle>;
+    using Work = FwdWork<D, kSingle, kOwn>;
     const Work wk{n_blocks * BH, BH, n_blocks, (T + kBlockK - 1) / kBlockK, T, H, chunk, orders, kCausal};
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(&bars->q_full[s], 1);
             // the store leaders of the two query tiles, or the UMMA issuer where O has buffers of its own
-            mbar_init(&bars->q_empty[s], kSingle || Cfg::kOwnStage ? 1 : 2);
+            mbar_init(&bars->q_empty[s], kSingle || kOwn ? 1 : 2);
             mbar_init(&bars->o_sent[s], 1);
             mbar_init(&bars->k_full[s], 1);
             mbar_init(&bars->k_empty[s], 1);
@@ -1065,17 +1072,26 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
                                  BH, s.H, orders, n_blocks, chunk, s.scale, wait_limit, inject, dev_status);
     };
     if (single)
-        return strided ? go(attn_fwd_kernel<D, kCausal, true, true>) : go(attn_fwd_kernel<D, kCausal, false, true>);
-    return strided ? go(attn_fwd_kernel<D, kCausal, true, false>) : go(attn_fwd_kernel<D, kCausal, false, false>);
+        return strided ? go(attn_fwd_kernel<D, kCausal, true, true, false>) : go(attn_fwd_kernel<D, kCausal, false, true, false>);
+    if constexpr (D == 128) {
+        if (static_cast<long long>(n_blocks) * BH > num_sms)
+            return strided ? go(attn_fwd_kernel<D, kCausal, true, false, true>)
+                           : go(attn_fwd_kernel<D, kCausal, false, false, true>);
+    }
+    return strided ? go(attn_fwd_kernel<D, kCausal, true, false, false>) : go(attn_fwd_kernel<D, kCausal, false, false, false>);
 }
 
 template <int D, bool kCausal, bool kStrided>
 cudaError_t configure_one() {
-    const cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<D, kCausal, kStrided, false>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<D>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(attn_fwd_kernel<D, kCausal, kStrided, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                FwdCfg<D>::kSmemBytes);
+    auto set = [](auto kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdCfg<D>::kSmemBytes);
+    };
+    cudaError_t e = set(attn_fwd_kernel<D, kCausal, kStrided, false, false>);
+    if (e == cudaSuccess) e = set(attn_fwd_kernel<D, kCausal, kStrided, true, false>);
+    if constexpr (D == 128) {
+        if (e == cudaSuccess) e = set(attn_fwd_kernel<D, kCausal, kStrided, false, true>);
+    }
+    return e;
 }
 
 }  // namespace
