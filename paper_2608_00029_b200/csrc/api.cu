@@ -579,9 +579,8 @@ int nova_lmhead_fwd(const void* X, const void* W, const int* targets, void* logi
     int rows_x = 0, rows_w = 0;
     const int box_k = lmhead_boxes(&rows_x, &rows_w);
     CUtensorMap tmX, tmW, tmWh, tmL;
-    if (M <= kLmHeadFewRows) {  // 24 rows: 18.7 against 45.7 us; the accumulator and the shuffles are laid out for 64
-        int ctas, tile_h, m_pad;
-        lmhead_rows_plan(M, N, st->num_sms, &ctas, &tile_h, &m_pad);
+    int ctas, tile_h, m_pad;
+    if (lmhead_rows_plan(M, N, st->num_sms, &ctas, &tile_h, &m_pad)) {
         if (int rc = encode_matrix_map(X, M, K, m_pad, box_k, &tmX)) return rc;
         if (int rc = encode_matrix_map(W, N, K, tile_h, box_k, &tmW)) return rc;
         const cudaError_t e = launch_lmhead_rows(tmX, tmW, targets, logits, lse, loss, M, N, K, ctas, tile_h, m_pad,

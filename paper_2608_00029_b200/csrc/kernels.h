@@ -148,11 +148,12 @@ float* lmhead_target_logits(void* workspace, int M, int N);  // the part of the 
 // Rows of the X and W boxes; returns the box width in k elements.
 int lmhead_boxes(int* box_rows_x, int* box_rows_w);
 
-// The same for at most kLmHeadFewRows rows (lmhead_rows.cu).  lmhead_rows_plan chooses the number of CTAs, the height
-// of a W tile (rows of the box of `tmW`) and the rows of the box of `tmX`; both boxes are 64 k elements wide.
+// The same for at most kLmHeadFewRows rows (lmhead_rows.cu).  lmhead_rows_plan says whether this kernel is the faster one and
+// chooses the number of CTAs, the height of a W tile (rows of the box of `tmW`) and the rows of the box of `tmX`; both boxes
+// are 64 k elements wide.
 constexpr int kLmHeadFewRows = 64;
 cudaError_t configure_lmhead_rows();
-void lmhead_rows_plan(int M, int N, int num_sms, int* ctas, int* tile_h, int* m_pad);
+bool lmhead_rows_plan(int M, int N, int num_sms, int* ctas, int* tile_h, int* m_pad);
 cudaError_t launch_lmhead_rows(const CUtensorMap& tmX, const CUtensorMap& tmW, const int* targets, void* logits,
                                float* lse, float* loss, int M, int N, int K, int ctas, int tile_h, int m_pad,
                                void* workspace, float* tgt_logit, int* dev_status, cudaStream_t stream);

@@ -17,7 +17,7 @@
 // 192 threads: warp 0 TMA producer, warp 1 UMMA issuer, warps 2-5 epilogue.
 // N = 50304, K = 768, M = 24, logits stored, back to back from a graph, merge included: 18.7 us, against 45.7 us for
 // lmhead_kernel (X padded to 128 rows, 256-entry tiles of W in two uneven rounds, 393 pairs per row merged by one
-// block), which is kept from 65 rows on.
+// block); lmhead_rows_plan says where that one is kept.
 #include "../../include/nova_lmhead.h"
 #include "kernels.h"
 #include "ptx.cuh"
@@ -307,7 +307,14 @@ cudaError_t configure_lmhead_rows() {
     return cudaFuncSetAttribute(lmhead_rows_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
 }
 
-void lmhead_rows_plan(int M, int N, int num_sms, int* ctas, int* tile_h, int* m_pad) {
+// When it pays.  This kernel against lmhead_kernel in us at N = 50304, K = 768, logits stored (part of W in L2): M = 24 15.0, 34.8;
+// 48 22.9, 34.7; 64 23.3, 34.2, where the accumulator and the shuffles end.  Up to 32 rows it is the faster one at every N
+// (1000 to 64000) and K (64 to 1600).  From 33 on a tile's epilogue has two groups of rows, which reading W has to pay for: not
+// below some 5000 entries (N = 4096 0.92 to 1.10 of the other kernel's time, N = 8000 0.85 to 0.96), nor where a second
+// round of tiles has only just begun and its tiles are low (N = 19000, tiles of 72: 0.74 to 1.14; N = 24000, tiles of 88:
+// 0.64 to 0.97).
+bool lmhead_rows_plan(int M, int N, int num_sms, int* ctas, int* tile_h, int* m_pad) {
+    if (M > kLmHeadFewRows) return false;
     const int limit = num_sms < 32 * kMergeSteps ? num_sms : 32 * kMergeSteps;
     const int full = (N + kTileV - 1) / kTileV;  // also what the workspace has room for: one pair per row and 128 entries
     *ctas = full < limit ? full : limit;
@@ -317,6 +324,7 @@ void lmhead_rows_plan(int M, int N, int num_sms, int* ctas, int* tile_h, int* m_
     const int n_tiles = (N + *tile_h - 1) / *tile_h;
     if (n_tiles < *ctas) *ctas = n_tiles;
     *m_pad = (M + 15) / 16 * 16;
+    return M <= 32 || (N > 40 * kTileV && (rounds == 1 || *tile_h >= 88));
 }
 
 cudaError_t launch_lmhead_rows(const CUtensorMap& tmX, const CUtensorMap& tmW, const int* targets, void* logits,

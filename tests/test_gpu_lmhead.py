@@ -70,8 +70,10 @@ def test_edge_shapes(M, N, K):
 
 # At most 64 rows: the kernel that streams W past swapped operands.  Group edges of the rows (16, 32), equal tile
 # heights below 128 (18952 = 148 * 128 + 8 entries: two rounds), a lone entry beyond a tile, a ragged k block, and
-# the first row count that goes to the other kernel.
-FEW_ROWS = [(1, 136, 8), (16, 18952, 64), (17, 2056, 72), (32, 50304, 128), (33, 1000, 200), (64, 18944, 64), (65, 264, 64)]
+# the first row count that goes to the other kernel.  From 33 rows on also by N: up to 5120 entries, and where tiles are
+# lower than 88 in several rounds, the other kernel.
+FEW_ROWS = [(1, 136, 8), (16, 18952, 64), (17, 2056, 72), (32, 50304, 128), (33, 1000, 200), (64, 18944, 64), (65, 264, 64),
+            (33, 5120, 72), (33, 5128, 72), (64, 18952, 64), (48, 24000, 64), (64, 50304, 128)]
 
 
 @pytest.mark.parametrize("M,N,K", FEW_ROWS)
