@@ -419,13 +419,16 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     if (int rc = get_bf16_map(dQ, s, sdq, strided, &tmdQ, &odq)) return rc;
     if (int rc = get_bf16_map(dK, s, sdk, strided, &tmdK, &odk)) return rc;
     if (int rc = get_bf16_map(dV, s, sdv, strided, &tmdV, &odv)) return rc;
+    if (s.D == 128) {
+        if (int rc = get_bf16_map(Q, s, sq, strided, &tmQs, &oq, kKeyStep)) return rc;
+        if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdOs, &odo, kKeyStep)) return rc;
+    }
+    // (every map is there before the first launch: a call that fails has launched nothing)
     const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12);
     cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders | (odq << 16), LSE, Delta, s, st.num_sms,
                                    st.dev_status, cs);
     if (e != cudaSuccess) return fail_cuda(e);
     if (s.D == 128) {
-        if (int rc = get_bf16_map(Q, s, sq, strided, &tmQs, &oq, kKeyStep)) return rc;
-        if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdOs, &odo, kKeyStep)) return rc;
         e = launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders | (odk << 16) | (odv << 20), LSE, Delta, s,
                              st.num_sms, st.dev_status, cs);
     } else {
@@ -461,11 +464,13 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
     const bool direct = T <= kBlockK && whole;
     if (whole && !direct && two_kernels_pay(BH, T, D, causal != 0, st->num_sms))
         return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv, *st, cs);
-    if ((steps & NOVA_ATTN_BWD_STEP_ZERO) && !direct) {
-        e = launch_zero(acc, need, st->num_sms, cs);
+    auto clear = [&]() {
+        return (steps & NOVA_ATTN_BWD_STEP_ZERO) && !direct ? launch_zero(acc, need, st->num_sms, cs) : cudaSuccess;
+    };
+    if (!(steps & NOVA_ATTN_BWD_STEP_MAIN)) {
+        e = clear();
         if (e != cudaSuccess) return fail_cuda(e);
-    }
-    if (steps & NOVA_ATTN_BWD_STEP_MAIN) {
+    } else {
         CUtensorMap tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV;
         uint32_t oq, ok, ov, odo, odk, odv, odq = 0;
         const bool strided = !(merges(s, sq) && merges(s, sk) && merges(s, sv) && merges(s, sdo) && merges(s, sdk) &&
@@ -482,7 +487,10 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
         if (int rc = get_bf16_map(dK, s, sdk, strided, &tmdK, &odk)) return rc;
         if (int rc = get_bf16_map(dV, s, sdv, strided, &tmdV, &odv)) return rc;
         const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12) | (odk << 16) | (odv << 20) | (odq << 24);
-        e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, direct ? DqMode::kDirect : DqMode::kAccumulate, LSE, Delta, static_cast<__nv_bfloat16*>(dK),
+        e = clear();  // every map is there: a call that fails has launched nothing
+        if (e != cudaSuccess) return fail_cuda(e);
+        e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders,
+                            direct ? DqMode::kDirect : DqMode::kAccumulate, LSE, Delta, static_cast<__nv_bfloat16*>(dK),
                             static_cast<__nv_bfloat16*>(dV), sdk, sdv, s, st->num_sms, st->dev_status, cs);
         if (e != cudaSuccess) return fail_cuda(e);
     }
