@@ -76,19 +76,20 @@ struct BwdCfg {
     static constexpr bool kBulkdQ = (D == 64);
     static constexpr int kStageBytes = 2 * kHalfTileBytes;
     // At D=64 the row terms enter S^T and dP^T through the tensor core: one more instruction per product multiplies a
-    // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale or -Delta, each as three bf16 numbers
-    // that add up to it exactly to 24 bits.  The two terms lie in tiles of their own, so that a Delta that is not finite
-    // does not reach S (0 * inf).  The compute warps then read no rows from shared memory (512 broadcasts of
+    // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale and -Delta, each as three bf16 numbers
+    // that add up to it exactly to 24 bits.  A Delta that is not finite must not reach S (0 * inf is NaN): it
+    // enters as kMostLse in a column of its own, times kMostLse for dP^T and times 0 for S.  The compute warps then read no rows from shared memory (512 broadcasts of
     // 16 bytes a tile, some 600 clocks of its one port, which the operands of the products need as well) and have an
     // fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at B=32, 337 -> 321 us at
     // B=1, T=8192, 214 -> 182 us at B=4, T=2048 without the mask.  D=128 has no shared memory left for the tiles.
     static constexpr bool kFold = (D == 64);
-    // An operand of 128 rows x 16 columns is two planes of 128 x 8: in order -LSE/scale (two stages), -Delta (two
-    // stages), ones in columns 0-2, zeros; the last is the second plane of all the others.
-    static constexpr int kExtPlane = 128 * 8 * 2;
-    static constexpr int kExtOnes = 4, kExtZeros = 5, kExtPlanes = 6;
-    static constexpr int kOffExt = kOffRow;                           // kFold: kExtPlanes planes
-    static constexpr int kOffStage = kOffRow + (kFold ? kExtPlanes * kExtPlane : 2 * 2 * 128 * 4);
+    // Each operand is 128 rows x 16 columns, unswizzled: core matrices of 8 rows x 8 columns (128 bytes), the two of 8 rows
+    // adjacent.  Queries: -LSE/scale in columns 0, 2, 4, -Delta in 1, 3, 5, the sign of a Delta that is not finite in 8.
+    static constexpr int kExtCore = 128;
+    static constexpr int kExtTile = 16 * 2 * kExtCore;
+    static constexpr int kExtConstS = 2 * kExtTile, kExtConstdP = 3 * kExtTile, kExtBytes = 4 * kExtTile;
+    static constexpr int kOffExt = kOffRow;                           // kFold: two stages, then the constants
+    static constexpr int kOffStage = kOffRow + (kFold ? kExtBytes : 2 * 2 * 128 * 4);
     static constexpr int kOffBar = kOffStage + kStageBytes;
     // At D=128 the tiles fill the 227 KB a CTA can have to within 512 bytes, so there is no room for
     // the padding that would let the kernel align its window itself: the kernel checks that the window
@@ -227,19 +228,18 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     // The whole warp runs this role in uniform control flow; one elected lane issues.
     const bool el = elect_one();
 
-    // The row terms of tile gq: unswizzled, 8 x 16-byte core matrices 128 bytes apart along M and N; along K the second one
-    // lies in the plane of zeros.  From one plane to the next the address grows by what that distance shrinks by.
-    const uint32_t ext_hi = umma_desc_hi_plain(128);
-    const uint32_t ext_0 = umma_desc_lo(smem_u32(smem + Cfg::kOffExt), Cfg::kExtZeros * Cfg::kExtPlane);
-    constexpr uint32_t kExtStep = (Cfg::kExtPlane >> 4) - ((Cfg::kExtPlane >> 4) << 16);
-    const uint32_t ext_ones = ext_0 + Cfg::kExtOnes * kExtStep;
-    (void)ext_hi, (void)ext_ones;
+    // The row terms of tile gq.
+    const uint32_t ext_hi = umma_desc_hi_plain(2 * Cfg::kExtCore);
+    const uint32_t ext_b = umma_desc_lo(smem_u32(smem + Cfg::kOffExt), Cfg::kExtCore);
+    constexpr uint32_t kExtStep = Cfg::kExtTile >> 4;
+    (void)ext_hi, (void)ext_b;
 
     auto issue_st = [&](int gq, uint32_t kd) {  // S^T = K Q^T: K tile `kd`, query tile in Q stage gq % kQStages
         const uint32_t b = q_k0 + (gq % Cfg::kQStages) * kQStageStep;
         if (el) {
             if (Cfg::kFold)
-                umma_ss(t_s, umma_desc_join(ext_ones, ext_hi), umma_desc_join(ext_0 + (gq & 1) * kExtStep, ext_hi), kIdescT, 0u);
+                umma_ss(t_s, umma_desc_join(ext_b + (Cfg::kExtConstS >> 4), ext_hi),
+                        umma_desc_join(ext_b + (gq & 1) * kExtStep, ext_hi), kIdescT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
                 const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
@@ -253,8 +253,8 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
         const uint32_t b = do_k[gq % Cfg::kdOStages];
         if (el) {
             if (Cfg::kFold)
-                umma_ss(t_dp, umma_desc_join(ext_ones, ext_hi), umma_desc_join(ext_0 + (2 + (gq & 1)) * kExtStep, ext_hi),
-                        kIdescT, 0u);
+                umma_ss(t_dp, umma_desc_join(ext_b + (Cfg::kExtConstdP >> 4), ext_hi),
+                        umma_desc_join(ext_b + (gq & 1) * kExtStep, ext_hi), kIdescT, 0u);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
                 const uint32_t off = ((k / 4) * kHalfTileBytes + (k % 4) * 32) >> 4;
@@ -420,46 +420,65 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
     }
 }
 
-// Three bf16 numbers that add up to v (to 24 bits), packed as columns 0-2 of a row of 8; an infinite or NaN v is itself.
-__device__ __forceinline__ uint4 split_bf16x3(float v) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    const float r = isinf(v) ? 0.f : v - __bfloat162float(h);
-    const __nv_bfloat16 m = __float2bfloat16_rn(r);
-    const __nv_bfloat16 l = __float2bfloat16_rn(r - __bfloat162float(m));
-    return make_uint4(__bfloat16_as_ushort(h) | (static_cast<uint32_t>(__bfloat16_as_ushort(m)) << 16),
-                      __bfloat16_as_ushort(l), 0u, 0u);
+// Three bf16 numbers each that add up to l and d (to 24 bits): columns 0, 2, 4 and 1, 3, 5 of a row of 8.
+__device__ __forceinline__ uint4 split_bf16x3(float l, float d) {
+    uint32_t w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        w[i] = pack_bf16x2(l, d);
+        l -= __uint_as_float(w[i] << 16);
+        d -= __uint_as_float(w[i] & 0xffff0000u);
+    }
+    return make_uint4(w[0], w[1], w[2], 0u);
 }
 
-// Row loader where the row terms go through the tensor core (kFold): one row of 8 columns per query in the plane of
-// -LSE/scale and in that of -Delta.  LSE/scale is held below kMostLse, which keeps what an infinite LSE means (P = 0 for
-// +inf, P = inf for -inf) without an infinity that would meet another in the sum; queries past the end of the sequence get
-// the same value, so that their P is 0.
+// Row loader where the row terms go through the tensor core (kFold): one row of 8 columns per query.  LSE/scale is held below
+// kMostLse, which keeps what an infinite LSE means (P = 0 for +inf, P = inf for -inf) without an infinity that would meet
+// another in the sum; queries past the end of the sequence get the same value, so that their P is 0.
 __device__ __forceinline__ void bwd_rows_folded(BwdBars* bars, uint8_t* ext, const float* __restrict__ LSE,
                                                 const float* __restrict__ Delta, int T, float inv_scale,
                                                 const WorkList& wl, int tid64) {
+    using Cfg = BwdCfg<64>;
     volatile int* abort_flag = &bars->abort_flag;
     int g = 0;
+    uint32_t dirty = 0;  // of the last two tiles: Deltas of this warp that are not finite (to be cleared by the next two)
     for (WorkCursor cur; !wl.done(cur); wl.advance(cur)) {
         int kt, bh, i0, n_it;
         if (!wl.get(cur, &kt, &bh, &i0, &n_it)) continue;
         const size_t row_base = static_cast<size_t>(bh) * T;
         for (int it = 0; it < n_it; ++it, ++g) {
             const int b = g & 1;
-            uint4 vl[2], vd[2];
+            float l[2], d[2], odd[2] = {0.f, 0.f};
+            bool rare = false;
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
                 const int q = (i0 + it) * kBlockQ + tid64 + 64 * x;
-                float l = (q < T) ? -LSE[row_base + q] * inv_scale : -kMostLse;
-                if (fabsf(l) > kMostLse) l = copysignf(kMostLse, l);  // (a NaN stays)
-                vl[x] = split_bf16x3(l);
-                vd[x] = split_bf16x3((q < T) ? -Delta[row_base + q] : 0.f);
+                l[x] = (q < T) ? -LSE[row_base + q] * inv_scale : -kMostLse;
+                d[x] = (q < T) ? -Delta[row_base + q] : 0.f;
+                rare = rare || !(fabsf(l[x]) <= kMostLse) || !(fabsf(d[x]) <= kMostLse);
             }
-            if (!mbar_wait(&bars->row_empty[b], ((g >> 1) & 1) ^ 1, abort_flag)) return;
+            const bool any_odd = __any_sync(0xffffffffu, rare);
+            if (any_odd) {
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                uint8_t* row = ext + b * BwdCfg<64>::kExtPlane + (tid64 + 64 * x) * 16;
-                *reinterpret_cast<uint4*>(row) = vl[x];
-                *reinterpret_cast<uint4*>(row + 2 * BwdCfg<64>::kExtPlane) = vd[x];
+                for (int x = 0; x < 2; ++x) {
+                    if (fabsf(l[x]) > kMostLse) l[x] = copysignf(kMostLse, l[x]);  // (a NaN stays)
+                    if (!(fabsf(d[x]) <= kMostLse)) {  // dP^T becomes infinite, for a NaN as well
+                        odd[x] = copysignf(kMostLse, d[x]);
+                        d[x] = 0.f;
+                    }
+                }
+            }
+            const uint4 v[2] = {split_bf16x3(l[0], d[0]), split_bf16x3(l[1], d[1])};
+            if (!mbar_wait(&bars->row_empty[b], ((g >> 1) & 1) ^ 1, abort_flag)) return;
+            uint8_t* row = ext + b * Cfg::kExtTile + (tid64 >> 3) * 2 * Cfg::kExtCore + (tid64 & 7) * 16;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) *reinterpret_cast<uint4*>(row + 16 * Cfg::kExtCore * x) = v[x];
+            if (any_odd || dirty != 0) {
+#pragma unroll
+                for (int x = 0; x < 2; ++x)
+                    *reinterpret_cast<uint4*>(row + Cfg::kExtCore + 16 * Cfg::kExtCore * x) =
+                        make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(odd[x])), 0u, 0u, 0u);
+                dirty = ((dirty << 1) | (any_odd ? 1u : 0u)) & 3u;
             }
             fence_proxy_async_smem();
             __syncwarp();
@@ -1079,10 +1098,16 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         tma_prefetch_desc(&tmdV);
     }
     if constexpr (Cfg::kFold) {
-        // the planes of constants (the stages are written whole)
-        for (int i = threadIdx.x; i < 2 * Cfg::kExtPlane / 16; i += Cfg::kThreads)
-            *reinterpret_cast<uint4*>(smem + Cfg::kOffExt + Cfg::kExtOnes * Cfg::kExtPlane + 16 * i) =
-                i < Cfg::kExtPlane / 16 ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+        // zeros in the stages, then the constants
+        for (int i = threadIdx.x; i < Cfg::kExtBytes / 16; i += Cfg::kThreads) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            const bool first_half = ((i >> 3) & 1) == 0;  // core matrix of columns 0-7
+            const int tile = i / (Cfg::kExtTile / 16);
+            if (tile == 2 && first_half) v = make_uint4(0x00003f80u, 0x00003f80u, 0x00003f80u, 0u);
+            if (tile == 3 && first_half) v = make_uint4(0x3f800000u, 0x3f800000u, 0x3f800000u, 0u);
+            if (tile == 3 && !first_half) v.x = __bfloat16_as_ushort(__float2bfloat16_rn(kMostLse));
+            *reinterpret_cast<uint4*>(smem + Cfg::kOffExt + 16 * i) = v;
+        }
         fence_proxy_async_smem();
     }
     if (warp == 1) {
