@@ -78,9 +78,9 @@ struct BwdCfg {
     // At D=64 the row terms enter S^T and dP^T through the tensor core: one more instruction per product multiplies a
     // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale and -Delta, each as three bf16 numbers
     // that add up to it exactly to 24 bits.  A Delta that is not finite must not reach S (0 * inf is NaN): it
-    // enters as kMostLse in a column of its own, times kMostLse for dP^T and times 0 for S.  The compute warps then read no rows from shared memory (512 broadcasts of
-    // 16 bytes a tile, some 600 clocks of its one port, which the operands of the products need as well) and have an
-    // fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at B=32, 337 -> 321 us at
+    // enters as kMostLse in a column of its own, times kMostLse for dP^T and times 0 for S.  The compute warps then read no
+    // rows from shared memory (512 broadcasts of 16 bytes a tile, some 600 clocks of its one port, which the operands of the
+    // products need as well) and have an fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at B=32, 337 -> 321 us at
     // B=1, T=8192, 214 -> 182 us at B=4, T=2048 without the mask.  D=128 has no shared memory left for the tiles.
     static constexpr bool kFold = (D == 64);
     // Each operand is 128 rows x 16 columns, unswizzled: core matrices of 8 rows x 8 columns (128 bytes), the two of 8 rows
@@ -461,7 +461,8 @@ __device__ __forceinline__ void bwd_rows_folded(BwdBars* bars, uint8_t* ext, con
             if (any_odd) {
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    if (fabsf(l[x]) > kMostLse) l[x] = copysignf(kMostLse, l[x]);  // (a NaN stays)
+                    // (a NaN, which would reach dP^T of keys behind the query, becomes P = inf where the query is kept)
+                    if (!(fabsf(l[x]) <= kMostLse)) l[x] = l[x] < 0.f ? -kMostLse : kMostLse;
                     if (!(fabsf(d[x]) <= kMostLse)) {  // dP^T becomes infinite, for a NaN as well
                         odd[x] = copysignf(kMostLse, d[x]);
                         d[x] = 0.f;
