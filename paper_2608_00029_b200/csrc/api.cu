@@ -434,8 +434,7 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     } else {
         // the fused kernel without its dQ product (the accumulator map is never used: any map will do)
         e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmQ, tmdK, tmdV, strided, orders | (odk << 16) | (odv << 20), DqMode::kNone,
-                            LSE, Delta, static_cast<__nv_bfloat16*>(dK), static_cast<__nv_bfloat16*>(dV), sdk, sdv, s,
-                            st.num_sms, st.dev_status, cs);
+                            LSE, Delta, s, st.num_sms, st.dev_status, cs);
     }
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
@@ -490,8 +489,8 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
         e = clear();  // every map is there: a call that fails has launched nothing
         if (e != cudaSuccess) return fail_cuda(e);
         e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders,
-                            direct ? DqMode::kDirect : DqMode::kAccumulate, LSE, Delta, static_cast<__nv_bfloat16*>(dK),
-                            static_cast<__nv_bfloat16*>(dV), sdk, sdv, s, st->num_sms, st->dev_status, cs);
+                            direct ? DqMode::kDirect : DqMode::kAccumulate, LSE, Delta, s, st->num_sms,
+                            st->dev_status, cs);
         if (e != cudaSuccess) return fail_cuda(e);
     }
     if ((steps & NOVA_ATTN_BWD_STEP_CONVERT) && !direct) {
@@ -541,8 +540,7 @@ int nova_attn_bwd_deterministic(const void* Q, const void* K, const void* V, con
     if (int rc = get_tensor_map(dK, D, T, BH, &tmdK)) return rc;
     if (int rc = get_tensor_map(dV, D, T, BH, &tmdV)) return rc;
     const cudaError_t e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmdQ, tmdK, tmdV, false, 0u, DqMode::kDirect, LSE, Delta,
-                                          static_cast<__nv_bfloat16*>(dK), static_cast<__nv_bfloat16*>(dV), c, c, s,
-                                          st->num_sms, st->dev_status, cs);
+                                          s, st->num_sms, st->dev_status, cs);
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 

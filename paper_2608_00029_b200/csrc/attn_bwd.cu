@@ -288,7 +288,7 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
         v_k = umma_desc_lo(smem_u32(smem + Cfg::kOffV + ks * Cfg::kTileBytes), 16);
         ok = mbar_wait(&bars->kv_full[ks], (w / Cfg::kKVStages) & 1, abort_flag);
         if (ok) ok = mbar_wait(&bars->q_full[g % Cfg::kQStages], (g / Cfg::kQStages) & 1, abort_flag);
-        if (ok && Cfg::kdQAliased && g > 0 && !wl.no_dq()) ok = mbar_wait(&bars->dq_free, (g - 1) & 1, abort_flag);
+        if (ok && Cfg::kdQAliased && g > 0) ok = mbar_wait(&bars->dq_free, (g - 1) & 1, abort_flag);
         if (ok) ok = mbar_wait(&bars->do_full[g % Cfg::kdOStages], (g / Cfg::kdOStages) & 1, abort_flag);
         // (queued already: its row terms may have been read, and their buffer filled again, by now)
         if (ok && Cfg::kFold && !first_queued) ok = mbar_wait(&bars->row_full[g & 1], (g >> 1) & 1, abort_flag);
@@ -343,13 +343,11 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
                 // dQ_i = dS K_j first, all D columns per instruction (the dP^T columns it lands in were read by the
                 // compute warps before they arrived on ds_ready), then dK += dS^T Q_i with dS^T from shared memory.
                 if (el) {
-                    if (!wl.no_dq()) {
 #pragma unroll
-                        for (int k = 0; k < kBlockK / 16; ++k)
-                            umma_ss(tmem_base + Cfg::kColdQ, umma_desc_join(ds_m + k * 128, hi),
-                                    umma_desc_join(k_m + k * 128, hi), kIdescdQWide, k > 0 ? 1u : 0u);
-                        tc_commit(&bars->dq_full);
-                    }
+                    for (int k = 0; k < kBlockK / 16; ++k)
+                        umma_ss(tmem_base + Cfg::kColdQ, umma_desc_join(ds_m + k * 128, hi),
+                                umma_desc_join(k_m + k * 128, hi), kIdescdQWide, k > 0 ? 1u : 0u);
+                    tc_commit(&bars->dq_full);
                     const uint32_t b = q_m0 + (g % Cfg::kQStages) * kQStageStep;
 #pragma unroll
                     for (int k = 0; k < kBlockQ / 16; ++k) {
@@ -393,7 +391,7 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
             __syncwarp();
             }
             if (more || cross) {
-                if (Cfg::kdQAliased && !wl.no_dq()) {  // dQ sits in the dP^T region until the dQ warps have read it
+                if (Cfg::kdQAliased) {  // dQ sits in the dP^T region until the dQ warps have read it
                     ok = mbar_wait(&bars->dq_free, g & 1, abort_flag);
                     if (!ok) break;
                 }
@@ -983,7 +981,7 @@ __device__ __forceinline__ void bwd_dq_tma_wide(uint8_t* smem, BwdBars* bars, ui
         return __all_sync(0xffffffffu, fine);  // also brings the warp together before its next TMEM instruction
     };
 
-    for (WorkCursor cur; !wl.done(cur) && ok && !wl.no_dq(); wl.advance(cur)) {
+    for (WorkCursor cur; !wl.done(cur) && ok; wl.advance(cur)) {
         int kt, bh, i0, n_it;
         if (!wl.get(cur, &kt, &bh, &i0, &n_it)) continue;
         for (int it = 0; it < n_it && ok; ++it, ++g) {
@@ -1044,8 +1042,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                 const __grid_constant__ CUtensorMap tmAcc, const __grid_constant__ CUtensorMap tmdK,
                 const __grid_constant__ CUtensorMap tmdV, const float* __restrict__ LSE,
-                const float* __restrict__ Delta, __nv_bfloat16* __restrict__ dK,
-                __nv_bfloat16* __restrict__ dV, const TensorStrides sdk, const TensorStrides sdv, int T,
+                const float* __restrict__ Delta, int T,
                 const __grid_constant__ WorkArgs wa, float scale, int* __restrict__ dev_status) {
     using Cfg = BwdCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -1163,8 +1160,7 @@ template <int D, bool kCausal>
 cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                        const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
                        const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,
-                       const float* Delta, __nv_bfloat16* dK, __nv_bfloat16* dV, const TensorStrides& sdk,
-                       const TensorStrides& sdv, const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream) {
+                       const float* Delta, const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream) {
     static_assert(kBlockK == 128 && kBlockQ == 128, "the work plan counts 128-row tiles");
     const int BH = s.B * s.H;
     int n_tiles = 0, n_ctas = 0;
@@ -1173,7 +1169,7 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     const WorkArgs wa{BH, n_tiles, s.H, orders, dq == DqMode::kNone ? 1 : 0, plan};
     auto go = [&](auto kernel) {
         return launch_overlapped(kernel, grid, dim3(BwdCfg<D>::kThreads), BwdCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO,
-                                 tmAcc, tmdK, tmdV, LSE, Delta, dK, dV, sdk, sdv, s.T, wa, s.scale, dev_status);
+                                 tmAcc, tmdK, tmdV, LSE, Delta, s.T, wa, s.scale, dev_status);
     };
     if (dq == DqMode::kDirect)
         return strided ? go(attn_bwd_kernel<D, kCausal, true, true>) : go(attn_bwd_kernel<D, kCausal, false, true>);
@@ -1204,15 +1200,13 @@ cudaError_t configure_attn_bwd() {
 cudaError_t launch_attn_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                             const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
                             const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,
-                            const float* Delta, __nv_bfloat16* dK, __nv_bfloat16* dV, const TensorStrides& sdk,
-                            const TensorStrides& sdv, const AttnShape& s, int num_sms, int* dev_status,
-                            cudaStream_t stream) {
-    if (s.D == 64) {
-        return s.causal ? launch_one<64, true>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream)
-                        : launch_one<64, false>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream);
-    }
-    return s.causal ? launch_one<128, true>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream)
-                    : launch_one<128, false>(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, dK, dV, sdk, sdv, s, num_sms, dev_status, stream);
+                            const float* Delta, const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream) {
+    if (s.D == 128 && dq == DqMode::kNone) return cudaErrorNotSupported;  // that half has a kernel of its own (attn_dkdv.cu)
+    auto go = [&](auto launch) {
+        return launch(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, s, num_sms, dev_status, stream);
+    };
+    if (s.D == 64) return s.causal ? go(launch_one<64, true>) : go(launch_one<64, false>);
+    return s.causal ? go(launch_one<128, true>) : go(launch_one<128, false>);
 }
 
 }  // namespace nova

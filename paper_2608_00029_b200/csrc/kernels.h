@@ -119,21 +119,19 @@ long long steps_until_done(long long items, int num_sms, F&& steps) {
 // What the backward main kernel does with its partial tiles of dQ.
 enum class DqMode {
     kAccumulate,  // adds them, unscaled, into the fp32 accumulator
-    kNone,        // nothing: dK and dV only (the dK/dV half of the two-kernel backward)
+    kNone,        // nothing: dK and dV only (the dK/dV half of the two-kernel backward; D = 64)
     kDirect,      // T <= kBlockK, a head has one key tile: its dQ tile is complete and is written scaled, as bf16
 };
 
 // Backward main kernel: adds unscaled dQ partial tiles into the fp32 accumulator [B,H,T,D] (zero on
 // entry) described by `tmAcc` (fp32 [D, T, B*H], box [32, 128, 1], 128-byte swizzle) and writes dK and dV
-// (`tmdK`, `tmdV`: the bf16 maps of the outputs, used for TMA stores at D=64; at D=128 the rows go out
-// with plain stores through `dK`, `dV` and their strides).  `strided`, `orders`: as in the forward, for
+// through TMA stores (`tmdK`, `tmdV`: the bf16 maps of the outputs).  `strided`, `orders`: as in the forward, for
 // Q, K, V, dO, dK, dV (and dQ).  `dq`: see above; `tmAcc` is the bf16 map of dQ with kDirect and never used with
 // kNone.  Persistent: launches at most `num_sms` CTAs.
 cudaError_t launch_attn_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                             const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
-                            const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE, const float* Delta,
-                            __nv_bfloat16* dK, __nv_bfloat16* dV, const TensorStrides& sdk, const TensorStrides& sdv,
-                            const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream);
+                            const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,
+                            const float* Delta, const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream);
 cudaError_t configure_attn_bwd();
 
 // Loss head (lmhead.cu): `tmX` is the 2-D map of X [K, M] with box [64, 128], `tmW` that of W [K, N] with box

@@ -179,12 +179,6 @@ struct WorkRing {
         if (lane == 0) mbar_arrive(&empty[w & 1]);
         return it;
     }
-    __device__ __forceinline__ int take_single(int w, volatile int* abort_flag, long long limit) {  // one thread
-        if (!mbar_wait(&full[w & 1], (w >> 1) & 1, abort_flag, limit)) return -2;
-        const int it = *reinterpret_cast<volatile int*>(&item[w & 1]);
-        mbar_arrive(&empty[w & 1]);
-        return it;
-    }
     // Has the w-th item been published yet?  Non-blocking; the same answer in every lane of a converged warp.
     __device__ __forceinline__ bool published(int w) {
         return __all_sync(0xffffffffu, mbar_test(&full[w & 1], (w >> 1) & 1));

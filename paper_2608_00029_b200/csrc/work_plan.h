@@ -30,7 +30,7 @@ struct WorkCursor {
 struct WorkArgs {
     int BH, n_tiles, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, dO, dK, dV, dQ tensor maps, four bits each
-    int no_dq;        // dK/dV half of the two-kernel backward: no dQ product, no accumulator traffic
+    int no_dq;        // dK/dV half of the two-kernel backward at D=64: no dQ product, no accumulator traffic
     WorkPlan plan;
 };
 struct WorkList {
