@@ -24,6 +24,7 @@ data: weak scaling, no data-path collective.  `--impl reference` times the CPU o
 from __future__ import annotations
 
 import argparse
+import ctypes
 import functools
 import json
 import os
@@ -216,6 +217,22 @@ def step(na, cfg, s):
     na.nova_attn_fwd(s.q, s.k, s.v, s.o, s.lse, cfg.scale, cfg.causal)
     na.nova_attn_bwd_preprocess(s.o, s.do, s.delta)
     na.nova_attn_bwd(s.q, s.k, s.v, s.o, s.do, s.lse, s.delta, s.dq, s.dk, s.dv, cfg.scale, cfg.causal, s.ws)
+
+
+def kernel_count(fn, dev):
+    """Kernels that `fn` launches: the nodes of a CUDA graph that it is captured into (the calls launch nothing else)."""
+    side = torch.cuda.Stream(device=dev)
+    with torch.cuda.stream(side):
+        fn()
+    side.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=side, capture_error_mode="thread_local"):
+        fn()
+    n = ctypes.c_size_t()
+    rc = ctypes.CDLL("libcudart.so.12").cudaGraphGetNodes(ctypes.c_void_p(g.raw_cuda_graph()), None, ctypes.byref(n))
+    if rc != 0:
+        raise RuntimeError(f"cudaGraphGetNodes returned {rc}")
+    return n.value
 
 
 def run_profile(args, na, cfg, dev):
@@ -533,11 +550,18 @@ def run_ours(args):
     stream = torch.cuda.current_stream()
     flops_step = cfg.fwd_flops + cfg.bwd_flops
 
+    # Which route the backward takes for this shape: one kernel (a single key tile), the dQ and the dK/dV kernel, or clear,
+    # main and conversion (see nova_attn_bwd).
+    launches_step = kernel_count(functools.partial(step, na, cfg, probe), dev)
+    launches_bwd = kernel_count(functools.partial(na.nova_attn_bwd, probe.q, probe.k, probe.v, probe.o, probe.do, probe.lse,
+                                                  probe.delta, probe.dq, probe.dk, probe.dv, cfg.scale, cfg.causal,
+                                                  probe.ws), dev)
+
     sampler = ClockSampler(local_rank)
     sampler.start()
 
     # ---- device-resident timing
-    # One step's five launches (the same C-ABI calls) are recorded once per buffer set into a CUDA graph
+    # One step's launches (the same C-ABI calls) are recorded once per buffer set into a CUDA graph
     # and replayed, as a training loop that has captured its step would run them; --launch eager issues
     # the calls one by one instead.
     run_step = [functools.partial(step, na, cfg, s) for s in sets]
@@ -602,15 +626,20 @@ def run_ours(args):
     #     timed steps (no host in between): `kernel_ms`, the figure the roofline uses;
     # (2) the calls issued one by one with an event on either side: `kernel_ms_eager`.  The host needs longer to
     #     issue a launch and two event records than these kernels run, so this figure contains idle time.
-    names = ["fwd", "bwd_preprocess", "bwd_zero", "bwd_main", "bwd_convert"]
+    # The steps of the backward are separate calls only where nova_attn_bwd itself takes them; its other routes are timed
+    # whole.
+    by_steps = launches_bwd == 3
+    names = ["fwd", "bwd_preprocess"] + (["bwd_zero", "bwd_main", "bwd_convert"] if by_steps else ["bwd_main"])
 
     def one_kernel(name, s):
         if name == "fwd":
             na.nova_attn_fwd(s.q, s.k, s.v, s.o, s.lse, cfg.scale, cfg.causal)
         elif name == "bwd_preprocess":
             na.nova_attn_bwd_preprocess(s.o, s.do, s.delta)
-        elif name == "bwd":  # the whole backward as the three calls make it: preprocess + clear + main + convert
+        elif name == "bwd":  # the whole backward as a caller makes it
             na.nova_attn_bwd_preprocess(s.o, s.do, s.delta)
+            na.nova_attn_bwd(s.q, s.k, s.v, s.o, s.do, s.lse, s.delta, s.dq, s.dk, s.dv, cfg.scale, cfg.causal, s.ws)
+        elif not by_steps:
             na.nova_attn_bwd(s.q, s.k, s.v, s.o, s.do, s.lse, s.delta, s.dq, s.dk, s.dv, cfg.scale, cfg.causal, s.ws)
         else:
             bit = {"bwd_zero": na.BWD_STEP_ZERO, "bwd_main": na.BWD_STEP_MAIN, "bwd_convert": na.BWD_STEP_CONVERT}[name]
@@ -675,7 +704,8 @@ def run_ours(args):
     fwd_tflops = cfg.fwd_flops / (fwd_seq_ms * 1e-3) / 1e12
     bwd_tflops = cfg.bwd_flops / (bwd_seq_ms * 1e-3) / 1e12
     roofline = {
-        "bound": "tensor", "kernel": "attn_bwd_kernel", "achieved": achieved, "peak": peak, "unit": UNIT,
+        "bound": "tensor", "kernel": "attn_dq_kernel + attn_dkdv_kernel" if launches_bwd == 2 else "attn_bwd_kernel",
+        "achieved": achieved, "peak": peak, "unit": UNIT,
         "frac": achieved / peak, "traffic": None, "traffic_source": None,
         "peak_source": f"{peak_src} bf16_tflops (burst)",
         "peak_sustained": peaks["bf16_tflops_sustained"],
@@ -684,7 +714,8 @@ def run_ours(args):
         "targets": {
             "fwd": {"what": "nova_attn_fwd", "ms": fwd_seq_ms, "tflops": fwd_tflops, "frac": fwd_tflops / peak,
                     "target": 0.50},
-            "bwd": {"what": "nova_attn_bwd_preprocess + nova_attn_bwd (clear, main, convert) in sequence",
+            "bwd": {"what": "nova_attn_bwd_preprocess + nova_attn_bwd "
+                            f"({'clear, main, convert' if by_steps else f'{launches_bwd} kernel(s)'}) in sequence",
                     "ms": bwd_seq_ms, "tflops": bwd_tflops, "frac": bwd_tflops / peak, "target": 0.35},
         },
         "preprocess_gbs": (4.0 * cfg.B * cfg.H * cfg.T * cfg.D + 4.0 * cfg.B * cfg.H * cfg.T)
@@ -697,7 +728,7 @@ def run_ours(args):
     # workload -> null.
     traffic_rel = os.path.join("profiles", f"attn_bwd_kernel_{base.name}.md")
     traffic_path = os.path.join(ROOT, traffic_rel)
-    if os.path.exists(traffic_path) and cfg.B == base.B:
+    if os.path.exists(traffic_path) and cfg.B == base.B and by_steps:
         try:
             with open(traffic_path) as f:
                 for line in f:
@@ -782,12 +813,12 @@ def run_ours(args):
                        "T": cfg.T, "D": cfg.D, "causal": True, "parallelism": f"dp{world} (batch split, no collective)",
                        "l2": f"rotating {n_sets} buffer sets of {probe.bytes() / 1e6:.0f} MB "
                              f"({n_sets * probe.bytes() / 1e6:.0f} MB > 126 MB L2)",
-                       "launch": (f"CUDA graph of one round over the {n_sets} buffer sets, replayed (5 kernels per step)"
-                                  if launch_mode == "graph" else "eager (5 launches per step)"),
+                       "launch": (f"CUDA graph of one round over the {n_sets} buffer sets, replayed ({launches_step} kernels per step)"
+                                  if launch_mode == "graph" else f"eager ({launches_step} launches per step)"),
                        "flops_per_step": flops_step, "frac_of_burst_peak": value / world / peaks["bf16_tflops"]},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "ms_per_step": e2e_ms, "steps": e2e_steps},
-            "gpu_launches": 5 * args.steps,
+            "gpu_launches": launches_step * args.steps,
             "clocks": clocks,
             "roofline": roofline,
             "cpu_baseline": cpu_baseline,

@@ -75,3 +75,13 @@ def test_device_arm_line(launch):
     assert 0 < e["value"] < d["value"]  # the copies are inside the timed region
     c = d["clocks"]
     assert c["sm_mhz"] > 0 and c["sm_max_mhz"] >= c["sm_mhz"] and isinstance(c["reasons"], list)
+
+
+@pytest.mark.gpu
+def test_device_arm_line_of_a_workload_without_an_accumulator():
+    """One key tile per head: three launches per step, and the backward is one kernel, timed as the step runs it."""
+    d = _run("--workload", "tiny", "--steps", "6", "--warmup", "3")
+    assert d["gpu_launches"] == 3 * 6 and "3 kernels per step" in d["config"]["launch"]
+    r = d["roofline"]
+    assert set(r["kernel_ms"]) == {"fwd", "bwd_preprocess", "bwd_main"} and r["kernel"] == "attn_bwd_kernel"
+    assert "1 kernel" in r["targets"]["bwd"]["what"] and r["traffic"] is None
