@@ -17,12 +17,21 @@ from paper_2608_00029_b200 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("name", ["tiny", "tiny_d128"])
+LIMITED = {
+    "tiny": W.CONFIGS["tiny"],
+    "tiny_d128": W.AttnConfig("tiny_d128", B=1, H=2, T=200, D=128, seed=5),
+    # pairs of query tiles, several items per SM: every one of them gives up
+    "pairs": W.AttnConfig("pairs", B=10, H=40, T=300, D=64, seed=6),
+    "pairs_d128": W.AttnConfig("pairs_d128", B=10, H=40, T=300, D=128, seed=7),
+}
+
+
+@pytest.mark.parametrize("name", sorted(LIMITED))
 def test_forward_wait_runs_out_and_the_library_recovers(name):
     import oracle
     from paper_2608_00029_b200 import nova_attn as na
     dev = torch.device("cuda:0")
-    cfg = W.CONFIGS["tiny"] if name == "tiny" else W.AttnConfig("tiny_d128", B=1, H=2, T=200, D=128, seed=5)
+    cfg = LIMITED[name]
     Q, K, V, dO = W.make_inputs(cfg)
     q, k, v = (x.to(dev) for x in (Q, K, V))
     o = torch.zeros_like(q)
