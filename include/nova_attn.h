@@ -128,7 +128,8 @@ int nova_attn_bwd(const void* Q, const void* K, const void* V, const void* O, co
  *   NOVA_ATTN_BWD_STEP_MAIN     the fused backward kernel: writes dK, dV, accumulates unscaled dQ
  *   NOVA_ATTN_BWD_STEP_CONVERT  dQ = bf16(scale * accumulator)
  * All three, in this order, give what nova_attn_bwd gives (which for some shapes uses kernels that write
- * dQ without the accumulator); any other combination leaves sequencing to the caller.  Arguments, validation and errors are those of nova_attn_bwd.
+ * dQ without the accumulator); any other combination leaves sequencing to the caller.  Arguments, validation
+ * and errors are those of nova_attn_bwd.
  */
 #define NOVA_ATTN_BWD_STEP_ZERO 1
 #define NOVA_ATTN_BWD_STEP_MAIN 2
@@ -177,9 +178,10 @@ int nova_attn_bwd_static_scratch(const void* Q, const void* K, const void* V, co
  * reduces dQ over keys, the other reduces dK and dV over queries; both rebuild the probability matrix from
  * the saved log-sum-exp).  Every output element is summed by one thread block in a fixed order, so dQ, dK
  * and dV are bitwise reproducible from run to run, and no workspace is needed.  The price: the score and
- * dP contractions are computed in both kernels (seven contractions for the five that are counted) and
- * the dQ kernel keeps one query tile in flight per SM, so it is slower than nova_attn_bwd; dK and dV are
- * bit-identical to nova_attn_bwd's, dQ differs from it in the last bits only (summation order).
+ * dP contractions are computed in both kernels (seven contractions for the five that are counted), which at
+ * D = 64 makes it slower than nova_attn_bwd.  Where nova_attn_bwd does without the accumulator (T <= 128, most
+ * shapes of D = 128 that fill the GPU) it launches these same kernels.  dK and dV are bit-identical to
+ * nova_attn_bwd's, dQ differs from it in the last bits at most (summation order).
  *   Q, K, V, dO : in,  bf16 [B,H,T,D]
  *   LSE, Delta  : in,  fp32 [B,H,T] from nova_attn_fwd / nova_attn_bwd_preprocess(_exact)
  *   dQ, dK, dV  : out, bf16 [B,H,T,D]

@@ -113,11 +113,13 @@ int get_tensor_map(const void* ptr, int D, long long T, long long BH, CUtensorMa
     if (st == 0) st = D;
     if (sh == 0) sh = T * D;
     const MapKey key{ptr, D, static_cast<int>(T), static_cast<int>(BH), dev, elem_bytes, box_rows, st, sh};
-    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull + (uint64_t(T) * 31 + uint64_t(BH) * 131 + D + box_rows) * 0xD6E8FEB86659FD93ull;
+    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull +
+                       (uint64_t(T) * 31 + uint64_t(BH) * 131 + D + box_rows) * 0xD6E8FEB86659FD93ull;
     std::lock_guard<std::mutex> lock(g_mutex);
     MapEntry& e = g_maps[(h >> 32) % kMapCache];
     if (e.valid && e.key.ptr == key.ptr && e.key.D == key.D && e.key.T == key.T && e.key.BH == key.BH &&
-        e.key.dev == key.dev && e.key.elem_bytes == key.elem_bytes && e.key.box_rows == box_rows && e.key.st == key.st && e.key.sh == key.sh) {
+        e.key.dev == key.dev && e.key.elem_bytes == key.elem_bytes && e.key.box_rows == box_rows && e.key.st == key.st &&
+        e.key.sh == key.sh) {
         *out = e.map;
         return NOVA_ATTN_OK;
     }
@@ -160,13 +162,14 @@ int get_tensor_map4(const void* ptr, const AttnShape& s, const TensorStrides& st
     int dev = 0;
     cudaGetDevice(&dev);
     const Map4Key key{ptr, s.D, s.T, s.H, s.B, dev, box_rows, st.b, st.h, st.t};
-    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull + 
+    const uint64_t h = (reinterpret_cast<uint64_t>(ptr) >> 8) * 0x9E3779B97F4A7C15ull +
                        (uint64_t(s.T) * 31 + uint64_t(s.B) * 131 + uint64_t(s.H) * 17 + uint64_t(st.t) * 7 + s.D + box_rows) *
                            0xD6E8FEB86659FD93ull;
     std::lock_guard<std::mutex> lock(g_mutex);
     Map4Entry& e = g_maps4[(h >> 32) % kMapCache];
     if (e.valid && e.key.ptr == key.ptr && e.key.D == key.D && e.key.T == key.T && e.key.H == key.H &&
-        e.key.B == key.B && e.key.dev == key.dev && e.key.box_rows == box_rows && e.key.sb == key.sb && e.key.sh == key.sh && e.key.st == key.st) {
+        e.key.B == key.B && e.key.dev == key.dev && e.key.box_rows == box_rows && e.key.sb == key.sb && e.key.sh == key.sh &&
+        e.key.st == key.st) {
         *out = e.map;
         *order = static_cast<uint32_t>(e.order);
         return NOVA_ATTN_OK;
@@ -375,7 +378,8 @@ int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, 
     if (int rc = get_tensor_map(dO, D, T, BH, &tmdO)) return rc;
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const cudaError_t e =
-        launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status, static_cast<cudaStream_t>(stream));
+        launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status,
+                          static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 

@@ -77,11 +77,13 @@ struct BwdCfg {
     static constexpr int kStageBytes = 2 * kHalfTileBytes;
     // At D=64 the row terms enter S^T and dP^T through the tensor core: one more instruction per product multiplies a
     // tile of constants (keys x 16) with a tile (queries x 16) that holds -LSE/scale and -Delta, each as three bf16 numbers
-    // that add up to it exactly to 24 bits.  A Delta that is not finite must not reach S (0 * inf is NaN): it
-    // enters as kMostLse in a column of its own, times kMostLse for dP^T and times 0 for S.  The compute warps then read no
-    // rows from shared memory (512 broadcasts of 16 bytes a tile, some 600 clocks of its one port, which the operands of the
-    // products need as well) and have an fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at B=32, 337 -> 321 us at
-    // B=1, T=8192, 214 -> 182 us at B=4, T=2048 without the mask.  D=128 has no shared memory left for the tiles.
+    // that add up to it exactly to 24 bits.  A Delta that is not finite must not reach S (0 * inf is NaN): it enters as
+    // kMostLse in a column of its own, times kMostLse for dP^T and times 0 for S.  The compute warps then read no rows from
+    // shared memory (512 broadcasts of 16 bytes a tile, some 600 clocks of its one port, which the operands of the products
+    // need as well) and have an fp32 addition less per element: 56.1 -> 55.0 us at B=8, H=12, T=1024, 210 -> 204.5 us at
+    // B=32, 337 -> 321 us at B=1, T=8192, 214 -> 182 us at B=4, T=2048 without the mask.  The row loader shares its schedulers
+    // with compute warps, so what it does per tile counts: a clamp per row was 0.3 %.  D=128 has no shared memory left
+    // for the tiles.
     static constexpr bool kFold = (D == 64);
     // Each operand is 128 rows x 16 columns, unswizzled: core matrices of 8 rows x 8 columns (128 bytes), the two of 8 rows
     // adjacent.  Queries: -LSE/scale in columns 0, 2, 4, -Delta in 1, 3, 5, the sign of a Delta that is not finite in 8.
@@ -661,8 +663,9 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
                         e23 = f32x2_add(e23, f32x2_pack(d4.z, d4.w));
                     }
                     float d0, d1, d2, d3;
-                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(pf[x + 4 * y + 0]), __uint_as_float(pf[x + 4 * y + 1])), e01), d0, d1);
-                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(pf[x + 4 * y + 2]), __uint_as_float(pf[x + 4 * y + 3])), e23), d2, d3);
+                    const uint32_t* p4 = pf + x + 4 * y;
+                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(p4[0]), __uint_as_float(p4[1])), e01), d0, d1);
+                    f32x2_unpack(f32x2_mul(f32x2_pack(__uint_as_float(p4[2]), __uint_as_float(p4[3])), e23), d2, d3);
                     dd[2 * y + 0] = pack_bf16x2(d0, d1);
                     dd[2 * y + 1] = pack_bf16x2(d2, d3);
                 }

@@ -50,7 +50,7 @@ struct FwdCfg {
     // Where O goes on its way out.  D=64: into the tile's Q buffer of the item, which has a second stage.  D=128: through
     // 16 KB per tile of its own, half of the columns at a time, so that the one Q stage can take the next item's Q as
     // soon as the last Q K^T has read it instead of after the item's O has left: 207 -> 188 us at B=16, H=32, T=1024, 66
-    // -> 59 us at B=4, H=32, T=1000, 33 -> 28 us at B=64, H=12, T=100. 
+    // -> 59 us at B=4, H=32, T=1000, 33 -> 28 us at B=64, H=12, T=100.
     // With an SM for every item no next Q tile is waiting, and O leaves sooner whole, through the Q buffers there too: 9.98 ->
     // 9.67 us at B=8, H=12, T=256 without the mask.
     static constexpr int kOffO = kOffV + kKVStages * kTileBytes;      // kOwn: [2 tiles]
@@ -480,7 +480,7 @@ __device__ __forceinline__ void fwd_softmax(uint8_t* smem, FwdBars* bars, uint32
                     ok = mbar_wait(&bars->pv_done[t], (cnt - 1) & 1, abort_flag, limit);
                     if (!ok) break;
                     tc_fence_after();
-                    #pragma unroll 1
+#pragma unroll 1
                     for (int cb = 0; cb < D; cb += 16) {
                         uint32_t o[16];
                         tmem_ld_x16(t_o + cb, o);

@@ -217,7 +217,8 @@ def nova_attn_bwd_strided(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, cau
 
 def nova_attn_bwd_deterministic(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: bool = True,
                                 stream=None) -> None:
-    """dQ, dK, dV by the two-kernel backward: bitwise reproducible, no workspace, slower than nova_attn_bwd."""
+    """dQ, dK, dV by the two-kernel backward: bitwise reproducible, no workspace.  At D = 64 and T > 128
+    slower than nova_attn_bwd, which elsewhere mostly takes the same kernels."""
     rc = _binding().bwd_deterministic(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_deterministic")
