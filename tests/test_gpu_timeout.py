@@ -46,6 +46,7 @@ def test_forward_wait_runs_out_and_the_library_recovers(name):
             na.nova_attn_poll_device_status()
         elapsed = time.perf_counter() - t0
         assert ei.value.status == na.ERR_TIMEOUT
+        del ei  # its traceback holds this frame, and the frame the tensors, until the next garbage collection
         assert elapsed < 1.0, f"the kernel took {elapsed:.2f} s to give up"
     finally:
         na.nova_attn_test_configure_waits(0, 0)
