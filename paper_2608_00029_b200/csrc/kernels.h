@@ -93,8 +93,12 @@ cudaError_t launch_attn_dkdv(const CUtensorMap& tmQ, const CUtensorMap& tmK, con
 cudaError_t configure_attn_dkdv();
 
 // Heads that the items of the kernels at D=128 are taken in together: enough items for two rounds of the SMs, and no more
-// than about 48 MB of Q, K, V and dO, so that what the tiles of a head share stays in L2.  All heads where everything
-// fits anyway (96 of the 126 MB): B=16, H=16, T=333 in two chunks lost 0.6 % to the uneven end of the first.
+// than about 48 MB of Q, K, V and dO, so that what the tiles of a head share stays in L2 (the forward re-reads K and V only,
+// half of that).  All heads in one list, chunks, in us, forward / exact Delta / deterministic backward: B=16, H=32, T=1024
+// 200, 174 / 173, 157 / 604, 547; B=4, H=32, T=2048 without the mask 280, 241 / 264, 240 / 908, 814.  Budgets of 24 and 96 MB
+// are within 3 % of it, most within 1 %, in either direction (the forward at the first shape 184 and 176).  All heads where
+// everything fits anyway (96 of the 126 MB): at 83 MB (B=16, H=16, T=333) 89.7 in one list, 92.2 us in two chunks, lost to
+// the uneven end of the first; at 100 to 128 MB the two differ by at most 3 %.
 inline int heads_per_chunk(int BH, int items_per_head, long long T, int D, int num_sms) {
     const long long per_head = T * D * 8;
     long long c = (48ll << 20) / per_head;
