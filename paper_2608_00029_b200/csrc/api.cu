@@ -78,6 +78,7 @@ int device_state(DeviceState** out) {
         if (e == cudaSuccess) e = configure_attn_bwd();
         if (e == cudaSuccess) e = configure_attn_dq();
         if (e == cudaSuccess) e = configure_attn_dkdv();
+        if (e == cudaSuccess) e = configure_attn_dkdv64();
         if (e == cudaSuccess) e = configure_lmhead();
         if (e == cudaSuccess) e = configure_lmhead_rows();
         if (e == cudaSuccess) e = cudaGetSymbolAddress(reinterpret_cast<void**>(&st.dev_status), g_dev_status);
@@ -423,23 +424,17 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     if (int rc = get_bf16_map(dQ, s, sdq, strided, &tmdQ, &odq)) return rc;
     if (int rc = get_bf16_map(dK, s, sdk, strided, &tmdK, &odk)) return rc;
     if (int rc = get_bf16_map(dV, s, sdv, strided, &tmdV, &odv)) return rc;
-    if (s.D == 128) {
-        if (int rc = get_bf16_map(Q, s, sq, strided, &tmQs, &oq, kKeyStep)) return rc;
-        if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdOs, &odo, kKeyStep)) return rc;
-    }
+    if (int rc = get_bf16_map(Q, s, sq, strided, &tmQs, &oq, kKeyStep)) return rc;
+    if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdOs, &odo, kKeyStep)) return rc;
     // (every map is there before the first launch: a call that fails has launched nothing)
     const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12);
     cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders | (odq << 16), LSE, Delta, s, st.num_sms,
                                    st.dev_status, cs);
     if (e != cudaSuccess) return fail_cuda(e);
-    if (s.D == 128) {
-        e = launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders | (odk << 16) | (odv << 20), LSE, Delta, s,
-                             st.num_sms, st.dev_status, cs);
-    } else {
-        // the fused kernel without its dQ product (the accumulator map is never used: any map will do)
-        e = launch_attn_bwd(tmQ, tmK, tmV, tmdO, tmQ, tmdK, tmdV, strided, orders | (odk << 16) | (odv << 20), DqMode::kNone,
-                            LSE, Delta, s, st.num_sms, st.dev_status, cs);
-    }
+    const uint32_t orders_kv = orders | (odk << 16) | (odv << 20);
+    e = s.D == 128 ? launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders_kv, LSE, Delta, s, st.num_sms,
+                                      st.dev_status, cs)
+                   : launch_attn_dkdv64(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders_kv, LSE, Delta, s, st.dev_status, cs);
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 
@@ -649,7 +644,7 @@ int nova_attn_bwd_work_list(int BH, long long T, int D, int causal, int n_ctas, 
         plan4[3] = plan.passes_last;
     }
     if (cta >= grid) return 0;  // fewer items than CTAs: the grid is that much smaller
-    const WorkArgs wa{BH, n_tiles, 1, 0u, 0, plan};
+    const WorkArgs wa{BH, n_tiles, 1, 0u, plan};
     const WorkList wl{wa, causal != 0};
     int n = 0;
     for (WorkCursor cur; !wl.done(cur); wl.advance(cur)) {

@@ -50,11 +50,6 @@ namespace nova {
 namespace {
 
 constexpr int kBwdTmemCols = 512;
-// LSE/scale has to be finite.  Below this scale the scores add nothing to P (|s| < 1e6 at most), with it or without.
-constexpr float kLeastScale = 1e-30f;
-// Largest |LSE/scale| (bf16 ends at 3.39e38): times kLeastScale it is still far past where 2^x becomes 0 or infinite.
-constexpr float kMostLse = 3e38f;
-
 template <int D>
 struct BwdCfg {
     static constexpr int kHalves = D / kBoxCols;
@@ -373,12 +368,12 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
             }
             __syncwarp();
             // dQ_i = dS K_j, 64 head-dim columns per accumulator half; 16 keys per instruction.
-            if (!Cfg::kdQAliased && !wl.no_dq()) {  // the dQ warps must have read the previous tile out of the dQ columns
+            if (!Cfg::kdQAliased) {  // the dQ warps must have read the previous tile out of the dQ columns
                 ok = mbar_wait(&bars->dq_free, (g & 1) ^ 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
             }
-            if (el && !wl.no_dq()) {
+            if (el) {
 #pragma unroll
                 for (int h = 0; h < Cfg::kHalves; ++h) {
                     const uint32_t t_dq = tmem_base + Cfg::kColdQ + h * 64;
@@ -418,18 +413,6 @@ __device__ __forceinline__ void bwd_mma(uint8_t* smem, BwdBars* bars, uint32_t t
         __syncwarp();
         (void)mbar_wait(&bars->drain, 0, &none);
     }
-}
-
-// Three bf16 numbers each that add up to l and d (to 24 bits): columns 0, 2, 4 and 1, 3, 5 of a row of 8.
-__device__ __forceinline__ uint4 split_bf16x3(float l, float d) {
-    uint32_t w[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        w[i] = pack_bf16x2(l, d);
-        l -= __uint_as_float(w[i] << 16);
-        d -= __uint_as_float(w[i] & 0xffff0000u);
-    }
-    return make_uint4(w[0], w[1], w[2], 0u);
 }
 
 // Row loader where the row terms go through the tensor core (kFold): one row of 8 columns per query.  LSE/scale is held below
@@ -671,11 +654,10 @@ __device__ __forceinline__ void bwd_compute(uint8_t* smem, BwdBars* bars, uint32
                 }
                 if (x + 16 < kQPT) tmem_ld_x16(t_dp + x + 16, dv);  // all of dv has been consumed above
                 if (!Cfg::kdKFromSmem) tmem_st_x8(t_dp + x / 2, dd);
-                if (Cfg::kdKFromSmem || !wl.no_dq()) {  // dS^T row r: two 16-byte chunks of one 128-byte swizzled row
-                    const int ch = ch0 + x / 8;
-                    *reinterpret_cast<uint4*>(sdS_row + (((ch + 0) ^ (r & 7)) << 4)) = make_uint4(dd[0], dd[1], dd[2], dd[3]);
-                    *reinterpret_cast<uint4*>(sdS_row + (((ch + 1) ^ (r & 7)) << 4)) = make_uint4(dd[4], dd[5], dd[6], dd[7]);
-                }
+                // dS^T row r: two 16-byte chunks of one 128-byte swizzled row
+                const int ch = ch0 + x / 8;
+                *reinterpret_cast<uint4*>(sdS_row + (((ch + 0) ^ (r & 7)) << 4)) = make_uint4(dd[0], dd[1], dd[2], dd[3]);
+                *reinterpret_cast<uint4*>(sdS_row + (((ch + 1) ^ (r & 7)) << 4)) = make_uint4(dd[4], dd[5], dd[6], dd[7]);
             }
             if (!Cfg::kdKFromSmem) tmem_wait_st();
             fence_proxy_async_smem();
@@ -844,7 +826,7 @@ __device__ __forceinline__ void bwd_dq_tma(uint8_t* smem, BwdBars* bars, uint32_
     for (WorkCursor cur; !wl.done(cur) && ok; wl.advance(cur)) {
         int kt, bh, i0, n_it;
         if (!wl.get(cur, &kt, &bh, &i0, &n_it)) continue;
-        for (int it = 0; it < n_it && !wl.no_dq(); ++it, ++g) {
+        for (int it = 0; it < n_it; ++it, ++g) {
             ok = mbar_wait(&bars->dq_full, g & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
@@ -1169,7 +1151,7 @@ cudaError_t launch_one(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     int n_tiles = 0, n_ctas = 0;
     const WorkPlan plan = bwd_work_plan(BH, s.T, D, kCausal, num_sms, &n_tiles, &n_ctas);
     const dim3 grid(static_cast<unsigned>(n_ctas));  // one persistent CTA per SM
-    const WorkArgs wa{BH, n_tiles, s.H, orders, dq == DqMode::kNone ? 1 : 0, plan};
+    const WorkArgs wa{BH, n_tiles, s.H, orders, plan};
     auto go = [&](auto kernel) {
         return launch_overlapped(kernel, grid, dim3(BwdCfg<D>::kThreads), BwdCfg<D>::kSmemBytes, stream, tmQ, tmK, tmV, tmdO,
                                  tmAcc, tmdK, tmdV, LSE, Delta, s.T, wa, s.scale, dev_status);
@@ -1204,7 +1186,6 @@ cudaError_t launch_attn_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmK, cons
                             const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
                             const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,
                             const float* Delta, const AttnShape& s, int num_sms, int* dev_status, cudaStream_t stream) {
-    if (s.D == 128 && dq == DqMode::kNone) return cudaErrorNotSupported;  // that half has a kernel of its own (attn_dkdv.cu)
     auto go = [&](auto launch) {
         return launch(tmQ, tmK, tmV, tmdO, tmAcc, tmdK, tmdV, strided, orders, dq, LSE, Delta, s, num_sms, dev_status, stream);
     };

@@ -91,6 +91,12 @@ cudaError_t launch_attn_dkdv(const CUtensorMap& tmQ, const CUtensorMap& tmK, con
                              uint32_t orders, const float* LSE, const float* Delta, const AttnShape& s, int num_sms,
                              int* dev_status, cudaStream_t stream);
 cudaError_t configure_attn_dkdv();
+// The same at D = 64 (attn_dkdv64.cu).
+cudaError_t launch_attn_dkdv64(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                               const CUtensorMap& tmdO, const CUtensorMap& tmdK, const CUtensorMap& tmdV, bool strided,
+                               uint32_t orders, const float* LSE, const float* Delta, const AttnShape& s, int* dev_status,
+                               cudaStream_t stream);
+cudaError_t configure_attn_dkdv64();
 
 // Heads that the items of the kernels at D=128 are taken in together: enough items for two rounds of the SMs, and no more
 // than about 48 MB of Q, K, V and dO, so that what the tiles of a head share stays in L2 (the forward re-reads K and V only,
@@ -123,15 +129,14 @@ long long steps_until_done(long long items, int num_sms, F&& steps) {
 // What the backward main kernel does with its partial tiles of dQ.
 enum class DqMode {
     kAccumulate,  // adds them, unscaled, into the fp32 accumulator
-    kNone,        // nothing: dK and dV only (the dK/dV half of the two-kernel backward; D = 64)
     kDirect,      // T <= kBlockK, a head has one key tile: its dQ tile is complete and is written scaled, as bf16
 };
 
 // Backward main kernel: adds unscaled dQ partial tiles into the fp32 accumulator [B,H,T,D] (zero on
 // entry) described by `tmAcc` (fp32 [D, T, B*H], box [32, 128, 1], 128-byte swizzle) and writes dK and dV
 // through TMA stores (`tmdK`, `tmdV`: the bf16 maps of the outputs).  `strided`, `orders`: as in the forward, for
-// Q, K, V, dO, dK, dV (and dQ).  `dq`: see above; `tmAcc` is the bf16 map of dQ with kDirect and never used with
-// kNone.  Persistent: launches at most `num_sms` CTAs.
+// Q, K, V, dO, dK, dV (and dQ).  `dq`: see above; `tmAcc` is the bf16 map of dQ with kDirect.
+// Persistent: launches at most `num_sms` CTAs.
 cudaError_t launch_attn_bwd(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                             const CUtensorMap& tmdO, const CUtensorMap& tmAcc, const CUtensorMap& tmdK,
                             const CUtensorMap& tmdV, bool strided, uint32_t orders, DqMode dq, const float* LSE,

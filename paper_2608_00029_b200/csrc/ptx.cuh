@@ -508,4 +508,22 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
+// ---- row terms of the backward that enter the products through the tensor core
+// LSE/scale has to be finite.  Below this scale the scores add nothing to P (|s| < 1e6 at most), with it or without.
+constexpr float kLeastScale = 1e-30f;
+// Largest |LSE/scale| (bf16 ends at 3.39e38): times kLeastScale it is still far past where 2^x becomes 0 or infinite.
+constexpr float kMostLse = 3e38f;
+
+// Three bf16 numbers each that add up to l and d (to 24 bits): columns 0, 2, 4 and 1, 3, 5 of a row of 8.
+__device__ __forceinline__ uint4 split_bf16x3(float l, float d) {
+    uint32_t w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        w[i] = pack_bf16x2(l, d);
+        l -= __uint_as_float(w[i] << 16);
+        d -= __uint_as_float(w[i] & 0xffff0000u);
+    }
+    return make_uint4(w[0], w[1], w[2], 0u);
+}
+
 }  // namespace nova

@@ -30,7 +30,6 @@ struct WorkCursor {
 struct WorkArgs {
     int BH, n_tiles, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, dO, dK, dV, dQ tensor maps, four bits each
-    int no_dq;        // dK/dV half of the two-kernel backward at D=64: no dQ product, no accumulator traffic
     WorkPlan plan;
 };
 struct WorkList {
@@ -38,7 +37,6 @@ struct WorkList {
     bool causal;
     __host__ __device__ __forceinline__ int H() const { return a.H; }
     __host__ __device__ __forceinline__ uint32_t orders() const { return a.orders; }
-    __host__ __device__ __forceinline__ bool no_dq() const { return a.no_dq != 0; }
     __host__ __device__ __forceinline__ bool done(const WorkCursor& c) const { return c.ck >= a.plan.n_chunks; }
     __host__ __device__ __forceinline__ void advance(WorkCursor& c) const {
         const int n = (c.ck == a.plan.n_chunks - 1) ? a.plan.passes_last : a.plan.passes_per_chunk;
@@ -81,7 +79,7 @@ inline WorkPlan work_plan_for_chunk(int BH, int n_tiles, int n_ctas, int chunk) 
 
 // Largest load of a CTA over the mean load (in tiles) when the items are dealt out by `wp`.
 inline double work_plan_imbalance(int BH, int n_tiles, bool causal, int n_ctas, const WorkPlan& wp) {
-    const WorkArgs wa{BH, n_tiles, 1, 0u, 0, wp};
+    const WorkArgs wa{BH, n_tiles, 1, 0u, wp};
     const WorkList wl{wa, causal};
     long long total = 0, worst = 0;
     for (int cta = 0; cta < n_ctas; ++cta) {

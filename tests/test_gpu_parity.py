@@ -632,6 +632,38 @@ def test_wide_heads_backward_routes(B, H, T, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"wide T={T}: ", dO=ref["dO_in"])
 
 
+# D=64: lengths around a step of 64, a tile of 128 and the ring of stages; items of one step, more items than SMs, several
+# items per SM that follow each other before the operands of the last have been released.
+TWO_KERNELS_64 = [(8, 30, 129, True), (8, 30, 191, False), (40, 30, 130, True), (5, 25, 449, False), (10, 8, 700, True),
+                  (7, 30, 200, True), (3, 50, 383, True), (2, 3, 1025, False)]
+
+
+@pytest.mark.parametrize("B,H,T,causal", TWO_KERNELS_64)
+def test_narrow_heads_two_kernel_backward(B, H, T, causal):
+    """The dQ and the dK/dV kernel at D=64: dK and dV have the bits of the fused kernel's (same arithmetic, same order; its
+    steps issued one by one), everything agrees with the oracle."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("narrow", B=B, H=H, T=T, D=64, seed=80 + T, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    got = h.run_gpu(Q, K, V, dO, cfg.scale, causal)
+    q, k, v, do = (x.to(dev) for x in (Q, K, V, dO))
+    o, lse, delta = got["O"].to(dev), got["LSE"].to(dev), got["Delta"].to(dev)
+    ws = torch.empty(nova_attn.nova_attn_bwd_workspace_bytes(B, H, T, 64), dtype=torch.uint8, device=dev)
+    fused = [torch.full_like(q, 7.0) for _ in range(3)]
+    for step in (nova_attn.BWD_STEP_ZERO, nova_attn.BWD_STEP_MAIN, nova_attn.BWD_STEP_CONVERT):
+        nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *fused, cfg.scale, causal, ws, steps=step)
+    two = [torch.full_like(q, 7.0) for _ in range(3)]
+    nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *two, cfg.scale, causal)
+    nova_attn.nova_attn_poll_device_status()
+    assert torch.equal(two[1], fused[1]) and torch.equal(two[2], fused[2])
+    got.update({"dQ": two[0].cpu(), "dK": two[1].cpu(), "dV": two[2].cpu()})
+    heads = [(0, 0), (B - 1, H - 1)]
+    ref = h.run_oracle(Q, K, V, dO, cfg.scale, causal, heads=heads)
+    h.compare(h.select_heads(got, heads), ref, label=f"narrow T={T}: ", dO=ref["dO_in"])
+
+
 # One of each backward kernel: the fused one (single key tile, several), with more heads than SMs, and at D=128 the pair of
 # kernels (which the deterministic entry point takes at every T > 128).
 NOT_FINITE = [(1, 2, 100, 64), (1, 2, 300, 64), (8, 30, 300, 64), (1, 2, 100, 128), (1, 2, 300, 128), (8, 30, 300, 128)]
