@@ -9,7 +9,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libnova_attn.so")
-SOURCES = ["api.cu", "attn_fwd.cu", "attn_bwd.cu", "attn_bwd_pre.cu", "attn_dq.cu", "attn_dkdv.cu", "attn_dkdv64.cu",
+SOURCES = ["api.cu", "attn_fwd.cu", "attn_bwd.cu", "attn_bwd_pre.cu", "attn_dq.cu", "attn_dq64.cu", "attn_dkdv.cu", "attn_dkdv64.cu",
            "attn_bwd_static.cu", "lmhead.cu", "lmhead_rows.cu"]
 BINDING = os.path.join(HERE, "_binding.so")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

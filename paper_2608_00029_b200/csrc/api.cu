@@ -77,6 +77,7 @@ int device_state(DeviceState** out) {
         e = configure_attn_fwd();
         if (e == cudaSuccess) e = configure_attn_bwd();
         if (e == cudaSuccess) e = configure_attn_dq();
+        if (e == cudaSuccess) e = configure_attn_dq64();
         if (e == cudaSuccess) e = configure_attn_dkdv();
         if (e == cudaSuccess) e = configure_attn_dkdv64();
         if (e == cudaSuccess) e = configure_lmhead();
@@ -378,9 +379,10 @@ int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, 
     if (int rc = get_tensor_map(V, D, T, BH, &tmV, 2, 0, 0, kKeyStep)) return rc;
     if (int rc = get_tensor_map(dO, D, T, BH, &tmdO)) return rc;
     const AttnShape s{B, H, T, D, causal != 0, scale};
+    const cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const cudaError_t e =
-        launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status,
-                          static_cast<cudaStream_t>(stream));
+        D == 128 ? launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status, cs)
+                 : launch_attn_delta64(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->dev_status, cs);
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 
@@ -428,8 +430,10 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     if (int rc = get_bf16_map(dO, s, sdo, strided, &tmdOs, &odo, kKeyStep)) return rc;
     // (every map is there before the first launch: a call that fails has launched nothing)
     const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12);
-    cudaError_t e = launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders | (odq << 16), LSE, Delta, s, st.num_sms,
-                                   st.dev_status, cs);
+    const uint32_t orders_dq = orders | (odq << 16);
+    cudaError_t e = s.D == 128 ? launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders_dq, LSE, Delta, s, st.num_sms,
+                                                st.dev_status, cs)
+                               : launch_attn_dq64(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders_dq, LSE, Delta, s, st.dev_status, cs);
     if (e != cudaSuccess) return fail_cuda(e);
     const uint32_t orders_kv = orders | (odk << 16) | (odv << 20);
     e = s.D == 128 ? launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders_kv, LSE, Delta, s, st.num_sms,

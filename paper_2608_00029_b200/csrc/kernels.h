@@ -69,7 +69,7 @@ cudaError_t launch_attn_bwd_preprocess(const __nv_bfloat16* O, const __nv_bfloat
                                        const AttnShape& s, const TensorStrides& so, const TensorStrides& sdo,
                                        int num_sms, cudaStream_t stream);
 
-// The query-major passes of the backward (attn_dq.cu): K and V maps with boxes of kKeyStep rows.
+// The query-major passes of the backward at D = 128 (attn_dq.cu): K and V maps with boxes of kKeyStep rows.
 constexpr int kKeyStep = 64;
 // Exact Delta_i = sum_j P_ij (dO_i . V_j) with P rebuilt from LSE (two contractions + exp2 per tile).
 cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
@@ -83,6 +83,14 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
                            const float* LSE, const float* Delta, const AttnShape& s, int num_sms, int* dev_status,
                            cudaStream_t stream);
 cudaError_t configure_attn_dq();
+// The same two at D = 64 (attn_dq64.cu).
+cudaError_t launch_attn_delta64(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                                const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s, int* dev_status,
+                                cudaStream_t stream);
+cudaError_t launch_attn_dq64(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
+                             const CUtensorMap& tmdO, const CUtensorMap& tmdQ, bool strided, uint32_t orders,
+                             const float* LSE, const float* Delta, const AttnShape& s, int* dev_status, cudaStream_t stream);
+cudaError_t configure_attn_dq64();
 
 // The dK/dV half of the two-kernel backward at D = 128 (attn_dkdv.cu): Q and dO maps with boxes of kKeyStep rows, the
 // others of 128.  `orders` for Q, K, V, dO, dK, dV.

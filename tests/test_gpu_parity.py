@@ -495,6 +495,34 @@ def test_query_major_passes_alone_and_in_a_crowd(T, D, causal):
     h.compare(h.select_heads(got, None), ref, label=f"crowd T={T} D={D}: ", dO=ref["dO_in"])
 
 
+@pytest.mark.parametrize("T", [1, 63, 64, 65, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_exact_delta_of_short_sequences(T, causal):
+    """Items of one or two steps, in which a compute group may have none: a head alone and 1500 copies (ten items per SM) have
+    the same bits, and the definition's value, sum_j P_ij (dO_i . V_j) in 64 bits, to within the fp32 sums and exponentials
+    (2e-6 of the largest terms, 64 in all; 1e-4 covers them with P read from an fp32 LSE)."""
+    from paper_2608_00029_b200 import nova_attn
+    h = _harness()
+    dev = torch.device("cuda:0")
+    cfg = W.AttnConfig("short", B=1, H=1, T=T, D=64, seed=20 + T, causal=causal)
+    Q, K, V, dO = W.make_inputs(cfg)
+    lse1 = h.run_gpu(Q, K, V, dO, cfg.scale, causal)["LSE"].to(dev)
+    first = None
+    for n in (1, 1500):
+        q, k, v, do = (x.to(dev).expand(1, n, T, 64).contiguous() for x in (Q, K, V, dO))
+        delta = torch.full((1, n, T), 7.0, device=dev)
+        nova_attn.nova_attn_bwd_preprocess_exact(q, k, v, do, lse1.expand(1, n, T).contiguous(), delta, cfg.scale, causal)
+        nova_attn.nova_attn_poll_device_status()
+        first = delta[0, 0].clone() if first is None else first
+        assert torch.equal(delta, first.expand_as(delta)), n
+    q, k, v, do = (x[0, 0].double() for x in (Q, K, V, dO))
+    s = (q @ k.T) * cfg.scale
+    if causal:
+        s = s.masked_fill(torch.ones(T, T).triu(1).bool(), float("-inf"))
+    want = (torch.softmax(s, -1) * (do @ v.T)).sum(-1)
+    assert (first.double().cpu() - want).abs().max() <= 1e-4 * max(1.0, float((do @ v.T).abs().max()))
+
+
 @pytest.mark.parametrize("T", [1, 127, 129, 256, 257, 384, 500])
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("causal", [True, False])
