@@ -401,17 +401,30 @@ namespace {
 // us; B=2, H=32, T=640, 192 blocks: 49 us both).  Without the mask every item of a head is as long as its longest, so that a
 // last round with few items costs as much as a full one: above T=2560 the two kernels then need more than three rounds of
 // blocks (H=28, T=4096: 763 -> 807 us, H=20: 539 -> 590 us; but H=32: 909 -> 843 us, H=40, T=3584: 827 -> 797 us).
+//
+// At D=64 the two kernels (with their operands in tensor memory, attn_dkdv64.cu) recompute S and dP but need neither the clear nor
+// the conversion (10 us of 74 at B=8, H=12, T=1024).  In small problems both ways are chains of launches, ramps and the longest
+// item and end within 3 % of each other (H=12, T=777: 21 us both; H=48, T=256: 13.2, 14.3 us); from 2.5 tiles of 128 rows per SM
+// on the two kernels are ahead (fused, two: H=96, T=512 27.9, 26.9 us; H=48, T=1024 38.9, 36.6; H=384, T=512 92, 76; H=12,
+// T=4096 95, 88), with two or three tiles a head, where items are short, from twice that (H=192, T=256 22.2, 22.9; H=768 74,
+// 66).  Large unmasked problems sit at the card's power limit, where two contractions more cost what the rest gains
+// (H=192, T=1500 364, 378 us; H=128, T=1500 252, 244).
 bool two_kernels_pay(long long BH, int T, int D, bool causal, int num_sms) {
+    if (D == 64) {
+        const long long tiles = BH * ((T + 127) / 128);
+        if (T <= 128 || tiles * 2 < (T > 256 ? 5ll : 11ll) * num_sms) return false;
+        return causal || tiles <= 14ll * num_sms;
+    }
     const long long blocks = BH * ((T + 255) / 256);
-    if (D != 128 || T > 4096) return false;
+    if (T > 4096) return false;
     return !causal && T > 2560 ? blocks * 3 >= 10ll * num_sms : blocks * 2 >= 3ll * num_sms;
 }
 
-// dQ, dK and dV by the two-kernel backward.
+// dQ, dK and dV by the two-kernel backward.  `terms`: room for the row terms of D=64 (32 bytes a row), or null.
 int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO, const float* LSE, const float* Delta,
                     void* dQ, void* dK, void* dV, const AttnShape& s, const TensorStrides& sq, const TensorStrides& sk,
                     const TensorStrides& sv, const TensorStrides& sdo, const TensorStrides& sdq, const TensorStrides& sdk,
-                    const TensorStrides& sdv, const DeviceState& st, cudaStream_t cs) {
+                    const TensorStrides& sdv, void* terms, const DeviceState& st, cudaStream_t cs) {
     const bool strided = !(merges(s, sq) && merges(s, sk) && merges(s, sv) && merges(s, sdo) && merges(s, sdq) &&
                            merges(s, sdk) && merges(s, sdv));
     // Each kernel takes what it streams in boxes of kKeyStep rows and what it holds in boxes of 128.
@@ -431,6 +444,10 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     // (every map is there before the first launch: a call that fails has launched nothing)
     const uint32_t orders = oq | (ok << 4) | (ov << 8) | (odo << 12);
     const uint32_t orders_dq = orders | (odq << 16);
+    if (terms != nullptr) {
+        const cudaError_t et = launch_row_terms64(LSE, Delta, terms, s, cs);
+        if (et != cudaSuccess) return fail_cuda(et);
+    }
     cudaError_t e = s.D == 128 ? launch_attn_dq(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders_dq, LSE, Delta, s, st.num_sms,
                                                 st.dev_status, cs)
                                : launch_attn_dq64(tmQ, tmKs, tmVs, tmdO, tmdQ, strided, orders_dq, LSE, Delta, s, st.dev_status, cs);
@@ -438,7 +455,8 @@ int bwd_two_kernels(const void* Q, const void* K, const void* V, const void* dO,
     const uint32_t orders_kv = orders | (odk << 16) | (odv << 20);
     e = s.D == 128 ? launch_attn_dkdv(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders_kv, LSE, Delta, s, st.num_sms,
                                       st.dev_status, cs)
-                   : launch_attn_dkdv64(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders_kv, LSE, Delta, s, st.dev_status, cs);
+                   : launch_attn_dkdv64(tmQs, tmK, tmV, tmdOs, tmdK, tmdV, strided, orders_kv, LSE, Delta, terms, s, st.dev_status,
+                                        cs);
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 
@@ -465,7 +483,7 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
     const bool whole = steps == (NOVA_ATTN_BWD_STEP_ZERO | NOVA_ATTN_BWD_STEP_MAIN | NOVA_ATTN_BWD_STEP_CONVERT);
     const bool direct = T <= kBlockK && whole;
     if (whole && !direct && two_kernels_pay(BH, T, D, causal != 0, st->num_sms))
-        return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv, *st, cs);
+        return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv, D == 64 ? workspace : nullptr, *st, cs);
     auto clear = [&]() {
         return (steps & NOVA_ATTN_BWD_STEP_ZERO) && !direct ? launch_zero(acc, need, st->num_sms, cs) : cudaSuccess;
     };
@@ -532,7 +550,7 @@ int nova_attn_bwd_deterministic(const void* Q, const void* K, const void* V, con
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const TensorStrides c = contiguous_strides(H, T, D);
-    if (T > kBlockK) return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, c, c, c, c, c, c, c, *st, cs);
+    if (T > kBlockK) return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, c, c, c, c, c, c, c, nullptr, *st, cs);
     // one key tile per head: nothing is summed across blocks, the fused kernel is deterministic too
     CUtensorMap tmQ, tmK, tmV, tmdO, tmdQ, tmdK, tmdV;
     if (int rc = get_tensor_map(Q, D, T, BH, &tmQ)) return rc;

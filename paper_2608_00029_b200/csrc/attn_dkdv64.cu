@@ -62,7 +62,7 @@ struct Kv64Bars {
     uint64_t dkv_full, dkv_free;          // dV and dK of an item complete; read out of TMEM
     uint64_t staged, stage_free;          // the write-out warps among themselves
     uint64_t drain[3];
-    WorkRing ring;
+    StepRing ring;
     int odd_rows[kQStages];  // the stage's row terms hold a Delta that is not finite
     uint32_t tmem_base;
     int abort_flag;
@@ -83,19 +83,62 @@ struct Kv64Work {
     }
 };
 
-template <bool kStrided>
+// The operand row of one query: 16 columns in two halves of 16 bytes.
+// LSE/scale is held below kMostLse, which keeps what an infinite LSE means (P = 0 for +inf, P = inf for -inf) without an
+// infinity that would meet another in the sum; queries past the end of the sequence count as +inf.  A NaN becomes P = inf where
+// the query is kept.  A Delta that is not finite must not reach S^T (0 * inf is NaN): it enters as kMostLse in a column of its
+// own, times kMostLse for dP^T (infinite, for a NaN as well) and times 0 for S^T.
+struct RowTerms {
+    uint4 first, second;
+    bool odd;  // the second half is not zero
+};
+__device__ __forceinline__ RowTerms row_terms(float l, float d) {
+    RowTerms t;
+    float odd = 0.f;
+    if (!(fabsf(l) <= kMostLse)) l = l < 0.f ? -kMostLse : kMostLse;
+    t.odd = !(fabsf(d) <= kMostLse);
+    if (t.odd) {
+        odd = copysignf(kMostLse, d);
+        d = 0.f;
+    }
+    t.first = split_bf16x3(l, d);
+    t.second = make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(odd)), 0u, 0u, 0u);
+    return t;
+}
+
+// The row terms of every step of every head, laid out as the kernel's stages hold them: once per row instead of once per row
+// and key tile, for callers that have room for them.
+__global__ void __launch_bounds__(256) row_terms64_kernel(const float* __restrict__ LSE, const float* __restrict__ Delta,
+                                                          uint8_t* __restrict__ terms, int T, int n_steps, long long rows,
+                                                          float inv_scale) {
+    griddep_launch_dependents();
+    griddep_wait();
+    const long long idx = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
+    if (idx >= rows) return;
+    const uint32_t tile = static_cast<uint32_t>(idx / kStep), r = static_cast<uint32_t>(idx % kStep);
+    const uint32_t bh = tile / n_steps, q = (tile - bh * n_steps) * kStep + r;
+    const bool in = q < static_cast<uint32_t>(T);
+    const size_t at = static_cast<size_t>(bh) * T + q;
+    const RowTerms t = row_terms(in ? -LSE[at] * inv_scale : -kMostLse, in ? -Delta[at] : 0.f);
+    uint8_t* const row = terms + static_cast<size_t>(tile) * kExtStep + (r >> 3) * 2 * kExtCore + (r & 7) * 16;
+    *reinterpret_cast<uint4*>(row) = t.first;
+    *reinterpret_cast<uint4*>(row + kExtCore) = t.second;
+}
+
+template <bool kStrided, bool kTerms>
 __device__ __forceinline__ void kv64_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                                              const CUtensorMap* tmdO, uint8_t* smem, Kv64Bars* bars, const Kv64Work& wk) {
+                                              const CUtensorMap* tmdO, const uint8_t* __restrict__ terms, uint8_t* smem,
+                                              Kv64Bars* bars, const Kv64Work& wk) {
     volatile int* abort_flag = &bars->abort_flag;
     bool ok = true, clc_pending = false;
     int w = 0, n_kv = 0, g = 0, st = 0;  // items, K and V requested; steps requested
     uint32_t ph = 0;
     int item = blockIdx.x;
     for (;;) {
-        ok = bars->ring.publish(w, item, abort_flag, kWaitLimitCycles);
+        int kt = 0, bh = 0, s0 = 0, n = -1;
+        if (item >= 0) wk.get(item, &kt, &bh, &s0, &n);
+        ok = bars->ring.publish_steps(w, item, n, abort_flag);
         if (!ok || item < 0) break;
-        int kt, bh, s0, n;
-        wk.get(item, &kt, &bh, &s0, &n);
         const int head = kStrided ? bh % wk.H : 0, batch = kStrided ? bh / wk.H : 0;
         const int ks = w & 1;
         ok = mbar_wait(&bars->kv_empty[ks], ((w >> 1) & 1) ^ 1, abort_flag);
@@ -109,8 +152,12 @@ __device__ __forceinline__ void kv64_producer(const CUtensorMap* tmQ, const CUte
         for (int s = 0; s < n; ++s) {
             ok = mbar_wait(&bars->q_empty[st], ph ^ 1, abort_flag);
             if (!ok) break;
-            mbar_expect_tx(&bars->q_full[st], 2 * kStepBytes);
+            mbar_expect_tx(&bars->q_full[st], 2 * kStepBytes + (kTerms ? kExtStep : 0));
             ++g;
+            if (kTerms)
+                bulk_load(smem + kOffExt + st * kExtStep,
+                          terms + (static_cast<size_t>(bh) * ((wk.T + kStep - 1) / kStep) + s0 + s) * kExtStep, kExtStep,
+                          &bars->q_full[st]);
             tma_load_tile<kStrided>(smem + kOffQ + st * kStepBytes, tmQ, &bars->q_full[st], wk.orders & 15, 0,
                                     (s0 + s) * kStep, head, batch, bh);
             tma_load_tile<kStrided>(smem + kOffdO + st * kStepBytes, tmdO, &bars->q_full[st], (wk.orders >> 12) & 15, 0,
@@ -136,7 +183,7 @@ __device__ __forceinline__ void kv64_producer(const CUtensorMap* tmQ, const CUte
         for (int x = g > kQStages ? g - kQStages : 0; x < g; ++x) {
             // the barrier counts the row terms too, which may never come: their share is made up for
             none = 0;
-            if (mbar_wait(&bars->q_full[x % kQStages], (x / kQStages) & 1, &none, 1 << 16)) continue;
+            if (mbar_wait(&bars->q_full[x % kQStages], (x / kQStages) & 1, &none, 1 << 16) || kTerms) continue;
             none = 0;
             mbar_arrive(&bars->q_full[x % kQStages]);
             (void)mbar_wait(&bars->q_full[x % kQStages], (x / kQStages) & 1, &none);
@@ -163,7 +210,7 @@ __device__ __forceinline__ void kv64_product(uint32_t t_acc, uint32_t t_a, uint3
 // S^T (kdP false): that of step g goes out as soon as the compute group has read that of step g - 2.
 // dP^T (kdP true): as soon as dK of step g - 2 has read the dS^T that lies in the same columns.
 template <bool kdP>
-__device__ __forceinline__ void kv64_mma_sp(uint8_t* smem, Kv64Bars* bars, uint32_t tmem_base, const Kv64Work& wk) {
+__device__ __forceinline__ void kv64_mma_sp(uint8_t* smem, Kv64Bars* bars, uint32_t tmem_base) {
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t b0 = umma_desc_lo(smem_u32(smem + (kdP ? kOffdO : kOffQ)), 16);
     const uint32_t ext0 = umma_desc_lo(smem_u32(smem + kOffExt), kExtCore);
@@ -176,13 +223,11 @@ __device__ __forceinline__ void kv64_mma_sp(uint8_t* smem, Kv64Bars* bars, uint3
     int g = 0, st = 0;
     uint32_t ph = 0;
     for (int w = 0;; ++w) {
-        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
-        if (item < 0) {
-            ok = (item == -1);
+        const int n = bars->ring.take_steps(w, lane, abort_flag);
+        if (n <= 0) {
+            ok = (n == 0);
             break;
         }
-        int kt, bh, s0, n;
-        wk.get(item, &kt, &bh, &s0, &n);
         ok = mbar_wait(&bars->op_full[kdP], w & 1, abort_flag);
         if (!ok) break;
         for (int s = 0; s < n; ++s, ++g) {
@@ -213,7 +258,7 @@ __device__ __forceinline__ void kv64_mma_sp(uint8_t* smem, Kv64Bars* bars, uint3
 }
 
 // dV and dK of each step, in order.
-__device__ __forceinline__ void kv64_mma_acc(uint8_t* smem, Kv64Bars* bars, uint32_t tmem_base, const Kv64Work& wk) {
+__device__ __forceinline__ void kv64_mma_acc(uint8_t* smem, Kv64Bars* bars, uint32_t tmem_base) {
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescKV = umma_idesc_bf16(128, D, 0, 1);  // A from TMEM, B MN-major
     const uint32_t hi = umma_desc_hi_sw128(1024);
@@ -224,13 +269,11 @@ __device__ __forceinline__ void kv64_mma_acc(uint8_t* smem, Kv64Bars* bars, uint
     bool ok = true;
     int g = 0, st = 0;
     for (int w = 0;; ++w) {
-        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
-        if (item < 0) {
-            ok = (item == -1);
+        const int n = bars->ring.take_steps(w, lane, abort_flag);
+        if (n <= 0) {
+            ok = (n == 0);
             break;
         }
-        int kt, bh, s0, n;
-        wk.get(item, &kt, &bh, &s0, &n);
         // the previous item's dV and dK must have been read out of TMEM before they are overwritten
         if (w > 0) ok = mbar_wait(&bars->dkv_free, (w - 1) & 1, abort_flag);
         if (!ok) break;
@@ -268,8 +311,7 @@ __device__ __forceinline__ void kv64_mma_acc(uint8_t* smem, Kv64Bars* bars, uint
 
 // Compute group `grp` (steps g with g % 2 == grp), warp `cwarp` of it.
 template <bool kCausal>
-__device__ __forceinline__ void kv64_compute(Kv64Bars* bars, uint32_t tmem_base, float scale, const Kv64Work& wk, int grp,
-                                             int cwarp, int lane) {
+__device__ __forceinline__ void kv64_compute(Kv64Bars* bars, uint32_t tmem_base, float scale, int grp, int cwarp, int lane) {
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * cwarp;
     const int r = lane_base + lane;  // local key row
@@ -282,13 +324,11 @@ __device__ __forceinline__ void kv64_compute(Kv64Bars* bars, uint32_t tmem_base,
     uint32_t ph = 0;   // phase of this group's barriers
 
     for (int w = 0;; ++w) {
-        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
-        if (item < 0) {
-            ok = (item == -1);
+        const int n = bars->ring.take_steps(w, lane, abort_flag);
+        if (n <= 0) {
+            ok = (n == 0);
             break;
         }
-        int kt, bh, s0, n;
-        wk.get(item, &kt, &bh, &s0, &n);
         for (int s = (g ^ grp) & 1; s < n; s += 2, ph ^= 1) {
             ok = mbar_wait(&bars->s_full[grp], ph, abort_flag);
             if (!ok) break;
@@ -362,11 +402,7 @@ __device__ __forceinline__ void kv64_compute(Kv64Bars* bars, uint32_t tmem_base,
 //   dV and dK * scale of a finished item as bf16 into shared memory and out with TMA stores.
 // The stages of an item's first kQStages steps are handed back by the item before, whose dV and dK may wait till then; the
 // later ones only after dV and dK have been read out.
-// Row terms: LSE/scale is held below kMostLse, which keeps what an infinite LSE means (P = 0 for +inf, P = inf for -inf)
-// without an infinity that would meet another in the sum; queries past the end of the sequence count as +inf.  A NaN becomes
-// P = inf where the query is kept.  A Delta that is not finite must not reach S^T (0 * inf is NaN): it enters as kMostLse in
-// a column of its own, times kMostLse for dP^T (infinite, for a NaN as well) and times 0 for S^T.
-template <bool kStrided>
+template <bool kStrided, bool kTerms>
 __device__ __forceinline__ void kv64_edges(uint8_t* smem, Kv64Bars* bars, uint32_t tmem_base, const CUtensorMap* tmdK,
                                            const CUtensorMap* tmdV, const float* __restrict__ LSE,
                                            const float* __restrict__ Delta, float scale, const Kv64Work& wk, int ow, int lane) {
@@ -408,36 +444,22 @@ __device__ __forceinline__ void kv64_edges(uint8_t* smem, Kv64Bars* bars, uint32
         constexpr int kNext32 = 32 / 8 * 2 * kExtCore;  // the row 32 queries on
         for (int s = from + ((ow - g0 - from) & 3); s < to; s += 4) {
             const int g = g0 + s, st = g % kQStages;
-            float l[2], d[2], odd[2] = {0.f, 0.f};
-            bool rare = false;
+            RowTerms t[2];
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
+            for (int x = 0; x < 2; ++x) {  // (past L1, which may hold what an earlier kernel saw there: there was no griddep_wait)
                 const int q = (s0 + s) * kStep + lane + 32 * x;
-                l[x] = (q < wk.T) ? -LSE[base + q] * inv_scale : -kMostLse;
-                d[x] = (q < wk.T) ? -Delta[base + q] : 0.f;
-                rare = rare || !(fabsf(l[x]) <= kMostLse) || !(fabsf(d[x]) <= kMostLse);
+                t[x] = row_terms((q < wk.T) ? -__ldcg(LSE + base + q) * inv_scale : -kMostLse,
+                                 (q < wk.T) ? -__ldcg(Delta + base + q) : 0.f);
             }
-            const bool any_odd = __any_sync(0xffffffffu, rare);
-            if (any_odd) {
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    if (!(fabsf(l[x]) <= kMostLse)) l[x] = l[x] < 0.f ? -kMostLse : kMostLse;
-                    if (!(fabsf(d[x]) <= kMostLse)) {
-                        odd[x] = copysignf(kMostLse, d[x]);
-                        d[x] = 0.f;
-                    }
-                }
-            }
-            const uint4 v[2] = {split_bf16x3(l[0], d[0]), split_bf16x3(l[1], d[1])};
+            const bool any_odd = __any_sync(0xffffffffu, t[0].odd || t[1].odd);
             if (!mbar_wait(&bars->q_empty[st], ((g / kQStages) & 1) ^ 1, abort_flag)) return false;
 #pragma unroll
-            for (int x = 0; x < 2; ++x) *reinterpret_cast<uint4*>(row + st * kExtStep + x * kNext32) = v[x];
+            for (int x = 0; x < 2; ++x) *reinterpret_cast<uint4*>(row + st * kExtStep + x * kNext32) = t[x].first;
             // (a stage is written by two of the warps in turn: the flag says what the one before left behind)
             if (any_odd || *reinterpret_cast<volatile int*>(&bars->odd_rows[st]) != 0) {
 #pragma unroll
                 for (int x = 0; x < 2; ++x)
-                    *reinterpret_cast<uint4*>(row + st * kExtStep + x * kNext32 + kExtCore) =
-                        make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(odd[x])), 0u, 0u, 0u);
+                    *reinterpret_cast<uint4*>(row + st * kExtStep + x * kNext32 + kExtCore) = t[x].second;
                 __syncwarp();
                 if (lane == 0) *reinterpret_cast<volatile int*>(&bars->odd_rows[st]) = any_odd;
             }
@@ -499,19 +521,20 @@ __device__ __forceinline__ void kv64_edges(uint8_t* smem, Kv64Bars* bars, uint32
 
     int g0 = 0, kt_out = 0, bh_out = 0;
     for (int w = 0; ok; ++w) {
-        const int item = bars->ring.take(w, lane, abort_flag, kWaitLimitCycles);
-        if (item < 0) {
-            if (item == -1 && w > 0) (void)write_out(w - 1, kt_out, bh_out);
+        int item = 0;
+        const int taken = bars->ring.take_steps(w, lane, abort_flag, &item);
+        if (taken <= 0) {
+            if (taken == 0 && w > 0) (void)write_out(w - 1, kt_out, bh_out);
             break;
         }
         int kt, bh, s0, n;
         wk.get(item, &kt, &bh, &s0, &n);
-        ok = rows(bh, s0, g0, 0, min(n, 2));
+        if (!kTerms) ok = rows(bh, s0, g0, 0, min(n, 2));
         if (ok) ok = operand(w, 0);
         if (ok) ok = operand(w, 1);
-        if (ok) ok = rows(bh, s0, g0, 2, min(n, kQStages));
+        if (ok && !kTerms) ok = rows(bh, s0, g0, 2, min(n, kQStages));
         if (ok && w > 0) ok = write_out(w - 1, kt_out, bh_out);
-        if (ok) ok = rows(bh, s0, g0, kQStages, n);
+        if (ok && !kTerms) ok = rows(bh, s0, g0, kQStages, n);
         kt_out = kt;
         bh_out = bh;
         g0 += n;
@@ -519,13 +542,13 @@ __device__ __forceinline__ void kv64_edges(uint8_t* smem, Kv64Bars* bars, uint32
     if (leader) bulk_wait_group<0>();  // dV and dK must be complete before the kernel ends
 }
 
-template <bool kCausal, bool kStrided>
+template <bool kCausal, bool kStrided, bool kTerms>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                    const __grid_constant__ CUtensorMap tmdK, const __grid_constant__ CUtensorMap tmdV,
-                   const float* __restrict__ LSE, const float* __restrict__ Delta, int T, int BH, int H, uint32_t orders,
-                   float scale, int* __restrict__ dev_status) {
+                   const float* __restrict__ LSE, const float* __restrict__ Delta, const uint8_t* __restrict__ terms, int T, int BH,
+                   int H, uint32_t orders, float scale, int* __restrict__ dev_status) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Kv64Bars* bars = reinterpret_cast<Kv64Bars*>(smem + kOffBar);
@@ -545,7 +568,7 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             mbar_init(&bars->op_free[s], 1);
         }
         for (int s = 0; s < kQStages; ++s) {
-            mbar_init(&bars->q_full[s], 2);  // the tiles and the row terms
+            mbar_init(&bars->q_full[s], kTerms ? 1 : 2);  // the producer, and the edge warp that writes the row terms
             mbar_init(&bars->q_empty[s], 1);
             bars->odd_rows[s] = 0;
         }
@@ -584,25 +607,27 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
     griddep_launch_dependents();
-    griddep_wait();  // everything above overlaps the previous kernel of the stream
+    // No griddep_wait() here: the kernel before this one in the stream is the dQ kernel, which lets this one start only when its
+    // own predecessor has completed, and nothing of what it writes is read here.
 
     if (warp == 0) {
-        if (lane == 0) kv64_producer<kStrided>(&tmQ, &tmK, &tmV, &tmdO, smem, bars, wk);
+        if (lane == 0) kv64_producer<kStrided, kTerms>(&tmQ, &tmK, &tmV, &tmdO, terms, smem, bars, wk);
     } else if (warp == 1) {
-        kv64_mma_sp<false>(smem, bars, tmem_base, wk);
+        kv64_mma_sp<false>(smem, bars, tmem_base);
     } else if (warp == 2) {
-        kv64_mma_sp<true>(smem, bars, tmem_base, wk);
+        kv64_mma_sp<true>(smem, bars, tmem_base);
     } else if (warp == 3) {
-        kv64_mma_acc(smem, bars, tmem_base, wk);
+        kv64_mma_acc(smem, bars, tmem_base);
     } else if (warp >= 12) {
-        kv64_edges<kStrided>(smem, bars, tmem_base, &tmdK, &tmdV, LSE, Delta, scale, wk, warp & 3, lane);
+        kv64_edges<kStrided, kTerms>(smem, bars, tmem_base, &tmdK, &tmdV, LSE, Delta, scale, wk, warp & 3, lane);
     } else {
-        kv64_compute<kCausal>(bars, tmem_base, scale, wk, (warp - 4) >> 2, warp & 3, lane);
+        kv64_compute<kCausal>(bars, tmem_base, scale, (warp - 4) >> 2, warp & 3, lane);
     }
 
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
+    griddep_wait();  // what waits for this kernel waits for dQ too
     if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
 }
 
@@ -612,25 +637,36 @@ cudaError_t configure_attn_dkdv64() {
     auto set = [](auto kernel) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     };
-    cudaError_t e = set(attn_dkdv64_kernel<true, false>);
-    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<true, true>);
-    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<false, false>);
-    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<false, true>);
+    cudaError_t e = set(attn_dkdv64_kernel<true, false, false>);
+    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<false, false, false>);
+    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<true, false, true>);
+    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<true, true, true>);
+    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<false, false, true>);
+    if (e == cudaSuccess) e = set(attn_dkdv64_kernel<false, true, true>);
     return e;
+}
+
+cudaError_t launch_row_terms64(const float* LSE, const float* Delta, void* terms, const AttnShape& s, cudaStream_t stream) {
+    const int n_steps = (s.T + kStep - 1) / kStep;
+    const long long rows = static_cast<long long>(s.B) * s.H * n_steps * kStep;
+    return launch_overlapped(row_terms64_kernel, dim3(static_cast<unsigned>((rows + 255) / 256)), dim3(256), 0, stream, LSE, Delta,
+                             static_cast<uint8_t*>(terms), s.T, n_steps, rows, 1.0f / fmaxf(s.scale, kLeastScale));
 }
 
 cudaError_t launch_attn_dkdv64(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                                const CUtensorMap& tmdO, const CUtensorMap& tmdK, const CUtensorMap& tmdV, bool strided,
-                               uint32_t orders, const float* LSE, const float* Delta, const AttnShape& s, int* dev_status,
-                               cudaStream_t stream) {
+                               uint32_t orders, const float* LSE, const float* Delta, const void* terms, const AttnShape& s,
+                               int* dev_status, cudaStream_t stream) {
+    if (strided && terms == nullptr) return cudaErrorNotSupported;  // (only the deterministic entry point has no workspace)
     const int n_tiles = (s.T + kBlockK - 1) / kBlockK, BH = s.B * s.H;
     const dim3 grid(static_cast<unsigned>(n_tiles) * BH);  // one CTA per item; those that do not start are taken over
     auto go = [&](auto kernel) {
         return launch_overlapped(kernel, grid, dim3(kThreads), kSmemBytes, stream, tmQ, tmK, tmV, tmdO, tmdK, tmdV, LSE, Delta,
-                                 s.T, BH, s.H, orders, s.scale, dev_status);
+                                 static_cast<const uint8_t*>(terms), s.T, BH, s.H, orders, s.scale, dev_status);
     };
-    if (s.causal) return strided ? go(attn_dkdv64_kernel<true, true>) : go(attn_dkdv64_kernel<true, false>);
-    return strided ? go(attn_dkdv64_kernel<false, true>) : go(attn_dkdv64_kernel<false, false>);
+    if (terms == nullptr) return s.causal ? go(attn_dkdv64_kernel<true, false, false>) : go(attn_dkdv64_kernel<false, false, false>);
+    if (s.causal) return strided ? go(attn_dkdv64_kernel<true, true, true>) : go(attn_dkdv64_kernel<true, false, true>);
+    return strided ? go(attn_dkdv64_kernel<false, true, true>) : go(attn_dkdv64_kernel<false, false, true>);
 }
 
 }  // namespace nova

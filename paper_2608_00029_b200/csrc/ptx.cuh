@@ -185,6 +185,30 @@ struct WorkRing {
     }
 };
 
+// The same ring carrying the number of steps of an item, which is all that most roles need (finding it out takes an integer
+// division, some 300 clocks for a warp beside busy ones), and beside it the item's number.
+struct StepRing : WorkRing {
+    int number[2];
+
+    // Producer: announces the CTA's w-th item (n < 0: there are no more).
+    __device__ __forceinline__ bool publish_steps(int w, int it, int n, volatile int* abort_flag) {
+        if (!mbar_wait(&empty[w & 1], ((w >> 1) & 1) ^ 1, abort_flag)) return false;
+        number[w & 1] = it;
+        item[w & 1] = n;
+        mbar_arrive(&full[w & 1]);
+        return true;
+    }
+    // A whole warp: steps of the CTA's w-th item; 0: there are no more; -1: the wait was given up.
+    __device__ __forceinline__ int take_steps(int w, int lane, volatile int* abort_flag, int* it = nullptr) {
+        if (!mbar_wait(&full[w & 1], (w >> 1) & 1, abort_flag)) return -1;
+        const int n = *reinterpret_cast<volatile int*>(&item[w & 1]);
+        if (it != nullptr) *it = *reinterpret_cast<volatile int*>(&number[w & 1]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[w & 1]);
+        return n < 0 ? 0 : n;
+    }
+};
+
 // ------------------------------------------------------------------------------------------ TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
@@ -269,6 +293,12 @@ __device__ __forceinline__ void tma_store_tile(const CUtensorMap* m, const void*
     tma_order_coords(order, t, h, b, c1, c2, c3);
     asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(m),
                  "r"(smem_u32(smem_src)), "r"(d), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+// Untiled load of `bytes` (a multiple of 16) from 16-byte aligned global memory, completion counted in bytes on `bar`.
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(smem_dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
 // 2-D tiled load and store (matrices).
