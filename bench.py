@@ -550,12 +550,18 @@ def run_ours(args):
     stream = torch.cuda.current_stream()
     flops_step = cfg.fwd_flops + cfg.bwd_flops
 
-    # Which route the backward takes for this shape: one kernel (a single key tile), the dQ and the dK/dV kernel, or clear,
-    # main and conversion (see nova_attn_bwd).
+    # Which route the backward takes for this shape: one kernel (a single key tile), the dQ and the dK/dV kernel (at D=64 with the
+    # row terms before them), or clear, main and conversion (see nova_attn_bwd); the last alone sums dQ in the workspace.
     launches_step = kernel_count(functools.partial(step, na, cfg, probe), dev)
     launches_bwd = kernel_count(functools.partial(na.nova_attn_bwd, probe.q, probe.k, probe.v, probe.o, probe.do, probe.lse,
                                                   probe.delta, probe.dq, probe.dk, probe.dv, cfg.scale, cfg.causal,
                                                   probe.ws), dev)
+
+    acc_end = 4 * cfg.B * cfg.H * cfg.T * cfg.D
+    probe.ws.view(torch.uint8)[acc_end - 16:acc_end].fill_(0x5a)
+    na.nova_attn_bwd(probe.q, probe.k, probe.v, probe.o, probe.do, probe.lse, probe.delta, probe.dq, probe.dk, probe.dv, cfg.scale,
+                     cfg.causal, probe.ws)
+    accumulates = bool((probe.ws.view(torch.uint8)[acc_end - 16:acc_end] != 0x5a).any())
 
     sampler = ClockSampler(local_rank)
     sampler.start()
@@ -628,7 +634,7 @@ def run_ours(args):
     #     issue a launch and two event records than these kernels run, so this figure contains idle time.
     # The steps of the backward are separate calls only where nova_attn_bwd itself takes them; its other routes are timed
     # whole.
-    by_steps = launches_bwd == 3
+    by_steps = accumulates
     names = ["fwd", "bwd_preprocess"] + (["bwd_zero", "bwd_main", "bwd_convert"] if by_steps else ["bwd_main"])
 
     def one_kernel(name, s):
@@ -704,7 +710,8 @@ def run_ours(args):
     fwd_tflops = cfg.fwd_flops / (fwd_seq_ms * 1e-3) / 1e12
     bwd_tflops = cfg.bwd_flops / (bwd_seq_ms * 1e-3) / 1e12
     roofline = {
-        "bound": "tensor", "kernel": "attn_dq_kernel + attn_dkdv_kernel" if launches_bwd == 2 else "attn_bwd_kernel",
+        "bound": "tensor", "kernel": ("attn_bwd_kernel" if by_steps or launches_bwd == 1 else
+                                      "attn_dq64_kernel + attn_dkdv64_kernel" if cfg.D == 64 else "attn_dq_kernel + attn_dkdv_kernel"),
         "achieved": achieved, "peak": peak, "unit": UNIT,
         "frac": achieved / peak, "traffic": None, "traffic_source": None,
         "peak_source": f"{peak_src} bf16_tflops (burst)",
