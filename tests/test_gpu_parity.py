@@ -351,6 +351,47 @@ def test_back_to_back_steps_on_shared_buffers():
         assert d <= 1e-2 * r["dQ"].float().abs().max()  # dQ: summation order of the reduce-adds
 
 
+@pytest.mark.parametrize("entry", ["plain", "deterministic"])
+@pytest.mark.parametrize("causal", [True, False])
+def test_back_to_back_two_kernel_backward_on_shared_buffers(entry, causal):
+    """The same where the dQ and the dK/dV kernel of D=64 run (768 tiles): the row terms that the next step puts into the one
+    workspace, its LSE and its Delta must not reach the dK/dV kernel of this one, nor the other way round.  Both kernels sum in
+    a fixed order, so all gradients have the bits of isolated runs."""
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    cfg = W.CONFIGS["gpt2_small"].replace(causal=causal)
+    B, H, T, D = cfg.B, cfg.H, cfg.T, cfg.D
+    assert B * H * ((T + 127) // 128) >= 2.5 * torch.cuda.get_device_properties(dev).multi_processor_count
+    g = torch.Generator(device="cuda").manual_seed(93)
+    dins = [[torch.randn((B, H, T, D), generator=g, device=dev).to(torch.bfloat16) for _ in range(4)] for _ in range(2)]
+    o = torch.empty_like(dins[0][0])
+    lse = torch.empty((B, H, T), dtype=torch.float32, device=dev)
+    delta = torch.empty_like(lse)
+    ws = torch.empty(nova_attn.nova_attn_bwd_workspace_bytes(B, H, T, D), dtype=torch.uint8, device=dev)
+
+    def step(s, grads):
+        q, k, v, do = dins[s]
+        nova_attn.nova_attn_fwd(q, k, v, o, lse, cfg.scale, causal)
+        nova_attn.nova_attn_bwd_preprocess(o, do, delta)
+        if entry == "plain":
+            nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *grads, cfg.scale, causal, ws)
+        else:
+            nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *grads, cfg.scale, causal)
+
+    alone = []
+    for s in range(2):
+        alone.append([torch.full_like(o, 7.0) for _ in range(3)])
+        torch.cuda.synchronize()
+        step(s, alone[s])
+        nova_attn.nova_attn_poll_device_status()
+    runs = [[torch.full_like(o, 7.0) for _ in range(3)] for _ in range(12)]
+    for i, grads in enumerate(runs):
+        step(i & 1, grads)
+    nova_attn.nova_attn_poll_device_status()
+    for i, grads in enumerate(runs):
+        assert all(torch.equal(a, b) for a, b in zip(grads, alone[i & 1])), i
+
+
 FUSED = [  # (B, H, T, D, causal)
     (2, 3, 300, 64, True),      # ragged T: partial tiles with TMA clipping on strided rows
     (2, 12, 1024, 64, True),    # the GPT-2 layout: H*D = 768
