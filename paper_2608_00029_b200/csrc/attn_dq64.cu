@@ -76,7 +76,7 @@ struct Dq64Work {
     }
 };
 
-template <bool kStrided, bool kDelta>
+template <bool kStrided>
 __device__ __forceinline__ void dq64_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
                                               const CUtensorMap* tmdO, uint8_t* smem, Dq64Bars* bars, const Dq64Work& wk) {
     volatile int* abort_flag = &bars->abort_flag;
@@ -87,12 +87,6 @@ __device__ __forceinline__ void dq64_producer(const CUtensorMap* tmQ, const CUte
     for (;;) {
         ok = bars->ring.publish(w, item, abort_flag, kWaitLimitCycles);
         if (!ok || item < 0) break;
-        if (w == 0) {
-            griddep_wait();
-            // The dK/dV kernel, which comes next, needs nothing of dQ and does not wait for it: it may start once what both
-            // read is there, that is now.  Its first items then run on the SMs that have no dQ item left.
-            if (!kDelta) griddep_launch_dependents();
-        }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
         const int head = kStrided ? bh % wk.H : 0, batch = kStrided ? bh / wk.H : 0;
@@ -438,7 +432,6 @@ __device__ __forceinline__ void dq64_edges(uint8_t* smem, Dq64Bars* bars, uint32
         }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
-        if (w == 0) griddep_wait();
         // Rows past the end of the sequence: LSE = +inf gives P = 0 everywhere.
         const int row = qt * kBlockQ + r;
         const size_t idx = static_cast<size_t>(bh) * wk.T + row;
@@ -509,12 +502,13 @@ __device__ __forceinline__ void dq64_body(const CUtensorMap* tmQ, const CUtensor
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
-    if (kDelta) griddep_launch_dependents();
-    // What reads or writes global memory, the producer and the edge warps, waits for the previous kernel of the stream where it
-    // first does; everything before overlaps that kernel.
+    griddep_launch_dependents();
+    // Everything above overlaps the previous kernel of the stream.  All roles wait here: a role that went ahead would wait for
+    // the others on barriers, whose waits are bounded, while the previous kernel may take as long as it likes.
+    griddep_wait();
 
     if (warp == 0) {
-        if (lane == 0) dq64_producer<kStrided, kDelta>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
+        if (lane == 0) dq64_producer<kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
     } else if (warp == 1) {
         dq64_mma_sp<false, kDelta>(smem, bars, tmem_base, wk);
     } else if (warp == 2) {

@@ -1,0 +1,44 @@
+"""Every kernel is launched while its predecessor in the stream may still run, so each has to wait for it by itself: all threads,
+before any role starts.  What a grid reads is promised to be visible only after its own wait; and a role that went ahead would
+wait for the others on barriers, whose waits are bounded, for as long as the predecessor takes."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_00029_b200", "csrc")
+
+
+def _functions(text):
+    """Name, body (without its comments) of every function at the start of a line whose closing brace stands alone in the first column."""
+    for m in re.finditer(r"^(?:template[^\n]*\n)?(?:__device__|__global__)[^{;]*\{\n.*?^\}", text, re.M | re.S):
+        head, body = re.sub(r"//[^\n]*", "", m.group(0)).split("{\n", 1)
+        yield re.findall(r"(\w+)\s*\(", re.sub(r"__launch_bounds__\([^)]*\)|__cluster_dims__\([^)]*\)", "", head))[0], body
+
+
+def _own_level(body):
+    """The statements of a function that stand in no block."""
+    depth, kept = 0, []
+    for line in body.split("\n"):
+        if depth == 0:
+            kept.append(line)
+        depth += line.count("{") - line.count("}")
+    return "\n" + "\n".join(kept)
+
+
+def test_every_kernel_waits_for_its_predecessor_before_its_roles():
+    kernels = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith(".cu"):
+            continue
+        with open(os.path.join(CSRC, name)) as f:
+            functions = list(_functions(f.read()))
+        waits = "|".join(["mbar_wait"] + [fn for fn, body in functions if "mbar_wait(" in body])
+        for fn, body in functions:
+            if "griddep_launch_dependents();" not in body:
+                assert "griddep_" not in body, (name, fn)
+                continue
+            kernels += 1
+            own = _own_level(body).split("\n    griddep_wait();")
+            assert len(own) == 2, (name, fn)
+            ahead = ("\n" + body).split("\n    griddep_wait();")[0]
+            assert not re.search(rf"\b(?:{waits})\s*[(<]", ahead), (name, fn)
+    assert kernels == 16, kernels
