@@ -85,10 +85,11 @@ __device__ __forceinline__ void dq64_producer(const CUtensorMap* tmQ, const CUte
     uint32_t ph = 0;
     int item = blockIdx.x;
     for (;;) {
-        ok = bars->ring.publish(w, item, abort_flag, kWaitLimitCycles);
+        if (w > 0) ok = bars->ring.publish(w, item, abort_flag, kWaitLimitCycles);
         if (!ok || item < 0) break;
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
+        if (w == 0) griddep_wait();
         const int head = kStrided ? bh % wk.H : 0, batch = kStrided ? bh / wk.H : 0;
         const int qs = w & 1;
         ok = mbar_wait(&bars->q_empty[qs], ((w >> 1) & 1) ^ 1, abort_flag);
@@ -152,6 +153,7 @@ __device__ __forceinline__ void dq64_mma_sp(uint8_t* smem, Dq64Bars* bars, uint3
         }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
+        if (w == 0) griddep_wait();
         ok = mbar_wait(&bars->op_full[kdP], w & 1, abort_flag);
         if (!ok) break;
         for (int s = 0; s < n; ++s, ++g) {
@@ -205,6 +207,7 @@ __device__ __forceinline__ void dq64_mma_dq(uint8_t* smem, Dq64Bars* bars, uint3
         }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
+        if (w == 0) griddep_wait();
         // the previous item's dQ must have been read out of TMEM before it is overwritten
         if (w > 0) ok = mbar_wait(&bars->out_free, (w - 1) & 1, abort_flag);
         if (!ok) break;
@@ -259,6 +262,7 @@ __device__ __forceinline__ void dq64_compute(uint8_t* smem, Dq64Bars* bars, uint
         }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
+        if (w == 0) griddep_wait();
         ok = mbar_wait(&bars->rows_full[w & 1], (w >> 1) & 1, abort_flag);
         if (!ok) break;
         const float2 row_terms = reinterpret_cast<const float2*>(smem + kOffRow)[(w & 1) * kBlockQ + r];
@@ -432,6 +436,7 @@ __device__ __forceinline__ void dq64_edges(uint8_t* smem, Dq64Bars* bars, uint32
         }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
+        if (w == 0) griddep_wait();
         // Rows past the end of the sequence: LSE = +inf gives P = 0 everywhere.
         const int row = qt * kBlockQ + r;
         const size_t idx = static_cast<size_t>(bh) * wk.T + row;
@@ -486,6 +491,7 @@ __device__ __forceinline__ void dq64_body(const CUtensorMap* tmQ, const CUtensor
         mbar_init(&bars->stage_free, 1);
         for (int s = 0; s < 3; ++s) mbar_init(&bars->drain[s], 1);
         bars->ring.init((kDelta ? 2 : 3) + 8 + 4);  // issuers, compute warps, edge warps
+        bars->ring.publish_first(blockIdx.x);
         bars->abort_flag = 0;
         fence_mbar_init();
         tma_prefetch_desc(tmQ);
@@ -503,9 +509,10 @@ __device__ __forceinline__ void dq64_body(const CUtensorMap* tmQ, const CUtensor
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
     griddep_launch_dependents();
-    // Everything above overlaps the previous kernel of the stream.  All roles wait here: a role that went ahead would wait for
-    // the others on barriers, whose waits are bounded, while the previous kernel may take as long as it likes.
-    griddep_wait();
+    // Everything above overlaps the previous kernel of the stream, and so does finding out what the first item is: with the wait
+    // here instead, forward, exact Delta and backward of H=148, T=192 took 27.0 us, not 26.2.  Every role waits then, those
+    // that touch no global memory too: they would wait for the others on barriers, whose waits are bounded, while the previous
+    // kernel may take as long as it likes.
 
     if (warp == 0) {
         if (lane == 0) dq64_producer<kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);

@@ -154,6 +154,12 @@ struct WorkRing {
         }
         mbar_init(&answer_bar, 1);
     }
+    // The thread that has initialised the ring announces the CTA's first item, its own index, at once, so that the roles can
+    // take it before they wait for the previous kernel of the stream.
+    __device__ __forceinline__ void publish_first(int it) {
+        item[0] = it;
+        mbar_arrive(&full[0]);
+    }
     // ---- producer (one thread)
     __device__ __forceinline__ bool publish(int w, int it, volatile int* abort_flag, long long limit) {
         if (!mbar_wait(&empty[w & 1], ((w >> 1) & 1) ^ 1, abort_flag, limit)) return false;

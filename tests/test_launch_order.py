@@ -1,6 +1,6 @@
 """Every kernel is launched while its predecessor in the stream may still run, so each has to wait for it by itself: all threads,
-before any role starts.  What a grid reads is promised to be visible only after its own wait; and a role that went ahead would
-wait for the others on barriers, whose waits are bounded, for as long as the predecessor takes."""
+before any of them waits for another.  What a grid reads is promised to be visible only after its own wait; and a role that went
+ahead would wait for the others on barriers, whose waits are bounded, for as long as the predecessor takes."""
 import os
 import re
 
@@ -8,7 +8,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 
 def _functions(text):
-    """Name, body (without its comments) of every function at the start of a line whose closing brace stands alone in the first column."""
+    """Name, body (without its comments) of every function that starts a line and ends with a brace in the first column."""
     for m in re.finditer(r"^(?:template[^\n]*\n)?(?:__device__|__global__)[^{;]*\{\n.*?^\}", text, re.M | re.S):
         head, body = re.sub(r"//[^\n]*", "", m.group(0)).split("{\n", 1)
         yield re.findall(r"(\w+)\s*\(", re.sub(r"__launch_bounds__\([^)]*\)|__cluster_dims__\([^)]*\)", "", head))[0], body
@@ -31,14 +31,24 @@ def test_every_kernel_waits_for_its_predecessor_before_its_roles():
             continue
         with open(os.path.join(CSRC, name)) as f:
             functions = list(_functions(f.read()))
-        waits = "|".join(["mbar_wait"] + [fn for fn, body in functions if "mbar_wait(" in body])
+        roles = {fn: body for fn, body in functions if "mbar_wait(" in body and "griddep_launch_dependents();" not in body}
+        in_roles = [fn for fn, body in roles.items() if "griddep_wait();" in body]
+        # either each role of the file waits once it has its first item, which it does not have to wait for, ...
+        for fn in in_roles:
+            assert sorted(in_roles) == sorted(roles), (name, set(roles) - set(in_roles))
+            loop = re.split(r"\n    for \((?:int w = 0)?; ?\w*;[^\n]*\{\n", roles[fn])[-1]
+            assert not re.search(r"mbar_wait\(", loop.split("        if (w == 0) griddep_wait();\n")[0]), (name, fn)
+            assert loop.count("griddep_wait();") == 1, (name, fn)
+        # ... or the kernel does, before it comes to its roles
         for fn, body in functions:
             if "griddep_launch_dependents();" not in body:
-                assert "griddep_" not in body, (name, fn)
+                assert fn in in_roles or "griddep_" not in body, (name, fn)
                 continue
             kernels += 1
-            own = _own_level(body).split("\n    griddep_wait();")
-            assert len(own) == 2, (name, fn)
+            if in_roles and any(f"{role}<" in body or f"{role}(" in body for role in in_roles):
+                assert "publish_first" in body and "griddep_wait" not in body, (name, fn)
+                continue
+            assert len(_own_level(body).split("\n    griddep_wait();")) == 2, (name, fn)
             ahead = ("\n" + body).split("\n    griddep_wait();")[0]
-            assert not re.search(rf"\b(?:{waits})\s*[(<]", ahead), (name, fn)
+            assert not re.search(r"\b(?:%s)\s*[(<]" % "|".join(["mbar_wait", *roles]), ahead), (name, fn)
     assert kernels == 16, kernels
