@@ -446,10 +446,10 @@ __device__ __forceinline__ void kv64_edges(uint8_t* smem, Kv64Bars* bars, uint32
             const int g = g0 + s, st = g % kQStages;
             RowTerms t[2];
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
+            for (int x = 0; x < 2; ++x) {  // (past L1: there was no griddep_wait)
                 const int q = (s0 + s) * kStep + lane + 32 * x;
-                t[x] = row_terms((q < wk.T) ? -LSE[base + q] * inv_scale : -kMostLse,
-                                 (q < wk.T) ? -Delta[base + q] : 0.f);
+                t[x] = row_terms((q < wk.T) ? -__ldcg(LSE + base + q) * inv_scale : -kMostLse,
+                                 (q < wk.T) ? -__ldcg(Delta + base + q) : 0.f);
             }
             const bool any_odd = __any_sync(0xffffffffu, t[0].odd || t[1].odd);
             if (!mbar_wait(&bars->q_empty[st], ((g / kQStages) & 1) ^ 1, abort_flag)) return false;
@@ -555,7 +555,10 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Kv64Work wk{BH, T, H, orders, kCausal};
 
-    if (threadIdx.x == 0) {
+    // The kernel before this one in the stream is the dQ kernel, of which nothing is needed: it need not have completed (ptx.cuh).
+    // The threads that will read global memory, the producer and the edge warps, see to it while the others set up.
+    if (threadIdx.x == 0 || (!kTerms && warp >= 12)) griddep_taken_over();
+    if (threadIdx.x == 64) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(&bars->kv_full[s], 1);
             mbar_init(&bars->kv_empty[s], 4);
@@ -607,7 +610,6 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
     griddep_launch_dependents();
-    griddep_wait();  // everything above overlaps the previous kernel of the stream
 
     if (warp == 0) {
         if (lane == 0) kv64_producer<kStrided, kTerms>(&tmQ, &tmK, &tmV, &tmdO, terms, smem, bars, wk);
@@ -626,6 +628,7 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
+    griddep_wait();  // what waits for this kernel waits for dQ too
     if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
 }
 

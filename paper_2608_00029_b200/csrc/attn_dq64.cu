@@ -207,7 +207,11 @@ __device__ __forceinline__ void dq64_mma_dq(uint8_t* smem, Dq64Bars* bars, uint3
         }
         int qt, bh, n;
         wk.get(item, &qt, &bh, &n);
-        if (w == 0) griddep_wait();
+        if (w == 0) {
+            griddep_wait();
+            if (el) griddep_launch_dependents();  // the dK/dV kernel, which needs nothing of dQ, but what was there before (ptx.cuh)
+            __syncwarp();
+        }
         // the previous item's dQ must have been read out of TMEM before it is overwritten
         if (w > 0) ok = mbar_wait(&bars->out_free, (w - 1) & 1, abort_flag);
         if (!ok) break;
@@ -508,7 +512,7 @@ __device__ __forceinline__ void dq64_body(const CUtensorMap* tmQ, const CUtensor
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
-    griddep_launch_dependents();
+    if (kDelta) griddep_launch_dependents();
     // Everything above overlaps the previous kernel of the stream, and so does finding out what the first item is: with the wait
     // here instead, forward, exact Delta and backward of H=148, T=192 took 27.0 us, not 26.2.  Every role waits then, those
     // that touch no global memory too: they would wait for the others on barriers, whose waits are bounded, while the previous

@@ -100,7 +100,8 @@ cudaError_t launch_attn_dkdv(const CUtensorMap& tmQ, const CUtensorMap& tmK, con
                              int* dev_status, cudaStream_t stream);
 cudaError_t configure_attn_dkdv();
 // The same at D = 64 (attn_dkdv64.cu).  `terms`: the row terms of every query as launch_row_terms64 leaves them (32 bytes for
-// each of B * H * ceil(T / 64) * 64 rows, 16-byte aligned), or null: the kernel makes them itself (plain layout only).
+// each of B * H * ceil(T / 64) * 64 rows, 16-byte aligned), or null: the kernel makes them itself (plain layout only).  Goes out
+// right after the dQ kernel, whose end it does not wait for (ptx.cuh).
 cudaError_t launch_row_terms64(const float* LSE, const float* Delta, void* terms, const AttnShape& s, cudaStream_t stream);
 cudaError_t launch_attn_dkdv64(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                                const CUtensorMap& tmdO, const CUtensorMap& tmdK, const CUtensorMap& tmdV, bool strided,

@@ -29,9 +29,22 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // that reads or writes global memory may come before it.  griddep_launch_dependents() lets the
 // successor be scheduled as soon as every CTA of this grid has issued it or exited.  Both are no-ops
 // in a kernel launched the ordinary way.
+//
+// One pair of kernels, dQ and dK/dV at D = 64, departs from this: the second needs nothing of the first, so it does not wait for
+// it before it reads, only before it ends (what waits for the second then waits for both).  Why what earlier kernels wrote is
+// there all the same: the first calls griddep_launch_dependents() only after its own griddep_wait(), i.e. when all earlier
+// kernels have completed and their writes have been performed; a CTA of the second runs only after every CTA of the first has
+// done so or has never started, so its reads come later than those writes; and what could answer a read with something older
+// is emptied or passed by: griddep_taken_over() in each thread that reads, before it does (a fence at device scope, and one
+// between generic writes and the asynchronous reads of TMA), and TMA or __ldcg for the reads, past L1.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void griddep_taken_over() {
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
 // ------------------------------------------------------------------------------------------ mbarrier
