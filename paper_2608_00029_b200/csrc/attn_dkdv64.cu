@@ -64,6 +64,8 @@ struct Kv64Bars {
     uint64_t drain[3];
     StepRing ring;
     int odd_rows[kQStages];  // the stage's row terms hold a Delta that is not finite
+    int rows_of[kQStages];   // 1 + the step whose row terms the edge warps have put into the stage last
+    int asked_items, asked_steps, asked_clc;  // what the producer has asked for: loads of items, of steps; answers of the ring
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -130,8 +132,8 @@ __device__ __forceinline__ void kv64_producer(const CUtensorMap* tmQ, const CUte
                                               const CUtensorMap* tmdO, const uint8_t* __restrict__ terms, uint8_t* smem,
                                               Kv64Bars* bars, const Kv64Work& wk) {
     volatile int* abort_flag = &bars->abort_flag;
-    bool ok = true, clc_pending = false;
-    int w = 0, n_kv = 0, g = 0, st = 0;  // items, K and V requested; steps requested
+    bool ok = true;
+    int w = 0, n_kv = 0, n_clc = 0, g = 0, st = 0;  // items; K and V, answers, steps requested
     uint32_t ph = 0;
     int item = blockIdx.x;
     for (;;) {
@@ -170,24 +172,28 @@ __device__ __forceinline__ void kv64_producer(const CUtensorMap* tmQ, const CUte
         if (!ok) break;
         // all loads of this item are on their way: claim the next one now, and no earlier
         bars->ring.request();
-        clc_pending = true;
+        ++n_clc;
         ok = bars->ring.answer(w, &item, abort_flag, kWaitLimitCycles);
         if (!ok) break;
-        clc_pending = false;
         ++w;
     }
-    if (!ok) {  // giving up: let what is in flight land before the CTA's shared memory goes away
-        int none = 0;
-        if (clc_pending) (void)mbar_wait(&bars->ring.answer_bar, w & 1, &none);
-        for (int x = n_kv > 2 ? n_kv - 2 : 0; x < n_kv; ++x) (void)mbar_wait(&bars->kv_full[x & 1], (x >> 1) & 1, &none);
-        for (int x = g > kQStages ? g - kQStages : 0; x < g; ++x) {
-            // the barrier counts the row terms too, which may never come: their share is made up for
-            none = 0;
-            if (mbar_wait(&bars->q_full[x % kQStages], (x / kQStages) & 1, &none, 1 << 16) || kTerms) continue;
-            none = 0;
-            mbar_arrive(&bars->q_full[x % kQStages]);
-            (void)mbar_wait(&bars->q_full[x % kQStages], (x / kQStages) & 1, &none);
-        }
+    bars->asked_items = n_kv;
+    bars->asked_steps = g;
+    bars->asked_clc = n_clc;
+}
+
+// After a wait has run out: what is in flight lands before the CTA's shared memory goes away.  One thread, once every role has
+// left: a stage's barrier counts the row terms of the edge warps too, and only then it is known which of them will not come.
+template <bool kTerms>
+__device__ __noinline__ void kv64_drain(Kv64Bars* bars) {
+    int none = 0;
+    const int n_clc = bars->asked_clc, n_kv = bars->asked_items, n_steps = bars->asked_steps;
+    if (n_clc > 0) (void)mbar_wait(&bars->ring.answer_bar, (n_clc - 1) & 1, &none);
+    for (int x = n_kv > 2 ? n_kv - 2 : 0; x < n_kv; ++x) (void)mbar_wait(&bars->kv_full[x & 1], (x >> 1) & 1, &none);
+    for (int x = n_steps > kQStages ? n_steps - kQStages : 0; x < n_steps; ++x) {
+        const int st = x % kQStages;
+        if (!kTerms && *reinterpret_cast<volatile int*>(&bars->rows_of[st]) <= x) mbar_arrive(&bars->q_full[st]);
+        (void)mbar_wait(&bars->q_full[st], (x / kQStages) & 1, &none);
     }
 }
 
@@ -465,7 +471,10 @@ __device__ __forceinline__ void kv64_edges(uint8_t* smem, Kv64Bars* bars, uint32
             }
             fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&bars->q_full[st]);
+            if (lane == 0) {
+                *reinterpret_cast<volatile int*>(&bars->rows_of[st]) = g + 1;
+                mbar_arrive(&bars->q_full[st]);
+            }
         }
         return true;
     };
@@ -574,6 +583,7 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             mbar_init(&bars->q_full[s], kTerms ? 1 : 2);  // the producer, and the edge warp that writes the row terms
             mbar_init(&bars->q_empty[s], 1);
             bars->odd_rows[s] = 0;
+            bars->rows_of[s] = 0;
         }
         mbar_init(&bars->dkv_full, 1);
         mbar_init(&bars->dkv_free, 4);
@@ -628,6 +638,7 @@ attn_dkdv64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
+    if (threadIdx.x == 0 && bars->abort_flag != 0) kv64_drain<kTerms>(bars);
     griddep_wait();  // what waits for this kernel waits for dQ too
     if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
 }
