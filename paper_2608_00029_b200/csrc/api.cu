@@ -363,6 +363,27 @@ int nova_attn_bwd_preprocess(const void* O, const void* dO, float* Delta, int B,
     return nova_attn_bwd_preprocess_strided(O, dO, Delta, B, H, T, D, &n, &n, stream);
 }
 
+}  // extern "C"
+
+namespace {
+// Does the exact Delta at D=64 take the kernel with its operands in tensor memory (attn_dq64.cu) or the one that multiplies out of
+// shared memory, a pair of query tiles or a single one at a time (attn_dq.cu)?  Both give the same bits.  The first has more
+// hands to pass an item through: with one tile a head and not more than one item per SM (three with at most 64 rows) the second
+// answers sooner, but for a few items of more than 64 rows (forward, exact Delta and backward: H=148, T=64 18.4, 17.4 us, H=148,
+// T=100 20.3, 19.1; but H=444, T=100 32.9, 33.5, H=4, T=100 14.4, 14.6).  Pairs load K and V once for two tiles, which shows
+// where the card is at its power limit, without the mask from 24 tiles per SM on (Delta alone: H=518, T=1024 240, 226 us,
+// H=370, T=2048 660, 610; but H=148, T=2048 196, 203), and where the second tile has a few rows (H=2960, T=129, causal 68.4,
+// 58.4 us, H=2960, T=192 76.1, 69.5; but H=592, T=192 16.0, 16.9).
+bool delta64_pays(long long BH, int T, bool causal, int num_sms) {
+    const long long tiles = BH * ((T + kBlockQ - 1) / kBlockQ);
+    if (T <= 64) return tiles > 3ll * num_sms;
+    if (T <= kBlockQ) return tiles > num_sms || tiles * 4 < num_sms;
+    return causal ? T > 192 || tiles <= 12ll * num_sms : tiles <= 24ll * num_sms;
+}
+}  // namespace
+
+extern "C" {
+
 int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, const void* dO, const float* LSE,
                                    float* Delta, int B, int H, int T, int D, float scale, int causal, void* stream) {
     if (!Q || !K || !V || !dO || !LSE || !Delta) return NOVA_ATTN_ERR_NULL;
@@ -381,8 +402,9 @@ int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, 
     const AttnShape s{B, H, T, D, causal != 0, scale};
     const cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const cudaError_t e =
-        D == 128 ? launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status, cs)
-                 : launch_attn_delta64(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->dev_status, cs);
+        D == 64 && delta64_pays(BH, T, causal != 0, st->num_sms)
+            ? launch_attn_delta64(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->dev_status, cs)
+            : launch_attn_delta(tmQ, tmK, tmV, tmdO, LSE, Delta, s, st->num_sms, st->dev_status, cs);
     return e == cudaSuccess ? NOVA_ATTN_OK : fail_cuda(e);
 }
 
@@ -483,7 +505,8 @@ int bwd_impl(const void* Q, const void* K, const void* V, const void* dO, const 
     const bool whole = steps == (NOVA_ATTN_BWD_STEP_ZERO | NOVA_ATTN_BWD_STEP_MAIN | NOVA_ATTN_BWD_STEP_CONVERT);
     const bool direct = T <= kBlockK && whole;
     if (whole && !direct && two_kernels_pay(BH, T, D, causal != 0, st->num_sms))
-        return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv, D == 64 ? workspace : nullptr, *st, cs);
+        return bwd_two_kernels(Q, K, V, dO, LSE, Delta, dQ, dK, dV, s, sq, sk, sv, sdo, sdq, sdk, sdv,
+                               D == 64 ? workspace : nullptr, *st, cs);
     auto clear = [&]() {
         return (steps & NOVA_ATTN_BWD_STEP_ZERO) && !direct ? launch_zero(acc, need, st->num_sms, cs) : cudaSuccess;
     };

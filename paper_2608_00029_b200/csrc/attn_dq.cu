@@ -5,6 +5,7 @@
 //   attn_delta_kernel  Delta_i = sum_j P_ij (dO_i . V_j): the exact softmax-Jacobian row term.  The cheap route to the
 //                      same quantity, rowsum(dO * O), inherits the bf16 rounding of the stored O, which with sharply
 //                      peaked rows (|O| ~ |V|) is the largest term in dQ and dK.
+// dQ at D=128 only, the exact Delta there and, in the smallest and the largest problems, at D=64 (elsewhere: attn_dq64.cu).
 // Both form S = Q K_j^T and dP = dO V_j^T tile by tile and differ in what becomes of the tile, so they are two builds of
 // one kernel.
 //
@@ -32,22 +33,21 @@
 namespace nova {
 namespace {
 
-constexpr int D = 128;  // (64: attn_dq64.cu)
 constexpr int kThreads = 384;
 constexpr int kTmemCols = 512;
 constexpr int kStep = kKeyStep;                  // keys per step
 constexpr int kHalfStepBytes = kStep * 128;      // one [64 keys x 64 bf16] box
 
 // kTiles: query tiles of a work item (see plan_of).
-template <int kTiles>
+template <int D, int kTiles>
 struct DqCfg {
     static constexpr int kBlockRows = kTiles * kBlockQ;   // query rows per work item
     static constexpr int kWorkConsumers = kTiles * 5;     // an issuer and four row warps per tile
     static constexpr int kHalves = D / kBoxCols;
     static constexpr int kTileBytes = kHalves * kHalfTileBytes;
     static constexpr int kStepBytes = kHalves * kHalfStepBytes;
-    static constexpr int kQStages = kTiles == 1 ? 2 : 1;  // Q and dO of an item
-    static constexpr int kKVStages = 3;
+    static constexpr int kQStages = (D == 64 || kTiles == 1) ? 2 : 1;  // Q and dO of an item
+    static constexpr int kKVStages = (D == 64) ? 5 : 3;
     static constexpr int kOffQ = 0;                                     // [kQStages][kTiles] of Q, then of dO
     static constexpr int kOffdO = kQStages * kTiles * kTileBytes;
     static constexpr int kOffK = 2 * kOffdO;                            // [kKVStages] of K, then of V
@@ -65,7 +65,7 @@ struct DqCfg {
 
 struct DqBars {
     uint64_t q_full[2][2], q_empty[2][2];  // [stage][tile]
-    uint64_t kv_full[3], kv_empty[3];
+    uint64_t kv_full[5], kv_empty[5];
     uint64_t sp_full[2][2], sp_free[2][2];  // [buffer][tile]; the second buffer is used by the Delta build only
     // Two ds_ready per tile, used in turn: where dS has columns of its own the row warps may finish step j + 1 before the
     // issuer has seen step j, and a single barrier two phases on looks as if it had not moved.
@@ -78,26 +78,32 @@ struct DqBars {
 };
 static_assert(sizeof(DqBars) <= 512, "barrier block");
 
-// Work items: blocks of kTiles query tiles, heaviest first (the last block of a causal problem sees every key).  Within
+// Work items: blocks of kTiles query tiles, heaviest first (the last block of a causal problem sees every key).  D=128: within
 // chunks of heads whose tensors stay in L2 together (the exact Delta at B=16, H=32, T=1024 175 -> 157 us, the
-// deterministic backward 650 -> 627 us).
-template <int kTiles>
+// deterministic backward 650 -> 627 us); at D=64 a head's K and V are half as large and the longer arithmetic costs
+// 1 % where there is nothing to gain.
+template <int D, int kTiles>
 struct DqWork {
     int BH, n_blocks, chunk, T, H;
     uint32_t orders;  // coordinate orders of the Q, K, V, dO, dQ tensor maps, four bits each
     bool causal;
     // Block index, head, and the number of key steps each tile visits (0: the tile lies past the end of the sequence).
     __device__ __forceinline__ void get(int idx, int* blk, int* bh, int* n_a, int* n_b) const {
-        int first = 0, in = idx, heads = BH;  // first head of the chunk, item within it, its heads
-        if (chunk < BH) {
-            const int per_chunk = chunk * n_blocks, ck = idx / per_chunk;
-            first = ck * chunk;
-            in = idx - ck * per_chunk;
-            heads = min(chunk, BH - first);
+        if constexpr (D == 128) {
+            int first = 0, in = idx, heads = BH;  // first head of the chunk, item within it, its heads
+            if (chunk < BH) {
+                const int per_chunk = chunk * n_blocks, ck = idx / per_chunk;
+                first = ck * chunk;
+                in = idx - ck * per_chunk;
+                heads = min(chunk, BH - first);
+            }
+            const int order = in / heads;
+            *blk = n_blocks - 1 - order;
+            *bh = first + in - order * heads;
+        } else {
+            *blk = n_blocks - 1 - idx / BH;
+            *bh = idx % BH;
         }
-        const int order = in / heads;
-        *blk = n_blocks - 1 - order;
-        *bh = first + in - order * heads;
         const int n_all = (T + kStep - 1) / kStep;
         const int qt_a = kTiles * (*blk), qt_b = qt_a + 1;
         *n_a = causal ? min((qt_a + 1) * (kBlockQ / kStep), n_all) : n_all;
@@ -105,10 +111,10 @@ struct DqWork {
     }
 };
 
-template <int kTiles, bool kStrided>
+template <int D, int kTiles, bool kStrided>
 __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
-                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork<kTiles>& wk) {
-    using Cfg = DqCfg<kTiles>;
+                                            const CUtensorMap* tmdO, uint8_t* smem, DqBars* bars, const DqWork<D, kTiles>& wk) {
+    using Cfg = DqCfg<D, kTiles>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr long long limit = kWaitLimitCycles;
     int armed_q[2][2] = {{-1, -1}, {-1, -1}}, armed_kv[Cfg::kKVStages];
@@ -185,9 +191,9 @@ __device__ __forceinline__ void dq_producer(const CUtensorMap* tmQ, const CUtens
 }
 
 // The issuer of query tile t: the whole warp in uniform control flow, one elected lane issues.
-template <int kTiles, bool kDelta>
-__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork<kTiles>& wk, int t) {
-    using Cfg = DqCfg<kTiles>;
+template <int D, int kTiles, bool kDelta>
+__device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const DqWork<D, kTiles>& wk, int t) {
+    using Cfg = DqCfg<D, kTiles>;
     volatile int* abort_flag = &bars->abort_flag;
     constexpr uint32_t kIdescT = umma_idesc_bf16(128, kStep, 0, 0);  // S, dP
     constexpr uint32_t kIdescdQ = umma_idesc_bf16(128, D, 0, 1);     // dQ: A from TMEM, B (K) MN-major
@@ -339,12 +345,12 @@ __device__ __forceinline__ void dq_mma(uint8_t* smem, DqBars* bars, uint32_t tme
 }
 
 // The row warps of query tile t.
-template <int kTiles, bool kCausal, bool kStrided, bool kDelta>
+template <int D, int kTiles, bool kCausal, bool kStrided, bool kDelta>
 __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tmem_base, const CUtensorMap* tmdQ,
                                         const float* __restrict__ LSE, const float* __restrict__ Delta,
-                                        float* __restrict__ Delta_out, float scale, const DqWork<kTiles>& wk, int t, int rwarp,
+                                        float* __restrict__ Delta_out, float scale, const DqWork<D, kTiles>& wk, int t, int rwarp,
                                         int lane) {
-    using Cfg = DqCfg<kTiles>;
+    using Cfg = DqCfg<D, kTiles>;
     volatile int* abort_flag = &bars->abort_flag;
     const uint32_t lane_base = 32u * rwarp;
     const int row_local = lane_base + lane;
@@ -391,6 +397,10 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
         const float ndelta = (!kDelta && row < T) ? -Delta[idx] : 0.f;
         const uint64_t nlse = f32x2_pack(nlse2, nlse2), nd = f32x2_pack(ndelta, ndelta);
         uint64_t acc0 = 0, acc1 = 0;
+        // D=64: steps in turn, as the two groups of the other kernel for this head dimension (attn_dq64.cu) sum them: which of the
+        // two a call takes depends on the number of heads, the bits of a head do not.
+        constexpr bool kInTurn = (D == 64);
+        uint64_t next0 = 0, next1 = 0;
 
         for (int j = 0; j < n_t; ++j, ++cnt) {
             const int buf = kDelta ? (cnt & 1) : 0;
@@ -434,6 +444,11 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
                     ds[i / 2 + 1] = pack_bf16x2(x2, x3);
                 }
             }
+            if constexpr (kDelta && kInTurn) {
+                const uint64_t a0 = acc0, a1 = acc1;
+                acc0 = next0, acc1 = next1;
+                next0 = a0, next1 = a1;
+            }
             if constexpr (!kDelta) {
                 // Single tiles: the dQ product of two steps ago, which read this buffer, was queued before S of this step, and
                 // the tensor pipe completes in order.
@@ -457,7 +472,13 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
             float a0, a1, a2, a3;
             f32x2_unpack(acc0, a0, a1);
             f32x2_unpack(acc1, a2, a3);
-            if (row < T) Delta_out[idx] = (a0 + a1) + (a2 + a3);
+            float sum = (a0 + a1) + (a2 + a3);
+            if constexpr (kInTurn) {
+                f32x2_unpack(next0, a0, a1);
+                f32x2_unpack(next1, a2, a3);
+                sum += (a0 + a1) + (a2 + a3);
+            }
+            if (row < T) Delta_out[idx] = sum;
             __syncwarp();
         } else {
             // ---- end of the item: scale * dQ_t as bf16 into this tile's Q buffer (no longer read: the last dQ product
@@ -516,12 +537,12 @@ __device__ __forceinline__ void dq_rows(uint8_t* smem, DqBars* bars, uint32_t tm
 }
 
 // Set-up and roles, shared by the two builds below.
-template <int kTiles, bool kCausal, bool kStrided, bool kDelta>
+template <int D, int kTiles, bool kCausal, bool kStrided, bool kDelta>
 __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMap* tmK, const CUtensorMap* tmV,
                                         const CUtensorMap* tmdO, const CUtensorMap* tmdQ, const float* __restrict__ LSE,
-                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork<kTiles>& wk,
+                                        const float* __restrict__ Delta, float* __restrict__ Delta_out, const DqWork<D, kTiles>& wk,
                                         float scale, int* __restrict__ dev_status) {
-    using Cfg = DqCfg<kTiles>;
+    using Cfg = DqCfg<D, kTiles>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     DqBars* bars = reinterpret_cast<DqBars*>(smem + Cfg::kOffBar);
@@ -566,12 +587,12 @@ __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMa
     griddep_wait();  // everything above overlaps the previous kernel of the stream
 
     if (warp == 0) {
-        if (lane == 0) dq_producer<kTiles, kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
+        if (lane == 0) dq_producer<D, kTiles, kStrided>(tmQ, tmK, tmV, tmdO, smem, bars, wk);
     } else if (warp == 1 || (kTiles == 2 && warp == 3)) {
-        dq_mma<kTiles, kDelta>(smem, bars, tmem_base, wk, warp >> 1);
+        dq_mma<D, kTiles, kDelta>(smem, bars, tmem_base, wk, warp >> 1);
     } else if (warp >= 4 && warp < 4 + 4 * kTiles) {
-        dq_rows<kTiles, kCausal, kStrided, kDelta>(smem, bars, tmem_base, tmdQ, LSE, Delta, Delta_out, scale, wk,
-                                              (warp - 4) >> 2, warp & 3, lane);
+        dq_rows<D, kTiles, kCausal, kStrided, kDelta>(smem, bars, tmem_base, tmdQ, LSE, Delta, Delta_out, scale, wk,
+                                                      (warp - 4) >> 2, warp & 3, lane);
     }
 
     tc_fence_before();
@@ -580,24 +601,24 @@ __device__ __forceinline__ void dq_body(const CUtensorMap* tmQ, const CUtensorMa
     if (threadIdx.x == 0 && bars->abort_flag != 0) atomicExch(dev_status, kDevTimeout);
 }
 
-template <int kTiles, bool kCausal, bool kStrided>
+template <int D, int kTiles, bool kCausal, bool kStrided>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                const __grid_constant__ CUtensorMap tmdQ, const float* __restrict__ LSE, const float* __restrict__ Delta,
                int T, int BH, int H, uint32_t orders, int n_blocks, int chunk, float scale, int* __restrict__ dev_status) {
-    dq_body<kTiles, kCausal, kStrided, false>(&tmQ, &tmK, &tmV, &tmdO, &tmdQ, LSE, Delta, nullptr,
-                                                 DqWork<kTiles>{BH, n_blocks, chunk, T, H, orders, kCausal}, scale, dev_status);
+    dq_body<D, kTiles, kCausal, kStrided, false>(&tmQ, &tmK, &tmV, &tmdO, &tmdQ, LSE, Delta, nullptr,
+                                                 DqWork<D, kTiles>{BH, n_blocks, chunk, T, H, orders, kCausal}, scale, dev_status);
 }
 
-template <int kTiles, bool kCausal>
+template <int D, int kTiles, bool kCausal>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_delta_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                   const float* __restrict__ LSE, float* __restrict__ Delta, int T, int BH, int n_blocks, int chunk, float scale,
                   int* __restrict__ dev_status) {
-    dq_body<kTiles, kCausal, false, true>(&tmQ, &tmK, &tmV, &tmdO, nullptr, LSE, nullptr, Delta,
-                                             DqWork<kTiles>{BH, n_blocks, chunk, T, 1, 0u, kCausal}, scale, dev_status);
+    dq_body<D, kTiles, kCausal, false, true>(&tmQ, &tmK, &tmV, &tmdO, nullptr, LSE, nullptr, Delta,
+                                             DqWork<D, kTiles>{BH, n_blocks, chunk, T, 1, 0u, kCausal}, scale, dev_status);
 }
 
 // Key steps after which the last SM is done.  Every item costs two besides its own.
@@ -615,7 +636,7 @@ long long span_of(const AttnShape& s, int tiles, int n_blocks, int num_sms) {
 // it; a tile alone takes a step in 0.6 of a pair's time, so it wins where the longest chain or the last round of items
 // decides.  The weights 5:8 are fitted to both forms' times over 688 shapes (T = 129 to 8192, 40 to 1200 tiles, with and
 // without the mask, both head dimensions): the slower form is taken at a mean cost of 0.3 %.  Pairs against single tiles,
-// exact Delta: H=8, T=4096: 69.4, 41.8 us.
+// exact Delta: H=8, T=4096: 69.4, 41.8 us.  (What comes here at D=64 is either one tile a head or many pairs.)
 struct Plan {
     int tiles, n_blocks, chunk;
     dim3 grid;  // one CTA per item; those that do not start at once are taken over by those that did
@@ -634,27 +655,32 @@ Plan plan_of(const AttnShape& s, int num_sms) {
     return p;
 }
 
-// Calls f with the tiles of an item and the mask as compile-time constants.
+// Calls f with the head dimension, the tiles of an item and the mask as compile-time constants.
 template <typename F>
-cudaError_t dispatch(int tiles, bool causal, F&& f) {
-    auto with_tiles = [&](auto t) { return causal ? f(t, std::true_type{}) : f(t, std::false_type{}); };
-    return tiles == 1 ? with_tiles(std::integral_constant<int, 1>{}) : with_tiles(std::integral_constant<int, 2>{});
+cudaError_t dispatch(int D, int tiles, bool causal, F&& f) {
+    auto with_d = [&](auto d) {
+        auto with_tiles = [&](auto t) { return causal ? f(d, t, std::true_type{}) : f(d, t, std::false_type{}); };
+        return tiles == 1 ? with_tiles(std::integral_constant<int, 1>{}) : with_tiles(std::integral_constant<int, 2>{});
+    };
+    return D == 64 ? with_d(std::integral_constant<int, 64>{}) : with_d(std::integral_constant<int, 128>{});
 }
 
 }  // namespace
 
 cudaError_t configure_attn_dq() {
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 4 && e == cudaSuccess; ++k)
-        e = dispatch(k & 1 ? 1 : 2, (k & 2) != 0, [](auto t, auto causal) {
-            constexpr int kTiles = decltype(t)::value;
+    for (int k = 0; k < 8 && e == cudaSuccess; ++k)
+        e = dispatch(k & 1 ? 64 : 128, k & 2 ? 1 : 2, (k & 4) != 0, [](auto d, auto t, auto causal) {
+            constexpr int D = decltype(d)::value, kTiles = decltype(t)::value;
             constexpr bool kCausal = decltype(causal)::value;
             auto set = [](auto kernel) {
-                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<kTiles>::kSmemBytes);
+                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<D, kTiles>::kSmemBytes);
             };
-            cudaError_t r = set(attn_dq_kernel<kTiles, kCausal, false>);
-            if (r == cudaSuccess) r = set(attn_dq_kernel<kTiles, kCausal, true>);
-            if (r == cudaSuccess) r = set(attn_delta_kernel<kTiles, kCausal>);
+            cudaError_t r = set(attn_delta_kernel<D, kTiles, kCausal>);
+            if constexpr (D == 128) {
+                if (r == cudaSuccess) r = set(attn_dq_kernel<D, kTiles, kCausal, false>);
+                if (r == cudaSuccess) r = set(attn_dq_kernel<D, kTiles, kCausal, true>);
+            }
             return r;
         });
     return e;
@@ -665,15 +691,19 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
                            const float* LSE, const float* Delta, const AttnShape& s, int num_sms, int* dev_status,
                            cudaStream_t stream) {
     const Plan p = plan_of(s, num_sms);
-    return dispatch(p.tiles, s.causal, [&](auto t, auto causal) {
-        constexpr int kTiles = decltype(t)::value;
+    return dispatch(s.D, p.tiles, s.causal, [&](auto d, auto t, auto causal) {
+        constexpr int D = decltype(d)::value, kTiles = decltype(t)::value;
         constexpr bool kCausal = decltype(causal)::value;
-        auto go = [&](auto kernel) {
-            return launch_overlapped(kernel, p.grid, dim3(kThreads), DqCfg<kTiles>::kSmemBytes, stream, tmQ, tmK, tmV,
-                                     tmdO, tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, p.n_blocks, p.chunk, s.scale,
-                                     dev_status);
-        };
-        return strided ? go(attn_dq_kernel<kTiles, kCausal, true>) : go(attn_dq_kernel<kTiles, kCausal, false>);
+        if constexpr (D == 64) {
+            return cudaErrorNotSupported;  // (attn_dq64.cu)
+        } else {
+            auto go = [&](auto kernel) {
+                return launch_overlapped(kernel, p.grid, dim3(kThreads), DqCfg<D, kTiles>::kSmemBytes, stream, tmQ, tmK, tmV,
+                                         tmdO, tmdQ, LSE, Delta, s.T, s.B * s.H, s.H, orders, p.n_blocks, p.chunk, s.scale,
+                                         dev_status);
+            };
+            return strided ? go(attn_dq_kernel<D, kTiles, kCausal, true>) : go(attn_dq_kernel<D, kTiles, kCausal, false>);
+        }
     });
 }
 
@@ -681,10 +711,10 @@ cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, co
                               const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s,
                               int num_sms, int* dev_status, cudaStream_t stream) {
     const Plan p = plan_of(s, num_sms);
-    return dispatch(p.tiles, s.causal, [&](auto t, auto causal) {
-        constexpr int kTiles = decltype(t)::value;
+    return dispatch(s.D, p.tiles, s.causal, [&](auto d, auto t, auto causal) {
+        constexpr int D = decltype(d)::value, kTiles = decltype(t)::value;
         constexpr bool kCausal = decltype(causal)::value;
-        return launch_overlapped(attn_delta_kernel<kTiles, kCausal>, p.grid, dim3(kThreads), DqCfg<kTiles>::kSmemBytes,
+        return launch_overlapped(attn_delta_kernel<D, kTiles, kCausal>, p.grid, dim3(kThreads), DqCfg<D, kTiles>::kSmemBytes,
                                  stream, tmQ, tmK, tmV, tmdO, LSE, Delta, s.T, s.B * s.H, p.n_blocks, p.chunk, s.scale,
                                  dev_status);
     });

@@ -387,6 +387,7 @@ __device__ __forceinline__ void dq64_edges(uint8_t* smem, Dq64Bars* bars, uint32
     auto write_out = [&](int w, int qt, int bh) -> bool {
         if (!mbar_wait(&bars->out_full[w & 1], (w >> 1) & 1, abort_flag)) return false;
         if constexpr (kDelta) {
+            // even steps, odd steps: the order in which attn_dq.cu sums them at D=64, too
             const float* sum = reinterpret_cast<const float*>(smem + kOffSum) + (w & 1) * 2 * kBlockQ;
             const int row = qt * kBlockQ + r;
             if (row < wk.T) Delta_out[static_cast<size_t>(bh) * wk.T + row] = sum[r] + sum[kBlockQ + r];

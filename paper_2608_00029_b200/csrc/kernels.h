@@ -69,7 +69,7 @@ cudaError_t launch_attn_bwd_preprocess(const __nv_bfloat16* O, const __nv_bfloat
                                        const AttnShape& s, const TensorStrides& so, const TensorStrides& sdo,
                                        int num_sms, cudaStream_t stream);
 
-// The query-major passes of the backward at D = 128 (attn_dq.cu): K and V maps with boxes of kKeyStep rows.
+// The query-major passes of the backward (attn_dq.cu; dQ at D = 128 only): K and V maps with boxes of kKeyStep rows.
 constexpr int kKeyStep = 64;
 // Exact Delta_i = sum_j P_ij (dO_i . V_j) with P rebuilt from LSE (two contractions + exp2 per tile).
 cudaError_t launch_attn_delta(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
@@ -83,7 +83,7 @@ cudaError_t launch_attn_dq(const CUtensorMap& tmQ, const CUtensorMap& tmK, const
                            const float* LSE, const float* Delta, const AttnShape& s, int num_sms, int* dev_status,
                            cudaStream_t stream);
 cudaError_t configure_attn_dq();
-// The same two at D = 64 (attn_dq64.cu).
+// The same two at D = 64, with their operands in tensor memory (attn_dq64.cu).  The same bits of Delta.
 cudaError_t launch_attn_delta64(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                                 const CUtensorMap& tmdO, const float* LSE, float* Delta, const AttnShape& s, int* dev_status,
                                 cudaStream_t stream);

@@ -564,6 +564,27 @@ def test_exact_delta_of_short_sequences(T, causal):
     assert (first.double().cpu() - want).abs().max() <= 1e-4 * max(1.0, float((do @ v.T).abs().max()))
 
 
+@pytest.mark.parametrize("T,causal", [(1, True), (64, False), (65, True), (128, False), (129, True), (192, True), (193, False),
+                                      (700, False), (1025, False)])
+def test_bits_of_exact_delta_do_not_depend_on_the_number_of_heads(T, causal):
+    """At D=64 two kernels compute it, by the number of tiles per SM: a head alone, in a crowd, in a large one."""
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device="cuda").manual_seed(T)
+    one = [torch.randn((1, 1, T, 64), generator=g, device=dev).to(torch.bfloat16) for _ in range(4)]
+    lse1, first = torch.empty((1, 1, T), device=dev), None
+    nova_attn.nova_attn_fwd(*one[:3], torch.empty_like(one[0]), lse1, 0.125, causal)
+    tiles = (T + 127) // 128
+    for per_sm in (0, 1, 4, 13, 30):
+        n = max(1, per_sm * 148 // tiles + per_sm)
+        q, k, v, do = (x.expand(1, n, T, 64).contiguous() for x in one)
+        delta = torch.full((1, n, T), 7.0, device=dev)
+        nova_attn.nova_attn_bwd_preprocess_exact(q, k, v, do, lse1.expand(1, n, T).contiguous(), delta, 0.125, causal)
+        nova_attn.nova_attn_poll_device_status()
+        first = delta[0, 0].clone() if first is None else first
+        assert torch.equal(delta, first.expand_as(delta)), n
+
+
 @pytest.mark.parametrize("T", [1, 127, 129, 256, 257, 384, 500])
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("causal", [True, False])
