@@ -425,17 +425,23 @@ namespace {
 // blocks (H=28, T=4096: 763 -> 807 us, H=20: 539 -> 590 us; but H=32: 909 -> 843 us, H=40, T=3584: 827 -> 797 us).
 //
 // At D=64 the two kernels (with their operands in tensor memory, attn_dkdv64.cu) recompute S and dP but need neither the clear nor
-// the conversion (10 us of 74 at B=8, H=12, T=1024).  In small problems both ways are chains of launches, ramps and the longest
-// item and end within 3 % of each other (H=12, T=777: 21 us both; H=48, T=256: 13.2, 14.3 us); from 2.5 tiles of 128 rows per SM
-// on the two kernels are ahead (fused, two: H=96, T=512 27.9, 26.9 us; H=48, T=1024 38.9, 36.6; H=384, T=512 92, 76; H=12,
-// T=4096 95, 88), with two or three tiles a head, where items are short, from twice that (H=192, T=256 22.2, 22.9; H=768 74,
-// 66).  Large unmasked problems sit at the card's power limit, where two contractions more cost what the rest gains
-// (H=192, T=1500 364, 378 us; H=128, T=1500 252, 244).
+// the conversion (10 us of 74 at B=8, H=12, T=1024).  Whole backward, fused against two kernels, a burst of calls after a pause:
+//   In small problems both ways are chains of launches, ramps and the longest item (H=99, T=300 21.8, 22.7 us; H=74, T=512 23.5,
+// 23.8).  From 2.5 tiles of 128 rows per SM on the two kernels are level or ahead (H=123, T=300 25.0, 24.4 us; H=123, T=384 26.6,
+// 27.2; H=46, T=1024 37.9, 36.1; H=346, T=257 69.8, 56.0), with two tiles a head, where items are short, from 5.5 on (H=296,
+// T=256 30.6, 31.8 us; H=407 43.0, 39.6; H=740 73.6, 59.7).
+//   Large problems run at the card's power limit, where two contractions more cost what the rest gains: the sooner, the longer the
+// items are.  In a burst of calls after a pause and, behind the slash, in a stretch of them, causal: H=92, T=8192 (40 tiles per SM)
+// 2407/2463, 2647/2711 us, H=46 (20) 1218/1221, 1211/1259; H=185, T=4096 (40) 1305/1328, 1453/1514, H=92 (20) 674/667,
+// 647/695; H=259, T=2048 (28) 547/522, 528/563, H=185 (20) 392/377, 358/381; H=493, T=1500 (40) 625/616, 612/654, H=247 (20)
+// 312/304, 288/303; H=1110, T=1024 (60) 730/732, 688/735.  Without the mask: H=32, T=8192 (14) 1578/1594, 1631/1706, H=23
+// (10) 1249/1219, 1133/1176; H=247, T=1500 (20) 482/515, 499/558, H=123 (10) 254/243, 238/254.
 bool two_kernels_pay(long long BH, int T, int D, bool causal, int num_sms) {
     if (D == 64) {
         const long long tiles = BH * ((T + 127) / 128);
         if (T <= 128 || tiles * 2 < (T > 256 ? 5ll : 11ll) * num_sms) return false;
-        return causal || tiles <= 14ll * num_sms;
+        if (!causal) return tiles <= (T > 4096 ? 12ll : 14ll) * num_sms;
+        return T <= 1024 || tiles <= (T <= 1536 ? 32ll : 24ll) * num_sms;
     }
     const long long blocks = BH * ((T + 255) / 256);
     if (T > 4096) return false;

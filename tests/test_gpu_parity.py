@@ -754,6 +754,27 @@ def test_narrow_heads_two_kernel_backward(B, H, T, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"narrow T={T}: ", dO=ref["dO_in"])
 
 
+@pytest.mark.parametrize("H,T,causal", [(394, 1500, True), (395, 1500, True), (273, 1600, True), (274, 1600, True),
+                                        (172, 1500, False), (173, 1500, False), (53, 4224, False), (54, 4224, False)])
+def test_narrow_heads_backward_around_the_limits_of_the_two_kernels(H, T, causal):
+    """On either side of 32 and 24 tiles per SM causal, 14 and 12 without the mask (148 SMs): dK and dV of the plain call have the
+    bits of the deterministic one, dQ is as close as the order of its sums allows."""
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device="cuda").manual_seed(H + T)
+    q, k, v, do = (torch.randn((1, H, T, 64), generator=g, device=dev).to(torch.bfloat16) for _ in range(4))
+    o, lse = torch.empty_like(q), torch.empty((1, H, T), device=dev)
+    delta = torch.empty_like(lse)
+    nova_attn.nova_attn_fwd(q, k, v, o, lse, 0.125, causal)
+    nova_attn.nova_attn_bwd_preprocess(o, do, delta)
+    plain, alike = ([torch.full_like(q, 7.0) for _ in range(3)] for _ in range(2))
+    nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *plain, 0.125, causal)
+    nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *alike, 0.125, causal)
+    nova_attn.nova_attn_poll_device_status()
+    assert torch.equal(plain[1], alike[1]) and torch.equal(plain[2], alike[2])
+    assert (plain[0].float() - alike[0].float()).abs().max() <= 1e-2 * alike[0].float().abs().max()
+
+
 # One of each backward kernel: the fused one (single key tile, several), with more heads than SMs, and at D=128 the pair of
 # kernels (which the deterministic entry point takes at every T > 128).
 NOT_FINITE = [(1, 2, 100, 64), (1, 2, 300, 64), (8, 30, 300, 64), (1, 2, 100, 128), (1, 2, 300, 128), (8, 30, 300, 128)]
