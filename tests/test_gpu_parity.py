@@ -754,6 +754,62 @@ def test_narrow_heads_two_kernel_backward(B, H, T, causal):
     h.compare(h.select_heads(got, heads), ref, label=f"narrow T={T}: ", dO=ref["dO_in"])
 
 
+# The same above the number of tiles from which nova_attn_bwd takes the two kernels (148 SMs: 370 tiles, 814 at T <= 256; without
+# the mask up to 2072), with the row terms in the workspace.
+ABOVE_64 = [(40, 30, 130, True), (4, 104, 200, True), (3, 140, 256, False), (3, 50, 383, True), (5, 25, 449, False),
+            (10, 8, 700, True), (6, 8, 1024, False)]
+
+
+@pytest.mark.parametrize("B,H,T,causal", ABOVE_64)
+def test_narrow_heads_two_kernel_backward_through_every_entry_point(B, H, T, causal):
+    """Plain: dK and dV have the bits of the fused kernel's (its steps issued one by one), dQ those of the deterministic entry
+    point, whatever the workspace held.  Strided: the same bits in three rounds of layouts (plain, [B,T,H,D], padded, heads or
+    tokens outermost, a different one for each tensor), nothing written between the rows.  Static scratch, where the problem
+    fits: the same bits right after a call on other inputs."""
+    from paper_2608_00029_b200 import nova_attn
+    dev = torch.device("cuda:0")
+    tiles, sms = B * H * ((T + 127) // 128), torch.cuda.get_device_properties(dev).multi_processor_count
+    assert (2.5 if T > 256 else 5.5) * sms <= tiles and (causal or tiles <= 14 * sms)
+    D, scale = 64, 0.125
+    g = torch.Generator(device="cuda").manual_seed(T)
+    q, k, v, do, do2 = (torch.randn((B, H, T, D), generator=g, device=dev).to(torch.bfloat16) for _ in range(5))
+    o, lse = torch.empty_like(q), torch.empty((B, H, T), device=dev)
+    delta, delta2 = torch.empty_like(lse), torch.empty_like(lse)
+    nova_attn.nova_attn_fwd(q, k, v, o, lse, scale, causal)
+    nova_attn.nova_attn_bwd_preprocess(o, do, delta)
+    nova_attn.nova_attn_bwd_preprocess(o, do2, delta2)
+    ws = torch.empty(nova_attn.nova_attn_bwd_workspace_bytes(B, H, T, D), dtype=torch.uint8, device=dev)
+    fused, alike, plain = ([torch.full_like(q, 7.0) for _ in range(3)] for _ in range(3))
+    for step in (nova_attn.BWD_STEP_ZERO, nova_attn.BWD_STEP_MAIN, nova_attn.BWD_STEP_CONVERT):
+        nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *fused, scale, causal, ws, steps=step)
+    nova_attn.nova_attn_bwd_deterministic(q, k, v, do, lse, delta, *alike, scale, causal)
+    nova_attn.nova_attn_bwd(q, k, v, o, do, lse, delta, *plain, scale, causal, ws.fill_(255))
+    nova_attn.nova_attn_poll_device_status()
+    assert torch.equal(plain[1], fused[1]) and torch.equal(plain[2], fused[2])
+    assert torch.equal(plain[0], alike[0])
+    assert (plain[0].float() - fused[0].float()).abs().max() <= 1e-2 * fused[0].float().abs().max()  # (dQ: order of the reduce-adds)
+
+    rng = np.random.default_rng(T)
+    kinds = ["bhtd", "bthd", "pad_t", "pad_h", "hbtd", "tbhd"]
+    for shift in range(3):
+        views = [_layout_view(x, kinds[(2 * shift + i) % 6], rng, dev)[0] for i, x in enumerate((q, k, v, do))]
+        outs = [_layout_view(torch.full_like(q, 7.0), kinds[(2 * shift + 4 + i) % 6], rng, dev) for i in range(3)]
+        nova_attn.nova_attn_bwd_strided(*views, lse, delta, *(view for view, _ in outs), scale, causal, ws.fill_(255))
+        nova_attn.nova_attn_poll_device_status()
+        for (view, storage), want in zip(outs, plain):
+            assert torch.equal(view, want), shift
+            view.fill_(7.0)  # what is left must be the untouched padding
+            assert bool((storage == 7.0).all()), shift
+
+    if ws.numel() <= nova_attn.nova_attn_static_scratch_bytes():
+        other, static = ([torch.full_like(q, 7.0) for _ in range(3)] for _ in range(2))
+        nova_attn.nova_attn_bwd_static_scratch(q, k, v, o, do2, lse, delta2, *other, scale, causal)
+        nova_attn.nova_attn_bwd_static_scratch(q, k, v, o, do, lse, delta, *static, scale, causal)
+        nova_attn.nova_attn_poll_device_status()
+        assert all(torch.equal(a, b) for a, b in zip(static, plain))
+        assert not torch.equal(other[0], plain[0])
+
+
 @pytest.mark.parametrize("H,T,causal", [(394, 1500, True), (395, 1500, True), (273, 1600, True), (274, 1600, True),
                                         (172, 1500, False), (173, 1500, False), (53, 4224, False), (54, 4224, False)])
 def test_narrow_heads_backward_around_the_limits_of_the_two_kernels(H, T, causal):
