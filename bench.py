@@ -12,10 +12,10 @@ training attention shape (B=8, H=12, T=1024, D=64, causal, bf16).  Prints ONE JS
              HBM, timed with CUDA events on the launching stream, max over ranks.
   e2e        the same metric with the step's inputs copied from pinned host memory and its results
              copied back inside the timed region.
-  roofline   tensor-core roofline of the dominant kernel (the fused backward) against the measured burst
-             bf16 peak, from a second pass that brackets each kernel with events, and the forward and the
-             whole backward (preprocess + clear + main + convert, timed in sequence) against the targets of
-             50 % and 35 % of that peak.
+  roofline   tensor-core roofline of the backward's main part (the fused kernel, or the dQ and the dK/dV kernel
+             with what they launch before them) against the measured burst bf16 peak, from a second pass
+             of back-to-back launches, and the forward and the whole backward (preprocess and all of
+             nova_attn_bwd, timed in sequence) against the targets of 50 % and 35 % of that peak.
   cpu_baseline  the fp64 oracle timed on the host cores on a bounded sample of the same workload.
 
 With N > 1 (launched by torchrun, one rank per GPU) every rank runs the same per-GPU batch on its own
@@ -730,12 +730,13 @@ def run_ours(args):
         "preprocess_frac_of_hbm_peak": (4.0 * cfg.B * cfg.H * cfg.T * cfg.D + 4.0 * cfg.B * cfg.H * cfg.T)
         / (kernel_ms["bwd_preprocess"] * 1e-3) / 1e9 / peaks["hbm_gbs"],
     }
-    # DRAM bytes of one launch of the dominant kernel are not measured by this run: they come from the
-    # committed ncu summary of this workload (its "traffic_bytes_per_launch: N" line); absent or another
+    # DRAM bytes of the backward's main part are not measured by this run: they come from the committed ncu
+    # summary of this workload and route (its "traffic_bytes_per_launch: N" line); absent or another
     # workload -> null.
-    traffic_rel = os.path.join("profiles", f"attn_bwd_kernel_{base.name}.md")
+    traffic_rel = os.path.join("profiles", f"attn_bwd_kernel_{base.name}.md" if by_steps else
+                               f"two_kernel_backward_d{cfg.D}_{base.name}.md")
     traffic_path = os.path.join(ROOT, traffic_rel)
-    if os.path.exists(traffic_path) and cfg.B == base.B and by_steps:
+    if os.path.exists(traffic_path) and cfg.B == base.B and (by_steps or launches_bwd > 1):
         try:
             with open(traffic_path) as f:
                 for line in f:

@@ -95,8 +95,8 @@ int nova_attn_bwd_preprocess_exact(const void* Q, const void* K, const void* V, 
                                    float scale, int causal, void* stream);
 
 /*
- * Bytes of scratch nova_attn_bwd needs: an fp32 accumulator for dQ, [B,H,T,D] (rounded up to
- * 256 bytes).  Returns 0 if the shape is invalid.
+ * Bytes of scratch nova_attn_bwd needs: room for an fp32 accumulator of dQ, [B,H,T,D] (rounded up to
+ * 256 bytes), whether the shape uses it or not.  Returns 0 if the shape is invalid.
  */
 size_t nova_attn_bwd_workspace_bytes(int B, int H, int T, int D);
 
@@ -109,12 +109,16 @@ size_t nova_attn_bwd_workspace_bytes(int B, int H, int T, int D);
  *   LSE, Delta  : in, fp32 [B,H,T] from nova_attn_fwd / nova_attn_bwd_preprocess
  *   dQ, dK, dV  : out, bf16 [B,H,T,D]; gradient of sum(O * dO) with respect to Q, K, V
  *   workspace   : device scratch of at least nova_attn_bwd_workspace_bytes(B,H,T,D) bytes, 16-byte
- *                 aligned; zeroed by the call itself on `stream` where it is used; contents afterwards
- *                 unspecified.
- * dQ is accumulated in fp32 across key tiles with floating-point reduce-adds whose order is not fixed,
- * so its low-order bits may differ from run to run; dK and dV are deterministic.  A final pass scales
- * the accumulator, rounds it once to bf16 and writes dQ.  Where it is faster (a single key tile, T <= 128;
- * most shapes of D = 128 that fill the GPU) dQ is summed in a fixed order without the accumulator.
+ *                 aligned; whatever it holds on entry does not matter; contents afterwards unspecified.
+ * Three routes, by shape:
+ *   - A single key tile, T <= 128: one kernel writes all three gradients; the workspace is not touched.
+ *   - Shapes that fill the GPU, where it is faster (most at D = 128 up to T = 4096, most at D = 64): one kernel
+ *     for dQ, one for dK and dV.  At D = 64 the workspace holds the row terms of the second (32 bytes a row,
+ *     rows of a head rounded up to 64), prepared by a small kernel; at D = 128 it is not touched.
+ *   - Otherwise one kernel that accumulates dQ in the workspace in fp32 across key tiles (zeroed by the call
+ *     itself on `stream`) with floating-point reduce-adds whose order is not fixed, so that its low-order bits
+ *     may differ from run to run; a final pass scales the accumulator, rounds it once to bf16 and writes dQ.
+ * dK and dV are deterministic in all three and do not depend on the route, dQ in the first two.
  */
 int nova_attn_bwd(const void* Q, const void* K, const void* V, const void* O, const void* dO,
                   const float* LSE, const float* Delta, void* dQ, void* dK, void* dV,
@@ -127,8 +131,8 @@ int nova_attn_bwd(const void* Q, const void* K, const void* V, const void* O, co
  *   NOVA_ATTN_BWD_STEP_ZERO     clear the fp32 dQ accumulator in `workspace`
  *   NOVA_ATTN_BWD_STEP_MAIN     the fused backward kernel: writes dK, dV, accumulates unscaled dQ
  *   NOVA_ATTN_BWD_STEP_CONVERT  dQ = bf16(scale * accumulator)
- * All three, in this order, give what nova_attn_bwd gives (which for some shapes uses kernels that write
- * dQ without the accumulator); any other combination leaves sequencing to the caller.  Arguments, validation
+ * All three in one call are nova_attn_bwd, its choice of route included (which for many shapes writes dQ
+ * without the accumulator); any other combination leaves sequencing to the caller.  Arguments, validation
  * and errors are those of nova_attn_bwd.
  */
 #define NOVA_ATTN_BWD_STEP_ZERO 1
@@ -145,8 +149,8 @@ int nova_attn_bwd_steps(const void* Q, const void* K, const void* V, const void*
  * Who needs it: code that runs where cudaMalloc is off limits - inside another framework's fixed
  * memory plan, in a plugin that only ever sees its input and output buffers, or in a loop that must
  * not touch the allocator once it is running.  Such callers cannot provide the `workspace` of
- * nova_attn_bwd.  This variant takes the same inputs and outputs and keeps the fp32 dQ accumulator in
- * a fixed array inside the library instead.
+ * nova_attn_bwd.  This variant takes the same inputs and outputs and keeps the workspace in a fixed
+ * array inside the library instead.
  *
  *   - The array holds nova_attn_static_scratch_bytes() = 32 MiB, i.e. B*H*T*D <= 8 Mi elements (the
  *     GPT-2-small training shape B=8, H=12, T=1024, D=64 fits).  Larger problems are rejected with
@@ -160,9 +164,9 @@ int nova_attn_bwd_steps(const void* Q, const void* K, const void* V, const void*
  *   - The call allocates nothing: no cudaMalloc, no cudaFree, no allocating library routine.
  *   - The first call on a device looks up the array's device address (one runtime query, cached per
  *     device).  Make that first call before starting any stream capture.
- *   - All calls on a device share the one array.  Each call clears the part it uses before use, so
+ *   - All calls on a device share the one array.  Each call clears or writes the part it uses before use, so
  *     what an earlier call left behind is harmless, but two calls whose GPU work overlaps (different
- *     streams, or different host threads) race on it and corrupt each other's dQ.  Serialise them.
+ *     streams, or different host threads) race on it and corrupt each other's dQ, or dK and dV.  Serialise them.
  *   - Arguments, validation, results and error codes are otherwise those of nova_attn_bwd, checked in
  *     the same order: a NULL pointer, a bad shape, alignment or scale is reported as such even when the
  *     problem is also too large for the array.
@@ -178,9 +182,9 @@ int nova_attn_bwd_static_scratch(const void* Q, const void* K, const void* V, co
  * reduces dQ over keys, the other reduces dK and dV over queries; both rebuild the probability matrix from
  * the saved log-sum-exp).  Every output element is summed by one thread block in a fixed order, so dQ, dK
  * and dV are bitwise reproducible from run to run, and no workspace is needed.  The price: the score and
- * dP contractions are computed in both kernels (seven contractions for the five that are counted), which at
- * D = 64 makes it slower than nova_attn_bwd.  Where nova_attn_bwd does without the accumulator (T <= 128, most
- * shapes of D = 128 that fill the GPU) it launches these same kernels.  dK and dV are bit-identical to
+ * dP contractions are computed in both kernels (seven contractions for the five that are counted).  Where
+ * that pays for itself nova_attn_bwd launches these same kernels (see there; at D = 64 with the row terms
+ * prepared in its workspace); elsewhere this entry point is slower.  dK and dV are bit-identical to
  * nova_attn_bwd's, dQ differs from it in the last bits at most (summation order).
  *   Q, K, V, dO : in,  bf16 [B,H,T,D]
  *   LSE, Delta  : in,  fp32 [B,H,T] from nova_attn_fwd / nova_attn_bwd_preprocess(_exact)

@@ -10,9 +10,13 @@
 // K_j and V_j are A operands in tensor memory, put there once per item: a product of M=128, N=64 with both operands in
 // shared memory takes 48 clocks per 16 k elements, 6 KB through the one 128-byte port; with A in tensor memory it takes
 // the 32 clocks of the arithmetic, and leaves three quarters of the port to the other users.
-// What bounds it: a step takes 608 clocks of the tensor pipe (of which the row terms 96), 512 of the exp2 unit and some 800 in
-// all; the rest is the chain dS^T -> dK -> dP^T of a group and the ends of items (1300 clocks each).  dK and dV at B=4,
-// H=12, T=1500: 55 us with the fused kernel without its dQ product, 40 so; B=32, T=1024: 213 with dQ, 127; B=1, T=8192: 283, 185.
+// What bounds it: a step takes 608 clocks of the tensor pipe (of which the row terms 96), 512 of the exp2 unit and some 780 in
+// all, the rest being the chain dS^T -> dK -> dP^T of a group; the end of an item costs 2000 clocks, a launch 10000 besides
+// (fitted to three of the shapes below), so that at T=1024, with nine steps an item, a step comes to 1200 of its SM's clocks.
+// dK and dV under ncu (us), with the fused kernel without its dQ product and so: H=12, B=8, T=1024: 52, 38; B=4, T=1500:
+// 53, 38; B=32, T=1024: 183, 125; B=1, T=8192: 286, 182; B=8, T=512: 22, 18.
+// All 128 registers that 512 threads may have are in use, and 64 bytes of stack besides (56 where the kernel makes the row
+// terms itself; 76 and 68 bytes of spill stores, 156 and 108 of loads in the code).
 // Items are handed out dynamically (WorkRing), heaviest first.  512 threads:
 //   warp 0      TMA producer: K_j and V_j double-buffered, Q_s and dO_s through a ring of 64-query stages
 //   warps 1-3   UMMA issuers of S^T, of dP^T, and of dV and dK

@@ -9,7 +9,9 @@
 // What bounds it: 64 exponentials per thread and step, 1024 clocks of the exp2 unit per 128 x 128 block; the products take
 // 768 with the A operands in tensor memory (1024 with all of them in shared memory, whose port a product of N = 64 then
 // saturates).  S and dP run ahead of the compute groups: the columns of a step are handed back as soon as they have been
-// read.  Items are handed out dynamically (WorkRing), heaviest first.  512 threads:
+// read.  A step takes some 670 clocks, the end of an item 1300, a launch 10000 besides.  Under ncu (us), the pairs of tiles of
+// attn_dq.cu and so: dQ at H=12, B=8, T=1024: 38, 33; B=4, T=1500: 37, 33; B=32, T=1024: 117, 103; B=1, T=8192: 189, 155; exact
+// Delta: 32, 30; 32, 30; 98, 94; 163, 143.  Items are handed out dynamically (WorkRing), heaviest first.  512 threads:
 //   warp 0      TMA producer: Q_i and dO_i double-buffered, K_s and V_s through a ring of 64-key stages
 //   warps 1-3   UMMA issuers of S, dP and dQ (why three: see attn_dkdv64.cu)
 //   warps 4-7   compute group 0, warps 8-11 group 1: a thread has one query row and the 64 keys of its step

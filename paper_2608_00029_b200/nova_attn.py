@@ -146,14 +146,14 @@ def nova_attn_bwd(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: 
 
 
 def nova_attn_static_scratch_bytes() -> int:
-    """Size of the library's built-in dQ accumulator (bytes)."""
+    """Size of the library's built-in workspace (bytes)."""
     return int(load().nova_attn_static_scratch_bytes())
 
 
 def nova_attn_bwd_static_scratch(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: bool = True,
                                  stream=None) -> None:
     """nova_attn_bwd for callers that cannot allocate: no workspace argument, nothing is allocated here
-    or in the library.  The dQ accumulator is a fixed 32 MiB array inside the library, shared by all
+    or in the library.  The workspace is a fixed 32 MiB array inside the library, shared by all
     calls on the device, so B*H*T*D must not exceed 8 Mi elements and calls must not overlap on the
     GPU.  Make the first call on a device before any stream capture."""
     rc = _binding().bwd_static_scratch(Q, K, V, O, dO, LSE, Delta, dQ, dK, dV, scale, causal, stream)
@@ -217,8 +217,8 @@ def nova_attn_bwd_strided(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, cau
 
 def nova_attn_bwd_deterministic(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale: float, causal: bool = True,
                                 stream=None) -> None:
-    """dQ, dK, dV by the two-kernel backward: bitwise reproducible, no workspace.  At D = 64 and T > 128
-    slower than nova_attn_bwd, which elsewhere mostly takes the same kernels."""
+    """dQ, dK, dV by the two-kernel backward: bitwise reproducible, no workspace.  nova_attn_bwd takes the same
+    kernels where they are faster than summing dQ in the workspace, i.e. for most shapes that fill the GPU."""
     rc = _binding().bwd_deterministic(Q, K, V, dO, LSE, Delta, dQ, dK, dV, scale, causal, stream)
     if rc != OK:
         raise NovaAttnError(rc, "nova_attn_bwd_deterministic")

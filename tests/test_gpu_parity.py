@@ -479,9 +479,10 @@ def test_single_key_tile_writes_dq_directly(T, D, causal):
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("causal", [True, False])
 def test_query_major_passes_at_step_edges(T, D, causal):
-    """The deterministic dQ and the exact Delta walk the keys in steps of 64 for pairs of 128-row tiles: sequence lengths
-    around the edges of a step, of a tile and of a pair (a second tile with one row, or none), more items than SMs so
-    that CTAs take over further ones; twelve calls back to back give the same bits every time."""
+    """The deterministic dQ and the exact Delta walk the keys in steps of 64, for pairs of 128-row tiles or (D=64) for one tile
+    in two groups that take turns: sequence lengths around the edges of a step, of a tile and of a pair (a second tile with
+    one row, or none), more items than SMs so that CTAs take over further ones; twelve calls back to back give the same bits
+    every time."""
     from paper_2608_00029_b200 import nova_attn
     h = _harness()
     dev = torch.device("cuda:0")
